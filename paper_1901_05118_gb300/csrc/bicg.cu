@@ -80,6 +80,10 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // kernel of the small grids keeps a separate direction-update phase
     const bool fuse = ctx->schedule == EXCMG_SCHEDULE_FUSED;
     const bool dir_fused = fused && fuse && !persistent;
+    // r*_0 = r_0: with every vector on chip; a caller-chosen r*_0, or no room
+    // for the exchange words: the general cooperative kernel
+    void* words = persistent && shadow == nullptr && resident_fits(n) ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
+    const bool resident = words != nullptr;
     double* p2 = dir_fused ? ctx_buffer(ctx, "bicg_p2", bytes, &st) : nullptr;
     double* ps2 = (dir_fused && !elide && !st) ? ctx_buffer(ctx, "bicg_ps2", bytes, &st) : nullptr;
     if (st) return st;
@@ -118,11 +122,12 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
             if (e != cudaSuccess) return ctx_cuda(ctx, e, "Bi-CG state read");
             if (ctx->host_state->done) break;
-            int chunk = 256;
+            int chunk = resident ? 1024 : 256;
             const int left = max_iter - ctx->host_state->iter;
             if (chunk > left) chunk = left;
-            e = launch_bicg_persistent(x, r, rs, p, ps, q, qs, n, bc_kind, chunk, ctx->partials, ctx->state,
-                                       ctx->barrier, s, elide);
+            e = resident ? launch_bicg_resident<double>(x, r, rs, p, ps, n, bc_kind, chunk, ctx->state, words, s, elide)
+                         : launch_bicg_persistent(x, r, rs, p, ps, q, qs, n, bc_kind, chunk, ctx->partials,
+                                                  ctx->state, ctx->barrier, s, elide);
             note_launches(1);
             if (e != cudaSuccess) return ctx_cuda(ctx, e, "cooperative Bi-CG launch");
         }

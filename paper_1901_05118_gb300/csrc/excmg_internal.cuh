@@ -74,6 +74,14 @@ bool persistent_pointwise(int n);
 cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, double* ps, double* q, double* qs,
                                    int n, int bc_kind, int iters, double* partials, BicgState* st,
                                    unsigned int* barrier_words, cudaStream_t s, bool elide);
+// The same with every vector on chip (resident.cuh), for calls that start
+// from r*_0 = p*_0 = r_0 = p_0.  words: resident_bytes(n) of device memory for
+// the exchanges between CTAs, not shared with a launch that may run at the same time.
+bool resident_fits(int n);
+size_t resident_bytes(int n);
+template <typename T>
+cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
+                                 void* words, cudaStream_t s, bool elide);
 // Shadow-elided mode (r* = r, p* = p, A^T p* = A p not stored): the one-field
 // operator launches with sigma = (p, A p) and alpha (the second also forms
 // p = r + beta p_prev into p), and the matching set-up and update kernels.
@@ -219,6 +227,11 @@ int ctx_cuda(excmg_ctx* ctx, cudaError_t err, const char* what);
 // host_scalar), written by a kernel; the caller synchronises the stream.
 cudaError_t ctx_read_back(excmg_ctx* ctx, void* host_mirror, const void* dev_src, size_t bytes);
 double* ctx_buffer(excmg_ctx* ctx, const char* name, size_t bytes, int* status);
+// At least `bytes` of device memory whose contents a caller may rely on to be
+// its own or zero (the exchange words of resident.cuh): null where the budget
+// or the device has no room.  It is given up first when a buffer needs the room.
+void* ctx_scratch(excmg_ctx* ctx, size_t bytes);
+bool ctx_drop_scratch(excmg_ctx* ctx);   // false: there was none
 // Bi-CG driver (bicg.cu): iterates on the context's stream.
 int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, double tol,
              double bnorm, int max_iter, int check_every, int* iters_out, double* relres_out,

@@ -1,0 +1,71 @@
+// Host side of the resident Bi-CG kernels (resident.cuh).
+#include "excmg_internal.cuh"
+#include "resident.cuh"
+
+#include <atomic>
+#include <map>
+#include <mutex>
+
+namespace excmg {
+namespace {
+
+template <typename T, bool kElide, int NI>
+const void* resident_fn(int np) {
+    switch (np) {
+        case 1: return (const void*)resident_bicg_kernel<T, 1, 2, kElide, NI>;
+        case 2: return (const void*)resident_bicg_kernel<T, 2, 3, kElide, NI>;
+        default: return (const void*)resident_bicg_kernel<T, 4, 5, kElide, NI>;
+    }
+}
+
+std::mutex g_geom_mu;
+std::map<std::pair<int, int>, ResidentGeom> g_geom;   // at most one entry per size and CTA limit
+
+}  // namespace
+
+ResidentGeom resident_geometry_cached(int n, int max_ctas) {
+    std::lock_guard<std::mutex> lock(g_geom_mu);
+    auto it = g_geom.find({n, max_ctas});
+    if (it == g_geom.end()) it = g_geom.emplace(std::make_pair(n, max_ctas), resident_geometry(n, max_ctas)).first;
+    return it->second;
+}
+
+bool resident_fits(int n) { return n <= kPersistentMaxN && resident_geometry_cached(n, device_sms()).ctas > 0; }
+
+namespace {
+size_t slot_bytes() { return (kResWords * sizeof(ulonglong2) + 255) / 256 * 256; }
+
+// The launch's tag: unique in the process, so no word left by another launch matches.
+unsigned next_serial() {
+    static std::atomic<unsigned> serial{0};
+    unsigned v = ++serial;
+    while (v == 0) v = ++serial;
+    return v;
+}
+}  // namespace
+
+size_t resident_bytes(int n) { return slot_bytes() + node_count(n) * sizeof(ulonglong2); }
+
+template <typename T>
+cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
+                                 void* words, cudaStream_t s, bool elide) {
+    ResidentGeom g = resident_geometry_cached(n, device_sms());
+    ResidentTable<T, 1> tab;
+    tab.inst[0] = ResidentInst<T>{x, r, rs, p, ps, st, (ulonglong2*)words, (ulonglong2*)((char*)words + slot_bytes()), n, bc_kind == 1 ? 1 : -1};
+    const size_t smem = (size_t)g.tile * (sizeof(T) == 8 ? sizeof(long long) : sizeof(float));
+    const void* fn;
+    if constexpr (sizeof(T) == 8)
+        fn = elide ? resident_fn<T, true, 1>(g.np) : resident_fn<T, false, 1>(g.np);
+    else
+        fn = resident_fn<T, false, 1>(g.np);
+    (void)kernel_occupancy(fn, kResThreads, smem);   // opts in to the shared memory
+    unsigned serial = next_serial();
+    long long limit = kBarrierSpinLimit;
+    void* args[] = {&tab, &g, &iters, &serial, &limit};
+    return cudaLaunchCooperativeKernel(fn, dim3(g.ctas), dim3(kResThreads), args, smem, s);
+}
+
+template cudaError_t launch_bicg_resident<double>(double*, double*, double*, double*, double*, int, int, int,
+                                                  BicgState*, void*, cudaStream_t, bool);
+
+}  // namespace excmg
