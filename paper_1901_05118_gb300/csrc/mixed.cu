@@ -218,13 +218,25 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
     note_launches(1);
     if (err != cudaSuccess) return ctx_cuda(ctx, err, "FP32 Bi-CG setup");
     if (check_every < 1) check_every = 1;
+    // grids up to 64^3: many iterations per launch with every vector on chip
+    // (48^3: 5 us per iteration, against 25 us for the three launches,
+    // each of them a few microseconds of latency for 0.5 MB vectors); larger
+    // ones, or no room for the exchange words: the launched kernels
+    void* words = resident_fits(n) ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
     for (;;) {
         err = ctx_read_back(ctx, ctx->host_state, ctx->state, sizeof(BicgState));
         if (err == cudaSuccess) err = cudaStreamSynchronize(s);
         if (err != cudaSuccess) return ctx_cuda(ctx, err, "FP32 Bi-CG state read");
         if (ctx->host_state->done) break;
-        int batch = check_every;
         const int left = max_iter - ctx->host_state->iter;
+        if (words) {
+            err = launch_bicg_resident<float>(e, r, rs, p, ps, n, bc_kind, left < 1024 ? left : 1024, ctx->state, words,
+                                              s, false);
+            note_launches(1);
+            if (err != cudaSuccess) return ctx_cuda(ctx, err, "cooperative FP32 Bi-CG launch");
+            continue;
+        }
+        int batch = check_every;
         if (batch > left) batch = left;
         for (int it = 0; it < batch && err == cudaSuccess; ++it) {
             stencil_f32_kernel<2, true><<<g.grid, g.block, 0, s>>>(p, ps, q, qs, n, sigma, g.kz_per_cta,
@@ -240,6 +252,8 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
     if (iters_out) *iters_out = ctx->host_state->iter;
     if (!std::isfinite(ctx->host_state->rr)) return ctx_fail(ctx, EXCMG_ERR_NAN, "FP32 Bi-CG residual is not finite");
     if (ctx->host_state->status == kBreakdown) return ctx_fail(ctx, EXCMG_ERR_BREAKDOWN, "FP32 Bi-CG breakdown");
+    if (ctx->host_state->status == kTimeout)
+        return ctx_fail(ctx, EXCMG_ERR_TIMEOUT, "an exchange of the cooperative FP32 Bi-CG gave up");
     return EXCMG_OK;
 }
 

@@ -58,7 +58,7 @@ cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_k
         fn = elide ? resident_fn<T, true, 1>(g.np) : resident_fn<T, false, 1>(g.np);
     else
         fn = resident_fn<T, false, 1>(g.np);
-    (void)kernel_occupancy(fn, kResThreads, smem);   // opts in to the shared memory
+    (void)kernel_occupancy(fn, kResThreads, kResTileBytes);   // opts in to the shared memory
     unsigned serial = next_serial();
     long long limit = kBarrierSpinLimit;
     void* args[] = {&tab, &g, &iters, &serial, &limit};
@@ -67,5 +67,7 @@ cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_k
 
 template cudaError_t launch_bicg_resident<double>(double*, double*, double*, double*, double*, int, int, int,
                                                   BicgState*, void*, cudaStream_t, bool);
+template cudaError_t launch_bicg_resident<float>(float*, float*, float*, float*, float*, int, int, int, BicgState*,
+                                                 void*, cudaStream_t, bool);
 
 }  // namespace excmg

@@ -34,6 +34,10 @@ struct ResidentGeom {
 // the 4-byte entries of the FP32 kernel share the layout).
 constexpr int kResPad = 16;
 
+// Shared memory for the tile; the kernels are opted in to this much once, as
+// the launches of different grids share them.
+constexpr size_t kResTileBytes = 160 * 1024;
+
 // Nodes around the brick per thread of the variant with np nodes per thread.
 inline int resident_nh(int np) { return np == 1 ? 2 : np == 2 ? 3 : 5; }
 
@@ -113,14 +117,15 @@ inline ResidentGeom resident_geometry(int n, int max_ctas) {
                 for (int np = 1; np <= 4; np *= 2) {
                     const int threads = bx * by * ((bz + np - 1) / np);
                     const int nh = resident_nh(np);
-                    if (threads > kResThreads || halo > nh * kResHaloThreads) continue;
+                    const int runs = (bz + np - 1) / np * np;
+                    const int tile = (bx + kResPad) * (by + 4) * (runs + 4);
+                    if (threads > kResThreads || halo > nh * kResHaloThreads ||
+                        (size_t)tile * 8 > kResTileBytes)
+                        continue;
                     const long long cost = 5LL * np * ((threads + 127) / 128) * 128 + halo + 40LL * cx * cy * cz;
                     if (best_cost < 0 || cost < best_cost) {
                         best_cost = cost;
-                        const int runs = (bz + np - 1) / np * np;
-                        best = ResidentGeom{cx, cy, cz, bx, by, bz, np, nh, halo, bx + kResPad,
-                                            (bx + kResPad) * (by + 4) * (runs + 4),
-                                            cx * cy * cz};
+                        best = ResidentGeom{cx, cy, cz, bx, by, bz, np, nh, halo, bx + kResPad, tile, cx * cy * cz};
                     }
                 }
             }

@@ -1,0 +1,97 @@
+"""The resident Bi-CG kernels (grids up to 64^3, every vector on chip) at the
+edges of their brick decompositions: smallest and largest grids, bricks cut
+short by the boundary, one to four nodes per thread, a call longer than one
+launch, the FP32 correction solves."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1901_05118_gb300 import problems as P
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU machines only
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1901_05118_gb300 import binding as B  # noqa: E402
+
+DEV = torch.device("cuda", 0)
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+
+
+def rel_max(got, ref):
+    return float(np.abs(got - ref).max() / np.abs(ref).max())
+
+
+@pytest.mark.parametrize("n,bc_kind,iters", [(4, 1, 9), (5, 2, 12), (9, 1, 20), (14, 2, 20), (23, 1, 20), (33, 2, 20),
+                                             (41, 1, 20), (47, 2, 20), (53, 1, 20), (58, 2, 20), (63, 1, 20),
+                                             (64, 2, 20)])
+def test_iterates_match_the_oracle(n, bc_kind, iters):
+    """Fixed iteration counts from random data: entry by entry within the
+    1e-10 that a few dozen FP64 Bi-CG steps in another summation order keep."""
+    b = P.random_field(n, 301)
+    x0 = P.random_field(n, 302) * 0.1
+    x = dev(x0)
+    it, rel, _ = B.bicg_solve(B.Level(n, bc_kind), dev(b), x, 0.0, iters)
+    xr, itr, relr, _ = oracle.bicg(n, bc_kind, b, x0, 0.0, max_iter=iters)
+    assert it == itr == iters
+    assert rel == pytest.approx(relr, rel=1e-8)
+    assert rel_max(x.cpu().numpy(), xr) <= 1e-10
+
+
+def test_call_longer_than_one_launch():
+    """1100 iterations of one call (a launch takes up to 1024): the residual
+    of the recurrence, carried over from launch to launch, is still the true
+    residual.  The two part by rounding of the order eps |A| |x| / |b| <
+    eps cond = 3e-11 here, times a growth factor; had a vector or scalar not
+    been carried over, they would part by the residual itself."""
+    n = 30
+    b = P.random_field(n, 303)
+    b[[0, -1]] = 0
+    b[:, [0, -1]] = 0
+    b[:, :, [0, -1]] = 0
+    lvl = B.Level(n, 1)
+    tb = dev(b)
+    x = torch.zeros((n + 1,) * 3, dtype=torch.float64, device=DEV)
+    it, rel, rc = B.bicg_solve(lvl, tb, x, 0.0, 1100)
+    assert it == 1100 and rc == -4
+    true = float((tb - B.stencil_apply(lvl, x)).norm() / tb.norm())
+    assert abs(true - rel) <= 1e-8
+
+
+def test_general_kernel_where_the_budget_has_no_room():
+    """A budget that holds the Bi-CG vectors but not the exchange words: the
+    call still runs, on the general cooperative kernel."""
+    n = 40
+    b = P.random_field(n, 304)
+    want = None
+    for budget in (0, 6 * 8 * (n + 1) ** 3):
+        x = torch.zeros((n + 1,) * 3, dtype=torch.float64, device=DEV)
+        ctx = B.Context(hbm_budget_bytes=budget)
+        B.bicg_solve(B.Level(n, 2, ctx), dev(b), x, 0.0, 20)
+        if budget:
+            assert ctx.bytes <= budget
+        got = x.cpu().numpy()
+        want = got if want is None else want
+        assert rel_max(got, want) <= 1e-10
+
+
+@pytest.mark.parametrize("n,nc,bc_kind", [(16, 4, 1), (28, 7, 2), (40, 5, 1), (64, 8, 2)])
+def test_mixed_levels(n, nc, bc_kind):
+    """FP32 correction solves on resident levels: what the mixed solve promises
+    is an FP64 residual below the tolerance on every level; on the finest one
+    it is formed again here from u_h."""
+    prob = P.exp_sum()
+    f, g1, g2 = (dev(a) for a in prob.data(n, bc_kind))
+    uh = torch.empty((n + 1,) * 3, dtype=torch.float64, device=DEV)
+    _, stats = B.excmg_solve(n, nc, bc_kind, f, g1, g2, 1e-10, u_h_out=uh, return_stats=True, precision="mixed")
+    for s in stats[2:]:
+        assert s["relres"] <= 1e-10 and not s["stagnated"]
+    lvl = B.Level(n, bc_kind)
+    fh = B.excmg_assemble_rhs(lvl, n, f, g1, g2)
+    rel = float((fh - B.stencil_apply(lvl, uh)).norm() / fh.norm())
+    assert rel <= 1e-10 * (1 + 1e-3)
