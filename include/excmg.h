@@ -289,10 +289,10 @@ int excmg_dsolve(const excmg_level *level, const double *fh, double *u);
  * correction solves, see EXCMG_PRECISION_MIXED).  Every instance keeps its
  * level hierarchy resident; the Bi-CG iterations of the instances that need
  * them run per level group (instances of one precision at one grid size),
- * each group on its own stream and taken back as soon as it completes: one
- * cooperative launch for all members of a group on grids up to 64^3 (and
- * for FP32 correction solves), the single solver's kernels per member on
- * larger FP64 grids.  Instances may be submitted at any time and leave when
+ * each group on its own stream and taken back as soon as it completes: on
+ * grids up to 64^3 one launch per member that keeps its vectors on chip, on
+ * larger grids one cooperative launch for all members of a group of FP32
+ * correction solves, the single solver's kernels per member in FP64.  Instances may be submitted at any time and leave when
  * done, so the batch refills continuously. */
 typedef struct excmg_batch excmg_batch;
 
@@ -319,7 +319,7 @@ int excmg_batch_submit(excmg_batch *batch, int n_finest, int n_coarsest, int bc_
                        int *id_out);
 
 /* Advance every live instance (all pending per-instance steps, then one
- * batched launch of FP32 Bi-CG iterations).  *n_live (may be NULL) receives
+ * round of Bi-CG launches).  *n_live (may be NULL) receives
  * the number of instances still running. */
 int excmg_batch_step(excmg_batch *batch, int *n_live);
 

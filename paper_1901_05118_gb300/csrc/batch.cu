@@ -9,7 +9,10 @@
 // EXP_true.  The Bi-CG iterations (Alg. 2, M = I, r*_0 = r_0) of the
 // instances waiting for them run per level group -- instances of one
 // precision at one grid size -- each group on its own stream:
-//  * grids up to 64^3 and FP32 correction solves: one cooperative launch for
+//  * grids up to 64^3 (both precisions): one launch of the resident kernel
+//    (resident.cuh) per member, on as many CTAs as resident_batch_limit
+//    gives that grid, side by side as far as the GPU's SMs go;
+//  * FP32 correction solves above 64^3: one cooperative launch for
 //    all members; CTAs take operator tiles and vector chunks from every
 //    member, members advance in lock step one iteration per grid-barrier
 //    round, and each member's scalars are formed by the CTA that completes
@@ -31,8 +34,6 @@
 #include "excmg_internal.cuh"
 #include "grid_sync.cuh"
 #include "march_f32.cuh"
-#include "march_fx.cuh"
-#include "march_pair.cuh"
 #include "reduce.cuh"
 
 namespace excmg {
@@ -42,63 +43,15 @@ constexpr int kChunk = 8192;          // vector entries per chunk of the batched
 constexpr int kLd = 2;                // vector entries per thread loaded together
 constexpr int kBatchMaxInst = 1024;
 
-template <typename T>
-struct BatchInst {     // device table entry, one per instance in the Bi-CG phase
+struct BatchInst {     // device table entry, one per instance of a cooperative FP32 group
     int n;
     int sigma;
     int gx, gy, kz_per, nunits, unit_begin;
     int nchunks, chunk_begin;
     int slot;          // index into the state array
     long long len;
-    T *x, *r, *rs, *p, *ps, *q, *qs;
-    T *p2, *ps2;       // FP64: second direction pair (p_k in p for even k, in p2 for odd k)
+    float *x, *r, *rs, *p, *ps, *q, *qs;
 };
-
-// One tile's operator pair (A p, A p* -- A is symmetric) and this thread's
-// share of (p*, A p): FP32 arithmetic for the correction solves; for FP64
-// solves the integer evaluation by the copy-ahead march (p* equals p bit for
-// bit: every call starts from r*_0 = p_0 = p*_0 = r_0), with the general
-// two-field march where a tile holds p* != p.  Called uniformly by the CTA.
-__device__ __forceinline__ float march_pair(const BatchInst<float>& in, int bx, int by, int kz0, int kz1,
-                                            unsigned char*) {
-    return f32_march<2, true>(in.p, in.ps, in.q, in.qs, in.n, (float)in.sigma, bx, by, kz0, kz1);
-}
-__device__ __forceinline__ double march_pair(const BatchInst<double>& in, int bx, int by, int kz0, int kz1,
-                                             unsigned char* smem) {
-    __syncthreads();   // the CTA's previous unit is done with the shared buffers
-    double d = 0.0;
-    if (pp_march<false, true>(in.p, in.ps, in.q, in.qs, in.n, in.sigma, bx, by, kz0, kz1, smem, &d)) return d;
-    __syncthreads();
-    const FxFields fl{{in.p, in.ps}, {in.q, in.qs}, {nullptr, nullptr}, {nullptr, nullptr}, 0.0};
-    return fx_march<2, true>(fl, nullptr, in.n, in.sigma, bx, by, kz0, kz1);
-}
-
-// FP64, iteration k >= 1 of a Bi-CG call: p_k = r_k + beta p_{k-1} (and p*_k)
-// formed on every loaded node from the pair holding p_{k-1}, the CTA's own
-// nodes written to the other pair, then the operator pair on p_k.
-__device__ __forceinline__ double march_pair_dir(const BatchInst<double>& in, int k, double beta, int bx, int by,
-                                                 int kz0, int kz1, unsigned char* smem) {
-    const bool odd = k & 1;
-    const double* pp = odd ? in.p : in.p2;
-    const double* psp = odd ? in.ps : in.ps2;
-    double* pn = odd ? in.p2 : in.p;
-    double* psn = odd ? in.ps2 : in.ps;
-    __syncthreads();   // the CTA's previous unit is done with the shared buffers
-    double d = 0.0;
-    const PairDir dir{in.r, in.rs, pn, psn, beta};
-    if (pp_march<false, true, true>(pp, psp, in.q, in.qs, in.n, in.sigma, bx, by, kz0, kz1, smem, &d, dir))
-        return d;
-    __syncthreads();
-    const FxFields fl{{pp, psp}, {in.q, in.qs}, {in.r, in.rs}, {pn, psn}, beta};
-    return fx_march<2, true, true>(fl, nullptr, in.n, in.sigma, bx, by, kz0, kz1);
-}
-
-// dynamic shared memory of the batched kernel: the copy-ahead march's stages
-// and tiles for FP64 instances, none for the FP32 march
-template <typename T>
-constexpr size_t batch_smem() {
-    return sizeof(T) == sizeof(double) ? pp_smem_bytes<4>() : 0;
-}
 
 struct BatchState {    // device, one per slot
     double rho, rr, alpha, beta, sigma, tol;
@@ -141,19 +94,14 @@ __device__ __forceinline__ double sum_range(const double* v, int begin, int coun
     return block_sum(s, sh);
 }
 
-template <typename T>
 __global__ void __launch_bounds__(S_NT, 2)
-batch_bicg_kernel(const BatchInst<T>* __restrict__ inst, const int* __restrict__ unit_begin,
+batch_bicg_kernel(const BatchInst* __restrict__ inst, const int* __restrict__ unit_begin,
                     const int* __restrict__ chunk_begin, int ninst, int total_units, int total_chunks,
                     double* unit_part, double* chunk_part, BatchState* states, int iters, int* active,
                     GridBarrier gb, int* rounds) {
     __shared__ double sh[32];
-    __shared__ T shf[32];
+    __shared__ float shf[32];
     __shared__ bool flag;
-    extern __shared__ __align__(128) unsigned char batch_smem_buf[];
-    // FP64 groups fold the direction update into the operator phase (two
-    // grid barriers per round); FP32 groups keep a separate phase C
-    constexpr bool kFused = sizeof(T) == sizeof(double);
     const unsigned int G = gridDim.x;
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     const int nt = blockDim.x * blockDim.y;
@@ -165,23 +113,16 @@ batch_bicg_kernel(const BatchInst<T>* __restrict__ inst, const int* __restrict__
         // instance's last tile forms sigma and alpha
         for (int u = blockIdx.x; u < total_units; u += G) {
             const int i = owner(unit_begin, ninst, u);
-            const BatchInst<T>& in = inst[i];
+            const BatchInst& in = inst[i];
             BatchState& st = states[in.slot];
             if (*(volatile int*)&st.done) continue;
             const int loc = u - in.unit_begin;
             const int bx = loc % in.gx, by = (loc / in.gx) % in.gy, bz = loc / (in.gx * in.gy);
             const int kz0 = 1 + bz * in.kz_per;
-            T d;
-            if constexpr (kFused) {
-                // the state's iteration count is this call's k until phase B
-                // of this round completes
-                const int k = st.iter;
-                d = k == 0 ? march_pair(in, bx, by, kz0, min(kz0 + in.kz_per, in.n), batch_smem_buf)
-                           : march_pair_dir(in, k, st.beta, bx, by, kz0, min(kz0 + in.kz_per, in.n),
-                                            batch_smem_buf);
-            } else {
-                d = march_pair(in, bx, by, kz0, min(kz0 + in.kz_per, in.n), batch_smem_buf);
-            }
+            // one tile's operator pair (A p, A p*: A is symmetric) and this
+            // thread's share of (p*, A p)
+            const float d = f32_march<2, true>(in.p, in.ps, in.q, in.qs, in.n, (float)in.sigma, bx, by, kz0,
+                                               min(kz0 + in.kz_per, in.n));
             const double ds = (double)block_sum(d, shf);
             if (thread0()) unit_part[u] = ds;
             if (take_last(&st.ticket_a, (unsigned)in.nunits, &flag)) {
@@ -205,7 +146,7 @@ batch_bicg_kernel(const BatchInst<T>* __restrict__ inst, const int* __restrict__
         // tests convergence
         for (int c = blockIdx.x; c < total_chunks; c += G) {
             const int i = owner(chunk_begin, ninst, c);
-            const BatchInst<T>& in = inst[i];
+            const BatchInst& in = inst[i];
             BatchState& st = states[in.slot];
             if (*(volatile int*)&st.done) {
                 // an instance that broke down in phase A of this round: its
@@ -219,21 +160,20 @@ batch_bicg_kernel(const BatchInst<T>* __restrict__ inst, const int* __restrict__
                 }
                 continue;
             }
-            const T alpha = (T)st.alpha;
-            const T* const pk = (kFused && (st.iter & 1)) ? in.p2 : in.p;   // p_k
+            const float alpha = (float)st.alpha;
             const long long t0 = (long long)(c - in.chunk_begin) * kChunk;
             const long long t1 = min(t0 + kChunk, in.len);
-            T vr = 0, vrr = 0;
+            float vr = 0, vrr = 0;
             // kLd entries per thread loaded together, then updated and summed
             // in index order
             for (long long tb = t0 + tid; tb < t1; tb += (long long)kLd * nt) {
-                T xv[kLd], pv[kLd], rv[kLd], qv[kLd], rsv[kLd], qsv[kLd];
+                float xv[kLd], pv[kLd], rv[kLd], qv[kLd], rsv[kLd], qsv[kLd];
 #pragma unroll
                 for (int k = 0; k < kLd; ++k) {
                     const long long t = tb + (long long)k * nt;
                     if (t < t1) {
                         xv[k] = in.x[t];
-                        pv[k] = pk[t];
+                        pv[k] = in.p[t];
                         rv[k] = in.r[t];
                         qv[k] = in.q[t];
                         rsv[k] = in.rs[t];
@@ -245,8 +185,8 @@ batch_bicg_kernel(const BatchInst<T>* __restrict__ inst, const int* __restrict__
                     const long long t = tb + (long long)k * nt;
                     if (t >= t1) break;
                     in.x[t] = xv[k] + alpha * pv[k];
-                    const T rn = rv[k] - alpha * qv[k];
-                    const T rsn = rsv[k] - alpha * qsv[k];
+                    const float rn = rv[k] - alpha * qv[k];
+                    const float rsn = rsv[k] - alpha * qsv[k];
                     in.r[t] = rn;
                     in.rs[t] = rsn;
                     vr += rsn * rn;
@@ -284,39 +224,37 @@ batch_bicg_kernel(const BatchInst<T>* __restrict__ inst, const int* __restrict__
         // the counter changes only in phase B: between this barrier and the
         // next phase B every CTA reads the same value
         if (*(volatile int*)active <= 0) break;
-        if constexpr (!kFused) {
-            // phase C: p = r + beta p; p* = r* + beta p*
-            for (int c = blockIdx.x; c < total_chunks; c += G) {
-                const int i = owner(chunk_begin, ninst, c);
-                const BatchInst<T>& in = inst[i];
-                const BatchState& st = states[in.slot];
-                if (*(volatile const int*)&st.done) continue;
-                const T beta = (T)st.beta;
-                const long long t0 = (long long)(c - in.chunk_begin) * kChunk;
-                const long long t1 = min(t0 + kChunk, in.len);
-                for (long long tb = t0 + tid; tb < t1; tb += (long long)kLd * nt) {
-                    T rv[kLd], pv[kLd], rsv[kLd], psv[kLd];
+        // phase C: p = r + beta p; p* = r* + beta p*
+        for (int c = blockIdx.x; c < total_chunks; c += G) {
+            const int i = owner(chunk_begin, ninst, c);
+            const BatchInst& in = inst[i];
+            const BatchState& st = states[in.slot];
+            if (*(volatile const int*)&st.done) continue;
+            const float beta = (float)st.beta;
+            const long long t0 = (long long)(c - in.chunk_begin) * kChunk;
+            const long long t1 = min(t0 + kChunk, in.len);
+            for (long long tb = t0 + tid; tb < t1; tb += (long long)kLd * nt) {
+                float rv[kLd], pv[kLd], rsv[kLd], psv[kLd];
 #pragma unroll
-                    for (int k = 0; k < kLd; ++k) {
-                        const long long t = tb + (long long)k * nt;
-                        if (t < t1) {
-                            rv[k] = in.r[t];
-                            pv[k] = in.p[t];
-                            rsv[k] = in.rs[t];
-                            psv[k] = in.ps[t];
-                        }
-                    }
-#pragma unroll
-                    for (int k = 0; k < kLd; ++k) {
-                        const long long t = tb + (long long)k * nt;
-                        if (t >= t1) break;
-                        in.p[t] = rv[k] + beta * pv[k];
-                        in.ps[t] = rsv[k] + beta * psv[k];
+                for (int k = 0; k < kLd; ++k) {
+                    const long long t = tb + (long long)k * nt;
+                    if (t < t1) {
+                        rv[k] = in.r[t];
+                        pv[k] = in.p[t];
+                        rsv[k] = in.rs[t];
+                        psv[k] = in.ps[t];
                     }
                 }
+#pragma unroll
+                for (int k = 0; k < kLd; ++k) {
+                    const long long t = tb + (long long)k * nt;
+                    if (t >= t1) break;
+                    in.p[t] = rv[k] + beta * pv[k];
+                    in.ps[t] = rsv[k] + beta * psv[k];
+                }
             }
-            if (!(ok = grid_sync(gb, G))) break;
         }
+        if (!(ok = grid_sync(gb, G))) break;
     }
     if (blockIdx.x == 0 && thread0()) {
         if (!ok) *active = -1;   // barrier gave up
@@ -329,7 +267,8 @@ batch_bicg_kernel(const BatchInst<T>* __restrict__ inst, const int* __restrict__
 __global__ void __launch_bounds__(kVecThreads)
 batch_init32_kernel(const double* __restrict__ r64, double inv_s, float* __restrict__ r32, float* __restrict__ e,
                     float* __restrict__ rs, float* __restrict__ p, float* __restrict__ ps, size_t len,
-                    double* partials, unsigned int* ticket, BatchState* st, double tol, int max_iter) {
+                    double* partials, unsigned int* ticket, BatchState* st, BicgState* bst, double tol,
+                    int max_iter) {
     __shared__ float shf[32];
     __shared__ double sh[32];
     __shared__ bool am_last;
@@ -357,6 +296,15 @@ batch_init32_kernel(const double* __restrict__ r64, double inv_s, float* __restr
             st->done = conv ? 1 : 0;
             st->status = conv ? kConverged : kRunning;
             st->ticket_a = st->ticket_b = 0;
+            // the same call in the single solver's state layout (resident kernel)
+            bst->rho = bst->rr = tot;
+            bst->alpha = bst->beta = bst->sigma = 0.0;
+            bst->bnorm = sqrt(tot);
+            bst->tol = tol;
+            bst->iter = 0;
+            bst->max_iter = max_iter;
+            bst->done = st->done;
+            bst->status = st->status;
             *ticket = 0;
         }
     }
@@ -368,12 +316,8 @@ batch_correct_kernel(double* __restrict__ u, const float* __restrict__ e, size_t
         u[t] = u[t] + s * (double)e[t];
 }
 
-// The cooperative grid: every SM of the current device, at most two CTAs each.
-template <typename T>
-int batch_resident_ctas() {
-    const int occ = min(2, kernel_occupancy((const void*)batch_bicg_kernel<T>, S_NT, batch_smem<T>()));
-    return device_sms() * occ;
-}
+// CTAs of the cooperative FP32 kernel per SM: at most two.
+int batch_ctas_per_sm() { return min(2, kernel_occupancy((const void*)batch_bicg_kernel, S_NT, 0)); }
 
 }  // namespace
 }  // namespace excmg
@@ -408,6 +352,7 @@ struct Instance {
     // Bi-CG call enqueued so far, and which direction pair holds p_k
     long long launched_k = 0;
     bool dir_in_p2 = false;
+    bool no_resident = false;   // the current call runs without the resident kernel (no room for its words)
     // FP32 correction solve vectors
     float *r32 = nullptr, *e = nullptr, *r = nullptr, *rs = nullptr, *p = nullptr, *ps = nullptr, *q = nullptr,
           *qs = nullptr;
@@ -476,10 +421,13 @@ struct excmg_batch {
         cudaStream_t stream = nullptr;
         cudaEvent_t start = nullptr, done = nullptr;
         bool busy = false;
-        bool launched = false;   // launched mode: per-member kernels, no grid barrier
+        bool launched = false;   // members' states are in the single solver's layout (launched mode, resident kernel)
+        int sm_share = 0;        // CTA places held while busy, in CTAs of the cooperative FP32 kernel
+        void* words = nullptr;   // exchange words of the resident kernel
+        size_t words_cap = 0;
         int prec = 0, n = 0, ctas = 0, cand = -1;
         std::vector<Instance*> members;
-        void* d_inst = nullptr;        // BatchInst<T>[max_instances]
+        void* d_inst = nullptr;        // BatchInst[max_instances]
         int *d_unit_begin = nullptr, *d_chunk_begin = nullptr, *d_active = nullptr, *d_rounds = nullptr;
         int *h_active = nullptr, *h_rounds = nullptr;
         unsigned int* d_barrier = nullptr;
@@ -606,10 +554,9 @@ bool grow(excmg_batch* b, double** buf, size_t* cap, size_t need) {
 }
 
 // Tile / chunk geometry of one instance's current level.
-template <typename T>
-BatchInst<T> geometry(Instance* in, int slot, int* units, int* chunks) {
+BatchInst geometry(Instance* in, int slot, int* units, int* chunks) {
     const int N = in->nc << in->level, m = N - 1;
-    BatchInst<T> t{};
+    BatchInst t{};
     t.n = N;
     t.sigma = in->bc == 1 ? 1 : -1;
     t.gx = (m + S_TX - 1) / S_TX;
@@ -633,9 +580,8 @@ constexpr int kTuneItems[kTuneCands] = {1, 2, 4, 8, 16};   // tiles or chunks pe
 // CTAs per instance of candidate c for an instance with W work items.
 int tune_cpi(int W, int c) { return (W + kTuneItems[c] - 1) / kTuneItems[c]; }
 
-int capacity_of(int prec) {
-    return prec == EXCMG_PRECISION_FP64 ? batch_resident_ctas<double>() : batch_resident_ctas<float>();
-}
+// CTA places of the GPU, in CTAs of the cooperative FP32 kernel.
+int capacity() { return device_sms() * batch_ctas_per_sm(); }
 
 // The group record's stream, events and fixed tables (made once).
 int group_init(excmg_batch* b, excmg_batch::Group& g) {
@@ -643,7 +589,7 @@ int group_init(excmg_batch* b, excmg_batch::Group& g) {
     const size_t mi = (size_t)b->max_instances;
     bool ok = cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreate(&g.start) == cudaSuccess && cudaEventCreate(&g.done) == cudaSuccess &&
-              cudaMalloc(&g.d_inst, mi * sizeof(BatchInst<double>)) == cudaSuccess &&
+              cudaMalloc(&g.d_inst, mi * sizeof(BatchInst)) == cudaSuccess &&
               cudaMalloc(&g.d_unit_begin, mi * sizeof(int)) == cudaSuccess &&
               cudaMalloc(&g.d_chunk_begin, mi * sizeof(int)) == cudaSuccess &&
               cudaMalloc(&g.d_active, sizeof(int)) == cudaSuccess &&
@@ -669,6 +615,7 @@ void group_free(excmg_batch::Group& g) {
     cudaFree(g.d_barrier);
     cudaFree(g.d_unit_part);
     cudaFree(g.d_chunk_part);
+    cudaFree(g.words);
     if (g.start) cudaEventDestroy(g.start);
     if (g.done) cudaEventDestroy(g.done);
     if (g.stream) cudaStreamDestroy(g.stream);
@@ -678,34 +625,21 @@ void group_free(excmg_batch::Group& g) {
 // One cooperative launch of up to b->inner_chunk Bi-CG iterations for the
 // instances `list` (one precision, one grid size) on group record g, with
 // `ctas` CTAs, after the context stream's state uploads.
-template <typename T>
 int launch_group(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instance*>& list, int ctas, int cand) {
     int st = group_init(b, g);
     if (st) return st;
-    std::vector<BatchInst<T>> tab;
+    std::vector<BatchInst> tab;
     std::vector<int> ub, cb;
     int units = 0, chunks = 0;
     for (Instance* in : list) {
-        BatchInst<T> t = geometry<T>(in, in->slot, &units, &chunks);
-        if (sizeof(T) == sizeof(double)) {
-            t.x = (T*)in->u[in->level];
-            t.r = (T*)in->res;
-            t.rs = (T*)in->rs64;
-            t.p = (T*)in->p64;
-            t.ps = (T*)in->ps64;
-            t.q = (T*)in->q64;
-            t.qs = (T*)in->qs64;
-            t.p2 = (T*)in->p2_64;
-            t.ps2 = (T*)in->ps2_64;
-        } else {
-            t.x = (T*)in->e;
-            t.r = (T*)in->r;
-            t.rs = (T*)in->rs;
-            t.p = (T*)in->p;
-            t.ps = (T*)in->ps;
-            t.q = (T*)in->q;
-            t.qs = (T*)in->qs;
-        }
+        BatchInst t = geometry(in, in->slot, &units, &chunks);
+        t.x = in->e;
+        t.r = in->r;
+        t.rs = in->rs;
+        t.p = in->p;
+        t.ps = in->ps;
+        t.q = in->q;
+        t.qs = in->qs;
         ub.push_back(t.unit_begin);
         cb.push_back(t.chunk_begin);
         tab.push_back(t);
@@ -719,7 +653,7 @@ int launch_group(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instan
     *g.h_active = (int)tab.size();
     cudaError_t e = cudaStreamWaitEvent(s, b->host_ready, 0);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(g.d_inst, tab.data(), tab.size() * sizeof(BatchInst<T>), cudaMemcpyHostToDevice, s);
+        e = cudaMemcpyAsync(g.d_inst, tab.data(), tab.size() * sizeof(BatchInst), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(g.d_unit_begin, ub.data(), ub.size() * sizeof(int), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(g.d_chunk_begin, cb.data(), cb.size() * sizeof(int), cudaMemcpyHostToDevice, s);
@@ -728,7 +662,7 @@ int launch_group(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instan
     if (e != cudaSuccess) return bcuda(b, e, "batch table upload");
     int iters = b->inner_chunk;
     int ninst = (int)tab.size();
-    const BatchInst<T>* di = (const BatchInst<T>*)g.d_inst;
+    const BatchInst* di = (const BatchInst*)g.d_inst;
     const int* d_ub = g.d_unit_begin;
     const int* d_cb = g.d_chunk_begin;
     double* up = g.d_unit_part;
@@ -742,17 +676,17 @@ int launch_group(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instan
                     (void*)&rounds};
     e = cudaEventRecord(g.start, s);
     if (e == cudaSuccess)
-        e = cudaLaunchCooperativeKernel((const void*)batch_bicg_kernel<T>, dim3(ctas), dim3(S_TX, S_TY, 1), args,
-                                        batch_smem<T>(), s);
+        e = cudaLaunchCooperativeKernel((const void*)batch_bicg_kernel, dim3(ctas), dim3(S_TX, S_TY, 1), args, 0, s);
     bnote(b, 1);
     if (e == cudaSuccess) e = cudaMemcpyAsync(g.h_active, g.d_active, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(g.h_rounds, g.d_rounds, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaEventRecord(g.done, s);
     if (e != cudaSuccess) return bcuda(b, e, "batched Bi-CG launch");
     g.busy = true;
-    g.prec = sizeof(T) == sizeof(double) ? EXCMG_PRECISION_FP64 : EXCMG_PRECISION_MIXED;
+    g.prec = EXCMG_PRECISION_MIXED;
     g.n = list.empty() ? 0 : (list[0]->nc << list[0]->level);
     g.ctas = ctas;
+    g.sm_share = ctas;
     g.cand = cand;
     g.members = list;
     for (Instance* in : list) in->in_flight = true;
@@ -764,8 +698,62 @@ int launch_group(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instan
 // launch with the direction update folded in, then the update), with the
 // member's own state and partial sums, so that a large level moves its
 // bytes as fast as in a single solve.
-bool launched_level(const Instance* in) {
-    return in->prec == EXCMG_PRECISION_FP64 && (in->nc << in->level) > kPersistentMaxN;
+bool launched_level(const Instance* in) { return in->prec == EXCMG_PRECISION_FP64; }
+
+// One launch of the resident kernel for instance `in`: up to b->inner_chunk
+// iterations of its current call.  Returns false where the exchange words
+// find no room at the start of a call: the call then takes the path of larger
+// grids to its end (the two keep different state).
+bool launch_resident(excmg_batch* b, excmg_batch::Group& g, Instance* in, int ctas, int* status) {
+    *status = group_init(b, g);
+    if (*status) return true;
+    const int N = in->nc << in->level;
+    cudaStream_t s = g.stream;
+    const size_t need = resident_bytes(N);
+    if (g.words_cap < need) {
+        cudaFree(g.words);
+        g.words = nullptr;
+        g.words_cap = 0;
+        if (cudaMalloc(&g.words, need) != cudaSuccess || cudaMemsetAsync(g.words, 0, need, s) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(g.words);
+            g.words = nullptr;
+            if (in->call_iter > 0) *status = bfail(b, EXCMG_ERR_OOM, "exchange words of the resident kernel");
+            in->no_resident = true;
+            return in->call_iter > 0;
+        }
+        g.words_cap = need;
+    }
+    BicgState* bs = b->d_bstate + in->slot;
+    cudaError_t e = cudaStreamWaitEvent(s, b->host_ready, 0);
+    if (e == cudaSuccess) e = cudaEventRecord(g.start, s);
+    const int limit = resident_batch_limit(N);
+    if (e == cudaSuccess) {
+        if (in->prec == EXCMG_PRECISION_FP64)
+            e = launch_bicg_resident<double>(in->u[in->level], in->res, in->rs64, in->p64, in->ps64, N, in->bc,
+                                             b->inner_chunk, bs, g.words, s, false, limit);
+        else
+            e = launch_bicg_resident<float>(in->e, in->r, in->rs, in->p, in->ps, N, in->bc, b->inner_chunk, bs,
+                                            g.words, s, false, limit);
+    }
+    bnote(b, 1);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->h_bstate + in->slot, bs, sizeof(BicgState), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaEventRecord(g.done, s);
+    *status = bcuda(b, e, "resident batch launch");
+    if (*status) return true;
+    *g.h_active = 0;
+    *g.h_rounds = 0;   // the member's iterations, known at the harvest
+    g.busy = true;
+    g.launched = true;
+    g.prec = in->prec;
+    g.n = N;
+    g.ctas = ctas;
+    g.sm_share = ctas * batch_ctas_per_sm();   // one CTA fills an SM
+    g.cand = -1;
+    g.members.assign(1, in);
+    in->in_flight = true;
+    return true;
 }
 
 int launch_group_launched(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instance*>& list) {
@@ -816,6 +804,7 @@ int launch_group_launched(excmg_batch* b, excmg_batch::Group& g, const std::vect
     g.prec = EXCMG_PRECISION_FP64;
     g.n = list[0]->nc << list[0]->level;
     g.ctas = 0;
+    g.sm_share = 0;
     g.cand = -1;
     g.members = list;
     for (Instance* in : list) in->in_flight = true;
@@ -857,12 +846,14 @@ int harvest(excmg_batch* b, excmg_batch::Group& g) {
             hs.iter = bs.iter;
             hs.rr = bs.rr;
             hs.rho = bs.rho;
+            if (bs.status == kTimeout) *g.h_active = -1;   // an exchange gave up
+            if (g.ctas > 0) *g.h_rounds = bs.iter - in->call_iter;
         }
         g.launched = false;
     }
     g.busy = false;
     for (Instance* in : g.members) in->in_flight = false;
-    if (*g.h_active < 0) return bfail(b, EXCMG_ERR_TIMEOUT, "grid barrier of the batched Bi-CG gave up");
+    if (*g.h_active < 0) return bfail(b, EXCMG_ERR_TIMEOUT, "a grid-wide wait of the batched Bi-CG gave up");
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, g.start, g.done) != cudaSuccess) {
         cudaGetLastError();
@@ -1247,7 +1238,7 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
                 if (e == cudaSuccess)
                     e = cudaMemcpyAsync(b->d_states + slot, b->h_states + slot, sizeof(BatchState),
                                         cudaMemcpyHostToDevice, s);
-                if (launched_level(in)) {
+                {
                     // the same call in the single solver's state layout
                     BicgState& bs = b->h_bstate[slot];
                     bs = BicgState{};
@@ -1269,7 +1260,7 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
                 batch_init32_kernel<<<kVecBlocks, kVecThreads, 0, s>>>(in->res, 1.0 / rn, in->r32, in->e, in->rs,
                                                                        in->p, in->ps, node_count(N), ctx->partials,
                                                                        ctx->ticket, b->d_states + slot,
-                                                                       in->inner_tol, cap);
+                                                                       b->d_bstate + slot, in->inner_tol, cap);
                 bnote(b, 1);
                 e = cudaGetLastError();
                 if (e == cudaSuccess)
@@ -1278,6 +1269,7 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
             if (e != cudaSuccess) return bcuda(b, e, "Bi-CG call setup");
             in->phase = kInner;
             in->call_iter = 0;
+            in->no_resident = false;
         }
     }
     // 3. one cooperative launch per level group of instances waiting for
@@ -1303,29 +1295,43 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
                 b->groups.emplace_back();
                 return b->groups.back();
             };
+            auto held = [&]() {
+                int used = 0;
+                for (auto& g : b->groups)
+                    if (g.busy) used += g.sm_share;
+                return used;
+            };
+            const int res = resident_ctas(key.second, resident_batch_limit(key.second));
+            if (res > 0) {
+                // per member, as many as find their SMs free; the others
+                // wait for a step in which they do
+                std::vector<Instance*> rest;
+                for (Instance* in : list) {
+                    if (in->no_resident) {
+                        rest.push_back(in);
+                        continue;
+                    }
+                    if (res * batch_ctas_per_sm() > capacity() - held()) continue;
+                    if (!launch_resident(b, free_group(), in, res, &st)) rest.push_back(in);
+                    if (st) return st;
+                }
+                if (rest.empty()) continue;
+                list = rest;
+            }
             if (launched_level(list[0])) {
                 if ((st = launch_group_launched(b, free_group(), list))) return st;
                 continue;
             }
-            int used = 0;
-            for (auto& g : b->groups)
-                if (g.busy && g.prec == key.first) used += g.ctas;
-            // groups of the other precision run another kernel: count them too
-            for (auto& g : b->groups)
-                if (g.busy && g.prec != key.first) used += g.ctas;
-            const int cap = capacity_of(key.first) - used;
+            const int cap = capacity() - held();
             if (cap < 1) continue;
             int cand = -1, units = 0, chunks = 0;
-            geometry<double>(list[0], 0, &units, &chunks);
+            geometry(list[0], 0, &units, &chunks);
             int ctas = group_ctas(b, key.first, key.second, units > chunks ? units : chunks, (int)list.size(), &cand);
             if (ctas > cap) {
                 ctas = cap;
                 cand = -1;   // not the candidate's shape: not a tuning sample
             }
-            excmg_batch::Group* slot = &free_group();
-            st = key.first == EXCMG_PRECISION_FP64 ? launch_group<double>(b, *slot, list, ctas, cand)
-                                                   : launch_group<float>(b, *slot, list, ctas, cand);
-            if (st) return st;
+            if ((st = launch_group(b, free_group(), list, ctas, cand))) return st;
         }
     }
     // 4. finals (EXP_true)

@@ -82,7 +82,7 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     const bool dir_fused = fused && fuse && !persistent;
     // r*_0 = r_0: with every vector on chip; a caller-chosen r*_0, or no room
     // for the exchange words: the general cooperative kernel
-    void* words = persistent && shadow == nullptr && resident_fits(n) ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
+    void* words = persistent && shadow == nullptr && resident_ctas(n, 0) > 0 ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
     const bool resident = words != nullptr;
     double* p2 = dir_fused ? ctx_buffer(ctx, "bicg_p2", bytes, &st) : nullptr;
     double* ps2 = (dir_fused && !elide && !st) ? ctx_buffer(ctx, "bicg_ps2", bytes, &st) : nullptr;
@@ -125,7 +125,7 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
             int chunk = resident ? 1024 : 256;
             const int left = max_iter - ctx->host_state->iter;
             if (chunk > left) chunk = left;
-            e = resident ? launch_bicg_resident<double>(x, r, rs, p, ps, n, bc_kind, chunk, ctx->state, words, s, elide)
+            e = resident ? launch_bicg_resident<double>(x, r, rs, p, ps, n, bc_kind, chunk, ctx->state, words, s, elide, 0)
                          : launch_bicg_persistent(x, r, rs, p, ps, q, qs, n, bc_kind, chunk, ctx->partials,
                                                   ctx->state, ctx->barrier, s, elide);
             note_launches(1);

@@ -77,11 +77,14 @@ cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, 
 // The same with every vector on chip (resident.cuh), for calls that start
 // from r*_0 = p*_0 = r_0 = p_0.  words: resident_bytes(n) of device memory for
 // the exchanges between CTAs, not shared with a launch that may run at the same time.
-bool resident_fits(int n);
+// max_ctas: CTAs at most (0: one per SM).  resident_ctas: CTAs that the launch takes, 0 where it takes no
+// such grid.  resident_batch_limit: the batch engine's max_ctas.
+int resident_ctas(int n, int max_ctas);
+int resident_batch_limit(int n);
 size_t resident_bytes(int n);
 template <typename T>
 cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
-                                 void* words, cudaStream_t s, bool elide);
+                                 void* words, cudaStream_t s, bool elide, int max_ctas);
 // Shadow-elided mode (r* = r, p* = p, A^T p* = A p not stored): the one-field
 // operator launches with sigma = (p, A p) and alpha (the second also forms
 // p = r + beta p_prev into p), and the matching set-up and update kernels.

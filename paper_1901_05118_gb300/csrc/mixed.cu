@@ -222,7 +222,7 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
     // (48^3: 5 us per iteration, against 25 us for the three launches,
     // each of them a few microseconds of latency for 0.5 MB vectors); larger
     // ones, or no room for the exchange words: the launched kernels
-    void* words = resident_fits(n) ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
+    void* words = resident_ctas(n, 0) > 0 ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
     for (;;) {
         err = ctx_read_back(ctx, ctx->host_state, ctx->state, sizeof(BicgState));
         if (err == cudaSuccess) err = cudaStreamSynchronize(s);
@@ -231,7 +231,7 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
         const int left = max_iter - ctx->host_state->iter;
         if (words) {
             err = launch_bicg_resident<float>(e, r, rs, p, ps, n, bc_kind, left < 1024 ? left : 1024, ctx->state, words,
-                                              s, false);
+                                              s, false, 0);
             note_launches(1);
             if (err != cudaSuccess) return ctx_cuda(ctx, err, "cooperative FP32 Bi-CG launch");
             continue;

@@ -9,12 +9,12 @@
 namespace excmg {
 namespace {
 
-template <typename T, bool kElide, int NI>
+template <typename T, bool kElide>
 const void* resident_fn(int np) {
     switch (np) {
-        case 1: return (const void*)resident_bicg_kernel<T, 1, 2, kElide, NI>;
-        case 2: return (const void*)resident_bicg_kernel<T, 2, 3, kElide, NI>;
-        default: return (const void*)resident_bicg_kernel<T, 4, 5, kElide, NI>;
+        case 1: return (const void*)resident_bicg_kernel<T, 1, 2, kElide>;
+        case 2: return (const void*)resident_bicg_kernel<T, 2, 3, kElide>;
+        default: return (const void*)resident_bicg_kernel<T, 4, 5, kElide>;
     }
 }
 
@@ -30,7 +30,15 @@ ResidentGeom resident_geometry_cached(int n, int max_ctas) {
     return it->second;
 }
 
-bool resident_fits(int n) { return n <= kPersistentMaxN && resident_geometry_cached(n, device_sms()).ctas > 0; }
+int resident_ctas(int n, int max_ctas) {
+    if (n > kPersistentMaxN) return 0;
+    return resident_geometry_cached(n, max_ctas > 0 ? max_ctas : device_sms()).ctas;
+}
+
+// CTAs of a grid in the batch engine: fewer than a single solve takes, so that several instances run side by
+// side, and a number that depends on the grid alone (the sums do, too).  32^3 on 16 CTAs takes about 1.5
+// times as long per iteration as on its own 64, and nine fit beside each other; 64^3 leaves no choice.
+int resident_batch_limit(int n) { return n <= 32 ? 16 : n <= 52 ? 72 : 0; }
 
 namespace {
 size_t slot_bytes() { return (kResWords * sizeof(ulonglong2) + 255) / 256 * 256; }
@@ -48,26 +56,25 @@ size_t resident_bytes(int n) { return slot_bytes() + node_count(n) * sizeof(ulon
 
 template <typename T>
 cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
-                                 void* words, cudaStream_t s, bool elide) {
-    ResidentGeom g = resident_geometry_cached(n, device_sms());
-    ResidentTable<T, 1> tab;
-    tab.inst[0] = ResidentInst<T>{x, r, rs, p, ps, st, (ulonglong2*)words, (ulonglong2*)((char*)words + slot_bytes()), n, bc_kind == 1 ? 1 : -1};
+                                 void* words, cudaStream_t s, bool elide, int max_ctas) {
+    ResidentGeom g = resident_geometry_cached(n, max_ctas > 0 ? max_ctas : device_sms());
+    ResidentInst<T> in{x, r, rs, p, ps, st, (ulonglong2*)words, (ulonglong2*)((char*)words + slot_bytes()), n, bc_kind == 1 ? 1 : -1};
     const size_t smem = (size_t)g.tile * (sizeof(T) == 8 ? sizeof(long long) : sizeof(float));
     const void* fn;
     if constexpr (sizeof(T) == 8)
-        fn = elide ? resident_fn<T, true, 1>(g.np) : resident_fn<T, false, 1>(g.np);
+        fn = elide ? resident_fn<T, true>(g.np) : resident_fn<T, false>(g.np);
     else
-        fn = resident_fn<T, false, 1>(g.np);
+        fn = resident_fn<T, false>(g.np);
     (void)kernel_occupancy(fn, kResThreads, kResTileBytes);   // opts in to the shared memory
     unsigned serial = next_serial();
     long long limit = kBarrierSpinLimit;
-    void* args[] = {&tab, &g, &iters, &serial, &limit};
+    void* args[] = {&in, &g, &iters, &serial, &limit};
     return cudaLaunchCooperativeKernel(fn, dim3(g.ctas), dim3(kResThreads), args, smem, s);
 }
 
 template cudaError_t launch_bicg_resident<double>(double*, double*, double*, double*, double*, int, int, int,
-                                                  BicgState*, void*, cudaStream_t, bool);
+                                                  BicgState*, void*, cudaStream_t, bool, int);
 template cudaError_t launch_bicg_resident<float>(float*, float*, float*, float*, float*, int, int, int, BicgState*,
-                                                 void*, cudaStream_t, bool);
+                                                 void*, cudaStream_t, bool, int);
 
 }  // namespace excmg

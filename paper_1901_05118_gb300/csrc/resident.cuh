@@ -68,12 +68,6 @@ struct ResidentInst {
     int n, sigma;
 };
 
-// The calls of one launch: CTA b works on call b / ctas.
-template <typename T, int NI>
-struct ResidentTable {
-    ResidentInst<T> inst[NI];
-};
-
 namespace {
 
 // One 16-byte word, read and written as a whole.
@@ -147,9 +141,9 @@ __device__ __forceinline__ float sum_f32(float v) {
 }
 
 // NP: nodes of a thread's z-run; NH: nodes around the brick per thread.
-template <typename T, int NP, int NH, bool kElide, int NI>
+template <typename T, int NP, int NH, bool kElide>
 __global__ void __launch_bounds__(kResThreads, 1)
-resident_bicg_kernel(const __grid_constant__ ResidentTable<T, NI> tab, const ResidentGeom g, int iters,
+resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
                      unsigned serial, long long spin_limit) {
     constexpr bool kExact = std::is_same<T, double>::value;
     using Fix = typename std::conditional<kExact, long long, float>::type;
@@ -160,11 +154,9 @@ resident_bicg_kernel(const __grid_constant__ ResidentTable<T, NI> tab, const Res
     __shared__ double bcast[2];   // alpha or beta, rho
     __shared__ int flags[2];      // stop code of the last exchange, gave up
     __shared__ int lost;          // a thread gave up waiting for r
-    const ResidentInst<T>& in = tab.inst[NI == 1 ? 0 : blockIdx.x / g.ctas];
     BicgState* const st = in.st;
     if (st->done) return;
-    const int cta = NI == 1 ? (int)blockIdx.x : (int)(blockIdx.x % g.ctas);
-    const int G = g.ctas, n = in.n, np = n + 1;
+    const int cta = (int)blockIdx.x, G = g.ctas, n = in.n, np = n + 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int plane = np * np;
 
