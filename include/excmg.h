@@ -119,13 +119,14 @@ enum { EXCMG_STENCIL_EXACT = 0, EXCMG_STENCIL_FP64 = 1 };
 int excmg_ctx_set_stencil(excmg_ctx *ctx, int variant);
 
 /* Shadow sequence of Bi-CG (Alg. 2) on this context.
- * EXCMG_SHADOW_FULL (default): r*, p* and A^T p* are carried in memory as
- *   Alg. 2 prints them.
+ * EXCMG_SHADOW_FULL (default): r* and p* are carried in memory and updated
+ *   as Alg. 2 prints them.  With r*_0 = r_0 and the exact operator A^T p* is
+ *   A p bit for bit and both are read from one array.
  * EXCMG_SHADOW_ELIDED -- not the paper's algorithm as printed, a labelled
  *   variant: A_h is symmetric, and with r*_0 = r_0 and the exact operator
  *   (EXCMG_STENCIL_EXACT) A^T p* and A p are the same bits, so the shadow
  *   sequence equals the primal one bit for bit; it is then neither stored
- *   nor read (88 instead of 152 bytes per unknown and iteration on large
+ *   nor read (88 instead of 136 bytes per unknown and iteration on large
  *   grids) and every iterate, stopping decision and result is bit for bit
  *   that of EXCMG_SHADOW_FULL.  It applies to the exact operator only: with
  *   EXCMG_STENCIL_FP64, and in calls that pass their own r*_0
@@ -142,9 +143,9 @@ int excmg_ctx_set_shadow_mode(excmg_ctx *ctx, int mode);
  *   p = r + beta p and p* = r* + beta p* from the previous directions on
  *   every node it loads (writing the nodes it owns into a second buffer
  *   pair), then applies A and A^T with sigma and alpha; with the update
- *   (x, r, r*, rho, beta) that makes two launches and 136 bytes per unknown.
+ *   (x, r, r*, rho, beta) that makes two launches and 120 bytes per unknown.
  * EXCMG_SCHEDULE_SEPARATE: operator pair (A p, A^T p*, sigma, alpha), update
- *   and direction update (p, p*) as three launches, 152 bytes per unknown. */
+ *   and direction update (p, p*) as three launches, 136 bytes per unknown. */
 enum { EXCMG_SCHEDULE_SEPARATE = 0, EXCMG_SCHEDULE_FUSED = 1 };
 int excmg_ctx_set_schedule(excmg_ctx *ctx, int schedule);
 
@@ -166,7 +167,7 @@ const char *excmg_last_error(const excmg_ctx *ctx);
  * operator launches timed since and (bytes may be NULL) the algorithmic
  * bytes those launches read and wrote: 8 B per unknown for every field in
  * or out (a launch of the fused pair that also forms the directions moves
- * eight fields, the plain pair four, one FP64 application two). */
+ * seven fields, the plain pair three, one FP64 application two). */
 long long excmg_launch_count(void);
 int excmg_ctx_profile(excmg_ctx *ctx, int enable);
 int excmg_ctx_profile_read(const excmg_ctx *ctx, int n, double *ms_total, long long *launches,

@@ -346,7 +346,7 @@ struct Instance {
     std::vector<double*> u;    // per level
     double *fh = nullptr, *res = nullptr, *W = nullptr;
     // FP64 Bi-CG vectors (r is `res`)
-    double *rs64 = nullptr, *p64 = nullptr, *ps64 = nullptr, *q64 = nullptr, *qs64 = nullptr;
+    double *rs64 = nullptr, *p64 = nullptr, *ps64 = nullptr, *q64 = nullptr;
     double *p2_64 = nullptr, *ps2_64 = nullptr;   // second direction pair
     // launched mode (FP64 levels above 64^3): iterations of the current
     // Bi-CG call enqueued so far, and which direction pair holds p_k
@@ -383,7 +383,7 @@ size_t instance_bytes(int n, int nc, int prec) {
     b += 2 * align256(node_count(n) * sizeof(double));                                   // fh, res
     b += align256(node_count(n / 2) * sizeof(double));                                   // W
     if (prec == EXCMG_PRECISION_FP64)
-        b += 7 * align256(node_count(n) * sizeof(double));                   // r*, p, p*, q, q*, p2, p*2
+        b += 6 * align256(node_count(n) * sizeof(double));                   // r*, p, p*, q, p2, p*2
     else
         b += 8 * align256(node_count(n) * sizeof(float));                                // r32, e, 6 vectors
     return b;
@@ -514,7 +514,7 @@ int setup_level(excmg_batch* b, Instance* in) {
         if (in->prec == EXCMG_PRECISION_FP64) {
             // (the second direction pair as well: the operator phase writes
             // its interior entries only)
-            double* const zero[] = {in->q64, in->qs64, in->p2_64, in->ps2_64};
+            double* const zero[] = {in->q64, in->p2_64, in->ps2_64};
             for (double* z : zero)
                 if (e == cudaSuccess) e = cudaMemsetAsync(z, 0, len * sizeof(double), ctx->stream);
         } else {
@@ -774,17 +774,17 @@ int launch_group_launched(excmg_batch* b, excmg_batch::Group& g, const std::vect
             double* psc = in->dir_in_p2 ? in->ps2_64 : in->ps64;
             if (in->launched_k == 0) {
                 // p_0 = r_0: the operator pair on the fused schedule's grid
-                e = launch_bicg_stencil_pair(pc, in->q64, psc, in->qs64, N, in->bc, part, bs, s, true);
+                e = launch_bicg_stencil_pair(pc, in->q64, psc, nullptr, N, in->bc, part, bs, s);
             } else {
                 double* pn = in->dir_in_p2 ? in->p64 : in->p2_64;
                 double* psn = in->dir_in_p2 ? in->ps64 : in->ps2_64;
-                e = launch_bicg_stencil_pair_dir(in->res, in->rs64, pc, psc, pn, psn, in->q64, in->qs64, N, in->bc,
+                e = launch_bicg_stencil_pair_dir(in->res, in->rs64, pc, psc, pn, psn, in->q64, nullptr, N, in->bc,
                                                  part, bs, s);
                 in->dir_in_p2 = !in->dir_in_p2;
                 pc = pn;
             }
             if (e == cudaSuccess)
-                e = launch_bicg_update(in->u[in->level], pc, in->res, in->q64, in->rs64, in->qs64, node_count(N), part,
+                e = launch_bicg_update(in->u[in->level], pc, in->res, in->q64, in->rs64, nullptr, node_count(N), part,
                                        bs, s);
             ++in->launched_k;
             nl += 2;
@@ -1090,7 +1090,6 @@ int excmg_batch_submit(excmg_batch* b, int n_finest, int n_coarsest, int bc_kind
         in->p64 = (double*)take(n64);
         in->ps64 = (double*)take(n64);
         in->q64 = (double*)take(n64);
-        in->qs64 = (double*)take(n64);
         in->p2_64 = (double*)take(n64);
         in->ps2_64 = (double*)take(n64);
     } else {

@@ -66,7 +66,6 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     double* p = st ? nullptr : ctx_buffer(ctx, "bicg_p", bytes, &st);
     double* ps = (st || elide) ? nullptr : ctx_buffer(ctx, "bicg_ps", bytes, &st);
     double* q = st ? nullptr : ctx_buffer(ctx, "bicg_q", bytes, &st);
-    double* qs = (st || elide) ? nullptr : ctx_buffer(ctx, "bicg_qs", bytes, &st);
     if (st) return st;
     // the integer operator has a fused two-field kernel; the FP64 one runs
     // as two applications and a separate inner product
@@ -84,6 +83,12 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // for the exchange words: the general cooperative kernel
     void* words = persistent && shadow == nullptr && resident_ctas(n, 0) > 0 ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
     const bool resident = words != nullptr;
+    // the integer operator's A^T p* is A p bit for bit while p* = p, as it is
+    // from r*_0 = r_0 on: both are read from q (the general cooperative
+    // kernel keeps its second array)
+    const bool twin = fused && shadow == nullptr && (resident || !persistent);
+    double* qs = (elide || twin) ? nullptr : ctx_buffer(ctx, "bicg_qs", bytes, &st);
+    if (st) return st;
     double* p2 = dir_fused ? ctx_buffer(ctx, "bicg_p2", bytes, &st) : nullptr;
     double* ps2 = (dir_fused && !elide && !st) ? ctx_buffer(ctx, "bicg_ps2", bytes, &st) : nullptr;
     if (st) return st;
@@ -100,7 +105,7 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // interior entries only
     if (e == cudaSuccess) e = cudaMemsetAsync(r, 0, bytes, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, bytes, s);
-    if (e == cudaSuccess && !elide) e = cudaMemsetAsync(qs, 0, bytes, s);
+    if (e == cudaSuccess && qs) e = cudaMemsetAsync(qs, 0, bytes, s);
     // r_0 = b - A x_0; r*_0 = p_0 = p*_0 = r_0; rho_0
     if (e == cudaSuccess) e = launch_stencil(x, r, b, n, bc_kind, false, nullptr, s, ctx->stencil_variant);
     if (e == cudaSuccess)
@@ -184,19 +189,19 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
                     // from the second iteration on the launch first forms
                     // p_k = r_k + beta_{k-1} p_{k-1} (and p*_k) on the fly
                     if (enqueued == 0 || !dir_fused) {
-                        ee = elide ? launch_cg_stencil(pc, q, n, bc_kind, ctx->partials, ctx->state, ss, dir_fused)
+                        ee = elide ? launch_cg_stencil(pc, q, n, bc_kind, ctx->partials, ctx->state, ss)
                                    : launch_bicg_stencil_pair(pc, q, psc, qs, n, bc_kind, ctx->partials, ctx->state,
-                                                              ss, dir_fused);
-                        // p (, p*) in; q (, q*) out
-                        launch_bytes[it] = (elide ? 16.0 : 32.0) * unknowns;
+                                                              ss);
+                        // p (, p*) in; q (, q* of its own) out
+                        launch_bytes[it] = (elide ? 16.0 : qs ? 32.0 : 24.0) * unknowns;
                     } else {
                         ee = elide ? launch_cg_stencil_dir(r, pc, pn, q, n, bc_kind, ctx->partials, ctx->state, ss)
                                    : launch_bicg_stencil_pair_dir(r, rs, pc, psc, pn, psn, q, qs, n, bc_kind,
                                                                   ctx->partials, ctx->state, ss);
                         std::swap(pc, pn);
                         std::swap(psc, psn);
-                        // r (, r*), p_old (, p*_old) in; p (, p*), q (, q*) out
-                        launch_bytes[it] = (elide ? 32.0 : 64.0) * unknowns;
+                        // r (, r*), p_old (, p*_old) in; p (, p*), q (, q* of its own) out
+                        launch_bytes[it] = (elide ? 32.0 : qs ? 64.0 : 56.0) * unknowns;
                     }
                     if (ctx->profile) {
                         cudaEventRecord(ctx->prof_events[3 * it + 1], ss);

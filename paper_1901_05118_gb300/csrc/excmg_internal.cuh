@@ -57,8 +57,10 @@ cudaError_t launch_zero_boundary(double* y, int n, cudaStream_t s);
 // One z-march applying A to p (-> q) and A^T to p* (-> qs) with the integer
 // arithmetic, fused with sigma = (p*, q) and alpha = rho / sigma (Alg. 2).
 // Skips when st->done.  partials must hold stencil_cta_count(n) doubles.
+// qs null: the call started from r*_0 = p*_0 = r_0 = p_0, so p* = p and A^T p*
+// is q bit for bit and is not stored again; else (a caller-chosen r*_0) the two fields are marched apart.
 cudaError_t launch_bicg_stencil_pair(const double* p, double* q, const double* ps, double* qs, int n,
-                                     int bc_kind, double* partials, BicgState* st, cudaStream_t s, bool staged);
+                                     int bc_kind, double* partials, BicgState* st, cudaStream_t s);
 int stencil_cta_count(int n);
 // As launch_bicg_stencil_pair, with the direction update of the previous
 // iteration fused in: p = r + beta p_prev, p* = r* + beta p*_prev (beta from
@@ -92,7 +94,7 @@ cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_k
 // partial sums in the same order and the iterates are bit for bit those of
 // the full mode.
 cudaError_t launch_cg_stencil(const double* p, double* q, int n, int bc_kind, double* partials, BicgState* st,
-                              cudaStream_t s, bool staged);
+                              cudaStream_t s);
 cudaError_t launch_cg_pupdate(double* p, const double* r, size_t len, const BicgState* st, cudaStream_t s);
 cudaError_t launch_cg_stencil_dir(const double* r, const double* p_prev, double* p, double* q, int n, int bc_kind,
                                   double* partials, BicgState* st, cudaStream_t s);
@@ -111,6 +113,7 @@ cudaError_t launch_bicg_init(const double* r, const double* shadow, double* rs, 
                              double* partials, BicgState* st, cudaStream_t s);
 cudaError_t launch_bicg_sigma(const double* ps, const double* q, size_t len, double* partials,
                               BicgState* st, cudaStream_t s);
+// qs null: A^T p* = q.
 cudaError_t launch_bicg_update(double* x, const double* p, double* r, const double* q, double* rs,
                                const double* qs, size_t len, double* partials, BicgState* st,
                                cudaStream_t s);

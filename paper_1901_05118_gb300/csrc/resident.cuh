@@ -47,7 +47,7 @@
 #include <type_traits>
 
 #include "grid_sync.cuh"
-#include "march_pair.cuh"
+#include "march_lap.cuh"
 #include "resident_geom.h"
 
 namespace excmg {

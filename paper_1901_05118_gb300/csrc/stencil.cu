@@ -27,7 +27,7 @@
 #include "excmg_internal.cuh"
 #include "grid_sync.cuh"
 #include "march_fx.cuh"
-#include "march_pair.cuh"
+#include "march_lap.cuh"
 #include "reduce.cuh"
 
 namespace excmg {
@@ -98,54 +98,20 @@ stencil_f64_kernel(const double* __restrict__ u, double* __restrict__ y, const d
     }
 }
 
-// y = A u (or y = b - A u): the single-field march of march_fx.cuh, three
-// CTAs per SM (the march waits on each plane's loads, and 24 resident warps
-// hide more of that latency than 16).
-__global__ void __launch_bounds__(FX_NT, 3)
-stencil_fx_kernel(FxFields fl, const double* __restrict__ b, int n, int sigma, int kz_per_cta,
-                  const int* __restrict__ skip) {
+// y = A u, or y = b - A u.
+__global__ void __launch_bounds__(PP_NT, 3)
+stencil_apply_kernel(const double* __restrict__ u, double* __restrict__ y, const double* __restrict__ b, int n,
+                     int sigma, int kz_per_cta, const int* __restrict__ skip) {
+    extern __shared__ __align__(128) unsigned char march_smem[];
     if (skip != nullptr && *skip) return;
     const int kz0 = 1 + blockIdx.z * kz_per_cta;
-    const int kz1 = min(kz0 + kz_per_cta, n);
-    (void)fx_march<1, false>(fl, b, n, sigma, blockIdx.x, blockIdx.y, kz0, kz1);
+    const MarchArrays a{u, nullptr, nullptr, nullptr, b, y, nullptr, nullptr, 0.0};
+    (void)lap_march<kMarchApply, true>(a, n, sigma, blockIdx.x, blockIdx.y, kz0, min(kz0 + kz_per_cta, n),
+                                       march_smem);
 }
 
-// The operator launch of the default Bi-CG schedule on grids above 64^3:
-// q = A p, q* = A^T p*, sigma = (p*, q) and alpha = rho / sigma (Alg. 2),
-// with the copy-ahead march of march_pair.cuh (bit for bit the results of
-// fx_march<2, true>).  A CTA whose slab holds a node where p*
-// differs from p (a caller-chosen r*_0) runs the general two-field march
-// instead.  kElide: the shadow-elided mode (p only, q only; the same sums).
-constexpr bool kPairCvt = true;   // outputs rounded by the hardware conversion
-
-// the general two-field march, kept out of line: it runs only where p* != p
-__device__ __noinline__ double pair_two_field(const double* p, const double* ps, double* q, double* qs, int n,
-                                              int sigma, int bx, int by, int kz0, int kz1) {
-    const FxFields fl{{p, ps}, {q, qs}, {nullptr, nullptr}, {nullptr, nullptr}, 0.0};
-    return fx_march<2, true>(fl, nullptr, n, sigma, bx, by, kz0, kz1);
-}
-
-// Launch bounds: the two-field kernel at two CTAs per SM (up to 128
-// registers: measured 1.27 ms against 1.41 ms per 512^3 launch at three CTAs
-// and 80 registers, where the compiler recomputes values it cannot keep),
-// the elided one at three (1.02 against 1.06 ms).
-template <bool kElide>
-__global__ void __launch_bounds__(PP_NT, kElide ? 3 : 2)
-stencil_pair_kernel(const double* __restrict__ p, const double* __restrict__ ps, double* __restrict__ q,
-                    double* __restrict__ qs, int n, int sigma, int kz_per_cta, double* partials, BicgState* st) {
-    extern __shared__ __align__(128) unsigned char pp_smem[];
-    if (st->done) return;
-    const int kz0 = 1 + blockIdx.z * kz_per_cta;
-    const int kz1 = min(kz0 + kz_per_cta, n);
-    double dot = 0.0;
-    const bool fast = pp_march<kElide, kPairCvt>(p, ps, q, qs, n, sigma, blockIdx.x, blockIdx.y, kz0, kz1,
-                                                pp_smem, &dot);
-    if constexpr (!kElide) {
-        if (!fast) {
-            __syncthreads();
-            dot = pair_two_field(p, ps, q, qs, n, sigma, blockIdx.x, blockIdx.y, kz0, kz1);
-        }
-    }
+// Every CTA's share of sigma = (p*, A p); the last one forms alpha = rho / sigma (Alg. 2).
+__device__ __forceinline__ void finish_sigma(double dot, double* partials, BicgState* st) {
     __shared__ double sh[32];
     __shared__ bool am_last;
     const double sdot = block_sum(dot, sh);
@@ -165,55 +131,33 @@ stencil_pair_kernel(const double* __restrict__ p, const double* __restrict__ ps,
     }
 }
 
-// The fused schedule's operator launch: p = r + beta p_prev (and p*) formed
-// on every loaded node, the nodes the CTA owns written to (pn, psn), then
-// q = A p, q* = A^T p*, sigma and alpha, with the copy-ahead march (bit for
-// bit the results of fx_march<2, true, true>).  A CTA whose slab
-// holds a node where r* != r or p*_prev != p_prev runs the general march.
-__device__ __noinline__ double pair_two_field_dir(const double* r, const double* rs, const double* pp,
-                                                  const double* psp, double* pn, double* psn, double* q, double* qs,
-                                                  double beta, int n, int sigma, int kz0, int kz1) {
-    FxFields fl{{pp, psp}, {q, qs}, {r, rs}, {pn, psn}, beta};
-    return fx_march<2, true, true>(fl, nullptr, n, sigma, blockIdx.x, blockIdx.y, kz0, kz1);
-}
-
-template <bool kElide>
+// The operator launch of Bi-CG on grids above 64^3, for calls that start from
+// r*_0 = p*_0 = r_0 = p_0: q = A p (A^T p* is the same bits, as p* = p),
+// sigma and alpha; K = kMarchDir: p = r + beta p_{k-1} and p* formed first
+// (the fused schedule).  kElide: the shadow-elided mode (p, q only; the same
+// sums).
+template <MarchKind K, bool kElide>
 __global__ void __launch_bounds__(PP_NT, 2)
-stencil_pair_dir_kernel(const double* __restrict__ r, const double* __restrict__ rs, const double* __restrict__ pp,
-                        const double* __restrict__ psp, double* __restrict__ pn, double* __restrict__ psn,
-                        double* __restrict__ q, double* __restrict__ qs, int n, int sigma, int kz_per_cta,
-                        double* partials, BicgState* st) {
-    extern __shared__ __align__(128) unsigned char pp_smem[];
+stencil_step_kernel(MarchArrays a, int n, int sigma, int kz_per_cta, double* partials, BicgState* st) {
+    extern __shared__ __align__(128) unsigned char march_smem[];
     if (st->done) return;
     const int kz0 = 1 + blockIdx.z * kz_per_cta;
-    const int kz1 = min(kz0 + kz_per_cta, n);
-    const PairDir dir{r, rs, pn, psn, st->beta};
-    double dot = 0.0;
-    const bool fast = pp_march<kElide, kPairCvt, true>(pp, psp, q, qs, n, sigma, blockIdx.x, blockIdx.y, kz0, kz1,
-                                                      pp_smem, &dot, dir);
-    if constexpr (!kElide) {
-        if (!fast) {
-            __syncthreads();
-            dot = pair_two_field_dir(r, rs, pp, psp, pn, psn, q, qs, dir.beta, n, sigma, kz0, kz1);
-        }
-    }
-    __shared__ double sh[32];
-    __shared__ bool am_last;
-    const double sdot = block_sum(dot, sh);
-    if (publish_partials(&sdot, 1, partials, &st->ticket, &am_last)) {
-        const double sg = gather_partials(partials, 0, sh);
-        if (thread0()) {
-            const double rho = st->rho;
-            st->sigma = sg;
-            if (!(rho != 0.0 && isfinite(rho)) || !(sg != 0.0 && isfinite(sg))) {
-                st->status = kBreakdown;
-                st->done = 1;
-            } else {
-                st->alpha = rho / sg;
-            }
-            st->ticket = 0;
-        }
-    }
+    a.beta = st->beta;
+    finish_sigma(lap_march<K, kElide>(a, n, sigma, blockIdx.x, blockIdx.y, kz0, min(kz0 + kz_per_cta, n), march_smem),
+                 partials, st);
+}
+
+// The same for a caller-chosen r*_0: two fields, marched side by side
+// (march_fx.cuh).
+template <bool kDir>
+__global__ void __launch_bounds__(FX_NT, 2)
+stencil_two_field_kernel(MarchArrays a, double* qs, int n, int sigma, int kz_per_cta, double* partials, BicgState* st) {
+    if (st->done) return;
+    const int kz0 = 1 + blockIdx.z * kz_per_cta;
+    const FxFields fl{{a.in, a.ins}, {a.out, qs}, {a.r, a.rs}, {a.pn, a.psn}, st->beta};
+    finish_sigma(fx_march<2, true, kDir>(fl, nullptr, n, sigma, blockIdx.x, blockIdx.y, kz0,
+                                         min(kz0 + kz_per_cta, n)),
+                 partials, st);
 }
 
 // A u at one interior node (i, j, k) with the integer arithmetic, without
@@ -304,7 +248,6 @@ bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int 
     const int units = gx * gy * slabs;
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     const int nthreads = blockDim.x * blockDim.y;
-    extern __shared__ __align__(128) unsigned char persistent_stage_smem[];
     double rho = st->rho, rr = st->rr, alpha = st->alpha, beta = st->beta, sigma_s = st->sigma;
     int iter = st->iter, status = st->status, done = st->done;
     const int max_iter = st->max_iter;
@@ -334,17 +277,9 @@ bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int 
                 const int bx = u % gx, by = (u / gx) % gy, bz = u / (gx * gy);
                 const int kz0 = 1 + bz * kz_per;
                 const int kz1 = min(kz0 + kz_per, n);
-                // the copy-ahead march (same sums as fx_march<2, true>); the
-                // CTA's previous unit is done with the shared buffers
-                __syncthreads();
-                double dd = 0.0;
-                if (pp_march<kElide, kPairCvt>(v.p, v.ps, v.q, v.qs, n, sigma, bx, by, kz0, kz1,
-                                               persistent_stage_smem, &dd)) {
-                    dot += dd;
-                } else if constexpr (!kElide) {
-                    __syncthreads();
-                    dot += pair_two_field(v.p, v.ps, v.q, v.qs, n, sigma, bx, by, kz0, kz1);
-                }
+                __syncthreads();   // the CTA's previous unit is done with the shared buffers
+                const FxFields fl{{v.p, v.ps}, {v.q, v.qs}, {nullptr, nullptr}, {nullptr, nullptr}, 0.0};
+                dot += fx_march<kElide ? 1 : 2, true>(fl, nullptr, n, sigma, bx, by, kz0, kz1);
             }
         }
         dot = block_sum(dot, sh);
@@ -545,38 +480,29 @@ int resident_per_sm(K kernel, int threads, size_t smem = 0) {
     return kernel_occupancy((const void*)kernel, threads, smem);
 }
 
-template <typename K>
-void opt_in_smem(K kernel, size_t smem) {
-    (void)kernel_occupancy((const void*)kernel, FX_NT, smem);
+StencilGrid march_grid(int n, int per_sm, size_t smem) {
+    StencilGrid g = stencil_grid(n, PP_TX, PP_OY, per_sm);
+    g.block = dim3(PP_TX, PP_TY, 1);
+    g.smem = smem;
+    return g;
 }
 
 // The single-field operator launch (A u, b - A u).
-StencilGrid fx_grid(int n) {
-    const int occ1 = resident_per_sm(stencil_fx_kernel, FX_NT);
-    StencilGrid g = stencil_grid(n, FX_TX, FX_OY, occ1);
-    g.block = dim3(FX_TX, FX_TY, 1);
-    return g;
+StencilGrid apply_grid(int n) {
+    constexpr size_t smem = MarchStage<kMarchApply, true>::kSmem;
+    return march_grid(n, resident_per_sm(stencil_apply_kernel, PP_NT, smem), smem);
 }
 
-// The copy-ahead operator launch (both modes run on this grid, so that
-// sigma adds the same per-CTA partial sums).
-StencilGrid pair_grid(int n) {
-    const int occ = resident_per_sm(stencil_pair_kernel<false>, PP_NT, pp_smem_bytes<2>());
-    StencilGrid g = stencil_grid(n, PP_TX, PP_OY, occ);
-    g.block = dim3(PP_TX, PP_TY, 1);
-    g.smem = pp_smem_bytes<2>();
-    return g;
-}
-
-// The fused schedule's launches (both modes on this grid: the same sigma
-// partial sums); the first iteration of a call (no previous directions) runs
-// stencil_pair_kernel on the same grid.
-StencilGrid pair_dir_grid(int n) {
-    const int occ = resident_per_sm(stencil_pair_dir_kernel<false>, PP_NT, pp_smem_bytes<4>());
-    StencilGrid g = stencil_grid(n, PP_TX, PP_OY, occ);
-    g.block = dim3(PP_TX, PP_TY, 1);
-    g.smem = pp_smem_bytes<4>();
-    return g;
+// The operator step of Bi-CG: every form of it runs on the grid of the
+// two-field one with directions, so that sigma adds the same per-CTA
+// partial sums in the shadow-elided mode.
+template <MarchKind K, bool kElide>
+StencilGrid step_grid(int n) {
+    constexpr size_t full = MarchStage<kMarchDir, false>::kSmem;
+    const int occ = resident_per_sm(stencil_step_kernel<kMarchDir, false>, PP_NT, full);
+    constexpr size_t smem = MarchStage<K, kElide>::kSmem;
+    (void)resident_per_sm(stencil_step_kernel<K, kElide>, PP_NT, smem);
+    return march_grid(n, occ, smem);
 }
 
 StencilGrid f64_grid(int n) {
@@ -589,14 +515,8 @@ StencilGrid f64_grid(int n) {
 }  // namespace
 
 int stencil_cta_count(int n) {
-    unsigned most = 0;
-    const StencilGrid g1 = fx_grid(n);
-    most = max(most, g1.grid.x * g1.grid.y * g1.grid.z);
-    const StencilGrid g = pair_grid(n);
-    most = max(most, g.grid.x * g.grid.y * g.grid.z);
-    const StencilGrid gd = pair_dir_grid(n);
-    most = max(most, gd.grid.x * gd.grid.y * gd.grid.z);
-    return (int)most;
+    const StencilGrid g1 = apply_grid(n), g2 = step_grid<kMarchDir, false>(n);
+    return (int)max(g1.grid.x * g1.grid.y * g1.grid.z, g2.grid.x * g2.grid.y * g2.grid.z);
 }
 
 cudaError_t launch_stencil(const double* u, double* y, const double* b, int n, int bc_kind,
@@ -611,18 +531,13 @@ cudaError_t launch_stencil(const double* u, double* y, const double* b, int n, i
     } else {
         // A^T u == A u bit for bit in integer arithmetic (see above)
         (void)transpose;
-        const StencilGrid g = fx_grid(n);
-        FxFields fl{{u, nullptr}, {y, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}, 0.0};
-        stencil_fx_kernel<<<g.grid, g.block, 0, s>>>(fl, b, n, bc_kind == 1 ? 1 : -1, g.kz_per_cta, skip);
+        const StencilGrid g = apply_grid(n);
+        stencil_apply_kernel<<<g.grid, g.block, g.smem, s>>>(u, y, b, n, bc_kind == 1 ? 1 : -1, g.kz_per_cta, skip);
     }
     return cudaGetLastError();
 }
 
 constexpr int kPointwiseMaxN = 32;   // per-node operator on grids up to 32^3
-
-// dynamic shared memory of the z-march variant: the copy-ahead march's
-// stages and tiles
-size_t persistent_smem(bool pointwise) { return pointwise ? 0 : pp_smem_bytes<2>(); }
 
 int persistent_grid(int n, int* gx, int* gy, int* slabs, int* kz_per) {
     // the elided variants run on the grids of the full ones (same partial
@@ -676,67 +591,51 @@ cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, 
     if (pw) {
         fn = elide ? (const void*)bicg_persistent_kernel<true, true> : (const void*)bicg_persistent_kernel<true, false>;
     } else {
-        opt_in_smem(bicg_persistent_kernel<false, true>, pp_smem_bytes<2>());
-        opt_in_smem(bicg_persistent_kernel<false, false>, pp_smem_bytes<2>());
         fn = elide ? (const void*)bicg_persistent_kernel<false, true> : (const void*)bicg_persistent_kernel<false, false>;
     }
-    return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(FX_TX, FX_TY, 1), args, persistent_smem(pw), s);
+    return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(FX_TX, FX_TY, 1), args, 0, s);
 }
 
 cudaError_t launch_bicg_stencil_pair_dir(const double* r, const double* rs, const double* p_prev,
                                          const double* ps_prev, double* p, double* ps, double* q, double* qs, int n,
                                          int bc_kind, double* partials, BicgState* st, cudaStream_t s) {
+    const MarchArrays a{p_prev, r, ps_prev, rs, nullptr, q, p, ps, 0.0};
     const int sg = bc_kind == 1 ? 1 : -1;
-    const StencilGrid g = pair_dir_grid(n);
-    opt_in_smem(stencil_pair_dir_kernel<false>, g.smem);
-    stencil_pair_dir_kernel<false><<<g.grid, g.block, g.smem, s>>>(r, rs, p_prev, ps_prev, p, ps, q, qs, n, sg,
-                                                                   g.kz_per_cta, partials, st);
+    const StencilGrid g = step_grid<kMarchDir, false>(n);
+    if (qs == nullptr)
+        stencil_step_kernel<kMarchDir, false><<<g.grid, g.block, g.smem, s>>>(a, n, sg, g.kz_per_cta, partials, st);
+    else
+        stencil_two_field_kernel<true><<<g.grid, g.block, 0, s>>>(a, qs, n, sg, g.kz_per_cta, partials, st);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bicg_stencil_pair(const double* p, double* q, const double* ps, double* qs, int n,
-                                     int bc_kind, double* partials, BicgState* st, cudaStream_t s, bool staged) {
+                                     int bc_kind, double* partials, BicgState* st, cudaStream_t s) {
+    const MarchArrays a{p, nullptr, ps, nullptr, nullptr, q, nullptr, nullptr, 0.0};
     const int sg = bc_kind == 1 ? 1 : -1;
-    if (staged) {   // the fused schedule's first iteration: its grid
-        const StencilGrid g = pair_dir_grid(n);
-        const size_t smem = pp_smem_bytes<2>();
-        opt_in_smem(stencil_pair_kernel<false>, smem);
-        stencil_pair_kernel<false><<<g.grid, g.block, smem, s>>>(p, ps, q, qs, n, sg, g.kz_per_cta, partials, st);
-    } else {
-        const StencilGrid g = pair_grid(n);
-        opt_in_smem(stencil_pair_kernel<false>, g.smem);
-        stencil_pair_kernel<false><<<g.grid, g.block, g.smem, s>>>(p, ps, q, qs, n, sg, g.kz_per_cta, partials, st);
-    }
+    const StencilGrid g = step_grid<kMarchPair, false>(n);
+    if (qs == nullptr)
+        stencil_step_kernel<kMarchPair, false><<<g.grid, g.block, g.smem, s>>>(a, n, sg, g.kz_per_cta, partials, st);
+    else
+        stencil_two_field_kernel<false><<<g.grid, g.block, 0, s>>>(a, qs, n, sg, g.kz_per_cta, partials, st);
     return cudaGetLastError();
 }
 
 cudaError_t launch_cg_stencil(const double* p, double* q, int n, int bc_kind, double* partials, BicgState* st,
-                              cudaStream_t s, bool staged) {
-    const int sg = bc_kind == 1 ? 1 : -1;
-    if (staged) {   // the fused schedule's first iteration: its grid
-        const StencilGrid g = pair_dir_grid(n);
-        const size_t smem = pp_smem_bytes<1>();
-        opt_in_smem(stencil_pair_kernel<true>, smem);
-        stencil_pair_kernel<true><<<g.grid, g.block, smem, s>>>(p, nullptr, q, nullptr, n, sg, g.kz_per_cta, partials,
-                                                               st);
-    } else {
-        const StencilGrid g = pair_grid(n);
-        const size_t smem = pp_smem_bytes<1>();
-        opt_in_smem(stencil_pair_kernel<true>, smem);
-        stencil_pair_kernel<true><<<g.grid, g.block, smem, s>>>(p, nullptr, q, nullptr, n, sg, g.kz_per_cta, partials,
-                                                               st);
-    }
+                              cudaStream_t s) {
+    const MarchArrays a{p, nullptr, nullptr, nullptr, nullptr, q, nullptr, nullptr, 0.0};
+    const StencilGrid g = step_grid<kMarchPair, true>(n);
+    stencil_step_kernel<kMarchPair, true><<<g.grid, g.block, g.smem, s>>>(a, n, bc_kind == 1 ? 1 : -1, g.kz_per_cta,
+                                                                         partials, st);
     return cudaGetLastError();
 }
 
 cudaError_t launch_cg_stencil_dir(const double* r, const double* p_prev, double* p, double* q, int n, int bc_kind,
                                   double* partials, BicgState* st, cudaStream_t s) {
-    const int sg = bc_kind == 1 ? 1 : -1;
-    const StencilGrid g = pair_dir_grid(n);
-    const size_t smem = pp_smem_bytes<2>();
-    opt_in_smem(stencil_pair_dir_kernel<true>, smem);
-    stencil_pair_dir_kernel<true><<<g.grid, g.block, smem, s>>>(r, nullptr, p_prev, nullptr, p, nullptr, q, nullptr,
-                                                                n, sg, g.kz_per_cta, partials, st);
+    const MarchArrays a{p_prev, r, nullptr, nullptr, nullptr, q, p, nullptr, 0.0};
+    const StencilGrid g = step_grid<kMarchDir, true>(n);
+    stencil_step_kernel<kMarchDir, true><<<g.grid, g.block, g.smem, s>>>(a, n, bc_kind == 1 ? 1 : -1, g.kz_per_cta,
+                                                                        partials, st);
     return cudaGetLastError();
 }
 

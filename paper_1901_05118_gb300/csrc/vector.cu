@@ -6,7 +6,8 @@
 // walks the vectors with a grid stride, each CTA reduces its values by a
 // fixed shuffle tree, and the last CTA to finish (atomic ticket) adds the
 // per-CTA partials in CTA order.  The same inputs therefore always give the
-// same bits, independent of scheduling.
+// same bits, independent of scheduling.  Multiply-adds are written out, so
+// that every variant of a kernel rounds alike.
 #include "excmg_internal.cuh"
 #include "reduce.cuh"
 
@@ -130,6 +131,8 @@ bicg_sigma_kernel(const double* __restrict__ ps, const double* __restrict__ q, s
 // once; a thread that meets a differing entry continues with separate sums
 // from the identical partial sums it has so far.  FP64 issue is scarce on
 // GB300: this saves two of the five FMAs per entry.
+// kOneQ: A^T p* is A p bit for bit and read once, from q.
+template <bool kOneQ>
 __global__ void __launch_bounds__(kVecThreads)
 bicg_update_kernel(double* __restrict__ x, const double* __restrict__ p, double* __restrict__ r,
                    const double* __restrict__ q, double* __restrict__ rs,
@@ -142,28 +145,28 @@ bicg_update_kernel(double* __restrict__ x, const double* __restrict__ p, double*
     bool twin = true;   // so far every entry of this thread was a twin: vr == vrr
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < len;
          t += (size_t)gridDim.x * blockDim.x) {
-        x[t] = x[t] + alpha * p[t];
-        const double rv = r[t], qv = q[t], rsv = rs[t], qsv = qs[t];
-        const double rn = rv - alpha * qv;
+        x[t] = __fma_rn(alpha, p[t], x[t]);
+        const double rv = r[t], qv = q[t], rsv = rs[t], qsv = kOneQ ? qv : qs[t];
+        const double rn = __fma_rn(-alpha, qv, rv);
         r[t] = rn;
         if (__double_as_longlong(rsv) == __double_as_longlong(rv) &&
             __double_as_longlong(qsv) == __double_as_longlong(qv)) {
             rs[t] = rn;
             if (twin) {
-                vrr += rn * rn;
+                vrr = __fma_rn(rn, rn, vrr);
             } else {
-                vr += rn * rn;
-                vrr += rn * rn;
+                vr = __fma_rn(rn, rn, vr);
+                vrr = __fma_rn(rn, rn, vrr);
             }
         } else {
             if (twin) {
                 vr = vrr;
                 twin = false;
             }
-            const double rsn = rsv - alpha * qsv;
+            const double rsn = __fma_rn(-alpha, qsv, rsv);
             rs[t] = rsn;
-            vr += rsn * rn;
-            vrr += rn * rn;
+            vr = __fma_rn(rsn, rn, vr);
+            vrr = __fma_rn(rn, rn, vrr);
         }
     }
     if (twin) vr = vrr;
@@ -200,12 +203,12 @@ bicg_pupdate_kernel(double* __restrict__ p, const double* __restrict__ r, double
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < len;
          t += (size_t)gridDim.x * blockDim.x) {
         const double rv = r[t], pv = p[t], rsv = rs[t], psv = ps[t];
-        const double pn = rv + beta * pv;
+        const double pn = __fma_rn(beta, pv, rv);
         p[t] = pn;
         if (__double_as_longlong(rsv) == __double_as_longlong(rv) && __double_as_longlong(psv) == __double_as_longlong(pv))
             ps[t] = pn;
         else
-            ps[t] = rsv + beta * psv;
+            ps[t] = __fma_rn(beta, psv, rsv);
     }
 }
 
@@ -254,10 +257,10 @@ cg_update_kernel(double* __restrict__ x, const double* __restrict__ p, double* _
     double vrr = 0.0;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < len;
          t += (size_t)gridDim.x * blockDim.x) {
-        x[t] = x[t] + alpha * p[t];
-        const double rn = r[t] - alpha * q[t];
+        x[t] = __fma_rn(alpha, p[t], x[t]);
+        const double rn = __fma_rn(-alpha, q[t], r[t]);
         r[t] = rn;
-        vrr += rn * rn;
+        vrr = __fma_rn(rn, rn, vrr);
     }
     double s[2];
     s[0] = block_sum(vrr, sh);
@@ -288,7 +291,7 @@ cg_pupdate_kernel(double* __restrict__ p, const double* __restrict__ r, size_t l
     const double beta = st->beta;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < len;
          t += (size_t)gridDim.x * blockDim.x)
-        p[t] = r[t] + beta * p[t];
+        p[t] = __fma_rn(beta, p[t], r[t]);
 }
 
 }  // namespace
@@ -336,7 +339,10 @@ cudaError_t launch_bicg_sigma(const double* ps, const double* q, size_t len, dou
 cudaError_t launch_bicg_update(double* x, const double* p, double* r, const double* q, double* rs,
                                const double* qs, size_t len, double* partials, BicgState* st,
                                cudaStream_t s) {
-    bicg_update_kernel<<<kVecBlocks, kVecThreads, 0, s>>>(x, p, r, q, rs, qs, len, partials, st);
+    if (qs)
+        bicg_update_kernel<false><<<kVecBlocks, kVecThreads, 0, s>>>(x, p, r, q, rs, qs, len, partials, st);
+    else
+        bicg_update_kernel<true><<<kVecBlocks, kVecThreads, 0, s>>>(x, p, r, q, rs, qs, len, partials, st);
     return cudaGetLastError();
 }
 
