@@ -439,13 +439,23 @@ int bicg2d_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, d
     if (e != cudaSuccess) return ctx_cuda(ctx, e, "2D Bi-CG setup");
     const int sg = bc_kind == 1 ? 1 : -1;
     if (check_every < 1) check_every = 1;
+    // grids up to 512^2: many iterations per launch with every vector on chip
+    // (512^2: 10 us per iteration, three launches 31 us); larger ones, or no room
+    // for the exchange words: three launches per iteration
+    void* words = resident2d_ctas(n) > 0 ? ctx_scratch(ctx, resident2d_bytes(n)) : nullptr;
     for (;;) {
         e = ctx_read_back(ctx, ctx->host_state, ctx->state, sizeof(BicgState));
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return ctx_cuda(ctx, e, "2D Bi-CG state read");
         if (ctx->host_state->done) break;
-        int batch = check_every;
         const int left = max_iter - ctx->host_state->iter;
+        if (words) {
+            e = launch_bicg2d_resident(x, r, rs, p, ps, n, bc_kind, left < 1024 ? left : 1024, ctx->state, words, s);
+            note_launches(1);
+            if (e != cudaSuccess) return ctx_cuda(ctx, e, "cooperative 2D Bi-CG launch");
+            continue;
+        }
+        int batch = check_every;
         if (batch > left) batch = left;
         for (int it = 0; it < batch && e == cudaSuccess; ++it) {
             stencil2d_kernel<2, true><<<g, dim3(Q_TX, Q_TY), 0, s>>>(p, ps, q, qs, nullptr, n, sg, ctx->partials,
@@ -463,6 +473,8 @@ int bicg2d_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, d
     if (relres_out) *relres_out = bnorm > 0.0 ? rn / bnorm : rn;
     if (!std::isfinite(h.rr)) return ctx_fail(ctx, EXCMG_ERR_NAN, "2D Bi-CG residual is not finite");
     if (h.status == kBreakdown) return ctx_fail(ctx, EXCMG_ERR_BREAKDOWN, "2D Bi-CG breakdown");
+    if (h.status == kTimeout)
+        return ctx_fail(ctx, EXCMG_ERR_TIMEOUT, "an exchange of the cooperative 2D Bi-CG gave up");
     if (h.status == kCapped) return EXCMG_ERR_NOCONV;
     return EXCMG_OK;
 }

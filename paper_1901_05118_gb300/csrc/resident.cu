@@ -9,31 +9,35 @@
 namespace excmg {
 namespace {
 
-template <typename T, bool kElide>
+template <typename T, int DIM, bool kElide>
 const void* resident_fn(int np) {
     switch (np) {
-        case 1: return (const void*)resident_bicg_kernel<T, 1, 2, kElide>;
-        case 2: return (const void*)resident_bicg_kernel<T, 2, 3, kElide>;
-        default: return (const void*)resident_bicg_kernel<T, 4, 5, kElide>;
+        case 1: return (const void*)resident_bicg_kernel<T, DIM, 1, DIM == 3 ? 2 : 1, kElide>;
+        case 2: return (const void*)resident_bicg_kernel<T, DIM, 2, DIM == 3 ? 3 : 1, kElide>;
+        default: return (const void*)resident_bicg_kernel<T, DIM, 4, DIM == 3 ? 5 : 1, kElide>;
     }
 }
 
 std::mutex g_geom_mu;
-std::map<std::pair<int, int>, ResidentGeom> g_geom;   // at most one entry per size and CTA limit
+std::map<std::pair<int, int>, ResidentGeom> g_geom;   // one entry per size (2D: negative) and CTA limit
 
 }  // namespace
 
-ResidentGeom resident_geometry_cached(int n, int max_ctas) {
+ResidentGeom resident_geometry_cached(int dim, int n, int max_ctas) {
     std::lock_guard<std::mutex> lock(g_geom_mu);
-    auto it = g_geom.find({n, max_ctas});
-    if (it == g_geom.end()) it = g_geom.emplace(std::make_pair(n, max_ctas), resident_geometry(n, max_ctas)).first;
+    const auto key = std::make_pair(dim == 3 ? n : -n, max_ctas);
+    auto it = g_geom.find(key);
+    if (it == g_geom.end())
+        it = g_geom.emplace(key, dim == 3 ? resident_geometry(n, max_ctas) : resident_geometry2d(n, max_ctas)).first;
     return it->second;
 }
 
 int resident_ctas(int n, int max_ctas) {
     if (n > kPersistentMaxN) return 0;
-    return resident_geometry_cached(n, max_ctas > 0 ? max_ctas : device_sms()).ctas;
+    return resident_geometry_cached(3, n, max_ctas > 0 ? max_ctas : device_sms()).ctas;
 }
+
+int resident2d_ctas(int n) { return n > kPersistentMaxN2d ? 0 : resident_geometry_cached(2, n, device_sms()).ctas; }
 
 // CTAs of a grid in the batch engine: fewer than a single solve takes, so that several instances run side by
 // side, and a number that depends on the grid alone (the sums do, too).  32^3 on 16 CTAs takes about 1.5
@@ -53,23 +57,37 @@ unsigned next_serial() {
 }  // namespace
 
 size_t resident_bytes(int n) { return slot_bytes() + node_count(n) * sizeof(ulonglong2); }
+size_t resident2d_bytes(int n) { return slot_bytes() + (size_t)(n + 1) * (n + 1) * sizeof(ulonglong2); }
 
+namespace {
 template <typename T>
-cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
-                                 void* words, cudaStream_t s, bool elide, int max_ctas) {
-    ResidentGeom g = resident_geometry_cached(n, max_ctas > 0 ? max_ctas : device_sms());
-    ResidentInst<T> in{x, r, rs, p, ps, st, (ulonglong2*)words, (ulonglong2*)((char*)words + slot_bytes()), n, bc_kind == 1 ? 1 : -1};
+cudaError_t launch(const void* fn, ResidentGeom g, T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters,
+                   BicgState* st, void* words, cudaStream_t s) {
+    ResidentInst<T> in{x, r, rs, p, ps, st, (ulonglong2*)words, (ulonglong2*)((char*)words + slot_bytes()), n,
+                       bc_kind == 1 ? 1 : -1};
     const size_t smem = (size_t)g.tile * (sizeof(T) == 8 ? sizeof(long long) : sizeof(float));
-    const void* fn;
-    if constexpr (sizeof(T) == 8)
-        fn = elide ? resident_fn<T, true>(g.np) : resident_fn<T, false>(g.np);
-    else
-        fn = resident_fn<T, false>(g.np);
     (void)kernel_occupancy(fn, kResThreads, kResTileBytes);   // opts in to the shared memory
     unsigned serial = next_serial();
     long long limit = kBarrierSpinLimit;
     void* args[] = {&in, &g, &iters, &serial, &limit};
     return cudaLaunchCooperativeKernel(fn, dim3(g.ctas), dim3(kResThreads), args, smem, s);
+}
+}  // namespace
+
+template <typename T>
+cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
+                                 void* words, cudaStream_t s, bool elide, int max_ctas) {
+    const ResidentGeom g = resident_geometry_cached(3, n, max_ctas > 0 ? max_ctas : device_sms());
+    const void* fn = resident_fn<T, 3, false>(g.np);
+    if constexpr (sizeof(T) == 8)
+        if (elide) fn = resident_fn<T, 3, true>(g.np);
+    return launch<T>(fn, g, x, r, rs, p, ps, n, bc_kind, iters, st, words, s);
+}
+
+cudaError_t launch_bicg2d_resident(double* x, double* r, double* rs, double* p, double* ps, int n, int bc_kind,
+                                   int iters, BicgState* st, void* words, cudaStream_t s) {
+    const ResidentGeom g = resident_geometry_cached(2, n, device_sms());
+    return launch<double>(resident_fn<double, 2, false>(g.np), g, x, r, rs, p, ps, n, bc_kind, iters, st, words, s);
 }
 
 template cudaError_t launch_bicg_resident<double>(double*, double*, double*, double*, double*, int, int, int,

@@ -29,13 +29,17 @@
 //    and no FP64 comparisons: they go through the same pipe;
 //  * outputs rounded with integer instructions (fx_result).
 // Measured: 200 iterations on 64^3 2.23 ms (the general cooperative kernel:
-// 5.63 ms), a whole 32^3 first-kind solve to 1e-10 5.4 ms (14.8 ms).
+// 5.63 ms), a whole 32^3 first-kind solve to 1e-10 5.4 ms (14.8 ms); 100
+// iterations of the 512^2 problem 1.00 ms (three launches each: 3.08 ms).
 //
 // Shadow sequence: the launches start from r*_0 = p*_0 = r_0 = p_0 (a
 // caller-chosen r*_0 takes the general kernel in stencil.cu).  A^T p* is A p
 // bit for bit where p* = p (march_fx.cuh), so q serves both; r* and p* are
 // updated entry by entry, with the primal result reused where the operands
 // agree bit for bit.  kElide: r*, p* are not kept (the same bits).
+//
+// DIM = 2: the 2D problem's 13-point rows (excmg2d.cu), with the second axis in
+// the place of z and no third one.
 //
 // T = float: the FP32 correction solves of the mixed-precision mode.  The
 // operator sums in FP32, inner products are FP32 inside a CTA and combined in
@@ -140,8 +144,8 @@ __device__ __forceinline__ float sum_f32(float v) {
     return v;
 }
 
-// NP: nodes of a thread's z-run; NH: nodes around the brick per thread.
-template <typename T, int NP, int NH, bool kElide>
+// NP: nodes of a thread's run along z; NH: nodes around the brick per thread.
+template <typename T, int DIM, int NP, int NH, bool kElide>
 __global__ void __launch_bounds__(kResThreads, 1)
 resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
                      unsigned serial, long long spin_limit) {
@@ -158,7 +162,7 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
     if (st->done) return;
     const int cta = (int)blockIdx.x, G = g.ctas, n = in.n, np = n + 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int plane = np * np;
+    const int plane = DIM == 3 ? np * np : np;
 
     // this thread's nodes: NP along z at one (x, y) of the brick
     const int kx = cta % g.cx, ky = (cta / g.cx) % g.cy, kz = cta / (g.cx * g.cy);
@@ -169,20 +173,22 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
     const int nz = min(g.bz, n - oz);            // planes of the brick
     const bool mine = lz < nz && ox + lx < n && oy + ly < n;
     const int cnt = mine ? min(NP, nz - lz) : 0;   // this thread's nodes
-    const int idx0 = mine ? ((oz + lz) * np + oy + ly) * np + ox + lx : 0;
-    const int tx = g.tx, tp = tx * (g.by + 4);
-    const int t0 = (lz + 2) * tp + (ly + 2) * tx + lx + 2;   // tile entry of the first one
+    const int idx0 = !mine ? 0 : DIM == 3 ? ((oz + lz) * np + oy + ly) * np + ox + lx : (oz + lz) * np + ox + lx;
+    const int tx = g.tx, tp = DIM == 3 ? tx * (g.by + 4) : tx;
+    const int t0 = (lz + 2) * tp + (DIM == 3 ? (ly + 2) * tx : 0) + lx + 2;   // tile entry of the first one
     int cc[NP];
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
         const int i = ox + lx, j = oy + ly, z = oz + lz + k;
-        cc[k] = in.sigma * ((i == 1) + (i == n - 1) + (j == 1) + (j == n - 1) + (z == 1) + (z == n - 1));
+        const int cy = DIM == 3 ? (j == 1) + (j == n - 1) : 0;
+        cc[k] = in.sigma * ((i == 1) + (i == n - 1) + cy + (z == 1) + (z == n - 1));
     }
     // nodes of this thread that other bricks' taps reach
     unsigned surf = 0u;
 #pragma unroll
     for (int k = 0; k < NP; ++k)
-        if (k < cnt && (lx < 2 || lx >= g.bx - 2 || ly < 2 || ly >= g.by - 2 || lz + k < 2 || lz + k >= g.bz - 2))
+        if (k < cnt && (lx < 2 || lx >= g.bx - 2 || (DIM == 3 && (ly < 2 || ly >= g.by - 2)) || lz + k < 2 ||
+                        lz + k >= g.bz - 2))
             surf |= 1u << k;
     // nodes around the brick, on the warps from 1 up (warp 0 has the
     // exchanges): node index (-1: none, or outside the interior), tile entry
@@ -193,11 +199,13 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
         hidx[k] = -1;
         htile[k] = 0;
         if (tid >= 32 && h < g.halo) {
-            int hx, hy, hz;
-            res_halo(h, g.bx, g.by, g.bz, &hx, &hy, &hz);
+            int hx, hy = 0, hz;
+            if (DIM == 3) res_halo(h, g.bx, g.by, g.bz, &hx, &hy, &hz);
+            else res_halo2(h, g.bx, g.bz, &hx, &hz);
             const int i = ox + hx, j = oy + hy, z = oz + hz;
-            if (i >= 1 && i < n && j >= 1 && j < n && z >= 1 && z < n) hidx[k] = (z * np + j) * np + i;
-            htile[k] = (hz + 2) * tp + (hy + 2) * tx + hx + 2;
+            if (i >= 1 && i < n && j >= 1 && j < n && z >= 1 && z < n)
+                hidx[k] = DIM == 3 ? (z * np + j) * np + i : z * np + i;
+            htile[k] = (hz + 2) * tp + (DIM == 3 ? (hy + 2) * tx : 0) + hx + 2;
         }
     }
     for (int t = tid; t < g.tile; t += kResThreads) tile[t] = Fix(0);
@@ -338,8 +346,9 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
                     tile[htile[k]] = hp[k];
             }
         __syncthreads();
-        // q = A p: the four axis neighbours' sum of a plane serves its own
-        // row (-12) and the rows above and below (+2)
+        // q = A p: the sum of the axis neighbours inside a plane (DIM = 2: row)
+        // serves its own row (-12, -8) and the rows above and below (+2)
+        constexpr int kCentre = DIM == 3 ? 42 : 20, kNear = DIM == 3 ? 12 : 8;
         T dot = T(0);
         if (cnt > 0) {
             Fix u[NP + 4], s4[NP + 2];
@@ -348,23 +357,26 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
 #pragma unroll
             for (int k = 0; k < NP + 2; ++k) {
                 const int o = t0 + (k - 1) * tp;
-                s4[k] = (tile[o - 1] + tile[o + 1]) + (tile[o - tx] + tile[o + tx]);
+                s4[k] = tile[o - 1] + tile[o + 1];
+                if (DIM == 3) s4[k] += tile[o - tx] + tile[o + tx];
             }
 #pragma unroll
             for (int k = 0; k < NP; ++k) {
                 const int o = t0 + k * tp;
-                const Fix f4 = (tile[o - 2] + tile[o + 2]) + (tile[o - 2 * tx] + tile[o + 2 * tx]);
-                const Fix d4 = (tile[o - tx - 1] + tile[o - tx + 1]) + (tile[o + tx - 1] + tile[o + tx + 1]);
                 const Fix n6 = s4[k + 1] + (u[k + 1] + u[k + 3]);
-                const Fix f6 = f4 + (u[k] + u[k + 4]);
-                const Fix d12 = d4 + (s4[k] + s4[k + 2]);
+                Fix f6 = (tile[o - 2] + tile[o + 2]) + (u[k] + u[k + 4]);
+                Fix d12 = s4[k] + s4[k + 2];
+                if (DIM == 3) {
+                    f6 += tile[o - 2 * tx] + tile[o + 2 * tx];
+                    d12 += (tile[o - tx - 1] + tile[o - tx + 1]) + (tile[o + tx - 1] + tile[o + tx + 1]);
+                }
                 if (k < cnt) {
                     if constexpr (kExact) {
                         const long long acc =
-                            mul_w(u[k + 2], (unsigned)(42 + cc[k])) - mul_w(n6, 12u) + f6 + (d12 + d12);
+                            mul_w(u[k + 2], (unsigned)(kCentre + cc[k])) - mul_w(n6, (unsigned)kNear) + f6 + (d12 + d12);
                         q[k] = fx_result(acc, E, E == 0x7FF);
                     } else {
-                        q[k] = mad(42.f + (float)cc[k], u[k + 2], mad(-12.f, n6, mad(2.f, d12, f6)));
+                        q[k] = mad((float)(kCentre + cc[k]), u[k + 2], mad(-(float)kNear, n6, mad(2.f, d12, f6)));
                     }
                     dot = mad(kElide ? p[k] : ps[k], q[k], dot);
                 }

@@ -92,6 +92,26 @@ EXCMG_HD void res_halo(int h, int bx, int by, int bz, int* lx, int* ly, int* lz)
     *ly = (l & 2) ? by : -1;
 }
 
+// The same in two dimensions (DIM = 2: x and z), corners at (+-1, +-1).
+EXCMG_HD void res_halo2(int h, int bx, int bz, int* lx, int* lz) {
+    if (h < 4 * bx) {
+        const int l = h / bx;
+        *lx = h - l * bx;
+        *lz = l < 2 ? l - 2 : bz + l - 2;
+        return;
+    }
+    h -= 4 * bx;
+    if (h < 4 * bz) {
+        const int l = h & 3;
+        *lz = h >> 2;
+        *lx = l < 2 ? l - 2 : bx + l - 2;
+        return;
+    }
+    h -= 4 * bz;
+    *lx = (h & 1) ? bx : -1;
+    *lz = (h & 2) ? bz : -1;
+}
+
 // The cut of a grid with n intervals into at most max_ctas bricks that fits
 // the kernel's variants, and of those the cheapest iteration.  Cost in
 // half cycles: five FP64 instructions for each of a thread's own nodes (p,
@@ -127,6 +147,34 @@ inline ResidentGeom resident_geometry(int n, int max_ctas) {
                         best_cost = cost;
                         best = ResidentGeom{cx, cy, cz, bx, by, bz, np, nh, halo, bx + kResPad, tile, cx * cy * cz};
                     }
+                }
+            }
+        }
+    }
+    return best;
+}
+
+// The same for a 2D grid (y empty; at most one node around the brick per thread).
+inline ResidentGeom resident_geometry2d(int n, int max_ctas) {
+    ResidentGeom best{};
+    long long best_cost = -1;
+    const int m = n - 1;
+    if (max_ctas > kResMaxCtas) max_ctas = kResMaxCtas;
+    for (int cx = 1; cx <= m && cx <= max_ctas; ++cx) {
+        const int bx = (m + cx - 1) / cx;
+        if ((m + bx - 1) / bx != cx) continue;
+        for (int cz = 1; cz <= m && cx * cz <= max_ctas; ++cz) {
+            const int bz = (m + cz - 1) / cz;
+            if ((m + bz - 1) / bz != cz) continue;
+            const int halo = 4 * (bx + bz) + 4, nh = 1;
+            for (int np = 1; np <= 4; np *= 2) {
+                const int threads = bx * ((bz + np - 1) / np), runs = (bz + np - 1) / np * np;
+                const int tile = (bx + kResPad) * (runs + 4);
+                if (threads > kResThreads || halo > nh * kResHaloThreads || (size_t)tile * 8 > kResTileBytes) continue;
+                const long long cost = 5LL * np * ((threads + 127) / 128) * 128 + halo + 40LL * cx * cz;
+                if (best_cost < 0 || cost < best_cost) {
+                    best_cost = cost;
+                    best = ResidentGeom{cx, 1, cz, bx, 1, bz, np, nh, halo, bx + kResPad, tile, cx * cz};
                 }
             }
         }

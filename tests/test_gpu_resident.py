@@ -43,6 +43,20 @@ def test_iterates_match_the_oracle(n, bc_kind, iters):
     assert rel_max(x.cpu().numpy(), xr) <= 1e-10
 
 
+@pytest.mark.parametrize("n,bc_kind,iters", [(4, 2, 5), (9, 1, 20), (31, 2, 20), (97, 1, 20), (200, 2, 20),
+                                             (333, 1, 20), (512, 2, 20), (513, 1, 20)])
+def test_2d_iterates_match_the_oracle(n, bc_kind, iters):
+    """The 2D form, up to its largest grid and one beyond it."""
+    b = P.random_field_2d(n, 305)
+    x0 = P.random_field_2d(n, 306) * 0.1
+    x = dev(x0)
+    it, rel, _ = B.bicg_solve2d(n, bc_kind, dev(b), x, 0.0, iters)
+    xr, itr, relr, _ = oracle.bicg2d(n, bc_kind, b, x0, 0.0, max_iter=iters)
+    assert it == itr == iters
+    assert rel == pytest.approx(relr, rel=1e-8)
+    assert rel_max(x.cpu().numpy(), xr) <= 1e-10
+
+
 def test_call_longer_than_one_launch():
     """1100 iterations of one call (a launch takes up to 1024): the residual
     of the recurrence, carried over from launch to launch, is still the true

@@ -68,6 +68,52 @@ int main() {
         for (int s : seen)
             if (s != 1) fail("cover", n);
     }
+    // 2D: the same with the second axis as z
+    for (int n = 4; n <= 520; n += n < 70 ? 1 : 25) {
+        const ResidentGeom g = resident_geometry2d(n, 152);
+        if (g.ctas == 0) {
+            if (n <= 512) fail("no 2D cut", n);
+            continue;
+        }
+        if (g.ctas != g.cx * g.cz || g.ctas > 152 || g.bx * ((g.bz + g.np - 1) / g.np) > kResThreads ||
+            g.halo > g.nh * kResHaloThreads) fail("2D threads", n);
+        const int m = n - 1, tx = g.tx;
+        std::vector<int> seen((size_t)m * m, 0);
+        for (int cta = 0; cta < g.ctas; ++cta) {
+            const int ox = 1 + cta % g.cx * g.bx, oz = 1 + cta / g.cx * g.bz, nz = g.bz < n - oz ? g.bz : n - oz;
+            std::vector<char> wr(g.tile, 0);
+            for (int h = 0; h < g.halo; ++h) {
+                int x, z;
+                res_halo2(h, g.bx, g.bz, &x, &z);
+                const int t = (z + 2) * tx + x + 2;
+                if (t < 0 || t >= g.tile || wr[t]++) fail("2D halo entry", n);
+            }
+            for (int pass = 0; pass < 2; ++pass)
+            for (int tid = 0; tid < kResThreads; ++tid) {
+                const int lz = tid / g.bx * g.np, lx = tid % g.bx, t0 = (lz + 2) * tx + lx + 2;
+                if (!(lz < nz && ox + lx < n)) continue;
+                if (t0 - 2 * tx - 2 < 0 || t0 + (g.np + 1) * tx >= g.tile || t0 + g.np * tx + 1 >= g.tile)
+                    fail("2D read outside the tile", n);
+                for (int k = 0; k < g.np && lz + k < nz; ++k) {
+                    const int t = t0 + k * tx, X = ox + lx, Z = oz + lz + k;
+                    if (pass == 0) {
+                        if (t >= g.tile || wr[t]++) fail("2D own entry", n);
+                        ++seen[(size_t)(Z - 1) * m + X - 1];
+                        continue;
+                    }
+                    const int d[][2] = {{1,0},{2,0},{0,1},{0,2},{1,1},{1,-1}};
+                    for (auto& v : d)
+                        for (int s = -1; s <= 1; s += 2) {
+                            const int a = X + s * v[0], c = Z + s * v[1];
+                            if (a < 1 || a > m || c < 1 || c > m) continue;
+                            if (!wr[t + s * (v[1] * tx + v[0])]) fail("2D tap not in the tile", n);
+                        }
+                }
+            }
+        }
+        for (int s : seen)
+            if (s != 1) fail("2D cover", n);
+    }
     return 0;
 }
 """
