@@ -35,62 +35,115 @@ struct Src {
 
 __device__ __forceinline__ bool on_boundary(int v, int n) { return v == 0 || v == n; }
 
-__global__ void assemble_rhs_kernel(double* __restrict__ fh, int n, int bc_kind,
-                                    const double* __restrict__ f, Src src) {
-    const int np = n + 1;
-    const size_t total = (size_t)np * np * np;
-    const double h = 1.0 / (double)n;
-    const double h4 = h * h * h * h;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t % np);
-        const int j = (int)((t / np) % np);
-        const int k = (int)(t / ((size_t)np * np));
-        if (i < 1 || i > n - 1 || j < 1 || j > n - 1 || k < 1 || k > n - 1) {
-            fh[t] = 0.0;
-            continue;
-        }
-        double rhs = h4 * f[((size_t)(k * src.stride) * src.np_src + (size_t)(j * src.stride)) * src.np_src +
-                            (size_t)(i * src.stride)];
-        if (i >= 3 && i <= n - 3 && j >= 3 && j <= n - 3 && k >= 3 && k <= n - 3) {
-            fh[t] = rhs;
-            continue;
-        }
-        const int p[3] = {i, j, k};
-        double moved = 0.0;
-        // axis taps: +-1 (weight -12) and +-2 (weight +1)
-        for (int ax = 0; ax < 3; ++ax) {
-            for (int s = -1; s <= 1; s += 2) {
-                int q[3] = {p[0], p[1], p[2]};
-                q[ax] = p[ax] + s;
-                if (on_boundary(q[ax], n)) moved += -12.0 * src.node(q[0], q[1], q[2]);
-                q[ax] = p[ax] + 2 * s;
-                if (on_boundary(q[ax], n)) {
-                    moved += src.node(q[0], q[1], q[2]);
-                } else if (q[ax] < 0 || q[ax] > n) {
-                    int bnode[3] = {p[0], p[1], p[2]};
-                    bnode[ax] = s < 0 ? 0 : n;
-                    const int face = 2 * ax + (s < 0 ? 0 : 1);
-                    const double g2v = src.face(face, bnode[0], bnode[1], bnode[2]);
-                    if (bc_kind == 1)
-                        moved += 2.0 * h * g2v;
-                    else
-                        moved += 2.0 * src.node(bnode[0], bnode[1], bnode[2]) + h * h * g2v;
-                }
+// f_h at the interior node (i, j, k): h^4 f minus what the 25 taps move over.
+__device__ __forceinline__ double rhs_near_boundary(int i, int j, int k, int n, int bc_kind, double h, double rhs,
+                                                    const Src& src) {
+    const int p[3] = {i, j, k};
+    double moved = 0.0;
+    // axis taps: +-1 (weight -12) and +-2 (weight +1)
+    for (int ax = 0; ax < 3; ++ax) {
+        for (int s = -1; s <= 1; s += 2) {
+            int q[3] = {p[0], p[1], p[2]};
+            q[ax] = p[ax] + s;
+            if (on_boundary(q[ax], n)) moved += -12.0 * src.node(q[0], q[1], q[2]);
+            q[ax] = p[ax] + 2 * s;
+            if (on_boundary(q[ax], n)) {
+                moved += src.node(q[0], q[1], q[2]);
+            } else if (q[ax] < 0 || q[ax] > n) {
+                int bnode[3] = {p[0], p[1], p[2]};
+                bnode[ax] = s < 0 ? 0 : n;
+                const int face = 2 * ax + (s < 0 ? 0 : 1);
+                const double g2v = src.face(face, bnode[0], bnode[1], bnode[2]);
+                if (bc_kind == 1)
+                    moved += 2.0 * h * g2v;
+                else
+                    moved += 2.0 * src.node(bnode[0], bnode[1], bnode[2]) + h * h * g2v;
             }
         }
-        // in-plane diagonal taps (weight +2)
-        for (int a = 0; a < 3; ++a)
-            for (int b = a + 1; b < 3; ++b)
-                for (int sa = -1; sa <= 1; sa += 2)
-                    for (int sb = -1; sb <= 1; sb += 2) {
-                        int q[3] = {p[0], p[1], p[2]};
-                        q[a] += sa;
-                        q[b] += sb;
-                        if (on_boundary(q[0], n) || on_boundary(q[1], n) || on_boundary(q[2], n))
-                            moved += 2.0 * src.node(q[0], q[1], q[2]);
-                    }
-        fh[t] = rhs - moved;
+    }
+    // in-plane diagonal taps (weight +2)
+    for (int a = 0; a < 3; ++a)
+        for (int b = a + 1; b < 3; ++b)
+            for (int sa = -1; sa <= 1; sa += 2)
+                for (int sb = -1; sb <= 1; sb += 2) {
+                    int q[3] = {p[0], p[1], p[2]};
+                    q[a] += sa;
+                    q[b] += sb;
+                    if (on_boundary(q[0], n) || on_boundary(q[1], n) || on_boundary(q[2], n))
+                        moved += 2.0 * src.node(q[0], q[1], q[2]);
+                }
+    return rhs - moved;
+}
+
+// h^4 f at the nodes that no boundary value reaches, zero on the boundary;
+// kNear: the nodes within two of a face as well (small grids: one launch).
+// A thread takes kPlanes nodes of one (x, y) column.  One index per node with
+// 64-bit divisions, and the boundary rows in the same launch, took 1.14 ms
+// at 512^3: the first and the last warp of every row waited for the taps
+// of four nodes.
+constexpr int kPlanes = 8;
+template <bool kNear>
+__global__ void __launch_bounds__(256)
+assemble_rhs_kernel(double* __restrict__ fh, int n, int bc_kind, const double* __restrict__ f, Src src) {
+    const int np = n + 1;
+    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y;
+    if (i > n || j > n) return;
+    const double h = 1.0 / (double)n;
+    const double h4 = h * h * h * h;
+    const int kz = blockIdx.z * kPlanes;
+    const bool in_xy = i >= 1 && i <= n - 1 && j >= 1 && j <= n - 1;
+    const bool deep_xy = i >= 3 && i <= n - 3 && j >= 3 && j <= n - 3;
+    double v[kPlanes];
+#pragma unroll
+    for (int c = 0; c < kPlanes; ++c) {
+        const int k = kz + c;
+        v[c] = in_xy && k >= 1 && k <= n - 1
+                   ? f[((size_t)(k * src.stride) * src.np_src + (size_t)(j * src.stride)) * src.np_src +
+                       (size_t)(i * src.stride)]
+                   : 0.0;
+    }
+#pragma unroll
+    for (int c = 0; c < kPlanes; ++c) {
+        const int k = kz + c;
+        if (k > n) break;
+        const size_t t = ((size_t)k * np + j) * np + i;
+        const bool inside = in_xy && k >= 1 && k <= n - 1;
+        const bool deep = deep_xy && k >= 3 && k <= n - 3;
+        if (!inside || deep) fh[t] = h4 * v[c];
+        else if (kNear) fh[t] = rhs_near_boundary(i, j, k, n, bc_kind, h, h4 * v[c], src);
+    }
+}
+
+// The nodes within two of a face, n >= 9: the layers 1, 2, n - 2, n - 1 along z,
+// then those along y of the planes between, then those along x of what is left.
+__global__ void __launch_bounds__(256)
+assemble_near_kernel(double* __restrict__ fh, int n, int bc_kind, const double* __restrict__ f, Src src) {
+    const int np = n + 1, m = n - 1, q = m - 4;
+    const int nz = 4 * m * m, ny = q * 4 * m, total = nz + ny + q * q * 4;
+    const double h = 1.0 / (double)n;
+    const double h4 = h * h * h * h;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        int i, j, k;
+        auto layer = [&](int l) { return l < 2 ? 1 + l : n - 4 + l; };
+        if (t < nz) {
+            const int l = t / (m * m), e = t - l * m * m;
+            k = layer(l);
+            j = 1 + e / m;
+            i = e - (j - 1) * m + 1;
+        } else if (t < nz + ny) {
+            const int e = t - nz, z = e / (4 * m), r = e - z * 4 * m, l = r / m;
+            k = 3 + z;
+            j = layer(l);
+            i = r - l * m + 1;
+        } else {
+            const int e = t - nz - ny, z = e / (4 * q), r = e - z * 4 * q;
+            k = 3 + z;
+            j = 3 + (r >> 2);
+            i = layer(r & 3);
+        }
+        const double rhs = h4 * f[((size_t)(k * src.stride) * src.np_src + (size_t)(j * src.stride)) * src.np_src +
+                                  (size_t)(i * src.stride)];
+        fh[((size_t)k * np + j) * np + i] = rhs_near_boundary(i, j, k, n, bc_kind, h, rhs, src);
     }
 }
 
@@ -111,6 +164,9 @@ __global__ void set_boundary_kernel(double* __restrict__ u, int n, Src src) {
     }
 }
 
+// One launch up to here: a second one costs more than the warps that wait in the first.
+constexpr int kOneLaunchMaxN = 64;
+
 int grid_for(size_t work) {
     size_t b = (work + 255) / 256;
     if (b > 152 * 16) b = 152 * 16;
@@ -123,7 +179,14 @@ int grid_for(size_t work) {
 cudaError_t launch_assemble_rhs(double* fh, int n, int bc_kind, const double* f, const double* g1,
                                 const double* g2, int stride, cudaStream_t s) {
     Src src{g1, g2, n * stride + 1, stride};
-    assemble_rhs_kernel<<<grid_for(node_count(n)), 256, 0, s>>>(fh, n, bc_kind, f, src);
+    const dim3 grid((n + 32) / 32, (n + 8) / 8, (n + kPlanes) / kPlanes), block(32, 8);
+    if (n <= kOneLaunchMaxN) {
+        assemble_rhs_kernel<true><<<grid, block, 0, s>>>(fh, n, bc_kind, f, src);
+        return cudaGetLastError();
+    }
+    assemble_rhs_kernel<false><<<grid, block, 0, s>>>(fh, n, bc_kind, f, src);
+    const size_t near = 4 * ((size_t)(n - 1) * (n - 1) + (size_t)(n - 5) * (n - 1) + (size_t)(n - 5) * (n - 5));
+    assemble_near_kernel<<<grid_for(near), 256, 0, s>>>(fh, n, bc_kind, f, src);
     return cudaGetLastError();
 }
 

@@ -7,8 +7,8 @@
 // 2 face diagonals / 4 space diagonals.  All four are one formula,
 //     W = u1 + (1/4) * (mean of d = u1 - u0 over the 2^m coarse nodes
 //                       around the node, m = number of odd coordinates),
-// which the first kernel evaluates once per middle-grid node (shared cells
-// agree by construction).  Step 5 is tri-quadratic Lagrange interpolation
+// which is EXP_true's formula with 1/4 in the place of 1/3 (one kernel serves
+// both; shared cells agree by construction).  Step 5 is tri-quadratic Lagrange interpolation
 // (eqs. (inter)-(iinter)) of W at the fine nodes: per axis the natural
 // coordinate 0, 1/4, 1/2, 3/4, 1 has weights (1,0,0), (3/8,3/4,-1/8),
 // (0,1,0), (-1/8,3/4,3/8), (0,0,1) on the cell's three middle-grid nodes.
@@ -27,183 +27,131 @@ __device__ __forceinline__ size_t nidx(int np, int i, int j, int k) {
     return ((size_t)k * np + j) * np + i;
 }
 
-// coarse indices around fine index v on one axis: 1 (v even) or 2 (v odd)
-__device__ __forceinline__ int around(int v, int* c) {
-    if (v & 1) {
-        c[0] = (v - 1) >> 1;
-        c[1] = (v + 1) >> 1;
-        return 2;
-    }
-    c[0] = v >> 1;
-    return 1;
-}
-
-__global__ void exp_finite_w_kernel(double* __restrict__ W, const double* __restrict__ u1,
-                                    const double* __restrict__ u0, int n1) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int k = blockIdx.z;
-    const int np1 = n1 + 1, np0 = n1 / 2 + 1;
-    if (i >= np1 || j >= np1 || k >= np1) return;
-    int ci[2], cj[2], ck[2];
-    const int ni = around(i, ci), nj = around(j, cj), nk = around(k, ck);
-    double sum = 0.0;
-    for (int c = 0; c < nk; ++c)
-        for (int b = 0; b < nj; ++b)
-            for (int a = 0; a < ni; ++a)
-                sum += u1[nidx(np1, 2 * ci[a], 2 * cj[b], 2 * ck[c])] - u0[nidx(np0, ci[a], cj[b], ck[c])];
-    // 1/(4 * 2^m), m = number of odd coordinates: a power of two, so the
-    // product is exact; an FP64 division would cost many of GB300's scarce
-    // FP64 instructions per node
-    const int m = (i & 1) + (j & 1) + (k & 1);
-    const double w = m == 0 ? 0.25 : (m == 1 ? 0.125 : (m == 2 ? 0.0625 : 0.03125));
-    W[nidx(np1, i, j, k)] = u1[nidx(np1, i, j, k)] + sum * w;
-}
-
-// Lagrange weights on the cell's middle-grid nodes for local offset o (0..4)
-__device__ __forceinline__ int quad_weights(int v, int n0, int* idx, double* w) {
-    int c = v >> 2;
-    if (c > n0 - 1) c = n0 - 1;
-    const int o = v - 4 * c;
-    if ((o & 1) == 0) {
-        idx[0] = 2 * c + (o >> 1);
-        w[0] = 1.0;
-        return 1;
-    }
-    idx[0] = 2 * c;
-    idx[1] = 2 * c + 1;
-    idx[2] = 2 * c + 2;
-    if (o == 1) { w[0] = 0.375; w[1] = 0.75; w[2] = -0.125; }
-    else { w[0] = -0.125; w[1] = 0.75; w[2] = 0.375; }
-    return 3;
-}
-
-// Tiled, separable forms of the two fine-grid passes.  A CTA of 32 x 8
-// threads owns a tile of TX x TY x TZ fine nodes; the coarse values its
-// nodes need are staged in shared memory and interpolated along x, then y,
-// then z, so each intermediate value is formed once instead of once per
-// fine node that uses it (about 4 instead of 14 FP64 operations per node for
-// Step 5; FP64 issue is scarce on GB300).
+// Both passes work on tiles of 32 x 8 x 8 fine nodes, one CTA of 32 x 8
+// threads each.  The coarser values that a tile needs (17 x 5 x 5) go through
+// shared memory, are interpolated along x there, and along y and z in the
+// registers of the thread that owns a fine (x, y) column of the tile, so that
+// every intermediate value is formed once per tile.  What bounds them: FP64
+// issue (a warp instruction takes 64 cycles of an SM sub-partition whatever
+// its active lanes), then the stores; the integer index arithmetic is kept to
+// constant divisors.
 constexpr int TT_X = 32, TT_Y = 8, TT_Z = 8;
 constexpr int TT_THREADS = 256;
 constexpr int TM_X = TT_X / 2 + 1, TM_Y = TT_Y / 2 + 1, TM_Z = TT_Z / 2 + 1;   // coarse extents (17, 5, 5)
 
-// Middle-grid cell of fine index v (Step 5 uses cells of 4 fine intervals).
-__device__ __forceinline__ int quad_cell(int v, int n0) { return min(v >> 2, n0 - 1); }
-
-// Step 5 at every fine node of the tile: per fine node the same products and
-// sums, in the same order, as the direct tri-quadratic sum with x innermost,
-// then y, then z.
+// out = u + kWeight * (mean of d = u - uc over the 1, 2, 4 or 8 coarse nodes
+// around each node), u on the grid with nf intervals, uc on the one with nf / 2:
+// EXP_true with weight 1/3, Steps 1-4 of EXP_finite with weight 1/4
+// (kQuarter), where every scaling is a power of two.
+// Measured on 256^3 (42 us of HBM traffic): see launch_exp_true.
+template <bool kQuarter>
 __global__ void __launch_bounds__(TT_THREADS)
-exp_finite_interp_tiled_kernel(double* __restrict__ w, const double* __restrict__ W, int nf) {
-    __shared__ double Ws[TM_Z][TM_Y][TM_X];
-    __shared__ double Tx[TM_Z][TM_Y][TT_X];
-    __shared__ double Txy[TM_Z][TT_Y][TT_X];
-    const int tid = threadIdx.x;
-    const int np = nf + 1, n0 = nf / 4, np1 = nf / 2 + 1;
-    const int xa = blockIdx.x * TT_X, ya = blockIdx.y * TT_Y, za = blockIdx.z * TT_Z;
-    const int xb = min(xa + TT_X, np), yb = min(ya + TT_Y, np), zb = min(za + TT_Z, np);
-    // middle-grid nodes used by the tile: from the first node of the first
-    // cell to the last node of the last cell (tiles start on cell bounds)
-    const int mx0 = 2 * quad_cell(xa, n0), my0 = 2 * quad_cell(ya, n0), mz0 = 2 * quad_cell(za, n0);
-    const int nmx = 2 * quad_cell(xb - 1, n0) + 3 - mx0;
-    const int nmy = 2 * quad_cell(yb - 1, n0) + 3 - my0;
-    const int nmz = 2 * quad_cell(zb - 1, n0) + 3 - mz0;
-    for (int e = tid; e < nmz * nmy * nmx; e += TT_THREADS) {
-        const int ex = e % nmx, ey = (e / nmx) % nmy, ez = e / (nmx * nmy);
-        Ws[ez][ey][ex] = W[nidx(np1, mx0 + ex, my0 + ey, mz0 + ez)];
-    }
-    __syncthreads();
-    // along x: vx at (fine x, middle y, middle z)
-    for (int e = tid; e < nmz * nmy * TT_X; e += TT_THREADS) {
-        const int fx = e % TT_X, ey = (e / TT_X) % nmy, ez = e / (TT_X * nmy);
-        const int i = xa + fx;
-        if (i >= xb) continue;
-        int xi[3];
-        double xw[3];
-        const int nx = quad_weights(i, n0, xi, xw);
-        double vx = 0.0;
-        for (int a = 0; a < nx; ++a) vx += xw[a] * Ws[ez][ey][xi[a] - mx0];
-        Tx[ez][ey][fx] = vx;
-    }
-    __syncthreads();
-    // along y: vy at (fine x, fine y, middle z)
-    for (int e = tid; e < nmz * TT_Y * TT_X; e += TT_THREADS) {
-        const int fx = e % TT_X, fy = (e / TT_X) % TT_Y, ez = e / (TT_X * TT_Y);
-        const int i = xa + fx, j = ya + fy;
-        if (i >= xb || j >= yb) continue;
-        int yi[3];
-        double yw[3];
-        const int ny = quad_weights(j, n0, yi, yw);
-        double vy = 0.0;
-        for (int b = 0; b < ny; ++b) vy += yw[b] * Tx[ez][yi[b] - my0][fx];
-        Txy[ez][fy][fx] = vy;
-    }
-    __syncthreads();
-    // along z: the fine values
-    for (int e = tid; e < TT_Z * TT_Y * TT_X; e += TT_THREADS) {
-        const int fx = e % TT_X, fy = (e / TT_X) % TT_Y, fz = e / (TT_X * TT_Y);
-        const int i = xa + fx, j = ya + fy, k = za + fz;
-        if (i >= xb || j >= yb || k >= zb) continue;
-        int zi[3];
-        double zw[3];
-        const int nz = quad_weights(k, n0, zi, zw);
-        double v = 0.0;
-        for (int c = 0; c < nz; ++c) v += zw[c] * Txy[zi[c] - mz0][fy][fx];
-        w[nidx(np, i, j, k)] = v;
-    }
-}
-
-// EXP_true at every fine node of the tile: d = u_h - u_2h at the coarse
-// nodes, then its sums over the 1, 2, 4 or 8 coarse nodes around each fine
-// node, formed along x, then y, then z.
-__global__ void __launch_bounds__(TT_THREADS)
-exp_true_tiled_kernel(double* __restrict__ ut, const double* __restrict__ uh, const double* __restrict__ u2h,
-                      int nf) {
-    __shared__ double Ds[TM_Z][TM_Y][TM_X];
-    __shared__ double Sx[TM_Z][TM_Y][TT_X];
-    __shared__ double Sxy[TM_Z][TT_Y][TT_X];
-    const int tid = threadIdx.x;
+extrapolate_tiled_kernel(double* __restrict__ out, const double* __restrict__ u, const double* __restrict__ uc,
+                         int nf) {
+    __shared__ double Ds[TM_Z * TM_Y][TM_X];
+    __shared__ double Sx[TM_Z * TM_Y][TT_X];
+    const int tid = threadIdx.x, fx = tid & 31, fy = tid >> 5;
     const int np = nf + 1, npc = nf / 2 + 1;
     const int xa = blockIdx.x * TT_X, ya = blockIdx.y * TT_Y, za = blockIdx.z * TT_Z;
-    const int xb = min(xa + TT_X, np), yb = min(ya + TT_Y, np), zb = min(za + TT_Z, np);
-    // coarse nodes around the tile's fine nodes: floor(v/2) .. ceil(v/2)
     const int cx0 = xa >> 1, cy0 = ya >> 1, cz0 = za >> 1;
-    const int ncx = (xb >> 1) + 1 - cx0, ncy = (yb >> 1) + 1 - cy0, ncz = (zb >> 1) + 1 - cz0;
-    for (int e = tid; e < ncz * ncy * ncx; e += TT_THREADS) {
-        const int ex = e % ncx, ey = (e / ncx) % ncy, ez = e / (ncx * ncy);
+    for (int e = tid; e < TM_Z * TM_Y * TM_X; e += TT_THREADS) {
+        const int row = e / TM_X, ex = e - row * TM_X, ez = row / TM_Y, ey = row - ez * TM_Y;
         const int ci = cx0 + ex, cj = cy0 + ey, ck = cz0 + ez;
-        if (ci < npc && cj < npc && ck < npc)
-            Ds[ez][ey][ex] = uh[nidx(np, 2 * ci, 2 * cj, 2 * ck)] - u2h[nidx(npc, ci, cj, ck)];
+        double d = 0.0;
+        if (ci < npc && cj < npc && ck < npc) d = u[nidx(np, 2 * ci, 2 * cj, 2 * ck)] - uc[nidx(npc, ci, cj, ck)];
+        Ds[row][ex] = d;
+    }
+    const int i = xa + fx, j = ya + fy;
+    const bool mine = i < np && j < np;
+    const int kz = min(TT_Z, np - za);   // planes of the tile
+    const size_t o = nidx(np, mine ? i : 0, mine ? j : 0, za);
+    const size_t plane = (size_t)np * np;
+    double uv[TT_Z];
+#pragma unroll
+    for (int k = 0; k < TT_Z; ++k) uv[k] = mine && k < kz ? u[o + k * plane] : 0.0;
+    __syncthreads();
+    for (int row = fy; row < TM_Z * TM_Y; row += TT_Y) {
+        const int c = fx >> 1;
+        Sx[row][fx] = (fx & 1) ? Ds[row][c] + Ds[row][c + 1] : Ds[row][c];
     }
     __syncthreads();
-    for (int e = tid; e < ncz * ncy * TT_X; e += TT_THREADS) {
-        const int fx = e % TT_X, ey = (e / TT_X) % ncy, ez = e / (TT_X * ncy);
-        const int i = xa + fx;
-        if (i >= xb || cy0 + ey >= npc || cz0 + ez >= npc) continue;
-        const int c = (i >> 1) - cx0;
-        Sx[ez][ey][fx] = (i & 1) ? Ds[ez][ey][c] + Ds[ez][ey][c + 1] : Ds[ez][ey][c];
+    if (!mine) return;
+    double s[TM_Z];
+#pragma unroll
+    for (int c = 0; c < TM_Z; ++c) {
+        const int row = c * TM_Y + (fy >> 1);
+        s[c] = (fy & 1) ? Sx[row][fx] + Sx[row + 1][fx] : Sx[row][fx];
+    }
+    // 1 / (3 2^m) or 1 / (4 2^m), m = number of odd coordinates (tiles start on even ones)
+    const int m = (fx & 1) + (fy & 1);
+    const double w0 = kQuarter ? (m == 0 ? 0.25 : m == 1 ? 0.125 : 0.0625)
+                               : (m == 0 ? 1.0 / 3.0 : m == 1 ? 1.0 / 6.0 : 1.0 / 12.0);
+    const double w1 = kQuarter ? (m == 0 ? 0.125 : m == 1 ? 0.0625 : 0.03125)
+                               : (m == 0 ? 1.0 / 6.0 : m == 1 ? 1.0 / 12.0 : 1.0 / 24.0);
+#pragma unroll
+    for (int k = 0; k < TT_Z; ++k)
+        if (k < kz) {
+            const int c = k >> 1;
+            out[o + k * plane] = (k & 1) ? __fma_rn(s[c] + s[c + 1], w1, uv[k]) : __fma_rn(s[c], w0, uv[k]);
+        }
+}
+
+// the Lagrange value at local offset 1 (first) or 3 of a cell of four fine
+// intervals with middle-grid values a, b, c
+__device__ __forceinline__ double quad_odd(bool first, double a, double b, double c) {
+    const double wa = first ? 0.375 : -0.125, wc = first ? -0.125 : 0.375;
+    return __fma_rn(wc, c, __fma_rn(0.75, b, wa * a));
+}
+
+// Step 5 at every fine node of the tile: even coordinates are middle-grid
+// nodes, odd ones take three products per axis.  Along x a warp forms the
+// odd nodes of two rows at a time.
+__global__ void __launch_bounds__(TT_THREADS)
+exp_finite_interp_tiled_kernel(double* __restrict__ w, const double* __restrict__ W, int nf) {
+    __shared__ double Ws[TM_Z * TM_Y][TM_X];
+    __shared__ double Tx[TM_Z * TM_Y + 1][TT_X];
+    const int tid = threadIdx.x, fx = tid & 31, fy = tid >> 5;
+    const int np = nf + 1, np1 = nf / 2 + 1;
+    const int xa = blockIdx.x * TT_X, ya = blockIdx.y * TT_Y, za = blockIdx.z * TT_Z;
+    const int mx0 = xa >> 1, my0 = ya >> 1, mz0 = za >> 1;
+    for (int e = tid; e < TM_Z * TM_Y * TM_X; e += TT_THREADS) {
+        const int row = e / TM_X, ex = e - row * TM_X, ez = row / TM_Y, ey = row - ez * TM_Y;
+        const int ci = mx0 + ex, cj = my0 + ey, ck = mz0 + ez;
+        const double v = ci < np1 && cj < np1 && ck < np1 ? W[nidx(np1, ci, cj, ck)] : 0.0;
+        Ws[row][ex] = v;
+        if (ex < TT_X / 2) Tx[row][2 * ex] = v;
     }
     __syncthreads();
-    for (int e = tid; e < ncz * TT_Y * TT_X; e += TT_THREADS) {
-        const int fx = e % TT_X, fy = (e / TT_X) % TT_Y, ez = e / (TT_X * TT_Y);
-        const int i = xa + fx, j = ya + fy;
-        if (i >= xb || j >= yb || cz0 + ez >= npc) continue;
-        const int c = (j >> 1) - cy0;
-        Sxy[ez][fy][fx] = (j & 1) ? Sx[ez][c][fx] + Sx[ez][c + 1][fx] : Sx[ez][c][fx];
+    for (int pair = fy; 2 * pair < TM_Z * TM_Y; pair += TT_Y) {
+        const int row = 2 * pair + (fx >> 4), c = fx & 15, cell = c >> 1;
+        if (row < TM_Z * TM_Y) {
+            const double* const v = &Ws[row][2 * cell];
+            Tx[row][2 * c + 1] = quad_odd((c & 1) == 0, v[0], v[1], v[2]);
+        }
     }
     __syncthreads();
-    for (int e = tid; e < TT_Z * TT_Y * TT_X; e += TT_THREADS) {
-        const int fx = e % TT_X, fy = (e / TT_X) % TT_Y, fz = e / (TT_X * TT_Y);
-        const int i = xa + fx, j = ya + fy, k = za + fz;
-        if (i >= xb || j >= yb || k >= zb) continue;
-        const int c = (k >> 1) - cz0;
-        const double sum = (k & 1) ? Sxy[c][fy][fx] + Sxy[c + 1][fy][fx] : Sxy[c][fy][fx];
-        const int m = (i & 1) + (j & 1) + (k & 1);
-        const double wt = m == 0 ? 1.0 / 3.0 : (m == 1 ? 1.0 / 6.0 : (m == 2 ? 1.0 / 12.0 : 1.0 / 24.0));
-        const size_t o = nidx(np, i, j, k);
-        ut[o] = uh[o] + sum * wt;
+    const int i = xa + fx, j = ya + fy;
+    if (i >= np || j >= np) return;
+    double t[TM_Z];
+#pragma unroll
+    for (int c = 0; c < TM_Z; ++c) {
+        const int row = c * TM_Y;
+        if (fy & 1) {
+            const int r0 = row + 2 * (fy >> 2);
+            t[c] = quad_odd((fy & 2) == 0, Tx[r0][fx], Tx[r0 + 1][fx], Tx[r0 + 2][fx]);
+        } else {
+            t[c] = Tx[row + (fy >> 1)][fx];
+        }
     }
+    const int kz = min(TT_Z, np - za);
+    const size_t o = nidx(np, i, j, za);
+    const size_t plane = (size_t)np * np;
+#pragma unroll
+    for (int k = 0; k < TT_Z; ++k)
+        if (k < kz) {
+            const int c = 2 * (k >> 2);
+            w[o + k * plane] = (k & 1) ? quad_odd((k & 2) == 0, t[c], t[c + 1], t[c + 2]) : t[k >> 1];
+        }
 }
 
 dim3 tiled_grid(int nf) {
@@ -216,9 +164,7 @@ dim3 tiled_grid(int nf) {
 cudaError_t launch_exp_finite(double* w, const double* u1, const double* u0, double* W_scratch,
                               int n_fine, cudaStream_t s) {
     const int n1 = n_fine / 2;
-    dim3 block(32, 4, 1);
-    dim3 g1((n1 + 1 + 31) / 32, (n1 + 1 + 3) / 4, n1 + 1);
-    exp_finite_w_kernel<<<g1, block, 0, s>>>(W_scratch, u1, u0, n1);
+    extrapolate_tiled_kernel<true><<<tiled_grid(n1), TT_THREADS, 0, s>>>(W_scratch, u1, u0, n1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     exp_finite_interp_tiled_kernel<<<tiled_grid(n_fine), TT_THREADS, 0, s>>>(w, W_scratch, n_fine);
@@ -227,7 +173,7 @@ cudaError_t launch_exp_finite(double* w, const double* u1, const double* u0, dou
 
 cudaError_t launch_exp_true(double* ut, const double* uh, const double* u2h, int n_fine,
                             cudaStream_t s) {
-    exp_true_tiled_kernel<<<tiled_grid(n_fine), TT_THREADS, 0, s>>>(ut, uh, u2h, n_fine);
+    extrapolate_tiled_kernel<false><<<tiled_grid(n_fine), TT_THREADS, 0, s>>>(ut, uh, u2h, n_fine);
     return cudaGetLastError();
 }
 
