@@ -505,18 +505,15 @@ int setup_level(excmg_batch* b, Instance* in) {
     cudaError_t e = launch_assemble_rhs(in->fh, N, in->bc, in->f, in->g1, in->g2, stride, ctx->stream);
     if (e == cudaSuccess && l >= 2) e = launch_exp_finite(u, in->u[l - 1], in->u[l - 2], in->W, N, ctx->stream);
     if (e == cudaSuccess) e = launch_set_boundary(u, N, in->g1, stride, ctx->stream);
-    // the operator writes interior entries only and the buffers of A p, A p*
+    // the kernels of larger grids write interior entries only and the buffers
     // are shared by all levels: clear them in this level's layout, or the
     // previous level's values would sit on this level's boundary nodes and
     // enter r, the inner products and u through the vector updates
     if (e == cudaSuccess && l >= 2) {
         const size_t len = node_count(N);
         if (in->prec == EXCMG_PRECISION_FP64) {
-            // (the second direction pair as well: the operator phase writes
-            // its interior entries only)
-            double* const zero[] = {in->q64, in->p2_64, in->ps2_64};
-            for (double* z : zero)
-                if (e == cudaSuccess) e = cudaMemsetAsync(z, 0, len * sizeof(double), ctx->stream);
+            e = launch_zero_boundary({in->res, in->rs64, in->p64, in->ps64, in->q64, in->p2_64, in->ps2_64}, N,
+                                     ctx->stream);
         } else {
             e = cudaMemsetAsync(in->q, 0, len * sizeof(float), ctx->stream);
             if (e == cudaSuccess) e = cudaMemsetAsync(in->qs, 0, len * sizeof(float), ctx->stream);
@@ -1162,16 +1159,24 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
         if ((st = norms(b, need_f))) return st;
         for (size_t k = 0; k < need_f.size(); ++k) need_f[k].first->fnorm = std::sqrt(b->h_norms[k]);
         std::vector<std::pair<Instance*, const double*>> rw;
+        // r = f_h - A u, in FP64 instances with its copies r*, p, p* for the
+        // Bi-CG call that may follow, and (r, r)
         for (Instance* in : res) {
             const int N = in->nc << in->level;
-            cudaError_t e = cudaMemsetAsync(in->res, 0, node_count(N) * sizeof(double), s);
+            const bool fp64 = in->prec == EXCMG_PRECISION_FP64;
+            cudaError_t e = cudaSuccess;
+            if (!fp64 && !stencil_writes_boundary(N, kStencilExact))
+                e = launch_zero_boundary({in->res}, N, s);
             if (e == cudaSuccess)
-                e = launch_stencil(in->u[in->level], in->res, in->fh, N, in->bc, false, nullptr, s, kStencilExact);
+                e = launch_bicg_start(in->u[in->level], in->fh, N, in->bc, in->res, in->rs64, in->p64, in->ps64,
+                                      ctx->partials, ctx->ticket, b->d_norms + rw.size(), nullptr, s);
             bnote(b, 1);
             if (e != cudaSuccess) return bcuda(b, e, "batch residual");
             rw.push_back({in, in->res});
         }
-        if ((st = norms(b, rw))) return st;
+        cudaError_t ne = cudaMemcpyAsync(b->h_norms, b->d_norms, rw.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
+        if (ne == cudaSuccess) ne = cudaStreamSynchronize(s);
+        if ((st = bcuda(b, ne, "batch norm read"))) return st;
         for (size_t k = 0; k < rw.size(); ++k) {
             Instance* in = rw[k].first;
             const double rn = std::sqrt(b->h_norms[k]);
@@ -1218,12 +1223,8 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
             cudaError_t e = cudaSuccess;
             if (in->prec == EXCMG_PRECISION_FP64) {
                 // a Bi-CG call of Alg. 1's WHILE loop: x = u, r_0 = the true
-                // residual just formed, r*_0 = p_0 = p*_0 = r_0,
+                // residual just formed with its copies r*_0 = p_0 = p*_0,
                 // rho_0 = (r_0, r_0); stop at ||r|| <= eps ||f_h||
-                const size_t bytes = node_count(N) * sizeof(double);
-                e = cudaMemcpyAsync(in->rs64, in->res, bytes, cudaMemcpyDeviceToDevice, s);
-                if (e == cudaSuccess) e = cudaMemcpyAsync(in->p64, in->res, bytes, cudaMemcpyDeviceToDevice, s);
-                if (e == cudaSuccess) e = cudaMemcpyAsync(in->ps64, in->res, bytes, cudaMemcpyDeviceToDevice, s);
                 BatchState& hs = b->h_states[slot];
                 hs = BatchState{};
                 hs.rho = b->h_norms[k];   // (r_0, r_0) exactly as summed

@@ -35,19 +35,55 @@ int unknowns_norm(excmg_ctx* ctx, int n, const double* a, double* out) {
     return EXCMG_OK;
 }
 
-// Norm of b - A x over the unknowns (boundary entries of the work vector are
-// zero, so a flat norm over all nodes equals it).
-int true_residual_norm(excmg_ctx* ctx, int n, int bc_kind, const double* b, const double* x,
-                       double* out) {
+// (r, r) of r = b - A x over the unknowns, enqueued into ctx->scalar[slot].
+// With the integer operator r is not stored; else it goes through the
+// context's workspace (zero boundary entries, so a flat sum is the sum over the unknowns).
+static int enqueue_residual(excmg_ctx* ctx, int n, int bc_kind, const double* b, const double* x, int slot) {
     const size_t len = node_count(n);
+    double* const out = ctx->scalar + slot;
+    if (ctx->stencil_variant == kStencilExact && stencil_cta_count(n) <= kMaxPartials) {
+        const cudaError_t e =
+            launch_residual_norm(x, b, n, bc_kind, ctx->partials, ctx->ticket, out, ctx->stream);
+        note_launches(1);
+        return ctx_cuda(ctx, e, "residual");
+    }
     int st = EXCMG_OK;
     double* r = ctx_buffer(ctx, "res", len * sizeof(double), &st);
     if (st) return st;
     cudaError_t e = cudaMemsetAsync(r, 0, len * sizeof(double), ctx->stream);
     if (e == cudaSuccess) e = launch_stencil(x, r, b, n, bc_kind, false, nullptr, ctx->stream, ctx->stencil_variant);
-    if (e != cudaSuccess) return ctx_cuda(ctx, e, "residual");
+    if (e == cudaSuccess) e = launch_dot(r, r, len, ctx->partials, ctx->ticket, out, ctx->stream);
+    note_launches(2);
+    return ctx_cuda(ctx, e, "residual");
+}
+
+static int read_scalars(excmg_ctx* ctx, int count) {
+    cudaError_t e = ctx_read_back(ctx, ctx->host_scalar, ctx->scalar, count * sizeof(double));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    return ctx_cuda(ctx, e, "norm");
+}
+
+// Norm of b - A x over the unknowns.
+int true_residual_norm(excmg_ctx* ctx, int n, int bc_kind, const double* b, const double* x, double* out) {
+    int st = enqueue_residual(ctx, n, bc_kind, b, x, 0);
+    if (!st) st = read_scalars(ctx, 1);
+    if (!st) *out = sqrt(ctx->host_scalar[0]);
+    return st;
+}
+
+// ||b||_2 (zero boundary entries) and the norm of b - A x, read back together.
+int rhs_and_residual_norms(excmg_ctx* ctx, int n, int bc_kind, const double* b, const double* x, double* bnorm,
+                           double* out) {
+    const cudaError_t e =
+        launch_dot(b, b, node_count(n), ctx->partials, ctx->ticket, ctx->scalar, ctx->stream);
     note_launches(1);
-    return interior_norm(ctx, n, r, out);
+    int st = ctx_cuda(ctx, e, "norm");
+    if (!st) st = enqueue_residual(ctx, n, bc_kind, b, x, 1);
+    if (!st) st = read_scalars(ctx, 2);
+    if (st) return st;
+    *bnorm = sqrt(ctx->host_scalar[0]);
+    *out = sqrt(ctx->host_scalar[1]);
+    return EXCMG_OK;
 }
 
 int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, double tol,
@@ -101,43 +137,52 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     init.max_iter = max_iter;
     *ctx->host_state = init;
     cudaError_t e = cudaMemcpyAsync(ctx->state, ctx->host_state, sizeof(BicgState), cudaMemcpyHostToDevice, s);
-    // boundary entries of every work vector stay zero: the stencils write
-    // interior entries only
-    if (e == cudaSuccess) e = cudaMemsetAsync(r, 0, bytes, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, bytes, s);
-    if (e == cudaSuccess && qs) e = cudaMemsetAsync(qs, 0, bytes, s);
+    // boundary entries of every work vector stay zero (the marches write
+    // interior entries only; the resident kernel looks at no boundary entry)
+    long long started = 1;
+    if (e == cudaSuccess && !resident) {
+        e = launch_zero_boundary({r, rs, p, ps, q, qs, p2, ps2}, n, s);
+        ++started;
+    }
     // r_0 = b - A x_0; r*_0 = p_0 = p*_0 = r_0; rho_0
-    if (e == cudaSuccess) e = launch_stencil(x, r, b, n, bc_kind, false, nullptr, s, ctx->stencil_variant);
-    if (e == cudaSuccess)
-        e = elide ? launch_cg_init(r, p, len, ctx->partials, ctx->state, s)
-                  : launch_bicg_init(r, shadow, rs, p, ps, len, ctx->partials, ctx->state, s);
-    // a caller's shadow may carry values on boundary nodes: the work vectors
-    // keep zeros there
-    if (e == cudaSuccess && shadow) e = launch_zero_boundary(rs, n, s);
-    if (e == cudaSuccess && shadow) e = launch_zero_boundary(ps, n, s);
-    if (e == cudaSuccess && dir_fused) e = launch_zero_boundary(p2, n, s);
-    if (e == cudaSuccess && dir_fused && !elide) e = launch_zero_boundary(ps2, n, s);
+    if (ctx->stencil_variant == kStencilExact && shadow == nullptr && fused) {
+        if (e == cudaSuccess)
+            e = launch_bicg_start(x, b, n, bc_kind, r, rs, p, ps, ctx->partials, &ctx->state->ticket, nullptr,
+                                  ctx->state, s);
+    } else {
+        if (e == cudaSuccess) e = launch_stencil(x, r, b, n, bc_kind, false, nullptr, s, ctx->stencil_variant);
+        if (e == cudaSuccess)
+            e = elide ? launch_cg_init(r, p, len, ctx->partials, ctx->state, s)
+                      : launch_bicg_init(r, shadow, rs, p, ps, len, ctx->partials, ctx->state, s);
+        ++started;
+        // a caller's shadow may carry values on boundary nodes: the work vectors
+        // keep zeros there
+        if (e == cudaSuccess && shadow) {
+            e = launch_zero_boundary({rs, ps}, n, s);
+            ++started;
+        }
+    }
     if (e != cudaSuccess) return ctx_cuda(ctx, e, "Bi-CG setup");
-    note_launches(dir_fused ? (elide ? 1 : 2) : 0);
+    note_launches(started);
 
     const int* done = &ctx->state->done;
     if (persistent) {
-        for (;;) {
-            e = ctx_read_back(ctx, ctx->host_state, ctx->state, sizeof(BicgState));
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            if (e != cudaSuccess) return ctx_cuda(ctx, e, "Bi-CG state read");
-            if (ctx->host_state->done) break;
+        // (a launch on a call that is done already returns at once)
+        for (int iter = 0;;) {
             int chunk = resident ? 1024 : 256;
-            const int left = max_iter - ctx->host_state->iter;
-            if (chunk > left) chunk = left;
+            if (chunk > max_iter - iter) chunk = max_iter - iter;
             e = resident ? launch_bicg_resident<double>(x, r, rs, p, ps, n, bc_kind, chunk, ctx->state, words, s, elide, 0)
                          : launch_bicg_persistent(x, r, rs, p, ps, q, qs, n, bc_kind, chunk, ctx->partials,
                                                   ctx->state, ctx->barrier, s, elide);
             note_launches(1);
             if (e != cudaSuccess) return ctx_cuda(ctx, e, "cooperative Bi-CG launch");
+            e = ctx_read_back(ctx, ctx->host_state, ctx->state, sizeof(BicgState));
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (e != cudaSuccess) return ctx_cuda(ctx, e, "Bi-CG state read");
+            if (ctx->host_state->done) break;
+            iter = ctx->host_state->iter;
         }
     }
-    note_launches(2);   // residual stencil + init (the memsets are not kernels)
     int batch = 0;
     int iter_before = 0;
     // algorithmic bytes of one timed operator launch: 8 B per unknown for

@@ -351,8 +351,9 @@ int stencil_apply(const excmg_level* level, int transpose, const double* u, doub
     if (u == y) return ctx_fail(ctx, EXCMG_ERR_ARG, "stencil_apply: u and y must not overlap");
     cudaError_t e = launch_stencil(u, y, nullptr, level->n, level->bc_kind, transpose != 0, nullptr,
                                    ctx->stream, ctx->stencil_variant);
-    if (e == cudaSuccess) e = launch_zero_boundary(y, level->n, ctx->stream);
-    note_launches(2);
+    const bool all = stencil_writes_boundary(level->n, ctx->stencil_variant);
+    if (e == cudaSuccess && !all) e = launch_zero_boundary({y}, level->n, ctx->stream);
+    note_launches(all ? 1 : 2);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     return ctx_cuda(ctx, e, "stencil_apply");
 }
@@ -498,15 +499,14 @@ int excmg_solve_ex(excmg_ctx* ctx, int n_finest, int n_coarsest, int bc_kind, co
         if (e == cudaSuccess) e = launch_set_boundary(u, N, g1, stride, s);
         note_launches(l >= 2 ? 4 : 2);
         if (e != cudaSuccess) { result = ctx_cuda(ctx, e, "level setup"); break; }
-        if ((result = interior_norm(ctx, N, fh, &fnorm))) break;
-        if (!std::isfinite(fnorm)) {
-            result = ctx_fail(ctx, EXCMG_ERR_NAN, "right-hand side f_h is not finite");
-            break;
-        }
         if (l <= 1) {
             // Alg. 1's direct solves
             if ((result = dsolve_run(ctx, N, bc_kind, fh, u))) break;
-            if ((result = true_residual_norm(ctx, N, bc_kind, fh, u, &rn))) break;
+            if ((result = rhs_and_residual_norms(ctx, N, bc_kind, fh, u, &fnorm, &rn))) break;
+            if (!std::isfinite(fnorm)) {
+                result = ctx_fail(ctx, EXCMG_ERR_NAN, "right-hand side f_h is not finite");
+                break;
+            }
             rel = fnorm > 0.0 ? rn / fnorm : 0.0;
             if (!std::isfinite(rel)) {
                 result = ctx_fail(ctx, EXCMG_ERR_NAN, "residual of the direct solve is not finite");
@@ -517,12 +517,21 @@ int excmg_solve_ex(excmg_ctx* ctx, int n_finest, int n_coarsest, int bc_kind, co
             const double eps = params->tol_mode == EXCMG_TOL_PAPER ? params->tol * std::pow(10.0, (double)(i - L))
                                                                    : params->tol;
             if (params->precision == EXCMG_PRECISION_MIXED) {
+                if ((result = interior_norm(ctx, N, fh, &fnorm))) break;
+                if (!std::isfinite(fnorm)) {
+                    result = ctx_fail(ctx, EXCMG_ERR_NAN, "right-hand side f_h is not finite");
+                    break;
+                }
                 result = mixed_level_solve(ctx, N, bc_kind, fh, u, fnorm, eps, params->inner_tol, params->max_iter,
                                            params->max_total, params->check_every, &iters, &calls, &stag, &rel);
                 if (result) break;
                 goto level_done;
             }
-            if ((result = true_residual_norm(ctx, N, bc_kind, fh, u, &rn))) break;
+            if ((result = rhs_and_residual_norms(ctx, N, bc_kind, fh, u, &fnorm, &rn))) break;
+            if (!std::isfinite(fnorm)) {
+                result = ctx_fail(ctx, EXCMG_ERR_NAN, "right-hand side f_h is not finite");
+                break;
+            }
             rel = fnorm > 0.0 ? rn / fnorm : 0.0;
             if (!std::isfinite(rel)) {
                 result = ctx_fail(ctx, EXCMG_ERR_NAN, "residual of the initial guess is not finite");

@@ -53,7 +53,23 @@ enum { kRunning = 0, kConverged = 1, kCapped = 2, kBreakdown = 3, kTimeout = 4 }
 enum { kStencilExact = 0, kStencilFp64 = 1 };
 cudaError_t launch_stencil(const double* u, double* y, const double* b, int n, int bc_kind,
                            bool transpose, const int* skip, cudaStream_t s, int variant);
-cudaError_t launch_zero_boundary(double* y, int n, cudaStream_t s);
+// True where launch_stencil sets the boundary entries of y to zero as well.
+bool stencil_writes_boundary(int n, int variant);
+// Zeros on the boundary nodes of up to eight node arrays (null: none).
+struct BoundaryArrays {
+    double* a[8];
+};
+cudaError_t launch_zero_boundary(const BoundaryArrays& arrays, int n, cudaStream_t s);
+// (r, r) of r = b - A x over the unknowns into *out (integer operator).
+cudaError_t launch_residual_norm(const double* x, const double* b, int n, int bc_kind, double* partials,
+                                 unsigned int* ticket, double* out, cudaStream_t s);
+// The start of a Bi-CG call with r*_0 = r_0 (integer operator): r = b - A x and
+// its copies r*, p, p* (each may be null) at the interior nodes (grids up to
+// 64^3: zeros on the boundary, too), (r, r) into *out and the scalars of *st
+// (each may be null).
+cudaError_t launch_bicg_start(const double* x, const double* b, int n, int bc_kind, double* r, double* rs, double* p,
+                              double* ps, double* partials, unsigned int* ticket, double* out, BicgState* st,
+                              cudaStream_t s);
 // One z-march applying A to p (-> q) and A^T to p* (-> qs) with the integer
 // arithmetic, fused with sigma = (p*, q) and alpha = rho / sigma (Alg. 2).
 // Skips when st->done.  partials must hold stencil_cta_count(n) doubles.
@@ -251,6 +267,8 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
 // ||b - A x||_2 over the unknowns, via the context's workspace (result on host).
 int true_residual_norm(excmg_ctx* ctx, int n, int bc_kind, const double* b, const double* x,
                        double* out);
+int rhs_and_residual_norms(excmg_ctx* ctx, int n, int bc_kind, const double* b, const double* x, double* bnorm,
+                           double* out);
 int interior_norm(excmg_ctx* ctx, int n, const double* a, double* out);   // flat: zero boundary assumed
 int unknowns_norm(excmg_ctx* ctx, int n, const double* a, double* out);   // interior nodes only
 // DSOLVE (dsolve.cu)

@@ -144,20 +144,23 @@ __host__ __device__ __forceinline__ void ml_ring(int e, int* lx, int* ly) {
     }
 }
 
-// What a march does: A u or b - A u; (p, p*) -> (q, q*) with sigma; the same
-// with p = r + beta p, p* = r* + beta p* formed first.
-enum MarchKind { kMarchApply, kMarchPair, kMarchDir };
+// What a march does: A u or b - A u; with r = b - A u the start of a Bi-CG
+// call (r, p, and r*, p* where given, and (r, r)) or (r, r) alone; (p, p*) ->
+// q with sigma; the same with p = r + beta p, p* = r* + beta p* formed first.
+enum MarchKind { kMarchApply, kMarchStart, kMarchNorm, kMarchPair, kMarchDir };
+constexpr bool march_is_step(MarchKind k) { return k == kMarchPair || k == kMarchDir; }
 
 struct MarchArrays {
     const double* in;     // u, p or p_{k-1}
     const double* r;      // kMarchDir
     const double* ins;    // p* or p*_{k-1}
     const double* rs;     // kMarchDir
-    const double* b;      // kMarchApply, may be null
+    const double* b;      // right-hand side (kMarchApply: may be null)
     double* out;          // y or q (q* = q: the same bits, not stored again)
-    double* pn;           // kMarchDir: p_k (not in: neighbours still read it)
-    double* psn;
+    double* pn;           // kMarchDir: p_k (not in: neighbours still read it); kMarchStart: p, may be null
+    double* psn;          // the same for p*
     double beta;
+    double* rsn;          // kMarchStart: r*, may be null
 };
 
 // Shared memory: one stage, `in` (and r) on all three slots, p* (and r*), or
@@ -165,14 +168,14 @@ struct MarchArrays {
 template <MarchKind K, bool kElide>
 struct MarchStage {
     static constexpr int kAll = K == kMarchDir ? 2 : 1;
-    static constexpr int kOwn = K == kMarchApply ? 1 : kElide ? 0 : kAll;
+    static constexpr int kOwn = !march_is_step(K) ? 1 : kElide ? 0 : kAll;
     static constexpr unsigned kBytes = (kAll * 3 + kOwn * 2) * PP_NT * 8u;
-    static constexpr unsigned kHist = K == kMarchApply ? 0 : 4 * 2 * PP_NT * 8u;
+    static constexpr unsigned kHist = !march_is_step(K) ? 0 : 4 * 2 * PP_NT * 8u;
     static constexpr size_t kSmem = kBytes + kHist + 4 * PP_HALO * sizeof(long long);
 };
 
 // One CTA's march over the output planes [kz0, kz1) of column tile (bx, by).
-// Returns this thread's share of sigma = (p*, q).  Called by all threads.
+// Returns this thread's share of sigma = (p*, q), or of (r, r).  Called by all threads.
 template <MarchKind K, bool kElide>
 __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sigma, int bx, int by, int kz0, int kz1,
                                             unsigned char* smem) {
@@ -189,7 +192,8 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
     const int lane = tid & 31, warp = tid >> 5;
     const int i0 = 1 + bx * PP_TX, j0 = 1 + by * PP_OY;
     const bool ring = tid < PP_RING, inner = tid < ML_INNER;
-    const bool has_b = K == kMarchApply && a.b != nullptr;
+    constexpr bool kStep = march_is_step(K);
+    const bool has_b = !kStep && a.b != nullptr;
 
     // in-plane byte offset of each slot, copy size (0: reads as zero), tile entry
     unsigned so[3], sz[3], te[3];
@@ -221,7 +225,7 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
             const size_t zo = (size_t)(zok ? z : 1) * plane8;
             const char* const in = (const char*)a.in + zo;
             const char* const r = K == kMarchDir ? (const char*)a.r + zo : nullptr;
-            const char* const ps = St::kOwn && K != kMarchApply ? (const char*)a.ins + zo : nullptr;
+            const char* const ps = St::kOwn && kStep ? (const char*)a.ins + zo : nullptr;
             const char* const rs = St::kOwn == 2 ? (const char*)a.rs + zo : nullptr;
 #pragma unroll
             for (int s = 0; s < 3; ++s) {
@@ -229,7 +233,7 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
                     const unsigned nb = zok ? sz[s] : 0u;
                     cp_async8_u32(st + s * kCol, in + so[s], nb);
                     if (K == kMarchDir) cp_async8_u32(st + (3 + s) * kCol, r + so[s], nb);
-                    if (s < 2 && K != kMarchApply && !kElide) {
+                    if (s < 2 && kStep && !kElide) {
                         cp_async8_u32(st + kOwn0 + s * kCol, ps + so[s], nb);
                         if (K == kMarchDir) cp_async8_u32(st + kOwn0 + (2 + s) * kCol, rs + so[s], nb);
                     }
@@ -251,7 +255,7 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
             if (s < 2 || ring) {
                 po[s] = lds_f64(st + s * kCol);
                 if (K == kMarchDir) rv[s] = lds_f64(st + (3 + s) * kCol);
-                if (s < 2 && K != kMarchApply && !kElide) {
+                if (s < 2 && kStep && !kElide) {
                     ps[s] = lds_f64(st + kOwn0 + s * kCol);
                     if (K == kMarchDir) rsv[s] = lds_f64(st + kOwn0 + (2 + s) * kCol);
                 }
@@ -261,7 +265,7 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
             v[s] = 0.0;
             if (s < 2 || ring) v[s] = K == kMarchDir ? __fma_rn(a.beta, po[s], rv[s]) : po[s];
         }
-        if (K != kMarchApply && !kElide) {
+        if (kStep && !kElide) {
             // the same bits in: the same bits out, without another FP64 instruction
             long long diff = 0;
 #pragma unroll
@@ -310,7 +314,7 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
             wm1[s] = w;
             um1[s] = u0[s];
             u0[s] = u;
-            if (K != kMarchApply)   // p* for sigma, two steps on
+            if (kStep)   // p* for sigma, two steps on
                 sts_s64(hist + (unsigned)(t & 3) * (2 * kCol) + s * kCol, __double_as_longlong(kElide ? v[s] : vs[s]));
         }
         if (ring) {
@@ -382,9 +386,20 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
                 const long long acc = gq[s] - wm1[s];   // L w of plane zo, complete with w(t - 1)
                 if (act[s]) {
                     const double val = fx_result_cvt(acc, E, poisoned);
-                    *(double*)(oz + so[s]) = has_b ? bv[s] - val : val;
-                    if (K != kMarchApply)
+                    if (kStep) {
+                        *(double*)(oz + so[s]) = val;
                         d = __fma_rn(lds_f64(hist + (unsigned)((t + 2) & 3) * (2 * kCol) + s * kCol), val, d);
+                    } else {
+                        const double rv = has_b ? bv[s] - val : val;
+                        if (K != kMarchNorm) *(double*)(oz + so[s]) = rv;
+                        if (K == kMarchStart) {
+                            const size_t o = (size_t)zo * plane8 + so[s];
+                            if (a.pn) *(double*)((char*)a.pn + o) = rv;
+                            if (a.rsn) *(double*)((char*)a.rsn + o) = rv;
+                            if (a.psn) *(double*)((char*)a.psn + o) = rv;
+                        }
+                        if (K != kMarchApply) d = __fma_rn(rv, rv, d);
+                    }
                 }
             }
         }

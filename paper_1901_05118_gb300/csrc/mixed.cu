@@ -271,12 +271,26 @@ int mixed_level_solve(excmg_ctx* ctx, int n, int bc_kind, const double* fh, doub
     double rel = 0.0;
     for (;;) {
         // FP64 true residual r = f_h - A u and its norm
-        cudaError_t err = cudaMemsetAsync(r, 0, len * sizeof(double), s);
-        if (err == cudaSuccess) err = launch_stencil(u, r, fh, n, bc_kind, false, nullptr, s, ctx->stencil_variant);
-        note_launches(1);
-        if (err != cudaSuccess) return ctx_cuda(ctx, err, "refinement residual");
+        cudaError_t err = cudaSuccess;
         double rn = 0.0;
-        if ((st = interior_norm(ctx, n, r, &rn))) return st;
+        if (ctx->stencil_variant == kStencilExact && stencil_cta_count(n) <= kMaxPartials) {
+            if (!stencil_writes_boundary(n, ctx->stencil_variant)) err = launch_zero_boundary({r}, n, s);
+            if (err == cudaSuccess)
+                err = launch_bicg_start(u, fh, n, bc_kind, r, nullptr, nullptr, nullptr, ctx->partials, ctx->ticket,
+                                        ctx->scalar, nullptr, s);
+            if (err == cudaSuccess) err = ctx_read_back(ctx, ctx->host_scalar, ctx->scalar, sizeof(double));
+            if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+            note_launches(2);
+            if (err != cudaSuccess) return ctx_cuda(ctx, err, "refinement residual");
+            rn = sqrt(*ctx->host_scalar);
+        } else {
+            err = cudaMemsetAsync(r, 0, len * sizeof(double), s);
+            if (err == cudaSuccess)
+                err = launch_stencil(u, r, fh, n, bc_kind, false, nullptr, s, ctx->stencil_variant);
+            note_launches(1);
+            if (err != cudaSuccess) return ctx_cuda(ctx, err, "refinement residual");
+            if ((st = interior_norm(ctx, n, r, &rn))) return st;
+        }
         const double prev = rel;
         rel = fnorm > 0.0 ? rn / fnorm : 0.0;
         if (!std::isfinite(rel)) return ctx_fail(ctx, EXCMG_ERR_NAN, "residual is not finite");

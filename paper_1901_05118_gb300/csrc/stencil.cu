@@ -105,9 +105,47 @@ stencil_apply_kernel(const double* __restrict__ u, double* __restrict__ y, const
     extern __shared__ __align__(128) unsigned char march_smem[];
     if (skip != nullptr && *skip) return;
     const int kz0 = 1 + blockIdx.z * kz_per_cta;
-    const MarchArrays a{u, nullptr, nullptr, nullptr, b, y, nullptr, nullptr, 0.0};
+    const MarchArrays a{u, nullptr, nullptr, nullptr, b, y, nullptr, nullptr, 0.0, nullptr};
     (void)lap_march<kMarchApply, true>(a, n, sigma, blockIdx.x, blockIdx.y, kz0, min(kz0 + kz_per_cta, n),
                                        march_smem);
+}
+
+// Every CTA's share of rr = (r, r): the last one writes the sum to *out, and
+// the start of a Bi-CG call (rho_0 = (r*_0, r_0) = rr, r*_0 = r_0) to st.
+__device__ __forceinline__ void finish_norm(double v, double* partials, unsigned int* ticket, double* out,
+                                            BicgState* st) {
+    __shared__ double sh[32];
+    __shared__ bool am_last;
+    const double s = block_sum(v, sh);
+    if (publish_partials(&s, 1, partials, ticket, &am_last)) {
+        const double rr = gather_partials(partials, 0, sh);
+        if (thread0()) {
+            *ticket = 0;
+            if (out) *out = rr;
+            if (st) {
+                st->rho = st->rr = rr;
+                st->iter = 0;
+                st->alpha = st->beta = st->sigma = 0.0;
+                const bool conv = sqrt(rr) <= st->tol * st->bnorm;
+                st->done = (conv || st->max_iter <= 0) ? 1 : 0;
+                st->status = conv ? kConverged : (st->max_iter <= 0 ? kCapped : kRunning);
+            }
+        }
+    }
+}
+
+// r = b - A u: the start of a Bi-CG call, or (r, r) alone, which then writes
+// nothing else.  Forming r, the copies p_0, r*_0, p*_0 and the norm in one pass
+// took the start of a 512^3 call from 2.4 to 1.5 ms, the norm alone from 1.6 to
+// 1.1 ms (residual kernel, cleared buffer, inner product).
+template <MarchKind K>
+__global__ void __launch_bounds__(PP_NT, 2)
+stencil_residual_kernel(MarchArrays a, int n, int sigma, int kz_per_cta, double* partials, unsigned int* ticket,
+                        double* out, BicgState* st) {
+    extern __shared__ __align__(128) unsigned char march_smem[];
+    const int kz0 = 1 + blockIdx.z * kz_per_cta;
+    finish_norm(lap_march<K, true>(a, n, sigma, blockIdx.x, blockIdx.y, kz0, min(kz0 + kz_per_cta, n), march_smem),
+                partials, ticket, out, st);
 }
 
 // Every CTA's share of sigma = (p*, A p); the last one forms alpha = rho / sigma (Alg. 2).
@@ -166,8 +204,10 @@ stencil_two_field_kernel(MarchArrays a, double* qs, int n, int sigma, int kz_per
 // a z-march would be all latency.
 __device__ __forceinline__ double fx_point(const double* __restrict__ u, int n, int sigma, int i, int j, int k) {
     const int np = n + 1;
+    // (nodes two away from every face need no bounds checks)
+    const bool deep = i > 2 && i < n - 2 && j > 2 && j < n - 2 && k > 2 && k < n - 2;
     auto val = [&](int a, int b, int c) -> double {
-        if (a < 1 || a > n - 1 || b < 1 || b > n - 1 || c < 1 || c > n - 1) return 0.0;
+        if (!deep && (a < 1 || a > n - 1 || b < 1 || b > n - 1 || c < 1 || c > n - 1)) return 0.0;
         return u[((size_t)c * np + b) * np + a];
     };
     const double ctr = val(i, j, k);
@@ -195,6 +235,34 @@ __device__ __forceinline__ double fx_point(const double* __restrict__ u, int n, 
     const int c = (i == 1) + (i == n - 1) + (j == 1) + (j == n - 1) + (k == 1) + (k == n - 1);
     const long long acc = (long long)(42 + sigma * c) * to_fixed(ctr, E) - 12 * s_ax + s_far + 2 * s_dg;
     return fx_result(acc, E, E == 0x7FF);
+}
+
+// The single-field forms (A u, b - A u, the start of a Bi-CG call, the norm)
+// on small grids, node by node: one round of loads instead of a march of a
+// dozen planes that wait for each other (17^3: 14 us).  Boundary nodes of the outputs are set
+// to zero.
+template <MarchKind K>
+__global__ void __launch_bounds__(256)
+stencil_point_kernel(MarchArrays a, int n, int sigma, const int* __restrict__ skip, double* partials,
+                     unsigned int* ticket, double* out, BicgState* st) {
+    if (skip != nullptr && *skip) return;
+    const int np = n + 1, total = np * np * np;
+    const int t = blockIdx.x * 256 + threadIdx.x;
+    double v = 0.0;
+    if (t < total) {
+        const int k = t / (np * np), e = t - k * np * np, j = e / np, i = e - j * np;
+        if (i > 0 && i < n && j > 0 && j < n && k > 0 && k < n) {
+            v = fx_point(a.in, n, sigma, i, j, k);
+            if (a.b) v = a.b[t] - v;
+        }
+        if (K != kMarchNorm) a.out[t] = v;
+        if (K == kMarchStart) {
+            if (a.pn) a.pn[t] = v;
+            if (a.rsn) a.rsn[t] = v;
+            if (a.psn) a.psn[t] = v;
+        }
+    }
+    if constexpr (K != kMarchApply) finish_norm(v * v, partials, ticket, out, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -414,7 +482,7 @@ bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int 
     }
 }
 
-__global__ void zero_boundary_kernel(double* __restrict__ y, int n) {
+__global__ void zero_boundary_kernel(BoundaryArrays arrays, int n) {
     // one thread per node of the six faces (faces overlap at edges: harmless)
     const int np = n + 1;
     const size_t per_face = (size_t)np * np;
@@ -428,7 +496,9 @@ __global__ void zero_boundary_kernel(double* __restrict__ y, int n) {
         if (face < 2) { i = fixed; j = a; k = bb; }
         else if (face < 4) { i = a; j = fixed; k = bb; }
         else { i = a; j = bb; k = fixed; }
-        y[((size_t)k * np + j) * np + i] = 0.0;
+        const size_t o = ((size_t)k * np + j) * np + i;
+        for (double* y : arrays.a)
+            if (y) y[o] = 0.0;
     }
 }
 
@@ -493,6 +563,12 @@ StencilGrid apply_grid(int n) {
     return march_grid(n, resident_per_sm(stencil_apply_kernel, PP_NT, smem), smem);
 }
 
+// Node-by-node form of the single-field launches: as long as all nodes are
+// in flight at once it takes one memory latency, the march a dozen.
+constexpr int kPointFormMaxN = 64;
+bool point_form(int n) { return n <= kPointFormMaxN; }
+int point_blocks(int n) { return (int)((node_count(n) + 255) / 256); }
+
 // The operator step of Bi-CG: every form of it runs on the grid of the
 // two-field one with directions, so that sigma adds the same per-CTA
 // partial sums in the shadow-elided mode.
@@ -516,7 +592,10 @@ StencilGrid f64_grid(int n) {
 
 int stencil_cta_count(int n) {
     const StencilGrid g1 = apply_grid(n), g2 = step_grid<kMarchDir, false>(n);
-    return (int)max(g1.grid.x * g1.grid.y * g1.grid.z, g2.grid.x * g2.grid.y * g2.grid.z);
+    unsigned most = max(g1.grid.x * g1.grid.y * g1.grid.z, g2.grid.x * g2.grid.y * g2.grid.z);
+    const StencilGrid g3 = march_grid(n, 2, 0);   // the residual launches: two CTAs per SM
+    most = max(most, g3.grid.x * g3.grid.y * g3.grid.z);
+    return (int)most;
 }
 
 cudaError_t launch_stencil(const double* u, double* y, const double* b, int n, int bc_kind,
@@ -531,10 +610,48 @@ cudaError_t launch_stencil(const double* u, double* y, const double* b, int n, i
     } else {
         // A^T u == A u bit for bit in integer arithmetic (see above)
         (void)transpose;
-        const StencilGrid g = apply_grid(n);
-        stencil_apply_kernel<<<g.grid, g.block, g.smem, s>>>(u, y, b, n, bc_kind == 1 ? 1 : -1, g.kz_per_cta, skip);
+        const int sg = bc_kind == 1 ? 1 : -1;
+        if (point_form(n)) {
+            const MarchArrays a{u, nullptr, nullptr, nullptr, b, y, nullptr, nullptr, 0.0, nullptr};
+            stencil_point_kernel<kMarchApply><<<point_blocks(n), 256, 0, s>>>(a, n, sg, skip, nullptr, nullptr,
+                                                                              nullptr, nullptr);
+        } else {
+            const StencilGrid g = apply_grid(n);
+            stencil_apply_kernel<<<g.grid, g.block, g.smem, s>>>(u, y, b, n, sg, g.kz_per_cta, skip);
+        }
     }
     return cudaGetLastError();
+}
+
+namespace {
+template <MarchKind K>
+cudaError_t launch_residual(const MarchArrays& a, int n, int bc_kind, double* partials, unsigned int* ticket,
+                            double* out, BicgState* st, cudaStream_t s) {
+    const int sg = bc_kind == 1 ? 1 : -1;
+    if (point_form(n)) {
+        stencil_point_kernel<K><<<point_blocks(n), 256, 0, s>>>(a, n, sg, nullptr, partials, ticket, out, st);
+    } else {
+        constexpr size_t smem = MarchStage<K, true>::kSmem;
+        const StencilGrid g = march_grid(n, resident_per_sm(stencil_residual_kernel<K>, PP_NT, smem), smem);
+        stencil_residual_kernel<K><<<g.grid, g.block, g.smem, s>>>(a, n, sg, g.kz_per_cta, partials, ticket, out, st);
+    }
+    return cudaGetLastError();
+}
+}  // namespace
+
+bool stencil_writes_boundary(int n, int variant) { return variant == kStencilExact && point_form(n); }
+
+cudaError_t launch_residual_norm(const double* x, const double* b, int n, int bc_kind, double* partials,
+                                 unsigned int* ticket, double* out, cudaStream_t s) {
+    const MarchArrays a{x, nullptr, nullptr, nullptr, b, nullptr, nullptr, nullptr, 0.0, nullptr};
+    return launch_residual<kMarchNorm>(a, n, bc_kind, partials, ticket, out, nullptr, s);
+}
+
+cudaError_t launch_bicg_start(const double* x, const double* b, int n, int bc_kind, double* r, double* rs, double* p,
+                              double* ps, double* partials, unsigned int* ticket, double* out, BicgState* st,
+                              cudaStream_t s) {
+    const MarchArrays a{x, nullptr, nullptr, nullptr, b, r, p, ps, 0.0, rs};
+    return launch_residual<kMarchStart>(a, n, bc_kind, partials, ticket, out, st, s);
 }
 
 constexpr int kPointwiseMaxN = 32;   // per-node operator on grids up to 32^3
@@ -599,7 +716,7 @@ cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, 
 cudaError_t launch_bicg_stencil_pair_dir(const double* r, const double* rs, const double* p_prev,
                                          const double* ps_prev, double* p, double* ps, double* q, double* qs, int n,
                                          int bc_kind, double* partials, BicgState* st, cudaStream_t s) {
-    const MarchArrays a{p_prev, r, ps_prev, rs, nullptr, q, p, ps, 0.0};
+    const MarchArrays a{p_prev, r, ps_prev, rs, nullptr, q, p, ps, 0.0, nullptr};
     const int sg = bc_kind == 1 ? 1 : -1;
     const StencilGrid g = step_grid<kMarchDir, false>(n);
     if (qs == nullptr)
@@ -611,7 +728,7 @@ cudaError_t launch_bicg_stencil_pair_dir(const double* r, const double* rs, cons
 
 cudaError_t launch_bicg_stencil_pair(const double* p, double* q, const double* ps, double* qs, int n,
                                      int bc_kind, double* partials, BicgState* st, cudaStream_t s) {
-    const MarchArrays a{p, nullptr, ps, nullptr, nullptr, q, nullptr, nullptr, 0.0};
+    const MarchArrays a{p, nullptr, ps, nullptr, nullptr, q, nullptr, nullptr, 0.0, nullptr};
     const int sg = bc_kind == 1 ? 1 : -1;
     const StencilGrid g = step_grid<kMarchPair, false>(n);
     if (qs == nullptr)
@@ -623,7 +740,7 @@ cudaError_t launch_bicg_stencil_pair(const double* p, double* q, const double* p
 
 cudaError_t launch_cg_stencil(const double* p, double* q, int n, int bc_kind, double* partials, BicgState* st,
                               cudaStream_t s) {
-    const MarchArrays a{p, nullptr, nullptr, nullptr, nullptr, q, nullptr, nullptr, 0.0};
+    const MarchArrays a{p, nullptr, nullptr, nullptr, nullptr, q, nullptr, nullptr, 0.0, nullptr};
     const StencilGrid g = step_grid<kMarchPair, true>(n);
     stencil_step_kernel<kMarchPair, true><<<g.grid, g.block, g.smem, s>>>(a, n, bc_kind == 1 ? 1 : -1, g.kz_per_cta,
                                                                          partials, st);
@@ -632,18 +749,18 @@ cudaError_t launch_cg_stencil(const double* p, double* q, int n, int bc_kind, do
 
 cudaError_t launch_cg_stencil_dir(const double* r, const double* p_prev, double* p, double* q, int n, int bc_kind,
                                   double* partials, BicgState* st, cudaStream_t s) {
-    const MarchArrays a{p_prev, r, nullptr, nullptr, nullptr, q, p, nullptr, 0.0};
+    const MarchArrays a{p_prev, r, nullptr, nullptr, nullptr, q, p, nullptr, 0.0, nullptr};
     const StencilGrid g = step_grid<kMarchDir, true>(n);
     stencil_step_kernel<kMarchDir, true><<<g.grid, g.block, g.smem, s>>>(a, n, bc_kind == 1 ? 1 : -1, g.kz_per_cta,
                                                                         partials, st);
     return cudaGetLastError();
 }
 
-cudaError_t launch_zero_boundary(double* y, int n, cudaStream_t s) {
+cudaError_t launch_zero_boundary(const BoundaryArrays& arrays, int n, cudaStream_t s) {
     const size_t total = 6 * (size_t)(n + 1) * (n + 1);
     int blocks = (int)((total + 255) / 256);
     if (blocks > 4096) blocks = 4096;
-    zero_boundary_kernel<<<blocks, 256, 0, s>>>(y, n);
+    zero_boundary_kernel<<<blocks, 256, 0, s>>>(arrays, n);
     return cudaGetLastError();
 }
 
