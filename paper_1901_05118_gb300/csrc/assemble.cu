@@ -41,7 +41,9 @@ __device__ __forceinline__ double rhs_near_boundary(int i, int j, int k, int n, 
     const int p[3] = {i, j, k};
     double moved = 0.0;
     // axis taps: +-1 (weight -12) and +-2 (weight +1)
+#pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
+#pragma unroll
         for (int s = -1; s <= 1; s += 2) {
             int q[3] = {p[0], p[1], p[2]};
             q[ax] = p[ax] + s;
@@ -62,9 +64,13 @@ __device__ __forceinline__ double rhs_near_boundary(int i, int j, int k, int n, 
         }
     }
     // in-plane diagonal taps (weight +2)
+#pragma unroll
     for (int a = 0; a < 3; ++a)
+#pragma unroll
         for (int b = a + 1; b < 3; ++b)
+#pragma unroll
             for (int sa = -1; sa <= 1; sa += 2)
+#pragma unroll
                 for (int sb = -1; sb <= 1; sb += 2) {
                     int q[3] = {p[0], p[1], p[2]};
                     q[a] += sa;
@@ -76,41 +82,40 @@ __device__ __forceinline__ double rhs_near_boundary(int i, int j, int k, int n, 
 }
 
 // h^4 f at the nodes that no boundary value reaches, zero on the boundary;
-// kNear: the nodes within two of a face as well (small grids: one launch).
-// A thread takes kPlanes nodes of one (x, y) column.  One index per node with
-// 64-bit divisions, and the boundary rows in the same launch, took 1.14 ms
-// at 512^3: the first and the last warp of every row waited for the taps
-// of four nodes.
-constexpr int kPlanes = 8;
+// kNear: the nodes within two of a face as well (small grids: one launch).  A
+// warp takes a row at a time.  One index per node with 64-bit divisions, and
+// the boundary rows in the same launch, took 1.14 ms at 512^3: the first and
+// the last warp of every row waited for the taps of four nodes.
 template <bool kNear>
 __global__ void __launch_bounds__(256)
 assemble_rhs_kernel(double* __restrict__ fh, int n, int bc_kind, const double* __restrict__ f, Src src) {
-    const int np = n + 1;
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y;
-    if (i > n || j > n) return;
+    const int np = n + 1, lane = threadIdx.x & 31;
     const double h = 1.0 / (double)n;
     const double h4 = h * h * h * h;
-    const int kz = blockIdx.z * kPlanes;
-    const bool in_xy = i >= 1 && i <= n - 1 && j >= 1 && j <= n - 1;
-    const bool deep_xy = i >= 3 && i <= n - 3 && j >= 3 && j <= n - 3;
-    double v[kPlanes];
+    const int warps = gridDim.x * 8, rows = np * np;
+    for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows; row += warps) {
+        const int k = row / np, j = row - k * np;
+        double* const out = fh + (size_t)row * np;
+        const bool in_yz = j >= 1 && j <= n - 1 && k >= 1 && k <= n - 1;
+        const bool deep_yz = j >= 3 && j <= n - 3 && k >= 3 && k <= n - 3;
+        const double* const fr = f + ((size_t)(k * src.stride) * src.np_src + (size_t)(j * src.stride)) * src.np_src;
+        constexpr int U = 4;   // loads of a lane in flight
+        for (int i0 = lane; i0 <= n; i0 += 32 * U) {
+            double v[U];
 #pragma unroll
-    for (int c = 0; c < kPlanes; ++c) {
-        const int k = kz + c;
-        v[c] = in_xy && k >= 1 && k <= n - 1
-                   ? f[((size_t)(k * src.stride) * src.np_src + (size_t)(j * src.stride)) * src.np_src +
-                       (size_t)(i * src.stride)]
-                   : 0.0;
-    }
+            for (int c = 0; c < U; ++c) {
+                const int i = i0 + 32 * c;
+                v[c] = in_yz && i >= 1 && i <= n - 1 ? fr[(size_t)i * src.stride] : 0.0;
+            }
 #pragma unroll
-    for (int c = 0; c < kPlanes; ++c) {
-        const int k = kz + c;
-        if (k > n) break;
-        const size_t t = ((size_t)k * np + j) * np + i;
-        const bool inside = in_xy && k >= 1 && k <= n - 1;
-        const bool deep = deep_xy && k >= 3 && k <= n - 3;
-        if (!inside || deep) fh[t] = h4 * v[c];
-        else if (kNear) fh[t] = rhs_near_boundary(i, j, k, n, bc_kind, h, h4 * v[c], src);
+            for (int c = 0; c < U; ++c) {
+                const int i = i0 + 32 * c;
+                if (i > n) break;
+                const bool inside = in_yz && i >= 1 && i <= n - 1;
+                if (!inside || (deep_yz && i >= 3 && i <= n - 3)) out[i] = h4 * v[c];
+                else if (kNear) out[i] = rhs_near_boundary(i, j, k, n, bc_kind, h, h4 * v[c], src);
+            }
+        }
     }
 }
 
@@ -179,7 +184,8 @@ int grid_for(size_t work) {
 cudaError_t launch_assemble_rhs(double* fh, int n, int bc_kind, const double* f, const double* g1,
                                 const double* g2, int stride, cudaStream_t s) {
     Src src{g1, g2, n * stride + 1, stride};
-    const dim3 grid((n + 32) / 32, (n + 8) / 8, (n + kPlanes) / kPlanes), block(32, 8);
+    const int rows = (n + 1) * (n + 1), want = (rows + 7) / 8;
+    const int grid = want < 152 * 8 ? want : 152 * 8, block = 256;
     if (n <= kOneLaunchMaxN) {
         assemble_rhs_kernel<true><<<grid, block, 0, s>>>(fh, n, bc_kind, f, src);
         return cudaGetLastError();

@@ -1,0 +1,56 @@
+"""The forms that a launch picks by size, on both sides of the lines between
+them: the node-by-node operator up to 64^3 and the march above (ragged tiles),
+the right-hand side with its boundary rows in one launch up to 64^3 and in two
+above, transfers on grids that end inside a tile."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1901_05118_gb300 import problems as P
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU machines only
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1901_05118_gb300 import binding as B  # noqa: E402
+
+DEV = torch.device("cuda", 0)
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+
+
+def rel_max(got, ref):
+    return float(np.abs(got - ref).max() / np.abs(ref).max())
+
+
+@pytest.mark.parametrize("n,bc_kind", [(6, 1), (64, 2), (65, 1), (66, 2), (98, 1), (129, 2)])
+def test_operator_overwrites_every_entry(n, bc_kind):
+    u = P.random_field(n, 400 + n)
+    y = torch.full((n + 1,) * 3, float("nan"), dtype=torch.float64, device=DEV)
+    B.stencil_apply(B.Level(n, bc_kind), dev(u), y)
+    assert rel_max(y.cpu().numpy(), oracle.stencil_apply(n, bc_kind, u)) <= 1e-12
+
+
+@pytest.mark.parametrize("n,stride", [(5, 1), (9, 2), (64, 1), (65, 1), (70, 2)])
+@pytest.mark.parametrize("bc_kind", [1, 2])
+def test_right_hand_side(n, stride, bc_kind):
+    ns = n * stride
+    f, g1 = P.random_field(ns, 410), P.random_field(ns, 411)
+    g2 = np.random.Generator(np.random.PCG64(412)).uniform(-1, 1, size=(6, ns + 1, ns + 1))
+    fh = B.excmg_assemble_rhs(B.Level(n, bc_kind), ns, dev(f), dev(g1), dev(g2)).cpu().numpy()
+    ref = oracle.assemble_rhs(n, bc_kind, oracle.inject_nodes(ns, stride, f), oracle.inject_nodes(ns, stride, g1),
+                              oracle.inject_faces(ns, stride, g2))
+    assert np.abs(fh - ref).max() <= 1e-13 * max(1.0, np.abs(ref).max())
+
+
+@pytest.mark.parametrize("nf", [12, 28, 64, 68, 100])
+def test_transfers(nf):
+    u1, u0, uh = P.random_field(nf // 2, 420), P.random_field(nf // 4, 421), P.random_field(nf, 422)
+    w = B.extrapolate_interpolate(nf, dev(u1), dev(u0)).cpu().numpy()
+    assert rel_max(w, oracle.exp_finite(nf, u1, u0)) <= 1e-13
+    ut = B.midpoint_extrapolate(nf, dev(uh), dev(u1)).cpu().numpy()
+    assert rel_max(ut, oracle.exp_true(nf, uh, u1)) <= 1e-13
