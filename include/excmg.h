@@ -135,10 +135,10 @@ int excmg_ctx_set_stencil(excmg_ctx *ctx, int variant);
 enum { EXCMG_SHADOW_FULL = 0, EXCMG_SHADOW_ELIDED = 1 };
 int excmg_ctx_set_shadow_mode(excmg_ctx *ctx, int mode);
 
-/* How a Bi-CG iteration is split into kernels on grids above 64^3 (integer
+/* How a Bi-CG iteration is split into kernels on grids above 81^3 (integer
  * operator); both give the same iterates up to the reduction order of sigma
- * (same bits within one schedule).  Grids up to 64^3 run a three-phase
- * cooperative launch in both.
+ * (same bits within one schedule).  Grids up to 81^3 keep their
+ * vectors on chip for many iterations of one cooperative launch in both.
  * EXCMG_SCHEDULE_FUSED (default): the operator launch first forms
  *   p = r + beta p and p* = r* + beta p* from the previous directions on
  *   every node it loads (writing the nodes it owns into a second buffer
@@ -150,7 +150,7 @@ enum { EXCMG_SCHEDULE_SEPARATE = 0, EXCMG_SCHEDULE_FUSED = 1 };
 int excmg_ctx_set_schedule(excmg_ctx *ctx, int schedule);
 
 /* CUDA graphs (default on): on grids solved by launched kernels (above
- * 64^3), every full batch of Bi-CG iterations after the first -- the same
+ * 81^3), every full batch of Bi-CG iterations after the first -- the same
  * sequence of launches each time, all of them reading their scalars and
  * their stop flag from the device -- is captured once into a CUDA graph (on
  * a private stream of the context) and replayed, cached per grid size,
@@ -291,7 +291,7 @@ int excmg_dsolve(const excmg_level *level, const double *fh, double *u);
  * level hierarchy resident; the Bi-CG iterations of the instances that need
  * them run per level group (instances of one precision at one grid size),
  * each group on its own stream and taken back as soon as it completes: on
- * grids up to 64^3 one launch per member that keeps its vectors on chip, on
+ * grids up to 81^3 one launch per member that keeps its vectors on chip, on
  * larger grids one cooperative launch for all members of a group of FP32
  * correction solves, the single solver's kernels per member in FP64.  Instances may be submitted at any time and leave when
  * done, so the batch refills continuously. */

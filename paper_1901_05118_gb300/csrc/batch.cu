@@ -9,15 +9,15 @@
 // EXP_true.  The Bi-CG iterations (Alg. 2, M = I, r*_0 = r_0) of the
 // instances waiting for them run per level group -- instances of one
 // precision at one grid size -- each group on its own stream:
-//  * grids up to 64^3 (both precisions): one launch of the resident kernel
+//  * grids up to 81^3 (both precisions): one launch of the resident kernel
 //    (resident.cuh) per member, on as many CTAs as resident_batch_limit
 //    gives that grid, side by side as far as the GPU's SMs go;
-//  * FP32 correction solves above 64^3: one cooperative launch for
+//  * FP32 correction solves above 81^3: one cooperative launch for
 //    all members; CTAs take operator tiles and vector chunks from every
 //    member, members advance in lock step one iteration per grid-barrier
 //    round, and each member's scalars are formed by the CTA that completes
 //    its last tile / chunk;
-//  * FP64 grids above 64^3 (launched mode): per member and round the single
+//  * FP64 grids above 81^3 (launched mode): per member and round the single
 //    solver's fused operator and update kernels with the member's own state.
 // Instances can be submitted at any time (the engine admits them against
 // its device-memory budget) and leave as soon as they are done, so the
@@ -348,7 +348,7 @@ struct Instance {
     // FP64 Bi-CG vectors (r is `res`)
     double *rs64 = nullptr, *p64 = nullptr, *ps64 = nullptr, *q64 = nullptr;
     double *p2_64 = nullptr, *ps2_64 = nullptr;   // second direction pair
-    // launched mode (FP64 levels above 64^3): iterations of the current
+    // launched mode (FP64 levels above 81^3): iterations of the current
     // Bi-CG call enqueued so far, and which direction pair holds p_k
     long long launched_k = 0;
     bool dir_in_p2 = false;

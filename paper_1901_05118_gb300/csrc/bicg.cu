@@ -106,8 +106,13 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // the integer operator has a fused two-field kernel; the FP64 one runs
     // as two applications and a separate inner product
     const bool fused = ctx->stencil_variant == kStencilExact && stencil_cta_count(n) <= kMaxPartials;
-    // small grids run whole iterations in one cooperative launch
-    const bool persistent = fused && n <= kPersistentMaxN;
+    // small grids run whole iterations in one cooperative launch: with every
+    // vector on chip from r*_0 = r_0; a caller-chosen r*_0, or no room for the
+    // exchange words, the general cooperative kernel up to 64^3
+    void* words =
+        fused && shadow == nullptr && resident_ctas(n, 0) > 0 ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
+    const bool resident = words != nullptr;
+    const bool persistent = resident || (fused && n <= kPersistentMaxN);
     // the fused schedule (the default on the launched levels) folds
     // p = r + beta p into the operator step, which reads the previous
     // directions from one buffer pair and writes the new ones to the other
@@ -115,10 +120,6 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // kernel of the small grids keeps a separate direction-update phase
     const bool fuse = ctx->schedule == EXCMG_SCHEDULE_FUSED;
     const bool dir_fused = fused && fuse && !persistent;
-    // r*_0 = r_0: with every vector on chip; a caller-chosen r*_0, or no room
-    // for the exchange words: the general cooperative kernel
-    void* words = persistent && shadow == nullptr && resident_ctas(n, 0) > 0 ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
-    const bool resident = words != nullptr;
     // the integer operator's A^T p* is A p bit for bit while p* = p, as it is
     // from r*_0 = r_0 on: both are read from q (the general cooperative
     // kernel keeps its second array)

@@ -103,6 +103,7 @@ size_t resident_bytes(int n);
 template <typename T>
 cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
                                  void* words, cudaStream_t s, bool elide, int max_ctas);
+constexpr int kResidentMaxN = 81;   // eight nodes per thread on 152 SMs
 // The 2D problem's form, on grids that fit on chip with four nodes per thread.
 constexpr int kPersistentMaxN2d = 512;
 int resident2d_ctas(int n);

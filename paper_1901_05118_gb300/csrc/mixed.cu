@@ -218,7 +218,7 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
     note_launches(1);
     if (err != cudaSuccess) return ctx_cuda(ctx, err, "FP32 Bi-CG setup");
     if (check_every < 1) check_every = 1;
-    // grids up to 64^3: many iterations per launch with every vector on chip
+    // grids up to 81^3: many iterations per launch with every vector on chip
     // (48^3: 5 us per iteration, against 25 us for the three launches,
     // each of them a few microseconds of latency for 0.5 MB vectors); larger
     // ones, or no room for the exchange words: the launched kernels

@@ -14,8 +14,13 @@ const void* resident_fn(int np) {
     switch (np) {
         case 1: return (const void*)resident_bicg_kernel<T, DIM, 1, DIM == 3 ? 2 : 1, kElide>;
         case 2: return (const void*)resident_bicg_kernel<T, DIM, 2, DIM == 3 ? 3 : 1, kElide>;
-        default: return (const void*)resident_bicg_kernel<T, DIM, 4, DIM == 3 ? 5 : 1, kElide>;
+        case 4: return (const void*)resident_bicg_kernel<T, DIM, 4, DIM == 3 ? 5 : 1, kElide>;
+        default: break;
     }
+    if constexpr (DIM == 3)
+        return np == 6 ? (const void*)resident_bicg_kernel<T, 3, 6, 6, kElide>
+                       : (const void*)resident_bicg_kernel<T, 3, 8, 7, kElide>;
+    return nullptr;
 }
 
 std::mutex g_geom_mu;
@@ -33,7 +38,7 @@ ResidentGeom resident_geometry_cached(int dim, int n, int max_ctas) {
 }
 
 int resident_ctas(int n, int max_ctas) {
-    if (n > kPersistentMaxN) return 0;
+    if (n > kResidentMaxN) return 0;
     return resident_geometry_cached(3, n, max_ctas > 0 ? max_ctas : device_sms()).ctas;
 }
 
@@ -41,7 +46,8 @@ int resident2d_ctas(int n) { return n > kPersistentMaxN2d ? 0 : resident_geometr
 
 // CTAs of a grid in the batch engine: fewer than a single solve takes, so that several instances run side by
 // side, and a number that depends on the grid alone (the sums do, too).  32^3 on 16 CTAs takes about 1.5
-// times as long per iteration as on its own 64, and nine fit beside each other; 64^3 leaves no choice.
+// times as long per iteration as on its own 64, and nine fit beside each other.  (64^3 on 72 CTAs: 18 against
+// 11 us per iteration; eight mixed requests then take 74 instead of 50 ms, as the last one waits for itself.)
 int resident_batch_limit(int n) { return n <= 32 ? 16 : n <= 52 ? 72 : 0; }
 
 namespace {
@@ -65,8 +71,8 @@ cudaError_t launch(const void* fn, ResidentGeom g, T* x, T* r, T* rs, T* p, T* p
                    BicgState* st, void* words, cudaStream_t s) {
     ResidentInst<T> in{x, r, rs, p, ps, st, (ulonglong2*)words, (ulonglong2*)((char*)words + slot_bytes()), n,
                        bc_kind == 1 ? 1 : -1};
-    const size_t smem = (size_t)g.tile * (sizeof(T) == 8 ? sizeof(long long) : sizeof(float));
-    (void)kernel_occupancy(fn, kResThreads, kResTileBytes);   // opts in to the shared memory
+    const size_t smem = (size_t)((g.tile + 1) & ~1) * sizeof(T) + resident_own_bytes(g.np) / 8 * sizeof(T);
+    (void)kernel_occupancy(fn, kResThreads, kResSmemBytes);   // opts in to the shared memory
     unsigned serial = next_serial();
     long long limit = kBarrierSpinLimit;
     void* args[] = {&in, &g, &iters, &serial, &limit};

@@ -31,7 +31,8 @@
 //    conversion goes through the FP64 pipe: the same time here).
 // Measured: 200 iterations on 64^3 2.23 ms (the general cooperative kernel:
 // 5.63 ms), a whole 32^3 first-kind solve to 1e-10 5.4 ms (14.8 ms); 100
-// iterations of the 512^2 problem 1.00 ms (three launches each: 3.08 ms).
+// iterations of the 512^2 problem 1.00 ms (three launches each: 3.08 ms); per
+// iteration 66^3 10.9 us, 72^3 14.0, 80^3 18.2 (launched kernels: 34.9, 36.1, 37.7).
 //
 // Shadow sequence: the launches start from r*_0 = p*_0 = r_0 = p_0 (a
 // caller-chosen r*_0 takes the general kernel in stencil.cu).  A^T p* is A p
@@ -145,6 +146,18 @@ __device__ __forceinline__ float sum_f32(float v) {
     return v;
 }
 
+// A thread's NP values of one vector: in registers, or (kShared) in shared
+// memory at v[k * kResThreads].
+template <typename T, int NP, bool kShared>
+struct OwnValues {
+    T reg[kShared ? 1 : NP];
+    T* v;
+    __device__ __forceinline__ T& operator[](int k) {
+        if constexpr (kShared) return v[k * kResThreads];
+        else return reg[k];
+    }
+};
+
 // NP: nodes of a thread's run along z; NH: nodes around the brick per thread.
 template <typename T, int DIM, int NP, int NH, bool kElide>
 __global__ void __launch_bounds__(kResThreads, 1)
@@ -213,7 +226,14 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
     if (tid == 0) lost = 0;
     __syncthreads();   // (FP32: the first tile is written without another barrier before it)
 
-    T x[NP], r[NP], p[NP], q[NP], rs[NP], ps[NP], hp[NH], hr[NH];
+    T r[NP], p[NP], q[NP], hp[NH], hr[NH];
+    OwnValues<T, NP, (NP > kResRegNodes)> x, rs, ps;
+    if constexpr (NP > kResRegNodes) {
+        T* const own = reinterpret_cast<T*>(res_smem + (size_t)((g.tile + 1) & ~1) * sizeof(Fix)) + tid;
+        x.v = own;
+        rs.v = own + NP * kResThreads;
+        ps.v = own + 2 * NP * kResThreads;
+    }
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
         x[k] = r[k] = p[k] = q[k] = rs[k] = ps[k] = T(0);

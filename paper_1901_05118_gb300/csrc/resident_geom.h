@@ -34,12 +34,16 @@ struct ResidentGeom {
 // the 4-byte entries of the FP32 kernel share the layout).
 constexpr int kResPad = 16;
 
-// Shared memory for the tile; the kernels are opted in to this much once, as
-// the launches of different grids share them.
-constexpr size_t kResTileBytes = 160 * 1024;
+// Shared memory of a CTA at most; the kernels are opted in to this much once,
+// as the launches of different grids share them.
+constexpr size_t kResSmemBytes = 212 * 1024;
 
 // Nodes around the brick per thread of the variant with np nodes per thread.
-inline int resident_nh(int np) { return np == 1 ? 2 : np == 2 ? 3 : 5; }
+inline int resident_nh(int np) { return np == 1 ? 2 : np == 2 ? 3 : np == 4 ? 5 : np == 6 ? 6 : 7; }
+
+// Variants with more nodes per thread keep x, r*, p* in shared memory.
+constexpr int kResRegNodes = 4;
+inline size_t resident_own_bytes(int np) { return np > kResRegNodes ? (size_t)3 * np * kResThreads * 8 : 0; }
 
 // Node h of the nodes around a brick that the taps of its nodes reach: two
 // layers on each face and one row along each edge.  Local coordinates
@@ -134,13 +138,13 @@ inline ResidentGeom resident_geometry(int n, int max_ctas) {
                 const int cz = (m + bz - 1) / bz;
                 if (cx * cy * cz > max_ctas || (m + cz - 1) / cz != bz) continue;
                 const int halo = 4 * (bx * by + bx * bz + by * bz) + 4 * (bx + by + bz);
-                for (int np = 1; np <= 4; np *= 2) {
+                for (int np = 1; np <= 8; np += np < 2 ? 1 : 2) {
                     const int threads = bx * by * ((bz + np - 1) / np);
                     const int nh = resident_nh(np);
                     const int runs = (bz + np - 1) / np * np;
                     const int tile = (bx + kResPad) * (by + 4) * (runs + 4);
                     if (threads > kResThreads || halo > nh * kResHaloThreads ||
-                        (size_t)tile * 8 > kResTileBytes)
+                        (size_t)tile * 8 + resident_own_bytes(np) > kResSmemBytes)
                         continue;
                     const long long cost = 5LL * np * ((threads + 127) / 128) * 128 + halo + 40LL * cx * cy * cz;
                     if (best_cost < 0 || cost < best_cost) {
@@ -170,7 +174,7 @@ inline ResidentGeom resident_geometry2d(int n, int max_ctas) {
             for (int np = 1; np <= 4; np *= 2) {
                 const int threads = bx * ((bz + np - 1) / np), runs = (bz + np - 1) / np * np;
                 const int tile = (bx + kResPad) * (runs + 4);
-                if (threads > kResThreads || halo > nh * kResHaloThreads || (size_t)tile * 8 > kResTileBytes) continue;
+                if (threads > kResThreads || halo > nh * kResHaloThreads || (size_t)tile * 8 > kResSmemBytes) continue;
                 const long long cost = 5LL * np * ((threads + 127) / 128) * 128 + halo + 40LL * cx * cz;
                 if (best_cost < 0 || cost < best_cost) {
                     best_cost = cost;

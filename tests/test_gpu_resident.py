@@ -28,8 +28,8 @@ def rel_max(got, ref):
 
 
 @pytest.mark.parametrize("n,bc_kind,iters", [(4, 1, 9), (5, 2, 12), (9, 1, 20), (14, 2, 20), (23, 1, 20), (33, 2, 20),
-                                             (41, 1, 20), (47, 2, 20), (53, 1, 20), (58, 2, 20), (63, 1, 20),
-                                             (64, 2, 20)])
+                                             (41, 1, 20), (47, 2, 20), (53, 1, 20), (58, 2, 20), (63, 1, 20), (65, 2, 20),
+                                             (64, 2, 20), (67, 1, 20), (74, 2, 20), (81, 1, 20), (82, 2, 20)])
 def test_iterates_match_the_oracle(n, bc_kind, iters):
     """Fixed iteration counts from random data: entry by entry within the
     1e-10 that a few dozen FP64 Bi-CG steps in another summation order keep."""

@@ -16,11 +16,11 @@ PROGRAM = r"""
 using namespace excmg;
 static void fail(const char* what, int n) { std::printf("%s at n = %d\n", what, n); std::exit(1); }
 int main() {
-    for (int limit : {152, 132, 40, 16, 1})
-    for (int n = 4; n <= 72; ++n) {
+    for (int limit : {152, 132, 72, 16, 1})
+    for (int n = 4; n <= 84; ++n) {
         const ResidentGeom g = resident_geometry(n, limit);
         if (g.ctas == 0) {
-            if (limit == 152 && n <= 64) fail("no cut", n);
+            if (limit == 152 && n <= 81) fail("no cut", n);
             continue;
         }
         if (g.ctas != g.cx * g.cy * g.cz || g.ctas > limit || g.ctas > kResMaxCtas) fail("CTAs", n);
