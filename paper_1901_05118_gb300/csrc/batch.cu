@@ -352,6 +352,7 @@ struct Instance {
     // Bi-CG call enqueued so far, and which direction pair holds p_k
     long long launched_k = 0;
     bool dir_in_p2 = false;
+    double t_ready = 0.0;       // when the instance last became ready for Bi-CG iterations
     bool no_resident = false;   // the current call runs without the resident kernel (no room for its words)
     // FP32 correction solve vectors
     float *r32 = nullptr, *e = nullptr, *r = nullptr, *rs = nullptr, *p = nullptr, *ps = nullptr, *q = nullptr,
@@ -886,7 +887,10 @@ int harvest(excmg_batch* b, excmg_batch::Group& g) {
     for (Instance* in : g.members) {
         if (in->phase != kInner) continue;
         const BatchState& hs = b->h_states[in->slot];
-        if (!hs.done) continue;   // the launch's iteration chunk ended first
+        if (!hs.done) {   // the launch's iteration chunk ended first
+            in->t_ready = now_s();
+            continue;
+        }
         if (hs.status == kBreakdown) {
             in->phase = kFailed;
             in->status = EXCMG_ERR_BREAKDOWN;
@@ -1268,6 +1272,7 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
             }
             if (e != cudaSuccess) return bcuda(b, e, "Bi-CG call setup");
             in->phase = kInner;
+            in->t_ready = now_s();
             in->call_iter = 0;
             in->no_resident = false;
         }
@@ -1286,21 +1291,48 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
         for (auto& kv : ready)
             order.push_back({-(long long)kv.second.size() * node_count(kv.first.second), kv.first});
         std::sort(order.begin(), order.end());
+        auto free_group = [&]() -> excmg_batch::Group& {
+            for (auto& g : b->groups)
+                if (!g.busy) return g;
+            b->groups.emplace_back();
+            return b->groups.back();
+        };
+        auto held = [&]() {
+            int used = 0;
+            for (auto& g : b->groups)
+                if (g.busy) used += g.sm_share;
+            return used;
+        };
+        // An on-chip level that needs most of the SMs could be kept out for
+        // good by a stream of small ones that take each SM as it comes free.
+        // So the one that has waited longest, if longer than kOverdue (some
+        // 2000 iterations at 64^3), goes first, and while it does not fit
+        // nothing else is started.  Eight mixed requests take as long as
+        // without the rule, and as long with small grids always first.
+        constexpr double kOverdue = 0.02;
+        Instance* late = nullptr;
+        for (auto& kv : ready)
+            for (Instance* in : kv.second)
+                if (!in->no_resident && resident_ctas(kv.first.second, resident_batch_limit(kv.first.second)) > 0 &&
+                    now_s() - in->t_ready > kOverdue && (!late || in->t_ready < late->t_ready))
+                    late = in;
+        if (late) {
+            const int N = late->nc << late->level, res = resident_ctas(N, resident_batch_limit(N));
+            if (res * batch_ctas_per_sm() > capacity() - held()) {
+                order.clear();
+            } else {
+                const bool taken = launch_resident(b, free_group(), late, res, &st);
+                if (st) return st;
+                if (taken) {
+                    std::vector<Instance*>& list = ready[{late->prec, N}];
+                    list.erase(std::find(list.begin(), list.end(), late));
+                }
+            }
+        }
         for (auto& o : order) {
             const auto key = o.second;
             std::vector<Instance*>& list = ready[key];
-            auto free_group = [&]() -> excmg_batch::Group& {
-                for (auto& g : b->groups)
-                    if (!g.busy) return g;
-                b->groups.emplace_back();
-                return b->groups.back();
-            };
-            auto held = [&]() {
-                int used = 0;
-                for (auto& g : b->groups)
-                    if (g.busy) used += g.sm_share;
-                return used;
-            };
+            if (list.empty()) continue;
             const int res = resident_ctas(key.second, resident_batch_limit(key.second));
             if (res > 0) {
                 // per member, as many as find their SMs free; the others

@@ -109,3 +109,23 @@ def test_mixed_levels(n, nc, bc_kind):
     fh = B.excmg_assemble_rhs(lvl, n, f, g1, g2)
     rel = float((fh - B.stencil_apply(lvl, uh)).norm() / fh.norm())
     assert rel <= 1e-10 * (1 + 1e-3)
+
+
+def test_batch_large_level_is_not_kept_out():
+    """A 64^3 level needs most of the SMs at once; a stream of 32^3 requests
+    that takes every SM as it comes free must not keep it waiting.  Each of
+    its Bi-CG calls may wait 20 ms plus one launch of a small level, in which
+    the stream finishes some 100 requests: 2000 are a wide margin."""
+    prob = P.by_name("random_sines:4")
+    big, small = ([dev(a) for a in prob.data(n, 2)] for n in (64, 32))
+    batch = B.Batch(max_instances=16)
+    ident, _ = batch.submit(64, 8, 2, *big, 1e-8, precision="fp64")
+    live = [batch.submit(32, 4, 2, *small, 1e-10, precision="fp64")[0] for _ in range(13)]
+    done = 0
+    while not batch.query(ident)["done"] and done < 2000:
+        batch.step()
+        left = [k for k in live if not batch.query(k)["done"]]
+        done += len(live) - len(left)
+        live = left + [batch.submit(32, 4, 2, *small, 1e-10, precision="fp64")[0] for _ in range(13 - len(left))]
+    assert batch.query(ident)["done"]
+    batch.run()
