@@ -45,6 +45,7 @@
 #include <cuda_runtime.h>
 
 #include "march_fx.cuh"
+#include "reduce.cuh"
 
 namespace excmg {
 namespace {
@@ -275,9 +276,13 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
                     diff |= (__double_as_longlong(ps[s]) ^ __double_as_longlong(po[s])) |
                             (__double_as_longlong(rsv[s]) ^ __double_as_longlong(rv[s]));
             }
-            if (K == kMarchDir && diff != 0) {
+            if (K == kMarchDir) {
+                const int rare = opaque(diff != 0);
+#pragma unroll 1
+                for (int once = 0; once < rare; ++once) {
 #pragma unroll
-                for (int s = 0; s < 2; ++s) vs[s] = __fma_rn(a.beta, ps[s], rsv[s]);
+                    for (int s = 0; s < 2; ++s) vs[s] = fma_here(a.beta, ps[s], rsv[s]);
+                }
             }
         }
     };

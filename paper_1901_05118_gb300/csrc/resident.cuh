@@ -29,16 +29,17 @@
 //    and no FP64 comparisons: they go through the same pipe;
 //  * outputs rounded with integer instructions (fx_result; the hardware
 //    conversion goes through the FP64 pipe: the same time here).
-// Measured: 200 iterations on 64^3 2.23 ms (the general cooperative kernel:
-// 5.63 ms), a whole 32^3 first-kind solve to 1e-10 5.4 ms (14.8 ms); 100
+// Measured: 200 iterations on 64^3 2.13 ms (the general cooperative kernel:
+// 5.63 ms), a whole 32^3 first-kind solve to 1e-10 4.9 ms (14.8 ms); 100
 // iterations of the 512^2 problem 1.00 ms (three launches each: 3.08 ms); per
-// iteration 66^3 10.9 us, 72^3 14.0, 80^3 18.2 (launched kernels: 34.9, 36.1, 37.7).
+// iteration 72^3 13.8 us, 80^3 18.0 (launched kernels: 36.1, 37.7).
 //
 // Shadow sequence: the launches start from r*_0 = p*_0 = r_0 = p_0 (a
 // caller-chosen r*_0 takes the general kernel in stencil.cu).  A^T p* is A p
 // bit for bit where p* = p (march_fx.cuh), so q serves both; r* and p* are
 // updated entry by entry, with the primal result reused where the operands
-// agree bit for bit.  kElide: r*, p* are not kept (the same bits).
+// of a thread agree bit for bit; the other case is kept out of the FP64 pipe's
+// way (opaque in reduce.cuh).  kElide: r*, p* are not kept (the same bits).
 //
 // DIM = 2: the 2D problem's 13-point rows (excmg2d.cu), with the second axis in
 // the place of z and no third one.
@@ -138,6 +139,10 @@ __device__ __noinline__ bool root_at_most(double a, double b) { return sqrt(a) <
 // a b + c, fused: written out so that every variant of the kernel rounds alike
 __device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
+// The same where it is rarely reached: not evaluated ahead of its branch.
+__device__ __forceinline__ double mad_here(double a, double b, double c) { return fma_here(a, b, c); }
+__device__ __forceinline__ float mad_here(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
 // a sum over the warp in FP32 (every lane gets it)
 __device__ __forceinline__ float sum_f32(float v) {
@@ -324,14 +329,25 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
         // p = r + beta p
         if (iter > 0) {
             const T b = (T)beta;
+            bool twin = kExact;
+            if (kExact && !kElide) {
 #pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                const T pn = mad(b, p[k], r[k]);
-                if (!kElide) {
-                    if (kExact && same_bits(rs[k], r[k]) && same_bits(ps[k], p[k])) ps[k] = pn;
-                    else ps[k] = mad(b, ps[k], rs[k]);
+                for (int k = 0; k < NP; ++k) twin = twin && same_bits(rs[k], r[k]) && same_bits(ps[k], p[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < NP; ++k) p[k] = mad(b, p[k], r[k]);
+            if (!kElide) {
+                T pn[NP];
+#pragma unroll
+                for (int k = 0; k < NP; ++k) pn[k] = p[k];
+                const int general = kExact ? opaque(!twin) : 1;
+#pragma unroll 1
+                for (int once = 0; once < general; ++once) {
+#pragma unroll
+                    for (int k = 0; k < NP; ++k) pn[k] = mad_here(b, ps[k], rs[k]);
                 }
-                p[k] = pn;
+#pragma unroll
+                for (int k = 0; k < NP; ++k) ps[k] = pn[k];
             }
 #pragma unroll
             for (int k = 0; k < NH; ++k) hp[k] = mad(b, hp[k], hr[k]);
@@ -425,20 +441,38 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
         // r -= alpha q, r* -= alpha q*
         const T a = (T)bcast[0];
         const unsigned long long rtag = tag0 | (unsigned)(it + 1);
-        T vr = T(0);
+        T vr = T(0), rn[NP];
+#pragma unroll
+        for (int k = 0; k < NP; ++k) rn[k] = mad(-a, q[k], r[k]);
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
-            const T rn = mad(-a, q[k], r[k]);
             if (surf >> k & 1u) {
-                if constexpr (kExact) st_word(in.rx + idx0 + k * plane, bits_of(rn), rtag);
-                else st_word(in.rx + idx0 + k * plane, (unsigned long long)__float_as_uint(rn), rtag);
+                if constexpr (kExact) st_word(in.rx + idx0 + k * plane, bits_of(rn[k]), rtag);
+                else st_word(in.rx + idx0 + k * plane, (unsigned long long)__float_as_uint(rn[k]), rtag);
             }
-            if (!kElide) {
-                if (kExact && same_bits(rs[k], r[k])) rs[k] = rn;
-                else rs[k] = mad(-a, q[k], rs[k]);
+        }
+        if (!kElide) {
+            bool twin = kExact;
+            if (kExact) {
+#pragma unroll
+                for (int k = 0; k < NP; ++k) twin = twin && same_bits(rs[k], r[k]);
             }
-            r[k] = rn;
-            vr = mad(kElide ? rn : rs[k], rn, vr);
+            T rsn[NP];
+#pragma unroll
+            for (int k = 0; k < NP; ++k) rsn[k] = rn[k];
+            const int general = kExact ? opaque(!twin) : 1;
+#pragma unroll 1
+            for (int once = 0; once < general; ++once) {
+#pragma unroll
+                for (int k = 0; k < NP; ++k) rsn[k] = mad_here(-a, q[k], rs[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < NP; ++k) rs[k] = rsn[k];
+        }
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            r[k] = rn[k];
+            vr = mad(kElide ? rn[k] : rs[k], rn[k], vr);
         }
         // exchange 2: rho (r* = r bit for bit, so (r, r) is the same sum),
         // beta, the stopping test; x += alpha p and the r of the nodes

@@ -197,21 +197,18 @@ bicg_update_kernel(double* __restrict__ x, const double* __restrict__ p, double*
             if (t >= len) break;
             const double rn = __fma_rn(-alpha, qv[k], rv[k]);
             r[t] = rn;
-            if (__double_as_longlong(rsv[k]) == __double_as_longlong(rv[k]) &&
-                __double_as_longlong(qsv[k]) == __double_as_longlong(qv[k])) {
-                rs[t] = rn;
-                if (!twin) vr = __fma_rn(rn, rn, vr);
-                vrr = __fma_rn(rn, rn, vrr);
-            } else {
+            double rsn = rn;
+            if (!twin || __double_as_longlong(rsv[k]) != __double_as_longlong(rv[k]) ||
+                __double_as_longlong(qsv[k]) != __double_as_longlong(qv[k])) {
                 if (twin) {
                     vr = vrr;
                     twin = false;
                 }
-                const double rsn = __fma_rn(-alpha, qsv[k], rsv[k]);
-                rs[t] = rsn;
-                vr = __fma_rn(rsn, rn, vr);
-                vrr = __fma_rn(rn, rn, vrr);
+                rsn = fma_here(-alpha, qsv[k], rsv[k]);
+                vr = fma_here(rsn, rn, vr);
             }
+            rs[t] = rsn;
+            vrr = __fma_rn(rn, rn, vrr);
             x[t] = __fma_rn(alpha, pv[k], xv[k]);
         }
     }
@@ -264,11 +261,11 @@ bicg_pupdate_kernel(double* __restrict__ p, const double* __restrict__ r, double
             if (t >= len) break;
             const double pn = __fma_rn(beta, pv[k], rv[k]);
             p[t] = pn;
-            if (__double_as_longlong(rsv[k]) == __double_as_longlong(rv[k]) &&
-                __double_as_longlong(psv[k]) == __double_as_longlong(pv[k]))
-                ps[t] = pn;
-            else
-                ps[t] = __fma_rn(beta, psv[k], rsv[k]);
+            double psn = pn;
+            if (__double_as_longlong(rsv[k]) != __double_as_longlong(rv[k]) ||
+                __double_as_longlong(psv[k]) != __double_as_longlong(pv[k]))
+                psn = fma_here(beta, psv[k], rsv[k]);
+            ps[t] = psn;
         }
     }
 }
