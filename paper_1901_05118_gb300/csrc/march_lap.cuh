@@ -145,10 +145,10 @@ __host__ __device__ __forceinline__ void ml_ring(int e, int* lx, int* ly) {
     }
 }
 
-// What a march does: A u or b - A u; with r = b - A u the start of a Bi-CG
+// What a march does: A u; b - A u; with r = b - A u the start of a Bi-CG
 // call (r, p, and r*, p* where given, and (r, r)) or (r, r) alone; (p, p*) ->
 // q with sigma; the same with p = r + beta p, p* = r* + beta p* formed first.
-enum MarchKind { kMarchApply, kMarchStart, kMarchNorm, kMarchPair, kMarchDir };
+enum MarchKind { kMarchApply, kMarchSub, kMarchStart, kMarchNorm, kMarchPair, kMarchDir };
 constexpr bool march_is_step(MarchKind k) { return k == kMarchPair || k == kMarchDir; }
 
 struct MarchArrays {
@@ -156,7 +156,7 @@ struct MarchArrays {
     const double* r;      // kMarchDir
     const double* ins;    // p* or p*_{k-1}
     const double* rs;     // kMarchDir
-    const double* b;      // right-hand side (kMarchApply: may be null)
+    const double* b;      // right-hand side (kMarchSub, kMarchStart, kMarchNorm)
     double* out;          // y or q (q* = q: the same bits, not stored again)
     double* pn;           // kMarchDir: p_k (not in: neighbours still read it); kMarchStart: p, may be null
     double* psn;          // the same for p*
@@ -169,7 +169,7 @@ struct MarchArrays {
 template <MarchKind K, bool kElide>
 struct MarchStage {
     static constexpr int kAll = K == kMarchDir ? 2 : 1;
-    static constexpr int kOwn = !march_is_step(K) ? 1 : kElide ? 0 : kAll;
+    static constexpr int kOwn = K == kMarchApply ? 0 : !march_is_step(K) ? 1 : kElide ? 0 : kAll;
     static constexpr unsigned kBytes = (kAll * 3 + kOwn * 2) * PP_NT * 8u;
     static constexpr unsigned kHist = !march_is_step(K) ? 0 : 4 * 2 * PP_NT * 8u;
     static constexpr size_t kSmem = kBytes + kHist + 4 * PP_HALO * sizeof(long long);
@@ -194,7 +194,7 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
     const int i0 = 1 + bx * PP_TX, j0 = 1 + by * PP_OY;
     const bool ring = tid < PP_RING, inner = tid < ML_INNER;
     constexpr bool kStep = march_is_step(K);
-    const bool has_b = !kStep && a.b != nullptr;
+    constexpr bool has_b = !kStep && K != kMarchApply;
 
     // in-plane byte offset of each slot, copy size (0: reads as zero), tile entry
     unsigned so[3], sz[3], te[3];
@@ -403,7 +403,7 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
                             if (a.rsn) *(double*)((char*)a.rsn + o) = rv;
                             if (a.psn) *(double*)((char*)a.psn + o) = rv;
                         }
-                        if (K != kMarchApply) d = __fma_rn(rv, rv, d);
+                        if (K != kMarchApply && K != kMarchSub) d = __fma_rn(rv, rv, d);
                     }
                 }
             }

@@ -98,16 +98,20 @@ stencil_f64_kernel(const double* __restrict__ u, double* __restrict__ y, const d
     }
 }
 
-// y = A u, or y = b - A u.
-__global__ void __launch_bounds__(PP_NT, 3)
+// y = A u (K = kMarchApply), or y = b - A u (kMarchSub; as a run-time choice the
+// subtraction went through the FP64 pipe in either case).  Two CTAs per SM, as
+// with three the register limit costs a fifth more instructions: A u on 100^3 / 133^3
+// / 512^3 37 / 50 / 969 us with two, 43 / 53 / 980 with three, 42 / 56 / 1006 with
+// four (three, with b at run time: 45 / 57 / 1082).
+template <MarchKind K>
+__global__ void __launch_bounds__(PP_NT, 2)
 stencil_apply_kernel(const double* __restrict__ u, double* __restrict__ y, const double* __restrict__ b, int n,
                      int sigma, int kz_per_cta, const int* __restrict__ skip) {
     extern __shared__ __align__(128) unsigned char march_smem[];
     if (skip != nullptr && *skip) return;
     const int kz0 = 1 + blockIdx.z * kz_per_cta;
     const MarchArrays a{u, nullptr, nullptr, nullptr, b, y, nullptr, nullptr, 0.0, nullptr};
-    (void)lap_march<kMarchApply, true>(a, n, sigma, blockIdx.x, blockIdx.y, kz0, min(kz0 + kz_per_cta, n),
-                                       march_smem);
+    (void)lap_march<K, true>(a, n, sigma, blockIdx.x, blockIdx.y, kz0, min(kz0 + kz_per_cta, n), march_smem);
 }
 
 // Every CTA's share of rr = (r, r): the last one writes the sum to *out, and
@@ -262,7 +266,7 @@ stencil_point_kernel(MarchArrays a, int n, int sigma, const int* __restrict__ sk
             if (a.psn) a.psn[t] = v;
         }
     }
-    if constexpr (K != kMarchApply) finish_norm(v * v, partials, ticket, out, st);
+    if constexpr (K != kMarchApply && K != kMarchSub) finish_norm(v * v, partials, ticket, out, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -558,9 +562,10 @@ StencilGrid march_grid(int n, int per_sm, size_t smem) {
 }
 
 // The single-field operator launch (A u, b - A u).
+template <MarchKind K>
 StencilGrid apply_grid(int n) {
-    constexpr size_t smem = MarchStage<kMarchApply, true>::kSmem;
-    return march_grid(n, resident_per_sm(stencil_apply_kernel, PP_NT, smem), smem);
+    constexpr size_t smem = MarchStage<K, true>::kSmem;
+    return march_grid(n, resident_per_sm(stencil_apply_kernel<K>, PP_NT, smem), smem);
 }
 
 // Node-by-node form of the single-field launches: as long as all nodes are
@@ -591,7 +596,7 @@ StencilGrid f64_grid(int n) {
 }  // namespace
 
 int stencil_cta_count(int n) {
-    const StencilGrid g1 = apply_grid(n), g2 = step_grid<kMarchDir, false>(n);
+    const StencilGrid g1 = apply_grid<kMarchApply>(n), g2 = step_grid<kMarchDir, false>(n);
     unsigned most = max(g1.grid.x * g1.grid.y * g1.grid.z, g2.grid.x * g2.grid.y * g2.grid.z);
     const StencilGrid g3 = march_grid(n, 2, 0);   // the residual launches: two CTAs per SM
     most = max(most, g3.grid.x * g3.grid.y * g3.grid.z);
@@ -616,8 +621,9 @@ cudaError_t launch_stencil(const double* u, double* y, const double* b, int n, i
             stencil_point_kernel<kMarchApply><<<point_blocks(n), 256, 0, s>>>(a, n, sg, skip, nullptr, nullptr,
                                                                               nullptr, nullptr);
         } else {
-            const StencilGrid g = apply_grid(n);
-            stencil_apply_kernel<<<g.grid, g.block, g.smem, s>>>(u, y, b, n, sg, g.kz_per_cta, skip);
+            const StencilGrid g = b ? apply_grid<kMarchSub>(n) : apply_grid<kMarchApply>(n);
+            (b ? stencil_apply_kernel<kMarchSub> : stencil_apply_kernel<kMarchApply>)<<<g.grid, g.block, g.smem, s>>>(
+                u, y, b, n, sg, g.kz_per_cta, skip);
         }
     }
     return cudaGetLastError();

@@ -19,6 +19,7 @@
 // which is (4 u_h - u_2h)/3 at coarse nodes and (chenlin) at 1D midpoints.
 
 #include "excmg_internal.cuh"
+#include "reduce.cuh"
 
 namespace excmg {
 namespace {
@@ -42,20 +43,24 @@ constexpr int TM_X = TT_X / 2 + 1, TM_Y = TT_Y / 2 + 1, TM_Z = TT_Z / 2 + 1;   /
 // Row of the tile of a warp: the even rows on warps 0 .. 3, the odd ones, which
 // have FP64 work along y, on warps 4 .. 7, one on each sub-partition (on
 // every second warp they kept two of the four FP64 pipes idle: 1.08 instead
-// of 0.8 ms for Step 5 at 512^3).
+// of 0.8 ms for Step 5 at 512^3).  The kernels skip that work on the even rows by a
+// loop of 0 or 1 trips (opaque in reduce.cuh): as a branch it became
+// predicated FP64 instructions, which hold the pipe on every row.
 __device__ __forceinline__ int tile_row(int warp) { return 2 * (warp & 3) + (warp >> 2); }
 
 // out = u + kWeight * (mean of d = u - uc over the 1, 2, 4 or 8 coarse nodes
 // around each node), u on the grid with nf intervals, uc on the one with nf / 2:
 // EXP_true with weight 1/3, Steps 1-4 of EXP_finite with weight 1/4
 // (kQuarter), where every scaling is a power of two.
-// Measured on 256^3 (42 us of HBM traffic): see launch_exp_true.
+// Measured, EXP_true on 256^3 / 512^3 (42 / 320 us of HBM traffic, about 60 / 480 of
+// FP64 issue): 107 / 614 us (124 / 747 with predicated sums along y and one row per warp
+// along x; 135 / - with every intermediate value through shared memory).
 template <bool kQuarter>
 __global__ void __launch_bounds__(TT_THREADS)
 extrapolate_tiled_kernel(double* __restrict__ out, const double* __restrict__ u, const double* __restrict__ uc,
                          int nf) {
     __shared__ double Ds[TM_Z * TM_Y][TM_X];
-    __shared__ double Sx[TM_Z * TM_Y][TT_X];
+    __shared__ double Sx[TM_Z * TM_Y + 1][TT_X];
     const int tid = threadIdx.x, fx = tid & 31, warp = tid >> 5, fy = tile_row(warp);
     const int np = nf + 1, npc = nf / 2 + 1;
     const int xa = blockIdx.x * TT_X, ya = blockIdx.y * TT_Y, za = blockIdx.z * TT_Z;
@@ -66,6 +71,7 @@ extrapolate_tiled_kernel(double* __restrict__ out, const double* __restrict__ u,
         double d = 0.0;
         if (ci < npc && cj < npc && ck < npc) d = u[nidx(np, 2 * ci, 2 * cj, 2 * ck)] - uc[nidx(npc, ci, cj, ck)];
         Ds[row][ex] = d;
+        if (ex < TT_X / 2) Sx[row][2 * ex] = d;
     }
     const int i = xa + fx, j = ya + fy;
     const bool mine = i < np && j < np;
@@ -76,17 +82,22 @@ extrapolate_tiled_kernel(double* __restrict__ out, const double* __restrict__ u,
 #pragma unroll
     for (int k = 0; k < TT_Z; ++k) uv[k] = mine && k < kz ? u[o + k * plane] : 0.0;
     __syncthreads();
-    for (int row = warp; row < TM_Z * TM_Y; row += TT_Y) {
-        const int c = fx >> 1;
-        Sx[row][fx] = (fx & 1) ? Ds[row][c] + Ds[row][c + 1] : Ds[row][c];
+    // along x: a warp forms the odd nodes of two rows at a time
+    for (int pair = warp; 2 * pair < TM_Z * TM_Y; pair += TT_Y) {
+        const int row = 2 * pair + (fx >> 4), c = fx & 15;
+        if (row < TM_Z * TM_Y) Sx[row][2 * c + 1] = Ds[row][c] + Ds[row][c + 1];
     }
     __syncthreads();
     if (!mine) return;
     double s[TM_Z];
 #pragma unroll
-    for (int c = 0; c < TM_Z; ++c) {
-        const int row = c * TM_Y + (fy >> 1);
-        s[c] = (fy & 1) ? Sx[row][fx] + Sx[row + 1][fx] : Sx[row][fx];
+    for (int c = 0; c < TM_Z; ++c) s[c] = Sx[c * TM_Y + (fy >> 1)][fx];
+    // (a loop in place of a branch: opaque in reduce.cuh)
+    const int odd = opaque(fy & 1);
+#pragma unroll 1
+    for (int once = 0; once < odd; ++once) {
+#pragma unroll
+        for (int c = 0; c < TM_Z; ++c) s[c] += Sx[c * TM_Y + (fy >> 1) + 1][fx];
     }
     // 1 / (3 2^m) or 1 / (4 2^m), m = number of odd coordinates (tiles start on even ones)
     const int m = (fx & 1) + (fy & 1);
@@ -110,7 +121,8 @@ __device__ __forceinline__ double quad_odd(bool first, double a, double b, doubl
 }
 
 // Step 5 at every fine node of the tile: even coordinates are middle-grid
-// nodes, odd ones take three products per axis.  Along x a warp forms the
+// nodes, odd ones take three products per axis.  EXP_finite at 512^3: 0.87 ms
+// (1.14 with predicated products along y).  Along x a warp forms the
 // odd nodes of two rows at a time.
 __global__ void __launch_bounds__(TT_THREADS)
 exp_finite_interp_tiled_kernel(double* __restrict__ w, const double* __restrict__ W, int nf) {
@@ -140,13 +152,14 @@ exp_finite_interp_tiled_kernel(double* __restrict__ w, const double* __restrict_
     if (i >= np || j >= np) return;
     double t[TM_Z];
 #pragma unroll
-    for (int c = 0; c < TM_Z; ++c) {
-        const int row = c * TM_Y;
-        if (fy & 1) {
-            const int r0 = row + 2 * (fy >> 2);
+    for (int c = 0; c < TM_Z; ++c) t[c] = Tx[c * TM_Y + (fy >> 1)][fx];
+    const int odd = opaque(fy & 1);   // (a loop in place of a branch)
+#pragma unroll 1
+    for (int once = 0; once < odd; ++once) {
+#pragma unroll
+        for (int c = 0; c < TM_Z; ++c) {
+            const int r0 = c * TM_Y + 2 * (fy >> 2);
             t[c] = quad_odd((fy & 2) == 0, Tx[r0][fx], Tx[r0 + 1][fx], Tx[r0 + 2][fx]);
-        } else {
-            t[c] = Tx[row + (fy >> 1)][fx];
         }
     }
     const int kz = min(TT_Z, np - za);
