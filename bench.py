@@ -39,7 +39,8 @@ METRIC = "EXCMG solve s @512³ FP64 vs FP32+refine; stencil HBM GB/s % peak; p99
 # DRAM bytes (read + write) per launch measured by ncu on 255^3 unknowns
 # (python bench.py --case bicg --n 256 --iters 4 [--schedule separate]; the
 # summaries under profiles/ give the full capture commands)
-TRAFFIC_255 = {"stencil_pair_kernel": 288.93e6 + 220.17e6, "stencil_pair_dir_kernel": 582.57e6 + 489.67e6}
+TRAFFIC_255 = {"stencil_step_kernel<kMarchPair>": 278.87e6 + 104.51e6,
+               "stencil_step_kernel<kMarchDir>": 577.18e6 + 361.64e6}
 ORACLE_COUNTS = os.path.join(ROOT, "oracle", "excmg_512_counts.json")
 
 
@@ -548,7 +549,7 @@ def run_ours(args):
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
     # algorithmic bytes per launch as the library counts them: 8 B per unknown
     # for every field read or written (the fused launch that also forms the
-    # directions: r, r*, p_old, p*_old in; p, p*, A p, A^T p* out)
+    # directions: r, r*, p_old, p*_old in; p, p*, A p out, which is A^T p* too)
     avg_ms = st_ms / st_cnt if st_cnt else float("nan")
     bytes_per_launch = st_bytes / st_cnt if st_cnt else None
     achieved = st_bytes / (st_ms * 1e-3) / 1e9 if st_cnt else None
@@ -556,9 +557,10 @@ def run_ours(args):
     if args.stencil != "exact":
         kernel = f"stencil_f64_kernel: A p or A^T p* on the {n}^3 grid"
     elif per_unknown > 48.0:
-        kernel = f"stencil_pair_dir_kernel (fused schedule): p, p* formed, A p, A^T p*, sigma on the {n}^3 grid"
+        kernel = (f"stencil_step_kernel<kMarchDir> (fused schedule): p, p* formed, A p (= A^T p*), sigma "
+                  f"on the {n}^3 grid")
     else:
-        kernel = f"stencil_pair_kernel: A p, A^T p*, sigma (operator pair) on the {n}^3 grid"
+        kernel = f"stencil_step_kernel<kMarchPair>: A p (= A^T p*), sigma on the {n}^3 grid"
     # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the kernel
     # from one ncu capture on 255^3 unknowns, scaled to this launch by the
     # unknowns it processes (traffic grows in proportion); None for a kernel

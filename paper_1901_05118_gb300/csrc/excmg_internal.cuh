@@ -84,7 +84,8 @@ int stencil_cta_count(int n);
 cudaError_t launch_bicg_stencil_pair_dir(const double* r, const double* rs, const double* p_prev,
                                          const double* ps_prev, double* p, double* ps, double* q, double* qs, int n,
                                          int bc_kind, double* partials, BicgState* st, cudaStream_t s);
-// Small grids: whole Bi-CG iterations (up to `iters`) in one cooperative
+// Grids up to 64^3 that the resident kernel does not take (a caller-chosen r*_0, no
+// room for its words): whole Bi-CG iterations (up to `iters`) in one cooperative
 // launch with bounded grid barriers; barrier_words: 3 device words.
 constexpr int kPersistentMaxN = 64;
 bool persistent_pointwise(int n);

@@ -17,13 +17,13 @@
 // accumulators.
 //
 // What bounds it: latency and instruction issue of two CTAs per SM (at 512^3
-// the step with directions moves 56 B per unknown in 1.3 times the time that HBM
-// takes for them; the single-field form is far from HBM).  Hence
+// the step with directions moves 56 B per unknown in 1.4 times the time that HBM
+// takes for them, 1.54 ms; A u, 0.97 ms, is far from HBM).  Hence
 //  * copies run one plane ahead of their use by 8-byte cp.async (rows of N + 1
 //    doubles have no 16-byte alignment) into one stage, which a thread refills
 //    as soon as it has read its own slots back, so completing the copies needs
 //    no CTA barrier.  More stages were slower (step with directions 1.69 ms
-//    with one stage, 1.75 with two, 2.69 with three and no L1 left), the
+//    with one stage then, 1.75 with two, 2.69 with three and no L1 left), the
 //    256-byte L2 prefetch hint is worth 4-6 %;
 //  * one CTA barrier per plane publishes the tile of u at plane t, the tile of
 //    w at plane t - 1 and the exponent maximum of plane t + 1, and between two

@@ -17,9 +17,9 @@ namespace {
 // Each thread loads kLd entries, one grid stride apart, before it works on
 // them in index order: the sums are those of one entry at a time, but twice as
 // many bytes are in flight.  At 512^3 the update moves 64 B per entry
-// at 0.97 of the measured copy bandwidth with two entries (1.31 ms; one entry:
-// 1.6 ms, four at four CTAs per SM: 1.61 ms), and more CTAs per SM do not
-// help (1.34-1.5 ms).
+// at 0.95 of the measured copy bandwidth or more with two entries (1.3 ms; one
+// entry: 1.6 ms, three 0.1 ms slower, four at four CTAs per SM: 1.61 ms), and more CTAs
+// per SM do not help (1.34-1.5 ms).
 constexpr int kLd = 2;
 #define EXCMG_STRIDED(t0, S) \
     const size_t S = (size_t)gridDim.x * blockDim.x; \

@@ -54,3 +54,18 @@ def test_transfers(nf):
     assert rel_max(w, oracle.exp_finite(nf, u1, u0)) <= 1e-13
     ut = B.midpoint_extrapolate(nf, dev(uh), dev(u1)).cpu().numpy()
     assert rel_max(ut, oracle.exp_true(nf, uh, u1)) <= 1e-13
+
+
+def test_start_from_a_guess_in_the_separate_schedule():
+    """The march that stores b - A u alone (the other schedule forms its
+    copies with it): three iterations from a nonzero guess, within the bound that
+    the repository's fixed-iteration comparisons have."""
+    n = 98
+    b, x0 = P.random_field(n, 81), P.random_field(n, 82)
+    ctx = B.Context(DEV)
+    ctx.set_schedule("separate")
+    x = dev(x0)
+    it, rel, rc = B.bicg_solve(B.Level(n, 1, ctx), dev(b), x, 0.0, 3)
+    xr, itr, relr, rcr = oracle.bicg(n, 1, b, x0, 0.0, max_iter=3)
+    assert it == itr == 3
+    assert rel_max(x.cpu().numpy(), xr) <= 1e-10
