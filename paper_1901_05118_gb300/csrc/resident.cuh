@@ -27,7 +27,7 @@
 //    about 510 cycles, the integer form about a third;
 //  * scalars formed by one warp and broadcast (a division takes 650 cycles),
 //    and no FP64 comparisons: they go through the same pipe;
-//  * outputs rounded with integer instructions (fx_result; the hardware
+//  * outputs rounded with integer instructions (brick_result; the hardware
 //    conversion goes through the FP64 pipe: the same time here).
 // Measured: 200 iterations on 64^3 2.13 ms (the general cooperative kernel:
 // 5.63 ms), a whole 32^3 first-kind solve to 1e-10 4.9 ms (14.8 ms); 100
@@ -135,6 +135,33 @@ __device__ __forceinline__ double sum_fx(const double (&v)[C]) {
 // cycles each -- on the way of every iteration.
 __device__ __noinline__ double divide_slow(double a, double b) { return a / b; }
 __device__ __noinline__ bool root_at_most(double a, double b) { return sqrt(a) <= b; }
+
+// v as an integer of 2^(E - 1077), E the largest biased exponent of the tile,
+// rounded to nearest: two bits below the last place of the tile's largest
+// values (144 * 2^55 < 2^63, the weights' sum times the largest integer); the
+// marches truncate at that place.  The per-node form of the general kernel has a
+// scale for the 25 taps of each node, a brick one for all of its nodes: truncated to
+// it, A p kept fewer bits.  The error of the iterates against 64 bits after 48
+// to 96 iterations on 16^3 .. 32^3 (geometric means of 16 right-hand sides) was then 1.57 times the
+// per-node form's (0.75 to 2.5 by grid and kind), it is 0.73 times now (0.43 to 0.99), for
+// 10.8 instead of 10.7 us per iteration on 64^3, 0.7 % of a 32^3 solve.
+__device__ __forceinline__ long long to_brick(double v, int E) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned e = (hi >> 20) & 0x7FFu;
+    const unsigned mh = ((hi & 0xFFFFFu) | (e != 0u ? 0x100000u : 0u)) << 3 | lo >> 29, ml = lo << 3;
+    const unsigned d = (unsigned)(E - (int)max(e, 1u));
+    const unsigned rlo = shr_clamp(__funnelshift_rc(ml, mh, d), (unsigned)max((int)d - 32, 0));
+    const unsigned rhi = shr_clamp(mh, d);
+    const unsigned long long m = ((((unsigned long long)rhi << 32) | rlo) + 1ull) >> 1;   // from half units
+    return (int)hi < 0 ? -(long long)m : (long long)m;
+}
+
+// Y * 2^(E - 1077) rounded to nearest even, |Y| < 2^63 (from_fixed's exponent
+// field holds for one less than with its |Y| < 2^62).
+__device__ __forceinline__ double brick_result(long long acc, int E) {
+    if (E >= 55 && E <= 2038) return from_fixed(acc, E - 2);
+    return fx_result_slow(acc, E - 2, E == 0x7FF);
+}
 
 // a b + c, fused: written out so that every variant of the kernel rounds alike
 __device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
@@ -352,7 +379,7 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
 #pragma unroll
             for (int k = 0; k < NH; ++k) hp[k] = mad(b, hp[k], hr[k]);
         }
-        // the tile of p: on one power-of-two scale as integers (march_fx.cuh), or FP32
+        // the tile of p: on one power-of-two scale as integers (to_brick), or FP32
         int E = 1;
         if constexpr (kExact) {
             unsigned em = 1u;
@@ -370,7 +397,7 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
         for (int k = 0; k < NP; ++k)
             if (k < cnt) {
                 if constexpr (kExact)
-                    tile[t0 + k * tp] = to_fixed_e(p[k], ((unsigned)__double2hiint(p[k]) >> 20) & 0x7FFu, E);
+                    tile[t0 + k * tp] = to_brick(p[k], E);
                 else
                     tile[t0 + k * tp] = p[k];
             }
@@ -378,7 +405,7 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
         for (int k = 0; k < NH; ++k)
             if (hidx[k] >= 0) {
                 if constexpr (kExact)
-                    tile[htile[k]] = to_fixed_e(hp[k], ((unsigned)__double2hiint(hp[k]) >> 20) & 0x7FFu, E);
+                    tile[htile[k]] = to_brick(hp[k], E);
                 else
                     tile[htile[k]] = hp[k];
             }
@@ -411,7 +438,7 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
                     if constexpr (kExact) {
                         const long long acc =
                             mul_w(u[k + 2], (unsigned)(kCentre + cc[k])) - mul_w(n6, (unsigned)kNear) + f6 + (d12 + d12);
-                        q[k] = fx_result(acc, E, E == 0x7FF);
+                        q[k] = brick_result(acc, E);
                     } else {
                         q[k] = mad((float)(kCentre + cc[k]), u[k + 2], mad(-(float)kNear, n6, mad(2.f, d12, f6)));
                     }

@@ -129,3 +129,62 @@ def test_batch_large_level_is_not_kept_out():
         live = left + [batch.submit(32, 4, 2, *small, 1e-10, precision="fp64")[0] for _ in range(13 - len(left))]
     assert batch.query(ident)["done"]
     batch.run()
+
+
+def _operator_ld(n, bc_kind, v):
+    """A_h on interior values v[k, j, i] in numpy's extended precision."""
+    m = n - 1
+    pad = np.zeros((m + 4,) * 3, dtype=np.longdouble)
+    pad[2:-2, 2:-2, 2:-2] = v
+
+    def at(*o):
+        return pad[tuple(slice(2 + a, 2 + a + m) for a in o)]
+
+    end = np.zeros(m, dtype=np.longdouble)
+    end[0] += 1
+    end[-1] += 1
+    faces = end[:, None, None] + end[None, :, None] + end[None, None, :]
+    y = (42 + (1 if bc_kind == 1 else -1) * faces) * at(0, 0, 0)
+    for a in range(3):
+        for s in (-1, 1):
+            o = [0, 0, 0]
+            o[a] = s
+            y = y - 12 * at(*o)
+            o[a] = 2 * s
+            y = y + at(*o)
+        for b in range(a + 1, 3):
+            for s in (-1, 1):
+                for t in (-1, 1):
+                    o = [0, 0, 0]
+                    o[a], o[b] = s, t
+                    y = y + 2 * at(*o)
+    return y
+
+
+@pytest.mark.parametrize("n,bc_kind", [(16, 1), (20, 2), (32, 1), (32, 2)])
+def test_small_entries_beside_large_ones(n, bc_kind):
+    """Two iterations from x_0 = 0 on a b of entries near 2^-10 with a 1 at every
+    fourth node along each axis, so that every brick's scale is that of 1.
+    x_2 = alpha_0 b + alpha_1 (b - alpha_0 A b + beta b) shows the A b of the
+    first iteration entry by entry.  Bound: each tap is off by at most half
+    of 2^-54 (two bits below the last place of 1), 144 in all, times alpha_0 alpha_1,
+    and 64 roundings of 2^-53 of the magnitudes in the sum (about 10 on the way of an entry, the
+    rest for the inner products).  Taps truncated to the last place of 1 are off by up
+    to 8 times as much (4 times the bound on this data)."""
+    r = np.random.Generator(np.random.PCG64(7))
+    b = np.ldexp(r.uniform(0.5, 1.0, (n + 1,) * 3), -10) * r.choice([-1.0, 1.0], (n + 1,) * 3)
+    b[2::4, 2::4, 2::4] = 1.0
+    x = torch.zeros((n + 1,) * 3, dtype=torch.float64, device=DEV)
+    B.bicg_solve(B.Level(n, bc_kind), dev(b), x, 0.0, 2)
+    i = slice(1, -1)
+    v = b[i, i, i].astype(np.longdouble)
+    q0 = _operator_ld(n, bc_kind, v)
+    a0 = (v * v).sum() / (v * q0).sum()
+    r1 = v - a0 * q0
+    beta = (r1 * r1).sum() / (v * v).sum()
+    p1 = r1 + beta * v
+    a1 = (r1 * r1).sum() / (p1 * _operator_ld(n, bc_kind, p1)).sum()
+    off = np.abs(x.cpu().numpy()[i, i, i] - (a0 * v + a1 * p1))
+    tap, eps = np.ldexp(np.longdouble(1), -55), np.ldexp(np.longdouble(1), -53)
+    bound = a0 * a1 * 144 * tap + 64 * eps * (a0 * np.abs(v) + a1 * ((1 + beta) * np.abs(v) + a0 * np.abs(q0)))
+    assert float((off / bound).max()) <= 1.0
