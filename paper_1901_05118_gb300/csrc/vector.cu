@@ -15,16 +15,26 @@ namespace excmg {
 namespace {
 
 // Each thread loads kLd entries, one grid stride apart, before it works on
-// them in index order: the sums are those of one entry at a time, but twice as
-// many bytes are in flight.  At 512^3 the update moves 64 B per entry
+// them in index order: the sums are those of one entry at a time, but with two
+// entries twice as many bytes are in flight.  At 512^3 the update moves 64 B per entry
 // at 0.95 of the measured copy bandwidth or more with two entries (1.3 ms; one
 // entry: 1.6 ms, three 0.1 ms slower, four at four CTAs per SM: 1.61 ms), and more CTAs
 // per SM do not help (1.34-1.5 ms).
-constexpr int kLd = 2;
+//
+// Vectors of fewer than kPairStrides grid strides (1.87 million entries) go one
+// entry at a time: they lie in L2, and a last group of two that is half empty costs a
+// whole one, as its predicated FP64 instructions hold the pipe.  One against two entries:
+// 60 2D iterations on 580^2 1.95 / 2.18 ms, on 900^2 2.64 / 2.77, on 1400^2 4.47 / 4.37;
+// 40 elided ones on 100^3 1.76 / 1.83, on 120^3 2.17 / 2.25, 40 of the separate schedule on
+// 130^3 3.50 / 3.40, on 160^3 5.38 / 5.13.  (A loop of its own for the entries that do
+// not fill a group: as fast as one below the line, 2 to 4 % slower than two above it.)
+constexpr size_t kPairStrides = 12;
+inline bool load_pairs(size_t len) { return len >= kPairStrides * kVecBlocks * kVecThreads; }
 #define EXCMG_STRIDED(t0, S) \
     const size_t S = (size_t)gridDim.x * blockDim.x; \
     for (size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t0 < len; t0 += kLd * S)
 
+template <int kLd>
 __global__ void __launch_bounds__(kVecThreads)
 dot_kernel(const double* __restrict__ a, const double* __restrict__ b, size_t len,
            double* partials, unsigned int* ticket, double* out) {
@@ -83,6 +93,7 @@ interior_dot_kernel(const double* __restrict__ a, int n, double* partials, unsig
 
 // r*_0 = shadow (or r_0), p_0 = r_0, p*_0 = r*_0; rho_0 = (r*_0, r_0),
 // rr = (r_0, r_0).
+template <int kLd>
 __global__ void __launch_bounds__(kVecThreads)
 bicg_init_kernel(const double* __restrict__ r, const double* __restrict__ shadow, double* __restrict__ rs,
                  double* __restrict__ p, double* __restrict__ ps, size_t len, double* partials, BicgState* st) {
@@ -166,7 +177,7 @@ bicg_sigma_kernel(const double* __restrict__ ps, const double* __restrict__ q, s
 // from the identical partial sums it has so far.  FP64 issue is scarce on
 // GB300: this saves two of the five FMAs per entry.
 // kOneQ: A^T p* is A p bit for bit and read once, from q.
-template <bool kOneQ>
+template <int kLd, bool kOneQ>
 __global__ void __launch_bounds__(kVecThreads)
 bicg_update_kernel(double* __restrict__ x, const double* __restrict__ p, double* __restrict__ r,
                    const double* __restrict__ q, double* __restrict__ rs,
@@ -238,6 +249,7 @@ bicg_update_kernel(double* __restrict__ x, const double* __restrict__ p, double*
 
 // p_{k+1} = r_{k+1} + beta p_k; p*_{k+1} = r*_{k+1} + beta p*_k (one FMA
 // where the shadow entries equal the primal ones bit for bit).
+template <int kLd>
 __global__ void __launch_bounds__(kVecThreads)
 bicg_pupdate_kernel(double* __restrict__ p, const double* __restrict__ r, double* __restrict__ ps,
                     const double* __restrict__ rs, size_t len, const BicgState* st) {
@@ -305,6 +317,7 @@ cg_init_kernel(const double* __restrict__ r, double* __restrict__ p, size_t len,
 // Shadow-elided update: x += alpha p; r -= alpha A p; rho_{k+1} = rr =
 // (r, r); beta; stopping test.  Same arithmetic and summation order as
 // bicg_update_kernel on twin entries.
+template <int kLd>
 __global__ void __launch_bounds__(kVecThreads)
 cg_update_kernel(double* __restrict__ x, const double* __restrict__ p, double* __restrict__ r,
                  const double* __restrict__ q, size_t len, double* partials, BicgState* st) {
@@ -358,6 +371,7 @@ cg_update_kernel(double* __restrict__ x, const double* __restrict__ p, double* _
 }
 
 // Shadow-elided direction update: p = r + beta p.
+template <int kLd>
 __global__ void __launch_bounds__(kVecThreads)
 cg_pupdate_kernel(double* __restrict__ p, const double* __restrict__ r, size_t len, const BicgState* st) {
     if (st->done) return;
@@ -383,7 +397,7 @@ cg_pupdate_kernel(double* __restrict__ p, const double* __restrict__ r, size_t l
 }  // namespace
 
 cudaError_t launch_cg_pupdate(double* p, const double* r, size_t len, const BicgState* st, cudaStream_t s) {
-    cg_pupdate_kernel<<<kVecBlocks, kVecThreads, 0, s>>>(p, r, len, st);
+    (load_pairs(len) ? cg_pupdate_kernel<2> : cg_pupdate_kernel<1>)<<<kVecBlocks, kVecThreads, 0, s>>>(p, r, len, st);
     return cudaGetLastError();
 }
 
@@ -394,13 +408,13 @@ cudaError_t launch_cg_init(const double* r, double* p, size_t len, double* parti
 
 cudaError_t launch_cg_update(double* x, const double* p, double* r, const double* q, size_t len, double* partials,
                              BicgState* st, cudaStream_t s) {
-    cg_update_kernel<<<kVecBlocks, kVecThreads, 0, s>>>(x, p, r, q, len, partials, st);
+    (load_pairs(len) ? cg_update_kernel<2> : cg_update_kernel<1>)<<<kVecBlocks, kVecThreads, 0, s>>>(x, p, r, q, len, partials, st);
     return cudaGetLastError();
 }
 
 cudaError_t launch_dot(const double* a, const double* b, size_t len, double* partials,
                        unsigned int* ticket, double* out, cudaStream_t s) {
-    dot_kernel<<<kVecBlocks, kVecThreads, 0, s>>>(a, b, len, partials, ticket, out);
+    (load_pairs(len) ? dot_kernel<2> : dot_kernel<1>)<<<kVecBlocks, kVecThreads, 0, s>>>(a, b, len, partials, ticket, out);
     return cudaGetLastError();
 }
 
@@ -412,7 +426,7 @@ cudaError_t launch_interior_dot(const double* a, int n, double* partials, unsign
 
 cudaError_t launch_bicg_init(const double* r, const double* shadow, double* rs, double* p, double* ps, size_t len,
                              double* partials, BicgState* st, cudaStream_t s) {
-    bicg_init_kernel<<<kVecBlocks, kVecThreads, 0, s>>>(r, shadow, rs, p, ps, len, partials, st);
+    (load_pairs(len) ? bicg_init_kernel<2> : bicg_init_kernel<1>)<<<kVecBlocks, kVecThreads, 0, s>>>(r, shadow, rs, p, ps, len, partials, st);
     return cudaGetLastError();
 }
 
@@ -425,16 +439,16 @@ cudaError_t launch_bicg_sigma(const double* ps, const double* q, size_t len, dou
 cudaError_t launch_bicg_update(double* x, const double* p, double* r, const double* q, double* rs,
                                const double* qs, size_t len, double* partials, BicgState* st,
                                cudaStream_t s) {
-    if (qs)
-        bicg_update_kernel<false><<<kVecBlocks, kVecThreads, 0, s>>>(x, p, r, q, rs, qs, len, partials, st);
-    else
-        bicg_update_kernel<true><<<kVecBlocks, kVecThreads, 0, s>>>(x, p, r, q, rs, qs, len, partials, st);
+    const bool two = load_pairs(len);
+    (qs ? (two ? bicg_update_kernel<2, false> : bicg_update_kernel<1, false>)
+        : (two ? bicg_update_kernel<2, true> : bicg_update_kernel<1, true>))<<<kVecBlocks, kVecThreads, 0, s>>>(
+        x, p, r, q, rs, qs, len, partials, st);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bicg_pupdate(double* p, const double* r, double* ps, const double* rs, size_t len,
                                 const BicgState* st, cudaStream_t s) {
-    bicg_pupdate_kernel<<<kVecBlocks, kVecThreads, 0, s>>>(p, r, ps, rs, len, st);
+    (load_pairs(len) ? bicg_pupdate_kernel<2> : bicg_pupdate_kernel<1>)<<<kVecBlocks, kVecThreads, 0, s>>>(p, r, ps, rs, len, st);
     return cudaGetLastError();
 }
 

@@ -69,3 +69,26 @@ def test_start_from_a_guess_in_the_separate_schedule():
     xr, itr, relr, rcr = oracle.bicg(n, 1, b, x0, 0.0, max_iter=3)
     assert it == itr == 3
     assert rel_max(x.cpu().numpy(), xr) <= 1e-10
+
+
+@pytest.mark.parametrize("n,dim", [(122, 3), (123, 3), (1365, 2), (1366, 2)])
+@pytest.mark.parametrize("mode", ["full", "elided"])
+def test_vector_kernels_on_both_sides_of_their_line(n, dim, mode):
+    """Twelve grid strides (1867776 entries) lie between each pair of sizes:
+    one entry per thread at a time below, two from there on."""
+    entries = (n + 1) ** dim
+    assert (entries >= 12 * 152 * 4 * 256) == (n in (123, 1366))
+    ctx = B.Context(DEV)
+    ctx.set_shadow_mode(mode)
+    ctx.set_schedule("separate")
+    if dim == 3:
+        b, x0 = P.random_field(n, 85), P.random_field(n, 86)
+        x = dev(x0)
+        B.bicg_solve(B.Level(n, 2, ctx), dev(b), x, 0.0, 3)
+        xr = oracle.bicg(n, 2, b, x0, 0.0, max_iter=3)[0]
+    else:
+        b, x0 = P.random_field_2d(n, 85), P.random_field_2d(n, 86)
+        x = dev(x0)
+        B.bicg_solve2d(n, 2, dev(b), x, 0.0, 3, ctx=ctx)
+        xr = oracle.bicg2d(n, 2, b, x0, 0.0, max_iter=3)[0]
+    assert rel_max(x.cpu().numpy(), xr) <= 1e-10
