@@ -154,7 +154,7 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
         if (e == cudaSuccess) e = launch_stencil(x, r, b, n, bc_kind, false, nullptr, s, ctx->stencil_variant);
         if (e == cudaSuccess)
             e = elide ? launch_cg_init(r, p, len, ctx->partials, ctx->state, s)
-                      : launch_bicg_init(r, shadow, rs, p, ps, len, ctx->partials, ctx->state, s);
+                      : launch_bicg_init(r, shadow, rs, p, ps, len, n, ctx->partials, ctx->state, s);
         ++started;
         // a caller's shadow may carry values on boundary nodes: the work vectors
         // keep zeros there
@@ -213,6 +213,8 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
             }
         }
         if (ctx->host_state->done) break;
+        // a given r*_0 that is r_0 bit for bit: A^T p* is A p as in a call without one
+        if (fused && shadow && ctx->host_state->twin) qs = nullptr;
         iter_before = ctx->host_state->iter;
         batch = check_every;
         const int left = max_iter - ctx->host_state->iter;

@@ -434,7 +434,7 @@ int bicg2d_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, d
     if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, bytes, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(qs, 0, bytes, s);
     if (e == cudaSuccess) e = launch_stencil2d(x, r, b, n, bc_kind, s);
-    if (e == cudaSuccess) e = launch_bicg_init(r, nullptr, rs, p, ps, len, ctx->partials, ctx->state, s);
+    if (e == cudaSuccess) e = launch_bicg_init(r, nullptr, rs, p, ps, len, n, ctx->partials, ctx->state, s);
     note_launches(3);
     if (e != cudaSuccess) return ctx_cuda(ctx, e, "2D Bi-CG setup");
     const int sg = bc_kind == 1 ? 1 : -1;

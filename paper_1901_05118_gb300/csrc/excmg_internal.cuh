@@ -23,7 +23,7 @@ inline size_t face_count(int n) { return 6 * (size_t)(n + 1) * (size_t)(n + 1); 
 // their reductions always combine the same partial sums in the same order.
 constexpr int kVecThreads = 256;
 constexpr int kVecBlocks = 152 * 4;     // 4 CTAs on each of GB300's 152 SMs
-constexpr int kMaxPartials = 8192;   // >= 2 * kVecBlocks and >= stencil CTAs
+constexpr int kMaxPartials = 8192;   // >= 3 * kVecBlocks and >= stencil CTAs
 
 // Bi-CG state kept on the device so that a whole iteration runs without the
 // host (Alg. 2 with M = I).
@@ -41,7 +41,8 @@ struct BicgState {
     int done;          // 1 once converged, capped or broken down
     int status;        // kRunning / kConverged / kCapped / kBreakdown
     unsigned int ticket;   // last-block counter of the reductions
-    int pad1[3];
+    int twin;          // a given r*_0 is r_0 bit for bit (bicg_init_kernel)
+    int pad1[2];
 };
 static_assert(sizeof(BicgState) % 8 == 0, "read back in 8-byte words");
 enum { kRunning = 0, kConverged = 1, kCapped = 2, kBreakdown = 3, kTimeout = 4 };
@@ -74,7 +75,7 @@ cudaError_t launch_bicg_start(const double* x, const double* b, int n, int bc_ki
 // arithmetic, fused with sigma = (p*, q) and alpha = rho / sigma (Alg. 2).
 // Skips when st->done.  partials must hold stencil_cta_count(n) doubles.
 // qs null: the call started from r*_0 = p*_0 = r_0 = p_0, so p* = p and A^T p*
-// is q bit for bit and is not stored again; else (a caller-chosen r*_0) the two fields are marched apart.
+// is q bit for bit and is not stored again; else (another r*_0) the two fields are marched apart.
 cudaError_t launch_bicg_stencil_pair(const double* p, double* q, const double* ps, double* qs, int n,
                                      int bc_kind, double* partials, BicgState* st, cudaStream_t s);
 int stencil_cta_count(int n);
@@ -133,8 +134,9 @@ cudaError_t launch_dot(const double* a, const double* b, size_t len, double* par
 // (a, a) over the interior nodes only (a's boundary entries are ignored).
 cudaError_t launch_interior_dot(const double* a, int n, double* partials, unsigned int* ticket, double* out,
                                 cudaStream_t s);
+// n: grid intervals, for a shadow's boundary entries (3D).
 cudaError_t launch_bicg_init(const double* r, const double* shadow, double* rs, double* p, double* ps, size_t len,
-                             double* partials, BicgState* st, cudaStream_t s);
+                             int n, double* partials, BicgState* st, cudaStream_t s);
 cudaError_t launch_bicg_sigma(const double* ps, const double* q, size_t len, double* partials,
                               BicgState* st, cudaStream_t s);
 // qs null: A^T p* = q.

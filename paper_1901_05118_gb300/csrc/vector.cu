@@ -92,14 +92,19 @@ interior_dot_kernel(const double* __restrict__ a, int n, double* partials, unsig
 }
 
 // r*_0 = shadow (or r_0), p_0 = r_0, p*_0 = r*_0; rho_0 = (r*_0, r_0),
-// rr = (r_0, r_0).
+// rr = (r_0, r_0); st->twin: the shadow is r_0 bit for bit at every unknown of a
+// grid with n intervals (the boundary entries may hold anything; the index of an entry is
+// split only where the bits differ, and once per thread where that is inside).
 template <int kLd>
 __global__ void __launch_bounds__(kVecThreads)
 bicg_init_kernel(const double* __restrict__ r, const double* __restrict__ shadow, double* __restrict__ rs,
-                 double* __restrict__ p, double* __restrict__ ps, size_t len, double* partials, BicgState* st) {
+                 double* __restrict__ p, double* __restrict__ ps, size_t len, int n, double* partials, BicgState* st) {
     __shared__ double sh[32];
     __shared__ bool am_last;
     double vr = 0.0, vrr = 0.0;
+    const size_t np = (size_t)n + 1;
+    auto inner = [&](size_t v) { return v >= 1 && v < (size_t)n; };
+    bool differs = false;
     EXCMG_STRIDED(t0, S) {
         double rv[kLd], sv[kLd];
 #pragma unroll
@@ -114,6 +119,8 @@ bicg_init_kernel(const double* __restrict__ r, const double* __restrict__ shadow
         for (int k = 0; k < kLd; ++k) {
             const size_t t = t0 + k * S;
             if (t >= len) break;
+            if (!differs && __double_as_longlong(sv[k]) != __double_as_longlong(rv[k]))
+                differs = inner(t % np) && inner(t / np % np) && inner(t / (np * np));
             rs[t] = sv[k];
             p[t] = rv[k];
             ps[t] = sv[k];
@@ -121,13 +128,16 @@ bicg_init_kernel(const double* __restrict__ r, const double* __restrict__ shadow
             vrr = __fma_rn(rv[k], rv[k], vrr);
         }
     }
-    double s2[2];
+    double s2[3];
     s2[0] = block_sum(vr, sh);
     s2[1] = block_sum(vrr, sh);
-    if (publish_partials(s2, 2, partials, &st->ticket, &am_last)) {
+    s2[2] = __syncthreads_or(differs) ? 1.0 : 0.0;
+    if (publish_partials(s2, 3, partials, &st->ticket, &am_last)) {
         const double rho = gather_partials(partials, 0, sh);
         const double rr = gather_partials(partials, 1, sh);
+        const double off = gather_partials(partials, 2, sh);
         if (thread0()) {
+            st->twin = off == 0.0;
             st->rho = rho;
             st->rr = rr;
             st->iter = 0;
@@ -425,8 +435,8 @@ cudaError_t launch_interior_dot(const double* a, int n, double* partials, unsign
 }
 
 cudaError_t launch_bicg_init(const double* r, const double* shadow, double* rs, double* p, double* ps, size_t len,
-                             double* partials, BicgState* st, cudaStream_t s) {
-    (load_pairs(len) ? bicg_init_kernel<2> : bicg_init_kernel<1>)<<<kVecBlocks, kVecThreads, 0, s>>>(r, shadow, rs, p, ps, len, partials, st);
+                             int n, double* partials, BicgState* st, cudaStream_t s) {
+    (load_pairs(len) ? bicg_init_kernel<2> : bicg_init_kernel<1>)<<<kVecBlocks, kVecThreads, 0, s>>>(r, shadow, rs, p, ps, len, n, partials, st);
     return cudaGetLastError();
 }
 

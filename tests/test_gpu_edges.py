@@ -92,3 +92,31 @@ def test_vector_kernels_on_both_sides_of_their_line(n, dim, mode):
         B.bicg_solve2d(n, 2, dev(b), x, 0.0, 3, ctx=ctx)
         xr = oracle.bicg2d(n, 2, b, x0, 0.0, max_iter=3)[0]
     assert rel_max(x.cpu().numpy(), xr) <= 1e-10
+
+
+@pytest.mark.parametrize("n", [72, 90])
+@pytest.mark.parametrize("schedule", ["separate", "fused"])
+def test_given_shadow_that_is_the_residual(n, schedule):
+    """r*_0 = r_0 given by the caller, with anything on its boundary nodes: A p serves
+    A^T p* as in a call without r*_0 (the bytes per launch say so), an r*_0 that differs at one
+    node has its own.  Iterates as in the repository's fixed-iteration comparisons."""
+    b = P.random_field(n, 87)
+    ctx = B.Context(DEV)
+    ctx.set_schedule(schedule)
+    ctx.profile()
+    lvl = B.Level(n, 1, ctx)
+    moved = {}
+    for what in ("same", "one node off"):
+        shadow = b.copy()
+        if what != "same":
+            shadow[n // 2, n // 3, 1] *= 1 + 2.0 ** -40
+        ctx.profile()   # clears the records
+        x = torch.zeros((n + 1,) * 3, dtype=torch.float64, device=DEV)
+        it, _, _ = B.bicg_solve(lvl, dev(b), x, 0.0, 4, shadow=dev(shadow))
+        _, launches, moved[what] = ctx.profile_read(n)
+        assert it == launches == 4
+        xr = oracle.bicg(n, 1, b, np.zeros_like(b), 0.0, max_iter=4)[0]
+        assert rel_max(x.cpu().numpy(), xr) <= 1e-10
+    fields = 4 * 3 if schedule == "separate" else 3 + 3 * 7
+    assert moved["same"] == fields * 8.0 * (n - 1) ** 3
+    assert moved["one node off"] == moved["same"] + 4 * 8.0 * (n - 1) ** 3
