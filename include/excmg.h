@@ -101,8 +101,8 @@ typedef struct {
 
 /* Create a context on the current device, bound to `cuda_stream` (a
  * cudaStream_t; NULL = legacy default stream).  hbm_budget_bytes caps the
- * workspace the context may hold (0 = no cap); requests beyond it fail with
- * EXCMG_ERR_BUDGET. */
+ * workspace the context may hold (0 = no cap) beside 0.3 MB of fixed tables;
+ * requests beyond it fail with EXCMG_ERR_BUDGET. */
 int excmg_ctx_create(void *cuda_stream, size_t hbm_budget_bytes, excmg_ctx **out);
 int excmg_ctx_destroy(excmg_ctx *ctx);
 /* Bytes of device workspace the context holds right now. */

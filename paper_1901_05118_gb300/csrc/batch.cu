@@ -729,10 +729,10 @@ bool launch_resident(excmg_batch* b, excmg_batch::Group& g, Instance* in, int ct
     if (e == cudaSuccess) {
         if (in->prec == EXCMG_PRECISION_FP64)
             e = launch_bicg_resident<double>(in->u[in->level], in->res, in->rs64, in->p64, in->ps64, N, in->bc,
-                                             b->inner_chunk, bs, g.words, s, false, limit);
+                                             b->inner_chunk, bs, g.words, (char*)g.words + resident_slot_bytes(), s, false, limit);
         else
             e = launch_bicg_resident<float>(in->e, in->r, in->rs, in->p, in->ps, N, in->bc, b->inner_chunk, bs,
-                                            g.words, s, false, limit);
+                                            g.words, (char*)g.words + resident_slot_bytes(), s, false, limit);
     }
     bnote(b, 1);
     if (e == cudaSuccess)
@@ -1173,7 +1173,7 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
                 e = launch_zero_boundary({in->res}, N, s);
             if (e == cudaSuccess)
                 e = launch_bicg_start(in->u[in->level], in->fh, N, in->bc, in->res, in->rs64, in->p64, in->ps64,
-                                      ctx->partials, ctx->ticket, b->d_norms + rw.size(), nullptr, s);
+                                      nullptr, ctx->partials, ctx->ticket, b->d_norms + rw.size(), nullptr, s);
             bnote(b, 1);
             if (e != cudaSuccess) return bcuda(b, e, "batch residual");
             rw.push_back({in, in->res});

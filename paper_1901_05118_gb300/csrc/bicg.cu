@@ -97,22 +97,21 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // ones bit for bit, so they are neither stored nor read
     const bool elide =
         ctx->shadow_mode == EXCMG_SHADOW_ELIDED && shadow == nullptr && ctx->stencil_variant == kStencilExact;
-    double* r = ctx_buffer(ctx, "bicg_r", bytes, &st);
-    double* rs = (st || elide) ? nullptr : ctx_buffer(ctx, "bicg_rs", bytes, &st);
-    double* p = st ? nullptr : ctx_buffer(ctx, "bicg_p", bytes, &st);
-    double* ps = (st || elide) ? nullptr : ctx_buffer(ctx, "bicg_ps", bytes, &st);
-    double* q = st ? nullptr : ctx_buffer(ctx, "bicg_q", bytes, &st);
-    if (st) return st;
     // the integer operator has a fused two-field kernel; the FP64 one runs
     // as two applications and a separate inner product
     const bool fused = ctx->stencil_variant == kStencilExact && stencil_cta_count(n) <= kMaxPartials;
-    // small grids run whole iterations in one cooperative launch: with every
-    // vector on chip from r*_0 = r_0; a caller-chosen r*_0, or no room for the
-    // exchange words, the general cooperative kernel up to 64^3
-    void* words =
-        fused && shadow == nullptr && resident_ctas(n, 0) > 0 ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
-    const bool resident = words != nullptr;
+    // small grids run whole iterations in one cooperative launch: from r*_0 = r_0
+    // with every vector on chip, else on the general kernel up to 64^3.  The node words of the
+    // first take the place of r and q, so that it needs no more memory than
+    // the others do (three vectors shadow-elided, five in full) and no budget and no
+    // earlier call decides between them.
+    const bool resident = fused && shadow == nullptr && resident_ctas(n, 0) > 0;
     const bool persistent = resident || (fused && n <= kPersistentMaxN);
+    double* r = resident ? nullptr : ctx_buffer(ctx, "bicg_r", bytes, &st);
+    double* rs = (st || elide) ? nullptr : ctx_buffer(ctx, "bicg_rs", bytes, &st);
+    double* p = st ? nullptr : ctx_buffer(ctx, "bicg_p", bytes, &st);
+    double* ps = (st || elide) ? nullptr : ctx_buffer(ctx, "bicg_ps", bytes, &st);
+    if (st) return st;
     // the fused schedule (the default on the launched levels) folds
     // p = r + beta p into the operator step, which reads the previous
     // directions from one buffer pair and writes the new ones to the other
@@ -124,8 +123,10 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // from r*_0 = r_0 on: both are read from q (the general cooperative
     // kernel keeps its second array)
     const bool twin = fused && shadow == nullptr && (resident || !persistent);
-    double* qs = (elide || twin) ? nullptr : ctx_buffer(ctx, "bicg_qs", bytes, &st);
+    const bool own_qs = !elide && !twin;
+    double* q = ctx_buffer(ctx, "bicg_q", resident || own_qs ? 2 * bytes : bytes, &st);
     if (st) return st;
+    double* qs = own_qs ? q + len : nullptr;
     double* p2 = dir_fused ? ctx_buffer(ctx, "bicg_p2", bytes, &st) : nullptr;
     double* ps2 = (dir_fused && !elide && !st) ? ctx_buffer(ctx, "bicg_ps2", bytes, &st) : nullptr;
     if (st) return st;
@@ -148,8 +149,8 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // r_0 = b - A x_0; r*_0 = p_0 = p*_0 = r_0; rho_0
     if (ctx->stencil_variant == kStencilExact && shadow == nullptr && fused) {
         if (e == cudaSuccess)
-            e = launch_bicg_start(x, b, n, bc_kind, r, rs, p, ps, ctx->partials, &ctx->state->ticket, nullptr,
-                                  ctx->state, s);
+            e = launch_bicg_start(x, b, n, bc_kind, r, rs, p, ps, resident ? q : nullptr, ctx->partials,
+                                  &ctx->state->ticket, nullptr, ctx->state, s);
     } else {
         if (e == cudaSuccess) e = launch_stencil(x, r, b, n, bc_kind, false, nullptr, s, ctx->stencil_variant);
         if (e == cudaSuccess)
@@ -172,7 +173,8 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
         for (int iter = 0;;) {
             int chunk = resident ? 1024 : 256;
             if (chunk > max_iter - iter) chunk = max_iter - iter;
-            e = resident ? launch_bicg_resident<double>(x, r, rs, p, ps, n, bc_kind, chunk, ctx->state, words, s, elide, 0)
+            e = resident ? launch_bicg_resident<double>(x, r, rs, p, ps, n, bc_kind, chunk, ctx->state, ctx->slots, q, s,
+                                                        elide, 0)
                          : launch_bicg_persistent(x, r, rs, p, ps, q, qs, n, bc_kind, chunk, ctx->partials,
                                                   ctx->state, ctx->barrier, s, elide);
             note_launches(1);

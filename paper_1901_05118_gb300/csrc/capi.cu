@@ -228,6 +228,8 @@ int excmg_ctx_create(void* cuda_stream, size_t hbm_budget_bytes, excmg_ctx** out
               cudaMalloc(&c->scalar, 8 * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&c->state, sizeof(BicgState)) == cudaSuccess &&
               cudaMalloc(&c->barrier, 4 * sizeof(unsigned int)) == cudaSuccess &&
+              cudaMalloc(&c->slots, resident_slot_bytes()) == cudaSuccess &&
+              cudaMemset(c->slots, 0, resident_slot_bytes()) == cudaSuccess &&
               cudaMemset(c->barrier, 0, 4 * sizeof(unsigned int)) == cudaSuccess &&
               cudaHostAlloc(&c->host_state, sizeof(BicgState), cudaHostAllocMapped) == cudaSuccess &&
               cudaHostAlloc(&c->host_scalar, 8 * sizeof(double), cudaHostAllocMapped) == cudaSuccess &&
@@ -257,6 +259,7 @@ int excmg_ctx_destroy(excmg_ctx* c) {
     if (c->scalar) cudaFree(c->scalar);
     if (c->state) cudaFree(c->state);
     if (c->barrier) cudaFree(c->barrier);
+    if (c->slots) cudaFree(c->slots);
     if (c->host_state) cudaFreeHost(c->host_state);
     if (c->host_scalar) cudaFreeHost(c->host_scalar);
     for (cudaEvent_t e : c->prof_events) cudaEventDestroy(e);

@@ -67,10 +67,11 @@ cudaError_t launch_residual_norm(const double* x, const double* b, int n, int bc
 // The start of a Bi-CG call with r*_0 = r_0 (integer operator): r = b - A x and
 // its copies r*, p, p* (each may be null) at the interior nodes (grids up to
 // 64^3: zeros on the boundary, too), (r, r) into *out and the scalars of *st
-// (each may be null).
+// (each may be null).  words: the node words of launch_bicg_resident, which then take r in the
+// place of the array r; may be null.
 cudaError_t launch_bicg_start(const double* x, const double* b, int n, int bc_kind, double* r, double* rs, double* p,
-                              double* ps, double* partials, unsigned int* ticket, double* out, BicgState* st,
-                              cudaStream_t s);
+                              double* ps, void* words, double* partials, unsigned int* ticket, double* out,
+                              BicgState* st, cudaStream_t s);
 // One z-march applying A to p (-> q) and A^T to p* (-> qs) with the integer
 // arithmetic, fused with sigma = (p*, q) and alpha = rho / sigma (Alg. 2).
 // Skips when st->done.  partials must hold stencil_cta_count(n) doubles.
@@ -95,16 +96,20 @@ cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, 
                                    int n, int bc_kind, int iters, double* partials, BicgState* st,
                                    unsigned int* barrier_words, cudaStream_t s, bool elide);
 // The same with every vector on chip (resident.cuh), for calls that start
-// from r*_0 = p*_0 = r_0 = p_0.  words: resident_bytes(n) of device memory for
-// the exchanges between CTAs, not shared with a launch that may run at the same time.
+// from r*_0 = p*_0 = r_0 = p_0.  For the exchanges between CTAs, not shared with a
+// launch that may run at the same time: slots, resident_slot_bytes() of device
+// memory that no one else writes, zero at first; node_words, 16 bytes per node of
+// the grid, 16-byte aligned, without a tag when a call starts.  r null (FP64): r is in
+// the node words, as launch_bicg_start leaves it.
 // max_ctas: CTAs at most (0: one per SM).  resident_ctas: CTAs that the launch takes, 0 where it takes no
 // such grid.  resident_batch_limit: the batch engine's max_ctas.
 int resident_ctas(int n, int max_ctas);
 int resident_batch_limit(int n);
-size_t resident_bytes(int n);
+size_t resident_slot_bytes();
+size_t resident_bytes(int n);   // slots and node words
 template <typename T>
 cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
-                                 void* words, cudaStream_t s, bool elide, int max_ctas);
+                                 void* slots, void* node_words, cudaStream_t s, bool elide, int max_ctas);
 constexpr int kResidentMaxN = 81;   // eight nodes per thread on 152 SMs
 // The 2D problem's form, on grids that fit on chip with four nodes per thread.
 constexpr int kPersistentMaxN2d = 512;
@@ -198,6 +203,7 @@ struct excmg_ctx {
     double* scalar = nullptr;                 // one-off reduction results (8 doubles)
     excmg::BicgState* state = nullptr;        // device
     unsigned int* barrier = nullptr;          // device words of the cooperative solver's grid barrier
+    void* slots = nullptr;                    // slot words of the on-chip solver's exchanges
     // pinned, mapped host mirrors of `state` and `scalar` and their device
     // addresses: a one-CTA kernel writes them (ctx_read_back), so reading the
     // state back uses no copy engine and never queues behind a caller's large

@@ -162,6 +162,8 @@ struct MarchArrays {
     double* psn;          // the same for p*
     double beta;
     double* rsn;          // kMarchStart: r*, may be null
+    ulonglong2* words;    // kMarchStart: the on-chip kernel's words, r in their values, no tag (out is
+                          // not written then); may be null
 };
 
 // Shared memory: one stage, `in` (and r) on all three slots, p* (and r*), or
@@ -396,9 +398,13 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
                         d = __fma_rn(lds_f64(hist + (unsigned)((t + 2) & 3) * (2 * kCol) + s * kCol), val, d);
                     } else {
                         const double rv = has_b ? bv[s] - val : val;
-                        if (K != kMarchNorm) *(double*)(oz + so[s]) = rv;
+                        if (K == kMarchApply || K == kMarchSub) *(double*)(oz + so[s]) = rv;
                         if (K == kMarchStart) {
                             const size_t o = (size_t)zo * plane8 + so[s];
+                            if (a.words)
+                                a.words[o / 8] = make_ulonglong2((unsigned long long)__double_as_longlong(rv), 0ull);
+                            else
+                                *(double*)(oz + so[s]) = rv;
                             if (a.pn) *(double*)((char*)a.pn + o) = rv;
                             if (a.rsn) *(double*)((char*)a.rsn + o) = rv;
                             if (a.psn) *(double*)((char*)a.psn + o) = rv;

@@ -231,7 +231,7 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
         const int left = max_iter - ctx->host_state->iter;
         if (words) {
             err = launch_bicg_resident<float>(e, r, rs, p, ps, n, bc_kind, left < 1024 ? left : 1024, ctx->state, words,
-                                              s, false, 0);
+                                              (char*)words + resident_slot_bytes(), s, false, 0);
             note_launches(1);
             if (err != cudaSuccess) return ctx_cuda(ctx, err, "cooperative FP32 Bi-CG launch");
             continue;
@@ -276,7 +276,7 @@ int mixed_level_solve(excmg_ctx* ctx, int n, int bc_kind, const double* fh, doub
         if (ctx->stencil_variant == kStencilExact && stencil_cta_count(n) <= kMaxPartials) {
             if (!stencil_writes_boundary(n, ctx->stencil_variant)) err = launch_zero_boundary({r}, n, s);
             if (err == cudaSuccess)
-                err = launch_bicg_start(u, fh, n, bc_kind, r, nullptr, nullptr, nullptr, ctx->partials, ctx->ticket,
+                err = launch_bicg_start(u, fh, n, bc_kind, r, nullptr, nullptr, nullptr, nullptr, ctx->partials, ctx->ticket,
                                         ctx->scalar, nullptr, s);
             if (err == cudaSuccess) err = ctx_read_back(ctx, ctx->host_scalar, ctx->scalar, sizeof(double));
             if (err == cudaSuccess) err = cudaStreamSynchronize(s);

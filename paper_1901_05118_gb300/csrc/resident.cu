@@ -51,8 +51,6 @@ int resident2d_ctas(int n) { return n > kPersistentMaxN2d ? 0 : resident_geometr
 int resident_batch_limit(int n) { return n <= 32 ? 16 : n <= 52 ? 72 : 0; }
 
 namespace {
-size_t slot_bytes() { return (kResWords * sizeof(ulonglong2) + 255) / 256 * 256; }
-
 // The launch's tag: unique in the process, so no word left by another launch matches.
 unsigned next_serial() {
     static std::atomic<unsigned> serial{0};
@@ -62,15 +60,15 @@ unsigned next_serial() {
 }
 }  // namespace
 
-size_t resident_bytes(int n) { return slot_bytes() + node_count(n) * sizeof(ulonglong2); }
-size_t resident2d_bytes(int n) { return slot_bytes() + (size_t)(n + 1) * (n + 1) * sizeof(ulonglong2); }
+size_t resident_slot_bytes() { return (kResWords * sizeof(ulonglong2) + 255) / 256 * 256; }
+size_t resident_bytes(int n) { return resident_slot_bytes() + node_count(n) * sizeof(ulonglong2); }
+size_t resident2d_bytes(int n) { return resident_slot_bytes() + (size_t)(n + 1) * (n + 1) * sizeof(ulonglong2); }
 
 namespace {
 template <typename T>
 cudaError_t launch(const void* fn, ResidentGeom g, T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters,
-                   BicgState* st, void* words, cudaStream_t s) {
-    ResidentInst<T> in{x, r, rs, p, ps, st, (ulonglong2*)words, (ulonglong2*)((char*)words + slot_bytes()), n,
-                       bc_kind == 1 ? 1 : -1};
+                   BicgState* st, void* slots, void* node_words, cudaStream_t s) {
+    ResidentInst<T> in{x, r, rs, p, ps, st, (ulonglong2*)slots, (ulonglong2*)node_words, n, bc_kind == 1 ? 1 : -1};
     const size_t smem = (size_t)((g.tile + 1) & ~1) * sizeof(T) + resident_own_bytes(g.np) / 8 * sizeof(T);
     (void)kernel_occupancy(fn, kResThreads, kResSmemBytes);   // opts in to the shared memory
     unsigned serial = next_serial();
@@ -82,23 +80,24 @@ cudaError_t launch(const void* fn, ResidentGeom g, T* x, T* r, T* rs, T* p, T* p
 
 template <typename T>
 cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
-                                 void* words, cudaStream_t s, bool elide, int max_ctas) {
+                                 void* slots, void* node_words, cudaStream_t s, bool elide, int max_ctas) {
     const ResidentGeom g = resident_geometry_cached(3, n, max_ctas > 0 ? max_ctas : device_sms());
     const void* fn = resident_fn<T, 3, false>(g.np);
     if constexpr (sizeof(T) == 8)
         if (elide) fn = resident_fn<T, 3, true>(g.np);
-    return launch<T>(fn, g, x, r, rs, p, ps, n, bc_kind, iters, st, words, s);
+    return launch<T>(fn, g, x, r, rs, p, ps, n, bc_kind, iters, st, slots, node_words, s);
 }
 
 cudaError_t launch_bicg2d_resident(double* x, double* r, double* rs, double* p, double* ps, int n, int bc_kind,
                                    int iters, BicgState* st, void* words, cudaStream_t s) {
     const ResidentGeom g = resident_geometry_cached(2, n, device_sms());
-    return launch<double>(resident_fn<double, 2, false>(g.np), g, x, r, rs, p, ps, n, bc_kind, iters, st, words, s);
+    return launch<double>(resident_fn<double, 2, false>(g.np), g, x, r, rs, p, ps, n, bc_kind, iters, st, words,
+                          (char*)words + resident_slot_bytes(), s);
 }
 
 template cudaError_t launch_bicg_resident<double>(double*, double*, double*, double*, double*, int, int, int,
-                                                  BicgState*, void*, cudaStream_t, bool, int);
+                                                  BicgState*, void*, void*, cudaStream_t, bool, int);
 template cudaError_t launch_bicg_resident<float>(float*, float*, float*, float*, float*, int, int, int, BicgState*,
-                                                 void*, cudaStream_t, bool, int);
+                                                 void*, void*, cudaStream_t, bool, int);
 
 }  // namespace excmg

@@ -59,9 +59,11 @@
 
 namespace excmg {
 
-// One Bi-CG call on one grid.  Vectors are node arrays with zero boundary
-// entries.  words: kResWords slot words; rx: one word per node (the r of the
-// brick surfaces).  No word holds a tag of this launch when it starts.
+// One Bi-CG call on one grid.  Vectors are node arrays, of which the interior
+// entries are used.  words: kResWords slot words; rx: one word per node (the r of
+// the brick surfaces).  No word holds a tag of this launch when it starts.
+// r null: r is in the value halves of rx between launches, the surfaces' as the
+// exchanges left it.
 template <typename T>
 struct ResidentInst {
     T* x;
@@ -266,13 +268,20 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
         rs.v = own + NP * kResThreads;
         ps.v = own + 2 * NP * kResThreads;
     }
+    // (the owner of a word writes it first after exchange 1, which every CTA
+    // enters with these values in use)
+    auto first_r = [&](int o) -> T {
+        if constexpr (kExact)
+            if (!in.r) return __longlong_as_double((long long)ld_word(in.rx + o).x);
+        return in.r[o];
+    };
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
         x[k] = r[k] = p[k] = q[k] = rs[k] = ps[k] = T(0);
         if (k < cnt) {
             const int o = idx0 + k * plane;
             x[k] = in.x[o];
-            r[k] = in.r[o];
+            r[k] = first_r(o);
             p[k] = in.p[o];
             if (!kElide) {
                 rs[k] = in.rs[o];
@@ -283,7 +292,7 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
 #pragma unroll
     for (int k = 0; k < NH; ++k) {
         hp[k] = hidx[k] >= 0 ? in.p[hidx[k]] : T(0);
-        hr[k] = hidx[k] >= 0 ? in.r[hidx[k]] : T(0);
+        hr[k] = hidx[k] >= 0 ? first_r(hidx[k]) : T(0);
     }
 
     double rho = st->rho, beta = st->beta;                      // every thread
@@ -561,7 +570,8 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
         if (k < cnt) {
             const int o = idx0 + k * plane;
             in.x[o] = x[k];
-            in.r[o] = r[k];
+            if (in.r) in.r[o] = r[k];
+            else if (kExact && !(surf >> k & 1u)) st_word(in.rx + o, bits_of(r[k]), 0ull);
             in.p[o] = p[k];
             if (!kElide) {
                 in.rs[o] = rs[k];

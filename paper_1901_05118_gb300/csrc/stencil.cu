@@ -260,8 +260,10 @@ stencil_point_kernel(MarchArrays a, int n, int sigma, const int* __restrict__ sk
             v = fx_point(a.in, n, sigma, i, j, k);
             if (a.b) v = a.b[t] - v;
         }
-        if (K != kMarchNorm) a.out[t] = v;
+        if (K == kMarchApply || K == kMarchSub) a.out[t] = v;
         if (K == kMarchStart) {
+            if (a.words) a.words[t] = make_ulonglong2((unsigned long long)__double_as_longlong(v), 0ull);
+            else a.out[t] = v;
             if (a.pn) a.pn[t] = v;
             if (a.rsn) a.rsn[t] = v;
             if (a.psn) a.psn[t] = v;
@@ -655,9 +657,9 @@ cudaError_t launch_residual_norm(const double* x, const double* b, int n, int bc
 }
 
 cudaError_t launch_bicg_start(const double* x, const double* b, int n, int bc_kind, double* r, double* rs, double* p,
-                              double* ps, double* partials, unsigned int* ticket, double* out, BicgState* st,
-                              cudaStream_t s) {
-    const MarchArrays a{x, nullptr, nullptr, nullptr, b, r, p, ps, 0.0, rs};
+                              double* ps, void* words, double* partials, unsigned int* ticket, double* out,
+                              BicgState* st, cudaStream_t s) {
+    const MarchArrays a{x, nullptr, nullptr, nullptr, b, r, p, ps, 0.0, rs, (ulonglong2*)words};
     return launch_residual<kMarchStart>(a, n, bc_kind, partials, ticket, out, st, s);
 }
 
