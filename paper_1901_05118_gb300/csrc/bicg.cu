@@ -101,12 +101,12 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // as two applications and a separate inner product
     const bool fused = ctx->stencil_variant == kStencilExact && stencil_cta_count(n) <= kMaxPartials;
     // small grids run whole iterations in one cooperative launch: from r*_0 = r_0
-    // with every vector on chip, else on the general kernel up to 64^3.  The node words of the
-    // first take the place of r and q, so that it needs no more memory than
-    // the others do (three vectors shadow-elided, five in full) and no budget and no
-    // earlier call decides between them.
+    // with every vector on chip, with a caller's r*_0 on the general kernel up to
+    // 64^3.  The node words of the first take the place of r and q, so that it needs no
+    // more memory than launched kernels do (three vectors shadow-elided, five in full)
+    // and no budget and no earlier call decides between them.
     const bool resident = fused && shadow == nullptr && resident_ctas(n, 0) > 0;
-    const bool persistent = resident || (fused && n <= kPersistentMaxN);
+    const bool persistent = resident || (fused && shadow != nullptr && n <= kPersistentMaxN);
     double* r = resident ? nullptr : ctx_buffer(ctx, "bicg_r", bytes, &st);
     double* rs = (st || elide) ? nullptr : ctx_buffer(ctx, "bicg_rs", bytes, &st);
     double* p = st ? nullptr : ctx_buffer(ctx, "bicg_p", bytes, &st);
@@ -120,9 +120,8 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     const bool fuse = ctx->schedule == EXCMG_SCHEDULE_FUSED;
     const bool dir_fused = fused && fuse && !persistent;
     // the integer operator's A^T p* is A p bit for bit while p* = p, as it is
-    // from r*_0 = r_0 on: both are read from q (the general cooperative
-    // kernel keeps its second array)
-    const bool twin = fused && shadow == nullptr && (resident || !persistent);
+    // from r*_0 = r_0 on: both are read from q
+    const bool twin = fused && shadow == nullptr;
     const bool own_qs = !elide && !twin;
     double* q = ctx_buffer(ctx, "bicg_q", resident || own_qs ? 2 * bytes : bytes, &st);
     if (st) return st;
@@ -176,7 +175,7 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
             e = resident ? launch_bicg_resident<double>(x, r, rs, p, ps, n, bc_kind, chunk, ctx->state, ctx->slots, q, s,
                                                         elide, 0)
                          : launch_bicg_persistent(x, r, rs, p, ps, q, qs, n, bc_kind, chunk, ctx->partials,
-                                                  ctx->state, ctx->barrier, s, elide);
+                                                  ctx->state, ctx->barrier, s);
             note_launches(1);
             if (e != cudaSuccess) return ctx_cuda(ctx, e, "cooperative Bi-CG launch");
             e = ctx_read_back(ctx, ctx->host_state, ctx->state, sizeof(BicgState));

@@ -86,15 +86,12 @@ int stencil_cta_count(int n);
 cudaError_t launch_bicg_stencil_pair_dir(const double* r, const double* rs, const double* p_prev,
                                          const double* ps_prev, double* p, double* ps, double* q, double* qs, int n,
                                          int bc_kind, double* partials, BicgState* st, cudaStream_t s);
-// Grids up to 64^3 that the resident kernel does not take (a caller-chosen r*_0, no
-// room for its words): whole Bi-CG iterations (up to `iters`) in one cooperative
-// launch with bounded grid barriers; barrier_words: 3 device words.
+// Grids up to 64^3 with a caller's r*_0: whole Bi-CG iterations (up to `iters`)
+// in one cooperative launch with bounded grid barriers; barrier_words: 3 device words.
 constexpr int kPersistentMaxN = 64;
-bool persistent_pointwise(int n);
-// elide: the shadow-elided mode (rs, ps, qs unused, may be null).
 cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, double* ps, double* q, double* qs,
                                    int n, int bc_kind, int iters, double* partials, BicgState* st,
-                                   unsigned int* barrier_words, cudaStream_t s, bool elide);
+                                   unsigned int* barrier_words, cudaStream_t s);
 // The same with every vector on chip (resident.cuh), for calls that start
 // from r*_0 = p*_0 = r_0 = p_0.  For the exchanges between CTAs, not shared with a
 // launch that may run at the same time: slots, resident_slot_bytes() of device

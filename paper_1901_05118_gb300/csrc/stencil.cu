@@ -308,13 +308,9 @@ __device__ __forceinline__ double all_partials(const double* partials, int c, do
     return v;
 }
 
-// kElide: the shadow-elided mode (not the paper's Alg. 2 as printed): r*,
-// p*, A^T p* are not stored because they equal r, p, A p bit for bit (the
-// integer operator is symmetric and r*_0 = r_0); v.rs, v.ps, v.ps2, v.qs are
-// unused and the iterates are the same bits as with kElide = false.
 // Three phases per iteration: operator pair with sigma; x, r, r* update
 // with (r*, r) and (r, r); direction update.
-template <bool kPointwise, bool kElide>
+template <bool kPointwise>
 __global__ void __launch_bounds__(FX_NT, 2)
 bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int gy, int slabs, int kz_per,
                        int iters, double* partials, BicgState* st, GridBarrier gb) {
@@ -340,12 +336,8 @@ bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int 
                 const size_t o = ((size_t)k * np + j) * np + i;
                 const double qv = fx_point(v.p, n, sigma, i, j, k);
                 v.q[o] = qv;
-                if (kElide) {
-                    dot += v.p[o] * qv;
-                } else {
-                    v.qs[o] = fx_point(v.ps, n, sigma, i, j, k);
-                    dot += v.ps[o] * qv;
-                }
+                v.qs[o] = fx_point(v.ps, n, sigma, i, j, k);
+                dot += v.ps[o] * qv;
             }
         } else {
             for (int u = blockIdx.x; u < units; u += G) {
@@ -354,7 +346,7 @@ bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int 
                 const int kz1 = min(kz0 + kz_per, n);
                 __syncthreads();   // the CTA's previous unit is done with the shared buffers
                 const FxFields fl{{v.p, v.ps}, {v.q, v.qs}, {nullptr, nullptr}, {nullptr, nullptr}, 0.0};
-                dot += fx_march<kElide ? 1 : 2, true>(fl, nullptr, n, sigma, bx, by, kz0, kz1);
+                dot += fx_march<2, true>(fl, nullptr, n, sigma, bx, by, kz0, kz1);
             }
         }
         dot = block_sum(dot, sh);
@@ -385,10 +377,8 @@ bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int 
                     pv[k] = pcur[t];
                     rv[k] = v.r[t];
                     qv[k] = v.q[t];
-                    if (!kElide) {
-                        rsv[k] = v.rs[t];
-                        qsv[k] = v.qs[t];
-                    }
+                    rsv[k] = v.rs[t];
+                    qsv[k] = v.qs[t];
                 }
             }
 #pragma unroll
@@ -398,10 +388,6 @@ bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int 
                 v.x[t] = xv[k] + alpha * pv[k];
                 const double rn = rv[k] - alpha * qv[k];
                 v.r[t] = rn;
-                if (kElide) {
-                    vrr += rn * rn;
-                    continue;
-                }
                 if (__double_as_longlong(rsv[k]) == __double_as_longlong(rv[k]) &&
                     __double_as_longlong(qsv[k]) == __double_as_longlong(qv[k])) {
                     v.rs[t] = rn;
@@ -456,10 +442,8 @@ bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int 
                     if (t < len) {
                         rv[k] = v.r[t];
                         pv[k] = v.p[t];
-                        if (!kElide) {
-                            rsv[k] = v.rs[t];
-                            psv[k] = v.ps[t];
-                        }
+                        rsv[k] = v.rs[t];
+                        psv[k] = v.ps[t];
                     }
                 }
 #pragma unroll
@@ -467,7 +451,7 @@ bicg_persistent_kernel(BicgVectors v, size_t len, int n, int sigma, int gx, int 
                     const size_t t = t0 + k * S;
                     if (t >= len) break;
                     v.p[t] = rv[k] + beta * pv[k];
-                    if (!kElide) v.ps[t] = rsv[k] + beta * psv[k];
+                    v.ps[t] = rsv[k] + beta * psv[k];
                 }
             }
             if (!(ok = grid_sync(gb, G))) break;
@@ -666,9 +650,7 @@ cudaError_t launch_bicg_start(const double* x, const double* b, int n, int bc_ki
 constexpr int kPointwiseMaxN = 32;   // per-node operator on grids up to 32^3
 
 int persistent_grid(int n, int* gx, int* gy, int* slabs, int* kz_per) {
-    // the elided variants run on the grids of the full ones (same partial
-    // sums)
-    const int occ_pt = min(2, resident_per_sm(bicg_persistent_kernel<true, false>, FX_NT));
+    const int occ_pt = min(2, resident_per_sm(bicg_persistent_kernel<true>, FX_NT));
     const int sms = device_sms();
     const int m = n - 1;
     *gx = (m + FX_TX - 1) / FX_TX;
@@ -698,12 +680,9 @@ int persistent_grid(int n, int* gx, int* gy, int* slabs, int* kz_per) {
     return (int)want;
 }
 
-bool persistent_pointwise(int n) { return n <= kPointwiseMaxN; }
-
 cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, double* ps, double* q, double* qs,
                                    int n, int bc_kind, int iters, double* partials, BicgState* st,
-                                   unsigned int* barrier_words, cudaStream_t s, bool elide) {
-    const bool pw = persistent_pointwise(n);
+                                   unsigned int* barrier_words, cudaStream_t s) {
     int gx, gy, slabs, kz_per;
     const int G = persistent_grid(n, &gx, &gy, &slabs, &kz_per);
     cudaError_t e = cudaMemsetAsync(barrier_words, 0, 3 * sizeof(unsigned int), s);
@@ -713,12 +692,8 @@ cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, 
     int sigma = bc_kind == 1 ? 1 : -1;
     GridBarrier gb{barrier_words, barrier_words + 1, (int*)(barrier_words + 2), kBarrierSpinLimit};
     void* args[] = {&v, &len, &n, &sigma, &gx, &gy, &slabs, &kz_per, &iters, &partials, &st, &gb};
-    const void* fn;
-    if (pw) {
-        fn = elide ? (const void*)bicg_persistent_kernel<true, true> : (const void*)bicg_persistent_kernel<true, false>;
-    } else {
-        fn = elide ? (const void*)bicg_persistent_kernel<false, true> : (const void*)bicg_persistent_kernel<false, false>;
-    }
+    const void* fn = n <= kPointwiseMaxN ? (const void*)bicg_persistent_kernel<true>
+                                         : (const void*)bicg_persistent_kernel<false>;
     return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(FX_TX, FX_TY, 1), args, 0, s);
 }
 
