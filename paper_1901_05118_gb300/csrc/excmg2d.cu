@@ -419,9 +419,12 @@ int bicg2d_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, d
     double* rs = st ? nullptr : ctx_buffer(ctx, "b2_rs", bytes, &st);
     double* p = st ? nullptr : ctx_buffer(ctx, "b2_p", bytes, &st);
     double* ps = st ? nullptr : ctx_buffer(ctx, "b2_ps", bytes, &st);
-    double* q = st ? nullptr : ctx_buffer(ctx, "b2_q", bytes, &st);
-    double* qs = st ? nullptr : ctx_buffer(ctx, "b2_qs", bytes, &st);
+    // q and q* in one buffer: on the on-chip kernel's grids it has that kernel's node
+    // words, so that no budget decides between the two kernels
+    double* q = st ? nullptr : ctx_buffer(ctx, "b2_q", 2 * bytes, &st);
     if (st) return st;
+    double* qs = q + len;
+    const bool resident = resident2d_ctas(n) > 0;
     const dim3 g = grid2d(n);
     if ((int)(g.x * g.y) > kMaxPartials) return ctx_fail(ctx, EXCMG_ERR_ARG, "2D grid too large");
     cudaStream_t s = ctx->stream;
@@ -431,8 +434,7 @@ int bicg2d_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, d
     init.max_iter = max_iter;
     *ctx->host_state = init;
     cudaError_t e = cudaMemcpyAsync(ctx->state, ctx->host_state, sizeof(BicgState), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, bytes, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(qs, 0, bytes, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, 2 * bytes, s);
     if (e == cudaSuccess) e = launch_stencil2d(x, r, b, n, bc_kind, s);
     if (e == cudaSuccess) e = launch_bicg_init(r, nullptr, rs, p, ps, len, n, ctx->partials, ctx->state, s);
     note_launches(3);
@@ -440,17 +442,17 @@ int bicg2d_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, d
     const int sg = bc_kind == 1 ? 1 : -1;
     if (check_every < 1) check_every = 1;
     // grids up to 512^2: many iterations per launch with every vector on chip
-    // (512^2: 10 us per iteration, three launches 31 us); larger ones, or no room
-    // for the exchange words: three launches per iteration
-    void* words = resident2d_ctas(n) > 0 ? ctx_scratch(ctx, resident2d_bytes(n)) : nullptr;
+    // (512^2: 10 us per iteration, three launches 31 us); larger ones: three
+    // launches per iteration
     for (;;) {
         e = ctx_read_back(ctx, ctx->host_state, ctx->state, sizeof(BicgState));
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return ctx_cuda(ctx, e, "2D Bi-CG state read");
         if (ctx->host_state->done) break;
         const int left = max_iter - ctx->host_state->iter;
-        if (words) {
-            e = launch_bicg2d_resident(x, r, rs, p, ps, n, bc_kind, left < 1024 ? left : 1024, ctx->state, words, s);
+        if (resident) {
+            e = launch_bicg2d_resident(x, r, rs, p, ps, n, bc_kind, left < 1024 ? left : 1024, ctx->state, ctx->slots,
+                                       q, s);
             note_launches(1);
             if (e != cudaSuccess) return ctx_cuda(ctx, e, "cooperative 2D Bi-CG launch");
             continue;

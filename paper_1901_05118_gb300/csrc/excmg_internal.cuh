@@ -111,9 +111,8 @@ constexpr int kResidentMaxN = 81;   // eight nodes per thread on 152 SMs
 // The 2D problem's form, on grids that fit on chip with four nodes per thread.
 constexpr int kPersistentMaxN2d = 512;
 int resident2d_ctas(int n);
-size_t resident2d_bytes(int n);
 cudaError_t launch_bicg2d_resident(double* x, double* r, double* rs, double* p, double* ps, int n, int bc_kind,
-                                   int iters, BicgState* st, void* words, cudaStream_t s);
+                                   int iters, BicgState* st, void* slots, void* node_words, cudaStream_t s);
 // Shadow-elided mode (r* = r, p* = p, A^T p* = A p not stored): the one-field
 // operator launches with sigma = (p, A p) and alpha (the second also forms
 // p = r + beta p_prev into p), and the matching set-up and update kernels.

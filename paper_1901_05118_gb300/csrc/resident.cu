@@ -62,7 +62,6 @@ unsigned next_serial() {
 
 size_t resident_slot_bytes() { return (kResWords * sizeof(ulonglong2) + 255) / 256 * 256; }
 size_t resident_bytes(int n) { return resident_slot_bytes() + node_count(n) * sizeof(ulonglong2); }
-size_t resident2d_bytes(int n) { return resident_slot_bytes() + (size_t)(n + 1) * (n + 1) * sizeof(ulonglong2); }
 
 namespace {
 template <typename T>
@@ -89,10 +88,10 @@ cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_k
 }
 
 cudaError_t launch_bicg2d_resident(double* x, double* r, double* rs, double* p, double* ps, int n, int bc_kind,
-                                   int iters, BicgState* st, void* words, cudaStream_t s) {
+                                   int iters, BicgState* st, void* slots, void* node_words, cudaStream_t s) {
     const ResidentGeom g = resident_geometry_cached(2, n, device_sms());
-    return launch<double>(resident_fn<double, 2, false>(g.np), g, x, r, rs, p, ps, n, bc_kind, iters, st, words,
-                          (char*)words + resident_slot_bytes(), s);
+    return launch<double>(resident_fn<double, 2, false>(g.np), g, x, r, rs, p, ps, n, bc_kind, iters, st, slots,
+                          node_words, s);
 }
 
 template cudaError_t launch_bicg_resident<double>(double*, double*, double*, double*, double*, int, int, int,

@@ -68,3 +68,30 @@ def test_repeated_solves_under_the_least_budget(n, nc, kind, mode):
     least = least_budget(solve, 1 << 14, 20 * 8 * (n + 1) ** 3 + (1 << 25))
     for got in solve(least, times=3):
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("n", [97, 512, 600])
+def test_2d_bicg_in_seven_vectors(n):
+    """The 2D call's right-hand side and six vectors are all that it needs."""
+    b = dev(P.random_field_2d(n, 502))
+    got = []
+    for budget in (0, 7 * 8 * (n + 1) ** 2):
+        ctx = B.Context(hbm_budget_bytes=budget)
+        for _ in range(2):
+            x = torch.zeros((n + 1,) * 2, dtype=torch.float64, device=DEV)
+            got.append((x, B.bicg_solve2d(n, 1, b, x, 0.0, 25, ctx=ctx)))
+    for x, info in got:
+        assert info == got[0][1] and torch.equal(x, got[0][0])
+
+
+def test_2d_solves_under_the_least_budget():
+    n, nc, kind = 128, 8, 2
+    data = [dev(a) for a in P.exp_sum_2d().data(n, kind)]
+
+    def solve(budget, times=1):
+        ctx = B.Context(hbm_budget_bytes=budget)
+        return [B.excmg_solve2d(n, nc, kind, *data, 1e-8, ctx=ctx) for _ in range(times)]
+
+    want = solve(0)[0]
+    for got in solve(least_budget(solve, 1 << 14, 20 * 8 * (n + 1) ** 2 + (1 << 25)), times=3):
+        assert torch.equal(got, want)
