@@ -120,45 +120,10 @@ cudaError_t ctx_read_back(excmg_ctx* ctx, void* host_mirror, const void* dev_src
     return cudaGetLastError();
 }
 
-namespace {
-constexpr const char* kScratch = "resident_words";
-}  // namespace
-
-bool ctx_drop_scratch(excmg_ctx* ctx) {
-    auto it = ctx->buffers.find(kScratch);
-    if (it == ctx->buffers.end() || !it->second.ptr) return false;
-    cudaFree(it->second.ptr);
-    ctx->bytes -= it->second.bytes;
-    it->second = excmg_buffer{};
-    return true;
-}
-
-void* ctx_scratch(excmg_ctx* ctx, size_t bytes) {
-    excmg_buffer& b = ctx->buffers[kScratch];
-    if (b.ptr && b.bytes >= bytes) return b.ptr;
-    ctx_drop_scratch(ctx);
-    if (ctx->budget && ctx->bytes + bytes > ctx->budget) return nullptr;
-    void* p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (cudaMemsetAsync(p, 0, bytes, ctx->stream) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(p);
-        return nullptr;
-    }
-    b.ptr = p;
-    b.bytes = bytes;
-    ctx->bytes += bytes;
-    return p;
-}
-
 double* ctx_buffer(excmg_ctx* ctx, const char* name, size_t bytes, int* status) {
     excmg_buffer& b = ctx->buffers[name];
     if (b.bytes >= bytes && b.ptr) return (double*)b.ptr;
     const size_t held = b.bytes;
-    if (ctx->budget && ctx->bytes - held + bytes > ctx->budget) ctx_drop_scratch(ctx);
     if (ctx->budget && ctx->bytes - held + bytes > ctx->budget) {
         *status = ctx_fail(ctx, EXCMG_ERR_BUDGET, std::string("HBM budget too small for buffer ") + name);
         return nullptr;
@@ -169,8 +134,7 @@ double* ctx_buffer(excmg_ctx* ctx, const char* name, size_t bytes, int* status) 
         b.ptr = nullptr;
         b.bytes = 0;
     }
-    if (cudaMalloc(&b.ptr, bytes) != cudaSuccess &&
-        (cudaGetLastError(), !ctx_drop_scratch(ctx) || cudaMalloc(&b.ptr, bytes) != cudaSuccess)) {
+    if (cudaMalloc(&b.ptr, bytes) != cudaSuccess) {
         cudaGetLastError();
         b.ptr = nullptr;
         *status = ctx_fail(ctx, EXCMG_ERR_OOM, std::string("cudaMalloc failed for buffer ") + name);

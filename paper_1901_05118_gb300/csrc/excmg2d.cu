@@ -349,7 +349,6 @@ int dsolve2d(excmg_ctx* ctx, int n, int bc_kind, const double* fh, double* u) {
     auto it = ctx->inverses.find(key);
     if (it == ctx->inverses.end()) {
         const size_t bytes = (size_t)nu * nu * sizeof(double);
-        if (ctx->budget && ctx->bytes + bytes > ctx->budget) ctx_drop_scratch(ctx);
         if (ctx->budget && ctx->bytes + bytes > ctx->budget)
             return ctx_fail(ctx, EXCMG_ERR_BUDGET, "HBM budget too small for the 2D DSOLVE inverse");
         excmg_buffer buf;

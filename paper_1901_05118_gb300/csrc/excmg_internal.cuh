@@ -96,8 +96,8 @@ cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, 
 // from r*_0 = p*_0 = r_0 = p_0.  For the exchanges between CTAs, not shared with a
 // launch that may run at the same time: slots, resident_slot_bytes() of device
 // memory that no one else writes, zero at first; node_words, 16 bytes per node of
-// the grid, 16-byte aligned, without a tag when a call starts.  r null (FP64): r is in
-// the node words, as launch_bicg_start leaves it.
+// the grid, 16-byte aligned, without a tag when a call starts.  r null: r is in the
+// node words, as launch_bicg_start leaves it.
 // max_ctas: CTAs at most (0: one per SM).  resident_ctas: CTAs that the launch takes, 0 where it takes no
 // such grid.  resident_batch_limit: the batch engine's max_ctas.
 int resident_ctas(int n, int max_ctas);
@@ -261,11 +261,6 @@ int ctx_cuda(excmg_ctx* ctx, cudaError_t err, const char* what);
 // host_scalar), written by a kernel; the caller synchronises the stream.
 cudaError_t ctx_read_back(excmg_ctx* ctx, void* host_mirror, const void* dev_src, size_t bytes);
 double* ctx_buffer(excmg_ctx* ctx, const char* name, size_t bytes, int* status);
-// At least `bytes` of device memory whose contents a caller may rely on to be
-// its own or zero (the exchange words of resident.cuh): null where the budget
-// or the device has no room.  It is given up first when a buffer needs the room.
-void* ctx_scratch(excmg_ctx* ctx, size_t bytes);
-bool ctx_drop_scratch(excmg_ctx* ctx);   // false: there was none
 // Bi-CG driver (bicg.cu): iterates on the context's stream.
 int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, double tol,
              double bnorm, int max_iter, int check_every, int* iters_out, double* relres_out,

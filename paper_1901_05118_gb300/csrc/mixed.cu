@@ -184,8 +184,11 @@ int stencil32_cta_count(int n) {
 }
 
 // FP32 Bi-CG on A e = b32 from e = 0 (Alg. 2, M = I, r*_0 = r_0).
-static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, float* e, double tol, int max_iter,
-                      int check_every, int* iters_out) {
+// q, qs: where A p and A^T p* go; words: the on-chip kernel's node words, which
+// may lie in the same memory (and do: with that of the residual in FP64, which is formed
+// again after the solve), so that no budget decides between the two paths.
+static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, float* e, float* q, float* qs, void* words,
+                      double tol, int max_iter, int check_every, int* iters_out) {
     const size_t len = node_count(n);
     const size_t bytes = len * sizeof(float);
     int st = EXCMG_OK;
@@ -193,9 +196,8 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
     float* rs = st ? nullptr : (float*)ctx_buffer(ctx, "b32_rs", bytes, &st);
     float* p = st ? nullptr : (float*)ctx_buffer(ctx, "b32_p", bytes, &st);
     float* ps = st ? nullptr : (float*)ctx_buffer(ctx, "b32_ps", bytes, &st);
-    float* q = st ? nullptr : (float*)ctx_buffer(ctx, "b32_q", bytes, &st);
-    float* qs = st ? nullptr : (float*)ctx_buffer(ctx, "b32_qs", bytes, &st);
     if (st) return st;
+    const bool resident = resident_ctas(n, 0) > 0;
     cudaStream_t s = ctx->stream;
     const Grid32 g = grid32(n);
     if ((int)(g.grid.x * g.grid.y * g.grid.z) > kMaxPartials)
@@ -207,8 +209,12 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
     init.max_iter = max_iter;
     *ctx->host_state = init;
     cudaError_t err = cudaMemcpyAsync(ctx->state, ctx->host_state, sizeof(BicgState), cudaMemcpyHostToDevice, s);
-    if (err == cudaSuccess) err = cudaMemsetAsync(q, 0, bytes, s);
-    if (err == cudaSuccess) err = cudaMemsetAsync(qs, 0, bytes, s);
+    if (resident) {
+        if (err == cudaSuccess) err = cudaMemsetAsync(words, 0, 16 * len, s);
+    } else {
+        if (err == cudaSuccess) err = cudaMemsetAsync(q, 0, bytes, s);
+        if (err == cudaSuccess) err = cudaMemsetAsync(qs, 0, bytes, s);
+    }
     // e = 0, so r_0 = b32
     if (err == cudaSuccess) err = cudaMemcpyAsync(r, b32, bytes, cudaMemcpyDeviceToDevice, s);
     if (err == cudaSuccess) {
@@ -221,17 +227,16 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
     // grids up to 81^3: many iterations per launch with every vector on chip
     // (48^3: 5 us per iteration, against 25 us for the three launches,
     // each of them a few microseconds of latency for 0.5 MB vectors); larger
-    // ones, or no room for the exchange words: the launched kernels
-    void* words = resident_ctas(n, 0) > 0 ? ctx_scratch(ctx, resident_bytes(n)) : nullptr;
+    // ones: the launched kernels
     for (;;) {
         err = ctx_read_back(ctx, ctx->host_state, ctx->state, sizeof(BicgState));
         if (err == cudaSuccess) err = cudaStreamSynchronize(s);
         if (err != cudaSuccess) return ctx_cuda(ctx, err, "FP32 Bi-CG state read");
         if (ctx->host_state->done) break;
         const int left = max_iter - ctx->host_state->iter;
-        if (words) {
-            err = launch_bicg_resident<float>(e, r, rs, p, ps, n, bc_kind, left < 1024 ? left : 1024, ctx->state, words,
-                                              (char*)words + resident_slot_bytes(), s, false, 0);
+        if (resident) {
+            err = launch_bicg_resident<float>(e, r, rs, p, ps, n, bc_kind, left < 1024 ? left : 1024, ctx->state,
+                                              ctx->slots, words, s, false, 0);
             note_launches(1);
             if (err != cudaSuccess) return ctx_cuda(ctx, err, "cooperative FP32 Bi-CG launch");
             continue;
@@ -262,7 +267,9 @@ int mixed_level_solve(excmg_ctx* ctx, int n, int bc_kind, const double* fh, doub
                       int* outer_out, int* stag_out, double* rel_out) {
     const size_t len = node_count(n);
     int st = EXCMG_OK;
-    double* r = ctx_buffer(ctx, "res", len * sizeof(double), &st);
+    // r, and behind it q and q* of the FP32 solves
+    double* r = ctx_buffer(ctx, "res", 2 * len * sizeof(double), &st);
+    float* const q = (float*)(r + len);
     float* r32 = st ? nullptr : (float*)ctx_buffer(ctx, "mx_r32", len * sizeof(float), &st);
     float* e = st ? nullptr : (float*)ctx_buffer(ctx, "mx_e", len * sizeof(float), &st);
     if (st) return st;
@@ -311,7 +318,7 @@ int mixed_level_solve(excmg_ctx* ctx, int n, int bc_kind, const double* fh, doub
         int cap = max_total - iters;
         if (cap > max_inner) cap = max_inner;
         int it = 0;
-        if ((st = bicg32_run(ctx, n, bc_kind, r32, e, inner_tol, cap, check_every, &it))) return st;
+        if ((st = bicg32_run(ctx, n, bc_kind, r32, e, q, q + len, r, inner_tol, cap, check_every, &it))) return st;
         iters += it;
         ++outer;
         add_correction_kernel<<<kVecBlocks, kVecThreads, 0, s>>>(u, e, len, rn);

@@ -60,10 +60,10 @@
 namespace excmg {
 
 // One Bi-CG call on one grid.  Vectors are node arrays, of which the interior
-// entries are used.  words: kResWords slot words; rx: one word per node (the r of
-// the brick surfaces).  No word holds a tag of this launch when it starts.
-// r null: r is in the value halves of rx between launches, the surfaces' as the
-// exchanges left it.
+// entries are used.  words: kResWords slot words, none with a tag of this launch
+// when it starts; rx: one word per node (the r of the brick surfaces), without a
+// tag when a call starts.  r null: r is in the value halves of rx between
+// launches, the surfaces' as the exchanges left it (FP64).
 template <typename T>
 struct ResidentInst {
     T* x;
@@ -91,6 +91,24 @@ __device__ __forceinline__ ulonglong2 ld_word(const ulonglong2* p) {
 __device__ __forceinline__ void st_word(ulonglong2* p, unsigned long long x, unsigned long long y) {
     asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p), "l"(x), "l"(y)
                  : "memory");
+}
+
+// a node's word: its value, and its tag as the result
+__device__ __forceinline__ unsigned long long ld_node(const ulonglong2* w, double* v) {
+    const ulonglong2 t = ld_word(w);
+    *v = __longlong_as_double((long long)t.x);
+    return t.y;
+}
+__device__ __forceinline__ void st_node(ulonglong2* w, double v, unsigned long long tag) {
+    st_word(w, (unsigned long long)__double_as_longlong(v), tag);
+}
+__device__ __forceinline__ unsigned long long ld_node(const ulonglong2* w, float* v) {
+    const ulonglong2 t = ld_word(w);
+    *v = __uint_as_float((unsigned)t.x);
+    return t.y;
+}
+__device__ __forceinline__ void st_node(ulonglong2* w, float v, unsigned long long tag) {
+    st_word(w, (unsigned long long)__float_as_uint(v), tag);
 }
 
 __device__ __forceinline__ unsigned long long bits_of(double v) { return (unsigned long long)__double_as_longlong(v); }
@@ -271,9 +289,10 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
     // (the owner of a word writes it first after exchange 1, which every CTA
     // enters with these values in use)
     auto first_r = [&](int o) -> T {
-        if constexpr (kExact)
-            if (!in.r) return __longlong_as_double((long long)ld_word(in.rx + o).x);
-        return in.r[o];
+        if (!kExact || in.r) return in.r[o];
+        T v;
+        (void)ld_node(in.rx + o, &v);
+        return v;
     };
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
@@ -304,7 +323,8 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
     double inv = 0.0;                                 // warp 0: 1 / rho
     int code = kRunning;
     bool gave_up = false;
-    // Tags: the launch's serial number above the exchange's number.  Slot
+    // Tags: the launch's serial number above the number of the exchange or
+    // iteration (64 bits; a 32-bit one of the iteration in its call was up to 2 % slower).  Slot
     // words come in two sets: a CTA that publishes exchange e + 2 has read
     // exchange e + 1 from every CTA, which each published after it had read
     // exchange e.  The word of a node needs no second one: its owner writes
@@ -482,10 +502,7 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
         for (int k = 0; k < NP; ++k) rn[k] = mad(-a, q[k], r[k]);
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
-            if (surf >> k & 1u) {
-                if constexpr (kExact) st_word(in.rx + idx0 + k * plane, bits_of(rn[k]), rtag);
-                else st_word(in.rx + idx0 + k * plane, (unsigned long long)__float_as_uint(rn[k]), rtag);
-            }
+            if (surf >> k & 1u) st_node(in.rx + idx0 + k * plane, rn[k], rtag);
         }
         if (!kElide) {
             bool twin = kExact;
@@ -543,12 +560,7 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
                 ok = true;
 #pragma unroll
                 for (int k = 0; k < NH; ++k)
-                    if (hidx[k] >= 0) {
-                        const ulonglong2 w = ld_word(in.rx + hidx[k]);
-                        ok = ok && w.y == rtag;
-                        if constexpr (kExact) hr[k] = __longlong_as_double((long long)w.x);
-                        else hr[k] = __uint_as_float((unsigned)w.x);
-                    }
+                    if (hidx[k] >= 0) ok = (ld_node(in.rx + hidx[k], &hr[k]) == rtag) && ok;
                 if (!ok && (++spins & 255) == 0 && (*err == serial || spins > spin_limit)) {
                     *err = serial;
                     lost = 1;
@@ -570,8 +582,8 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
         if (k < cnt) {
             const int o = idx0 + k * plane;
             in.x[o] = x[k];
-            if (in.r) in.r[o] = r[k];
-            else if (kExact && !(surf >> k & 1u)) st_word(in.rx + o, bits_of(r[k]), 0ull);
+            if (!kExact || in.r) in.r[o] = r[k];
+            else if (!(surf >> k & 1u)) st_node(in.rx + o, r[k], 0u);
             in.p[o] = p[k];
             if (!kElide) {
                 in.rs[o] = rs[k];

@@ -95,3 +95,17 @@ def test_2d_solves_under_the_least_budget():
     want = solve(0)[0]
     for got in solve(least_budget(solve, 1 << 14, 20 * 8 * (n + 1) ** 2 + (1 << 25)), times=3):
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("n,nc,kind", [(48, 6, 1), (80, 5, 2), (96, 6, 2)])
+def test_mixed_solves_under_the_least_budget(n, nc, kind):
+    """FP32 correction solves on chip up to 81^3, launched above."""
+    data = [dev(a) for a in P.exp_sum().data(n, kind)]
+
+    def solve(budget, times=1):
+        ctx = B.Context(hbm_budget_bytes=budget)
+        return [B.excmg_solve(n, nc, kind, *data, 1e-8, ctx=ctx, precision="mixed") for _ in range(times)]
+
+    want = solve(0)[0]
+    for got in solve(least_budget(solve, 1 << 14, 20 * 8 * (n + 1) ** 3 + (1 << 25)), times=3):
+        assert torch.equal(got, want)
