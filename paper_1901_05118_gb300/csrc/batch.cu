@@ -353,7 +353,6 @@ struct Instance {
     long long launched_k = 0;
     bool dir_in_p2 = false;
     double t_ready = 0.0;       // when the instance last became ready for Bi-CG iterations
-    bool no_resident = false;   // the current call runs without the resident kernel (no room for its words)
     // FP32 correction solve vectors
     float *r32 = nullptr, *e = nullptr, *r = nullptr, *rs = nullptr, *p = nullptr, *ps = nullptr, *q = nullptr,
           *qs = nullptr;
@@ -390,6 +389,16 @@ size_t instance_bytes(int n, int nc, int prec) {
     return b;
 }
 
+// The node words of the instance's current level, null where it does not run on
+// chip: 16 bytes per node, in memory that the on-chip kernel has no other use for: q64 and
+// the p2_64 behind it (FP64); res, formed again after the call, and the q and qs
+// behind it (FP32).
+void* node_words(const Instance* in) {
+    const int N = in->nc << in->level;
+    if (resident_ctas(N, resident_batch_limit(N)) == 0) return nullptr;
+    return in->prec == EXCMG_PRECISION_FP64 ? (void*)in->q64 : (void*)in->res;
+}
+
 }  // namespace
 
 struct excmg_batch {
@@ -424,8 +433,7 @@ struct excmg_batch {
         bool busy = false;
         bool launched = false;   // members' states are in the single solver's layout (launched mode, resident kernel)
         int sm_share = 0;        // CTA places held while busy, in CTAs of the cooperative FP32 kernel
-        void* words = nullptr;   // exchange words of the resident kernel
-        size_t words_cap = 0;
+        void* slots = nullptr;   // slot words of the resident kernel
         int prec = 0, n = 0, ctas = 0, cand = -1;
         std::vector<Instance*> members;
         void* d_inst = nullptr;        // BatchInst[max_instances]
@@ -593,7 +601,9 @@ int group_init(excmg_batch* b, excmg_batch::Group& g) {
               cudaMalloc(&g.d_active, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&g.d_rounds, sizeof(int)) == cudaSuccess &&
               cudaMallocHost(&g.h_active, 2 * sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&g.d_barrier, 4 * sizeof(unsigned int)) == cudaSuccess;
+              cudaMalloc(&g.d_barrier, 4 * sizeof(unsigned int)) == cudaSuccess &&
+              cudaMalloc(&g.slots, resident_slot_bytes()) == cudaSuccess &&
+              cudaMemsetAsync(g.slots, 0, resident_slot_bytes(), g.stream) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         return bfail(b, EXCMG_ERR_OOM, "batch group buffers");
@@ -613,7 +623,7 @@ void group_free(excmg_batch::Group& g) {
     cudaFree(g.d_barrier);
     cudaFree(g.d_unit_part);
     cudaFree(g.d_chunk_part);
-    cudaFree(g.words);
+    cudaFree(g.slots);
     if (g.start) cudaEventDestroy(g.start);
     if (g.done) cudaEventDestroy(g.done);
     if (g.stream) cudaStreamDestroy(g.stream);
@@ -699,47 +709,30 @@ int launch_group(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instan
 bool launched_level(const Instance* in) { return in->prec == EXCMG_PRECISION_FP64; }
 
 // One launch of the resident kernel for instance `in`: up to b->inner_chunk
-// iterations of its current call.  Returns false where the exchange words
-// find no room at the start of a call: the call then takes the path of larger
-// grids to its end (the two keep different state).
-bool launch_resident(excmg_batch* b, excmg_batch::Group& g, Instance* in, int ctas, int* status) {
-    *status = group_init(b, g);
-    if (*status) return true;
+// iterations of its current call.  Its node words lie in the instance
+// (node_words), so a call goes on with any group record and needs no further memory.
+int launch_resident(excmg_batch* b, excmg_batch::Group& g, Instance* in, int ctas) {
+    int st = group_init(b, g);
+    if (st) return st;
     const int N = in->nc << in->level;
     cudaStream_t s = g.stream;
-    const size_t need = resident_bytes(N);
-    if (g.words_cap < need) {
-        cudaFree(g.words);
-        g.words = nullptr;
-        g.words_cap = 0;
-        if (cudaMalloc(&g.words, need) != cudaSuccess || cudaMemsetAsync(g.words, 0, need, s) != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(g.words);
-            g.words = nullptr;
-            if (in->call_iter > 0) *status = bfail(b, EXCMG_ERR_OOM, "exchange words of the resident kernel");
-            in->no_resident = true;
-            return in->call_iter > 0;
-        }
-        g.words_cap = need;
-    }
     BicgState* bs = b->d_bstate + in->slot;
     cudaError_t e = cudaStreamWaitEvent(s, b->host_ready, 0);
     if (e == cudaSuccess) e = cudaEventRecord(g.start, s);
     const int limit = resident_batch_limit(N);
     if (e == cudaSuccess) {
         if (in->prec == EXCMG_PRECISION_FP64)
-            e = launch_bicg_resident<double>(in->u[in->level], in->res, in->rs64, in->p64, in->ps64, N, in->bc,
-                                             b->inner_chunk, bs, g.words, (char*)g.words + resident_slot_bytes(), s, false, limit);
+            e = launch_bicg_resident<double>(in->u[in->level], nullptr, in->rs64, in->p64, in->ps64, N, in->bc,
+                                             b->inner_chunk, bs, g.slots, node_words(in), s, false, limit);
         else
             e = launch_bicg_resident<float>(in->e, in->r, in->rs, in->p, in->ps, N, in->bc, b->inner_chunk, bs,
-                                            g.words, (char*)g.words + resident_slot_bytes(), s, false, limit);
+                                            g.slots, node_words(in), s, false, limit);
     }
     bnote(b, 1);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->h_bstate + in->slot, bs, sizeof(BicgState), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaEventRecord(g.done, s);
-    *status = bcuda(b, e, "resident batch launch");
-    if (*status) return true;
+    if (e != cudaSuccess) return bcuda(b, e, "resident batch launch");
     *g.h_active = 0;
     *g.h_rounds = 0;   // the member's iterations, known at the harvest
     g.busy = true;
@@ -751,7 +744,7 @@ bool launch_resident(excmg_batch* b, excmg_batch::Group& g, Instance* in, int ct
     g.cand = -1;
     g.members.assign(1, in);
     in->in_flight = true;
-    return true;
+    return EXCMG_OK;
 }
 
 int launch_group_launched(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instance*>& list) {
@@ -1084,13 +1077,13 @@ int excmg_batch_submit(excmg_batch* b, int n_finest, int n_coarsest, int bc_kind
     for (int l = 0; l < in->nl; ++l) in->u.push_back((double*)take(node_count(n_coarsest << l) * sizeof(double)));
     const size_t n64 = node_count(n_finest) * sizeof(double), n32 = node_count(n_finest) * sizeof(float);
     in->fh = (double*)take(n64);
-    in->res = (double*)take(n64);
     in->W = (double*)take(node_count(n_finest / 2) * sizeof(double));
     if (prec == EXCMG_PRECISION_FP64) {
+        in->res = (double*)take(n64);
         in->rs64 = (double*)take(n64);
         in->p64 = (double*)take(n64);
         in->ps64 = (double*)take(n64);
-        in->q64 = (double*)take(n64);
+        in->q64 = (double*)take(n64);   // followed by p2_64 (node_words)
         in->p2_64 = (double*)take(n64);
         in->ps2_64 = (double*)take(n64);
     } else {
@@ -1100,6 +1093,7 @@ int excmg_batch_submit(excmg_batch* b, int n_finest, int n_coarsest, int bc_kind
         in->rs = (float*)take(n32);
         in->p = (float*)take(n32);
         in->ps = (float*)take(n32);
+        in->res = (double*)take(n64);   // followed by q and qs (node_words)
         in->q = (float*)take(n32);
         in->qs = (float*)take(n32);
     }
@@ -1173,7 +1167,8 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
                 e = launch_zero_boundary({in->res}, N, s);
             if (e == cudaSuccess)
                 e = launch_bicg_start(in->u[in->level], in->fh, N, in->bc, in->res, in->rs64, in->p64, in->ps64,
-                                      nullptr, ctx->partials, ctx->ticket, b->d_norms + rw.size(), nullptr, s);
+                                      fp64 ? node_words(in) : nullptr, ctx->partials, ctx->ticket,
+                                      b->d_norms + rw.size(), nullptr, s);
             bnote(b, 1);
             if (e != cudaSuccess) return bcuda(b, e, "batch residual");
             rw.push_back({in, in->res});
@@ -1269,12 +1264,14 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
                 e = cudaGetLastError();
                 if (e == cudaSuccess)
                     e = cudaMemcpyAsync(in->r, in->r32, node_count(N) * sizeof(float), cudaMemcpyDeviceToDevice, s);
+                // (the words lie in the residual's memory, among others)
+                void* const words = node_words(in);
+                if (e == cudaSuccess && words) e = cudaMemsetAsync(words, 0, 16 * node_count(N), s);
             }
             if (e != cudaSuccess) return bcuda(b, e, "Bi-CG call setup");
             in->phase = kInner;
             in->t_ready = now_s();
             in->call_iter = 0;
-            in->no_resident = false;
         }
     }
     // 3. one cooperative launch per level group of instances waiting for
@@ -1313,7 +1310,7 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
         Instance* late = nullptr;
         for (auto& kv : ready)
             for (Instance* in : kv.second)
-                if (!in->no_resident && resident_ctas(kv.first.second, resident_batch_limit(kv.first.second)) > 0 &&
+                if (resident_ctas(kv.first.second, resident_batch_limit(kv.first.second)) > 0 &&
                     now_s() - in->t_ready > kOverdue && (!late || in->t_ready < late->t_ready))
                     late = in;
         if (late) {
@@ -1321,12 +1318,9 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
             if (res * batch_ctas_per_sm() > capacity() - held()) {
                 order.clear();
             } else {
-                const bool taken = launch_resident(b, free_group(), late, res, &st);
-                if (st) return st;
-                if (taken) {
-                    std::vector<Instance*>& list = ready[{late->prec, N}];
-                    list.erase(std::find(list.begin(), list.end(), late));
-                }
+                if ((st = launch_resident(b, free_group(), late, res))) return st;
+                std::vector<Instance*>& list = ready[{late->prec, N}];
+                list.erase(std::find(list.begin(), list.end(), late));
             }
         }
         for (auto& o : order) {
@@ -1337,18 +1331,10 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
             if (res > 0) {
                 // per member, as many as find their SMs free; the others
                 // wait for a step in which they do
-                std::vector<Instance*> rest;
-                for (Instance* in : list) {
-                    if (in->no_resident) {
-                        rest.push_back(in);
-                        continue;
-                    }
-                    if (res * batch_ctas_per_sm() > capacity() - held()) continue;
-                    if (!launch_resident(b, free_group(), in, res, &st)) rest.push_back(in);
-                    if (st) return st;
-                }
-                if (rest.empty()) continue;
-                list = rest;
+                for (Instance* in : list)
+                    if (res * batch_ctas_per_sm() <= capacity() - held())
+                        if ((st = launch_resident(b, free_group(), in, res))) return st;
+                continue;
             }
             if (launched_level(list[0])) {
                 if ((st = launch_group_launched(b, free_group(), list))) return st;

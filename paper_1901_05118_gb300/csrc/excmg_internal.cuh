@@ -103,7 +103,6 @@ cudaError_t launch_bicg_persistent(double* x, double* r, double* rs, double* p, 
 int resident_ctas(int n, int max_ctas);
 int resident_batch_limit(int n);
 size_t resident_slot_bytes();
-size_t resident_bytes(int n);   // slots and node words
 template <typename T>
 cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
                                  void* slots, void* node_words, cudaStream_t s, bool elide, int max_ctas);

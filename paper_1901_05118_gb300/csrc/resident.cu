@@ -61,7 +61,6 @@ unsigned next_serial() {
 }  // namespace
 
 size_t resident_slot_bytes() { return (kResWords * sizeof(ulonglong2) + 255) / 256 * 256; }
-size_t resident_bytes(int n) { return resident_slot_bytes() + node_count(n) * sizeof(ulonglong2); }
 
 namespace {
 template <typename T>

@@ -109,3 +109,24 @@ def test_mixed_solves_under_the_least_budget(n, nc, kind):
     want = solve(0)[0]
     for got in solve(least_budget(solve, 1 << 14, 20 * 8 * (n + 1) ** 3 + (1 << 25)), times=3):
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_batch_levels_on_chip_take_no_memory_beyond_the_instances(precision):
+    """Once its group records exist, a batch whose levels run on chip holds what its instances
+    were admitted with (free memory is counted in steps of up to 2 MB)."""
+    n, nc, kind = 80, 5, 2
+    big, small = ([dev(a) for a in P.exp_sum().data(m, kind)] for m in (n, 20))
+    batch = B.Batch(max_instances=8)
+    for _ in range(4):   # the records and the direct solves' tables
+        batch.submit(20, nc, kind, *small, 1e-8, precision=precision)
+    batch.run()
+    ids = [batch.submit(n, nc, kind, *big, 1e-8, precision=precision)[0] for _ in range(4)]
+    torch.cuda.synchronize()
+    before = least = torch.cuda.mem_get_info()[0]
+    while not all(batch.query(k)["done"] for k in ids):
+        batch.step()
+        least = min(least, torch.cuda.mem_get_info()[0])
+    assert before - least <= 2 << 20
+    assert all(batch.query(k)["status"] == 0 for k in ids)
+    batch.close()
