@@ -7,18 +7,17 @@
 // true residual, Bi-CG call (or FP32 correction solve and FP64 update),
 // until the level's tolerance (or the stagnation rule) is met, and finally
 // EXP_true.  The Bi-CG iterations (Alg. 2, M = I, r*_0 = r_0) of the
-// instances waiting for them run per level group -- instances of one
-// precision at one grid size -- each group on its own stream:
+// instances waiting for them run in launches of their own, each on its own stream:
 //  * grids up to 81^3 (both precisions): one launch of the resident kernel
 //    (resident.cuh) per member, on as many CTAs as resident_batch_limit
 //    gives that grid, side by side as far as the GPU's SMs go;
-//  * FP32 correction solves above 81^3: one cooperative launch for
-//    all members; CTAs take operator tiles and vector chunks from every
+//  * FP32 correction solves above 81^3: one cooperative launch for all
+//    members of a level group (instances at one grid size); CTAs take operator tiles and vector chunks from every
 //    member, members advance in lock step one iteration per grid-barrier
 //    round, and each member's scalars are formed by the CTA that completes
 //    its last tile / chunk;
-//  * FP64 grids above 81^3 (launched mode): per member and round the single
-//    solver's fused operator and update kernels with the member's own state.
+//  * FP64 grids above 81^3 (launched mode): per member the single solver's
+//    fused operator and update kernels with the member's own state.
 // Instances can be submitted at any time (the engine admits them against
 // its device-memory budget) and leave as soon as they are done, so the
 // batch continuously refills: the same engine serves the fixed batch and
@@ -701,11 +700,14 @@ int launch_group(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instan
     return EXCMG_OK;
 }
 
-// FP64 levels above the cooperative kernel's range run in launched mode:
-// per member and iteration the single solver's two kernels (the operator
-// launch with the direction update folded in, then the update), with the
-// member's own state and partial sums, so that a large level moves its
-// bytes as fast as in a single solve.
+// FP64 levels that do not fit on chip run in launched mode: per iteration the
+// single solver's two kernels (the operator launch with the direction update
+// folded in, then the update), with the member's own state and partial sums.
+// Every member has a stream of its own: a kernel on 96^3 leaves part of the GPU idle and
+// the tail of one on 128^3 does, which another member's kernel fills.  (Members
+// that became ready together used to share a stream, one kernel after the other, and
+// stay together from then on: six requests of 96^3 took 263 to 365 ms by chance of their
+// timing, 201 so; four of 112^3 398 and 262, four of 128^3 649 and 457 ms.)
 bool launched_level(const Instance* in) { return in->prec == EXCMG_PRECISION_FP64; }
 
 // One launch of the resident kernel for instance `in`: up to b->inner_chunk
@@ -747,58 +749,50 @@ int launch_resident(excmg_batch* b, excmg_batch::Group& g, Instance* in, int cta
     return EXCMG_OK;
 }
 
-int launch_group_launched(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instance*>& list) {
+int launch_member(excmg_batch* b, excmg_batch::Group& g, Instance* in) {
     int st = group_init(b, g);
     if (st) return st;
     cudaStream_t s = g.stream;
-    const int K = b->launched_rounds;
-    long long nl = 0;
+    const int K = b->launched_rounds, N = in->nc << in->level;
+    BicgState* bs = b->d_bstate + in->slot;
+    double* part = b->d_bpart + (size_t)in->slot * kMaxPartials;
     cudaError_t e = cudaStreamWaitEvent(s, b->host_ready, 0);
     if (e == cudaSuccess) e = cudaEventRecord(g.start, s);
     for (int k = 0; k < K && e == cudaSuccess; ++k) {
-        for (Instance* in : list) {
-            if (e != cudaSuccess) break;
-            const int N = in->nc << in->level;
-            BicgState* bs = b->d_bstate + in->slot;
-            double* part = b->d_bpart + (size_t)in->slot * kMaxPartials;
-            double* pc = in->dir_in_p2 ? in->p2_64 : in->p64;
-            double* psc = in->dir_in_p2 ? in->ps2_64 : in->ps64;
-            if (in->launched_k == 0) {
-                // p_0 = r_0: the operator pair on the fused schedule's grid
-                e = launch_bicg_stencil_pair(pc, in->q64, psc, nullptr, N, in->bc, part, bs, s);
-            } else {
-                double* pn = in->dir_in_p2 ? in->p64 : in->p2_64;
-                double* psn = in->dir_in_p2 ? in->ps64 : in->ps2_64;
-                e = launch_bicg_stencil_pair_dir(in->res, in->rs64, pc, psc, pn, psn, in->q64, nullptr, N, in->bc,
-                                                 part, bs, s);
-                in->dir_in_p2 = !in->dir_in_p2;
-                pc = pn;
-            }
-            if (e == cudaSuccess)
-                e = launch_bicg_update(in->u[in->level], pc, in->res, in->q64, in->rs64, nullptr, node_count(N), part,
-                                       bs, s);
-            ++in->launched_k;
-            nl += 2;
+        double* pc = in->dir_in_p2 ? in->p2_64 : in->p64;
+        double* psc = in->dir_in_p2 ? in->ps2_64 : in->ps64;
+        if (in->launched_k == 0) {
+            // p_0 = r_0: the operator pair on the fused schedule's grid
+            e = launch_bicg_stencil_pair(pc, in->q64, psc, nullptr, N, in->bc, part, bs, s);
+        } else {
+            double* pn = in->dir_in_p2 ? in->p64 : in->p2_64;
+            double* psn = in->dir_in_p2 ? in->ps64 : in->ps2_64;
+            e = launch_bicg_stencil_pair_dir(in->res, in->rs64, pc, psc, pn, psn, in->q64, nullptr, N, in->bc, part,
+                                             bs, s);
+            in->dir_in_p2 = !in->dir_in_p2;
+            pc = pn;
         }
-    }
-    bnote(b, nl);
-    for (Instance* in : list)
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(b->h_bstate + in->slot, b->d_bstate + in->slot, sizeof(BicgState),
-                                cudaMemcpyDeviceToHost, s);
+            e = launch_bicg_update(in->u[in->level], pc, in->res, in->q64, in->rs64, nullptr, node_count(N), part, bs,
+                                   s);
+        ++in->launched_k;
+    }
+    bnote(b, 2LL * K);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->h_bstate + in->slot, bs, sizeof(BicgState), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaEventRecord(g.done, s);
-    if (e != cudaSuccess) return bcuda(b, e, "launched batch group");
+    if (e != cudaSuccess) return bcuda(b, e, "launched batch member");
     *g.h_active = 0;
     *g.h_rounds = K;
     g.busy = true;
     g.launched = true;
     g.prec = EXCMG_PRECISION_FP64;
-    g.n = list[0]->nc << list[0]->level;
+    g.n = N;
     g.ctas = 0;
     g.sm_share = 0;
     g.cand = -1;
-    g.members = list;
-    for (Instance* in : list) in->in_flight = true;
+    g.members.assign(1, in);
+    in->in_flight = true;
     return EXCMG_OK;
 }
 
@@ -1337,7 +1331,8 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
                 continue;
             }
             if (launched_level(list[0])) {
-                if ((st = launch_group_launched(b, free_group(), list))) return st;
+                for (Instance* in : list)
+                    if ((st = launch_member(b, free_group(), in))) return st;
                 continue;
             }
             const int cap = capacity() - held();
