@@ -30,6 +30,7 @@
 #include <thread>
 #include <vector>
 
+#include "batch_places.h"
 #include "excmg_internal.cuh"
 #include "grid_sync.cuh"
 #include "march_f32.cuh"
@@ -431,7 +432,6 @@ struct excmg_batch {
         cudaEvent_t start = nullptr, done = nullptr;
         bool busy = false;
         bool launched = false;   // members' states are in the single solver's layout (launched mode, resident kernel)
-        int sm_share = 0;        // CTA places held while busy, in CTAs of the cooperative FP32 kernel
         void* slots = nullptr;   // slot words of the resident kernel
         int prec = 0, n = 0, ctas = 0, cand = -1;
         std::vector<Instance*> members;
@@ -585,8 +585,13 @@ constexpr int kTuneItems[kTuneCands] = {1, 2, 4, 8, 16};   // tiles or chunks pe
 // CTAs per instance of candidate c for an instance with W work items.
 int tune_cpi(int W, int c) { return (W + kTuneItems[c] - 1) / kTuneItems[c]; }
 
-// CTA places of the GPU, in CTAs of the cooperative FP32 kernel.
-int capacity() { return device_sms() * batch_ctas_per_sm(); }
+// What the launches under way hold of the GPU's SMs.
+SmPlaces places(const excmg_batch* b) {
+    SmPlaces p{device_sms(), batch_ctas_per_sm(), 0, 0};
+    for (const auto& g : b->groups)
+        if (g.busy) (g.launched ? p.resident : p.coop) += g.ctas;   // (0 for a launched member)
+    return p;
+}
 
 // The group record's stream, events and fixed tables (made once).
 int group_init(excmg_batch* b, excmg_batch::Group& g) {
@@ -693,7 +698,6 @@ int launch_group(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instan
     g.prec = EXCMG_PRECISION_MIXED;
     g.n = list.empty() ? 0 : (list[0]->nc << list[0]->level);
     g.ctas = ctas;
-    g.sm_share = ctas;
     g.cand = cand;
     g.members = list;
     for (Instance* in : list) in->in_flight = true;
@@ -742,7 +746,6 @@ int launch_resident(excmg_batch* b, excmg_batch::Group& g, Instance* in, int cta
     g.prec = in->prec;
     g.n = N;
     g.ctas = ctas;
-    g.sm_share = ctas * batch_ctas_per_sm();   // one CTA fills an SM
     g.cand = -1;
     g.members.assign(1, in);
     in->in_flight = true;
@@ -789,21 +792,20 @@ int launch_member(excmg_batch* b, excmg_batch::Group& g, Instance* in) {
     g.prec = EXCMG_PRECISION_FP64;
     g.n = N;
     g.ctas = 0;
-    g.sm_share = 0;
     g.cand = -1;
     g.members.assign(1, in);
     in->in_flight = true;
     return EXCMG_OK;
 }
 
-excmg_ctx::BatchTune& tune_of(excmg_batch* b, int prec, int n) {
+excmg_ctx::BatchTune& tune_of(excmg_batch* b, int n) {
     auto& table = b->ctx->batch_tune;
-    auto it = table.find({prec, n});
+    auto it = table.find(n);
     if (it == table.end()) {
         excmg_ctx::BatchTune t;
         for (int k = 0; k < 8; ++k) t.ms[k] = t.cta_ms[k] = -1.0;
         t.settled = false;
-        it = table.emplace(std::make_pair(prec, n), t).first;
+        it = table.emplace(n, t).first;
     }
     return it->second;
 }
@@ -855,7 +857,7 @@ int harvest(excmg_batch* b, excmg_batch::Group& g) {
     }
     if (g.cand >= 0 && *g.h_rounds > 0) {
         if (ms >= 0.f) {
-            excmg_ctx::BatchTune& t = tune_of(b, g.prec, g.n);
+            excmg_ctx::BatchTune& t = tune_of(b, g.n);
             const double per_round = (double)ms / (double)*g.h_rounds;
             const double c = per_round * g.ctas / (double)g.members.size();
             if (t.ms[g.cand] < 0.0 || per_round < t.ms[g.cand]) {
@@ -901,8 +903,8 @@ int harvest(excmg_batch* b, excmg_batch::Group& g) {
 // CTAs for a group of m instances of grid size n with W work items each:
 // the tuner's next candidate while it is still trying, else its choice; *cand
 // the candidate index.
-int group_ctas(excmg_batch* b, int prec, int n, int W, int m, int* cand) {
-    excmg_ctx::BatchTune& t = tune_of(b, prec, n);
+int group_ctas(excmg_batch* b, int n, int W, int m, int* cand) {
+    excmg_ctx::BatchTune& t = tune_of(b, n);
     int pick = -1;
     if (!t.settled) {
         for (int k = 0; k < kTuneCands && pick < 0; ++k) {
@@ -1268,10 +1270,9 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
             in->call_iter = 0;
         }
     }
-    // 3. one cooperative launch per level group of instances waiting for
-    // Bi-CG iterations, largest groups first, within the device's
-    // co-resident capacity (so that concurrent groups never wait on each
-    // other's CTAs)
+    // 3. launches for the instances waiting for Bi-CG iterations, largest
+    // groups (of one precision at one grid size) first, as far as their CTAs
+    // find places beside those under way (batch_places.h)
     std::map<std::pair<int, int>, std::vector<Instance*>> ready;
     for (Instance* in : b->live)
         if (!in->in_flight && in->phase == kInner) ready[{in->prec, in->nc << in->level}].push_back(in);
@@ -1288,63 +1289,61 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
             b->groups.emplace_back();
             return b->groups.back();
         };
-        auto held = [&]() {
-            int used = 0;
-            for (auto& g : b->groups)
-                if (g.busy) used += g.sm_share;
-            return used;
+        // per member on chip, as many as find their SMs free; the others wait
+        // for a step in which they do
+        auto start_on_chip = [&](Instance* in, int ctas) -> bool {
+            if (!on_chip_fits(places(b), ctas)) return false;
+            st = launch_resident(b, free_group(), in, ctas);
+            return true;
         };
-        // An on-chip level that needs most of the SMs could be kept out for
-        // good by a stream of small ones that take each SM as it comes free.
-        // So the one that has waited longest, if longer than kOverdue (some
-        // 2000 iterations at 64^3), goes first, and while it does not fit
-        // nothing else is started.  Eight mixed requests take as long as
+        // one cooperative launch for a group's FP32 correction solves
+        auto start_group = [&](const std::vector<Instance*>& list) -> bool {
+            int cand = -1, units = 0, chunks = 0;
+            geometry(list[0], 0, &units, &chunks);
+            const int want = group_ctas(b, list[0]->nc << list[0]->level, units > chunks ? units : chunks,
+                                        (int)list.size(), &cand);
+            const int ctas = coop_share(places(b), want);
+            if (ctas == 0) return false;
+            // (not the candidate's shape: not a tuning sample)
+            st = launch_group(b, free_group(), list, ctas, ctas == want ? cand : -1);
+            return true;
+        };
+        auto on_chip = [&](int n) { return resident_ctas(n, resident_batch_limit(n)); };
+        // What needs many SMs at once could be kept out for good by a stream of
+        // small levels that take each SM as it comes free.  So the instance that has
+        // waited longest, if longer than kOverdue (some 2000 iterations at 64^3), goes
+        // first (a cooperative group's with its group), and while it finds no place nothing
+        // else is started.  Eight mixed requests take as long as
         // without the rule, and as long with small grids always first.
         constexpr double kOverdue = 0.02;
         Instance* late = nullptr;
         for (auto& kv : ready)
             for (Instance* in : kv.second)
-                if (resident_ctas(kv.first.second, resident_batch_limit(kv.first.second)) > 0 &&
-                    now_s() - in->t_ready > kOverdue && (!late || in->t_ready < late->t_ready))
+                if ((on_chip(kv.first.second) > 0 || !launched_level(in)) && now_s() - in->t_ready > kOverdue &&
+                    (!late || in->t_ready < late->t_ready))
                     late = in;
         if (late) {
-            const int N = late->nc << late->level, res = resident_ctas(N, resident_batch_limit(N));
-            if (res * batch_ctas_per_sm() > capacity() - held()) {
-                order.clear();
-            } else {
-                if ((st = launch_resident(b, free_group(), late, res))) return st;
-                std::vector<Instance*>& list = ready[{late->prec, N}];
-                list.erase(std::find(list.begin(), list.end(), late));
-            }
+            const int N = late->nc << late->level, ctas = on_chip(N);
+            std::vector<Instance*>& list = ready[{late->prec, N}];
+            if (!(ctas > 0 ? start_on_chip(late, ctas) : start_group(list))) order.clear();
+            else if (ctas > 0) list.erase(std::find(list.begin(), list.end(), late));
+            else list.clear();
+            if (st) return st;
         }
         for (auto& o : order) {
-            const auto key = o.second;
-            std::vector<Instance*>& list = ready[key];
+            const std::vector<Instance*>& list = ready[o.second];
             if (list.empty()) continue;
-            const int res = resident_ctas(key.second, resident_batch_limit(key.second));
-            if (res > 0) {
-                // per member, as many as find their SMs free; the others
-                // wait for a step in which they do
-                for (Instance* in : list)
-                    if (res * batch_ctas_per_sm() <= capacity() - held())
-                        if ((st = launch_resident(b, free_group(), in, res))) return st;
-                continue;
+            const int ctas = on_chip(o.second.second);
+            if (ctas == 0 && !launched_level(list[0])) {
+                (void)start_group(list);
+            } else {
+                for (Instance* in : list) {
+                    if (ctas > 0) (void)start_on_chip(in, ctas);
+                    else st = launch_member(b, free_group(), in);
+                    if (st) return st;
+                }
             }
-            if (launched_level(list[0])) {
-                for (Instance* in : list)
-                    if ((st = launch_member(b, free_group(), in))) return st;
-                continue;
-            }
-            const int cap = capacity() - held();
-            if (cap < 1) continue;
-            int cand = -1, units = 0, chunks = 0;
-            geometry(list[0], 0, &units, &chunks);
-            int ctas = group_ctas(b, key.first, key.second, units > chunks ? units : chunks, (int)list.size(), &cand);
-            if (ctas > cap) {
-                ctas = cap;
-                cand = -1;   // not the candidate's shape: not a tuning sample
-            }
-            if ((st = launch_group(b, free_group(), list, ctas, cand))) return st;
+            if (st) return st;
         }
     }
     // 4. finals (EXP_true)

@@ -143,3 +143,30 @@ def test_batch_admission_respects_the_budget():
     assert batch.bytes == 0
     assert batch.submit(n, nc, 1, f, g1, g2, 1e-10) is not None  # room again
     batch.run()
+
+
+def test_correction_solves_above_the_on_chip_grids_beside_small_requests():
+    """Mixed-precision requests whose finest level takes cooperative groups beside a stream of
+    small on-chip ones: all end, each level at its tolerance, and the large ones give the bits
+    that they give alone."""
+    tol = 1e-8
+    _, big = data(96, 2, "exp_sum")
+    _, small = data(32, 2, "random_sines:1")
+    alone = B.Batch(max_instances=2)
+    _, want = alone.submit(96, 6, 2, *big, tol, precision="mixed")
+    alone.run()
+    batch = B.Batch(max_instances=20)
+    large = [batch.submit(96, 6, 2, *big, tol, precision="mixed") for _ in range(2)]
+    live = [batch.submit(32, 4, 2, *small, tol, precision="fp64")[0] for _ in range(12)]
+    done = 0
+    while not all(batch.query(k)["done"] for k, _ in large) and done < 2000:
+        batch.step()
+        left = [k for k in live if not batch.query(k)["done"]]
+        done += len(live) - len(left)
+        live = left + [batch.submit(32, 4, 2, *small, tol, precision="fp64")[0] for _ in range(12 - len(left))]
+    batch.run()
+    for k, u in large:
+        q = batch.query(k)
+        assert q["done"] and q["status"] == 0
+        assert all(s["relres"] <= tol for s in q["stats"][2:])
+        assert torch.equal(u, want)
