@@ -395,14 +395,17 @@ int excmg2d_solve(excmg_ctx *ctx, int n_finest, int n_coarsest, int bc_kind, con
 /* Failure-path self-test (the paper has no counterpart): makes one of the
  * library's bounded device-side waits run out on purpose -- without a fault,
  * trap or hang -- so that the path that reports EXCMG_ERR_TIMEOUT can be
- * tested.  which = 0 (the only wait kind): the grid barrier of the
+ * tested.  which = 0: the grid barrier of the
  * cooperative kernels; a cooperative launch of 8 CTAs waits for a ninth
  * arrival that never comes, and each CTA gives up after `limit` polls (at
- * least 32 ns each).  1 <= limit <= 10^8.
- * Returns EXCMG_ERR_TIMEOUT when the wait gave up as designed, EXCMG_OK if it
- * did not (the mechanism failed), EXCMG_ERR_ARG, or EXCMG_ERR_CUDA.  Uses
- * fixed device memory (allocates nothing), runs on the legacy default stream
- * and returns when done. */
+ * least 32 ns each).  which = 1, 2: the on-chip Bi-CG kernel on 9^3 as 3 of its
+ * 4 CTAs, whose first exchange (1), or second exchange and wait for r (2),
+ * misses the fourth.  1 <= limit <= 10^8.
+ * Returns EXCMG_ERR_TIMEOUT when the wait gave up as designed, another status
+ * if it did not (the mechanism failed; EXCMG_OK for which = 0), EXCMG_ERR_ARG,
+ * EXCMG_ERR_OOM or EXCMG_ERR_CUDA.  which = 0 uses fixed device memory
+ * (allocates nothing), 1 and 2 allocate 0.3 MB for the call; runs on the legacy
+ * default stream and returns when done. */
 int excmg_selftest_wait_timeout(int which, long long limit);
 
 #ifdef __cplusplus

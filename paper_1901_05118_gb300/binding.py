@@ -155,9 +155,10 @@ def launch_count() -> int:
 
 def selftest_wait_timeout(which: str, limit: int) -> int:
     """Make a bounded device wait run out on purpose ('barrier': the grid
-    barrier of the cooperative kernels, limit in polls).  Returns the library
+    barrier of the cooperative kernels; 'exchange 1', 'exchange 2': those of the
+    on-chip Bi-CG kernel; limit in polls).  Returns the library
     status (-7, EXCMG_ERR_TIMEOUT, when it gave up)."""
-    return int(_lib.excmg_selftest_wait_timeout({"barrier": 0}[which], int(limit)))
+    return int(_lib.excmg_selftest_wait_timeout({"barrier": 0, "exchange 1": 1, "exchange 2": 2}[which], int(limit)))
 
 
 # ----------------------------------------------------------------- checks

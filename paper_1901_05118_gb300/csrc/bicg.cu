@@ -325,11 +325,7 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     if (iters_out) *iters_out = h.iter;
     const double rn = sqrt(h.rr);
     if (relres_out) *relres_out = bnorm > 0.0 ? rn / bnorm : rn;
-    if (!std::isfinite(h.rr)) return ctx_fail(ctx, EXCMG_ERR_NAN, "Bi-CG residual is not finite");
-    if (h.status == kBreakdown) return ctx_fail(ctx, EXCMG_ERR_BREAKDOWN, "Bi-CG breakdown");
-    if (h.status == kTimeout) return ctx_fail(ctx, EXCMG_ERR_TIMEOUT, "grid barrier of the cooperative Bi-CG gave up");
-    if (h.status == kCapped) return EXCMG_ERR_NOCONV;
-    return EXCMG_OK;
+    return ctx_bicg_outcome(ctx, "Bi-CG");
 }
 
 }  // namespace excmg

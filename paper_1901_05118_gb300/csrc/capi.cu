@@ -79,6 +79,14 @@ int ctx_cuda(excmg_ctx* ctx, cudaError_t err, const char* what) {
     return ctx_fail(ctx, EXCMG_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(err));
 }
 
+int ctx_bicg_outcome(excmg_ctx* ctx, const char* what) {
+    const int st = bicg_outcome(*ctx->host_state);
+    if (st == EXCMG_OK || st == EXCMG_ERR_NOCONV) return st;
+    return ctx_fail(ctx, st, std::string(what) + (st == EXCMG_ERR_TIMEOUT ? ": a grid-wide wait gave up"
+                                                  : st == EXCMG_ERR_NAN   ? " residual is not finite"
+                                                                          : " breakdown"));
+}
+
 cudaGraphExec_t ctx_chunk_graph(excmg_ctx* ctx, const std::vector<uintptr_t>& key) {
     auto it = ctx->chunk_graphs.find(key);
     return it == ctx->chunk_graphs.end() ? nullptr : it->second;

@@ -472,12 +472,7 @@ int bicg2d_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, d
     if (iters_out) *iters_out = h.iter;
     const double rn = sqrt(h.rr);
     if (relres_out) *relres_out = bnorm > 0.0 ? rn / bnorm : rn;
-    if (!std::isfinite(h.rr)) return ctx_fail(ctx, EXCMG_ERR_NAN, "2D Bi-CG residual is not finite");
-    if (h.status == kBreakdown) return ctx_fail(ctx, EXCMG_ERR_BREAKDOWN, "2D Bi-CG breakdown");
-    if (h.status == kTimeout)
-        return ctx_fail(ctx, EXCMG_ERR_TIMEOUT, "an exchange of the cooperative 2D Bi-CG gave up");
-    if (h.status == kCapped) return EXCMG_ERR_NOCONV;
-    return EXCMG_OK;
+    return ctx_bicg_outcome(ctx, "2D Bi-CG");
 }
 
 cudaError_t launch_exp_finite2d(double* w, const double* u1, const double* u0, double* W, int nf, cudaStream_t s) {

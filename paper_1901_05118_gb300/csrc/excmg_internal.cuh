@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 #include <map>
@@ -46,6 +47,14 @@ struct BicgState {
 };
 static_assert(sizeof(BicgState) % 8 == 0, "read back in 8-byte words");
 enum { kRunning = 0, kConverged = 1, kCapped = 2, kBreakdown = 3, kTimeout = 4 };
+// What a Bi-CG call that ended in state h returns: a wait that gave up first, as
+// the sums of such a call mean nothing.
+inline int bicg_outcome(const BicgState& h) {
+    if (h.status == kTimeout) return EXCMG_ERR_TIMEOUT;
+    if (!std::isfinite(h.rr)) return EXCMG_ERR_NAN;
+    if (h.status == kBreakdown) return EXCMG_ERR_BREAKDOWN;
+    return h.status == kCapped ? EXCMG_ERR_NOCONV : EXCMG_OK;
+}
 
 // ------------------------------------------------------------- kernels
 // Stencil (eq. (method1) + reflections): y = A u, or y = b - A u when b is
@@ -107,6 +116,10 @@ template <typename T>
 cudaError_t launch_bicg_resident(T* x, T* r, T* rs, T* p, T* ps, int n, int bc_kind, int iters, BicgState* st,
                                  void* slots, void* node_words, cudaStream_t s, bool elide, int max_ctas);
 constexpr int kResidentMaxN = 81;   // eight nodes per thread on 152 SMs
+// A resident launch whose last CTA never comes: its first exchange (1), or, with that
+// CTA's word of the first in place, its second and the r of its nodes (2), gives up
+// after `limit` polls.  Returns what the call would return (selftest.cu).
+int resident_wait_selftest(int exchange, long long limit);
 // The 2D problem's form, on grids that fit on chip with four nodes per thread.
 constexpr int kPersistentMaxN2d = 512;
 int resident2d_ctas(int n);
@@ -255,6 +268,8 @@ cudaStream_t ctx_capture_stream(excmg_ctx* ctx);
 // Workspace helpers (capi.cu).
 int ctx_fail(excmg_ctx* ctx, int status, const std::string& msg);
 int ctx_cuda(excmg_ctx* ctx, cudaError_t err, const char* what);
+// bicg_outcome of the state read back, with its message where that is an error.
+int ctx_bicg_outcome(excmg_ctx* ctx, const char* what);
 // Enqueue on ctx's stream a copy of `bytes` (a multiple of 8) from device
 // memory to one of the context's mapped host mirrors (host_state or
 // host_scalar), written by a kernel; the caller synchronises the stream.

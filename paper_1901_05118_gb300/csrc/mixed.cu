@@ -255,11 +255,8 @@ static int bicg32_run(excmg_ctx* ctx, int n, int bc_kind, const float* b32, floa
         if (err != cudaSuccess) return ctx_cuda(ctx, err, "FP32 Bi-CG iteration");
     }
     if (iters_out) *iters_out = ctx->host_state->iter;
-    if (!std::isfinite(ctx->host_state->rr)) return ctx_fail(ctx, EXCMG_ERR_NAN, "FP32 Bi-CG residual is not finite");
-    if (ctx->host_state->status == kBreakdown) return ctx_fail(ctx, EXCMG_ERR_BREAKDOWN, "FP32 Bi-CG breakdown");
-    if (ctx->host_state->status == kTimeout)
-        return ctx_fail(ctx, EXCMG_ERR_TIMEOUT, "an exchange of the cooperative FP32 Bi-CG gave up");
-    return EXCMG_OK;
+    const int out = ctx_bicg_outcome(ctx, "FP32 Bi-CG");
+    return out == EXCMG_ERR_NOCONV ? EXCMG_OK : out;   // a capped correction is as good as another
 }
 
 int mixed_level_solve(excmg_ctx* ctx, int n, int bc_kind, const double* fh, double* u, double fnorm, double eps,

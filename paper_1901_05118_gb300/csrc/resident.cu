@@ -3,8 +3,10 @@
 #include "resident.cuh"
 
 #include <atomic>
+#include <cstring>
 #include <map>
 #include <mutex>
+#include <vector>
 
 namespace excmg {
 namespace {
@@ -97,5 +99,61 @@ template cudaError_t launch_bicg_resident<double>(double*, double*, double*, dou
                                                   BicgState*, void*, void*, cudaStream_t, bool, int);
 template cudaError_t launch_bicg_resident<float>(float*, float*, float*, float*, float*, int, int, int, BicgState*,
                                                  void*, void*, cudaStream_t, bool, int);
+
+int resident_wait_selftest(int exchange, long long limit) {
+    constexpr int n = 9;
+    const ResidentGeom g = resident_geometry(n, 8);   // four bricks of 4 x 4 x 8
+    if (g.ctas < 2 || g.np != 1) return EXCMG_ERR_CUDA;
+    const size_t nodes = node_count(n), slots = resident_slot_bytes();
+    // slot words, node words, x, r, r*, p, p*, state
+    std::vector<unsigned char> host(slots + nodes * 16 + 5 * nodes * 8 + sizeof(BicgState), 0);
+    unsigned char* dev = nullptr;
+    if (cudaMalloc(&dev, host.size()) != cudaSuccess) {
+        cudaGetLastError();
+        return EXCMG_ERR_OOM;
+    }
+    const unsigned serial = next_serial();
+    unsigned long long one;
+    const double v = 1.0;
+    memcpy(&one, &v, 8);
+    unsigned long long* const word = (unsigned long long*)host.data();
+    for (int c = 0; exchange == 2 && c < kResCopies; ++c) {
+        // the missing CTA's sum of exchange 1, and a NaN where that of exchange 2 would be
+        unsigned long long* const w1 = word + 2 * ((size_t)c * kResMaxCtas + g.ctas - 1);
+        unsigned long long* const w2 = w1 + 2 * (size_t)kResCopies * kResMaxCtas;
+        w1[0] = one;
+        w1[1] = (unsigned long long)serial << 32;
+        w2[0] = w2[1] = ~0ull;
+    }
+    double* const vec = (double*)(host.data() + slots + nodes * 16);
+    for (size_t t = 0; t < 5 * nodes; ++t) vec[t] = 1.0;
+    BicgState st{};
+    st.rho = st.rr = st.bnorm = 1.0;
+    st.beta = 0.5;
+    st.iter = 1;   // under way: rr is the kernel's to write
+    st.max_iter = 8;
+    memcpy(host.data() + host.size() - sizeof st, &st, sizeof st);
+    double* const dv = (double*)(dev + slots + nodes * 16);
+    BicgState* const ds = (BicgState*)(dv + 5 * nodes);
+    ResidentInst<double> in{dv,      dv + nodes, dv + 2 * nodes, dv + 3 * nodes, dv + 4 * nodes, ds, (ulonglong2*)dev,
+                            (ulonglong2*)(dev + slots), n, 1};
+    const void* fn = resident_fn<double, 3, false>(g.np);
+    (void)kernel_occupancy(fn, kResThreads, kResSmemBytes);
+    int iters = 8;
+    unsigned tag = serial;
+    void* args[] = {&in, (void*)&g, &iters, &tag, &limit};
+    cudaError_t e = cudaMemcpy(dev, host.data(), host.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaLaunchCooperativeKernel(fn, dim3(g.ctas - 1), dim3(kResThreads), args, (size_t)((g.tile + 1) & ~1) * 8,
+                                        nullptr);
+    note_launches(1);
+    if (e == cudaSuccess) e = cudaMemcpy(&st, ds, sizeof st, cudaMemcpyDeviceToHost);
+    cudaFree(dev);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return EXCMG_ERR_CUDA;
+    }
+    return bicg_outcome(st);
+}
 
 }  // namespace excmg

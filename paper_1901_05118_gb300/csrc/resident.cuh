@@ -593,7 +593,8 @@ resident_bicg_kernel(const ResidentInst<T> in, const ResidentGeom g, int iters,
     if (cta == 0 && tid == 0) {
         if (gave_up || *err == serial) code = kTimeout;
         st->rho = rho;
-        st->rr = iter > 0 ? rr : st->rr;
+        // (the sum of an exchange that gave up has words of other exchanges in it)
+        if (iter > 0 && code != kTimeout) st->rr = rr;
         st->alpha = alpha;
         st->beta = beta;
         st->sigma = sigma;

@@ -1,8 +1,9 @@
 // Failure-path self-test: make one of the library's bounded device-side
 // waits run out on purpose, without a fault, trap or hang, so that the path
 // that turns a wait that gave up into EXCMG_ERR_TIMEOUT can be tested.  The
-// wait is the one the cooperative kernels use (grid_sync); only the arrival
-// it waits for is one that nothing makes.
+// waits are those of the cooperative kernels (grid_sync) and of the on-chip
+// kernels' exchanges (resident.cuh); only the arrival they wait for is one that
+// nothing makes.
 #include "excmg_internal.cuh"
 #include "grid_sync.cuh"
 
@@ -29,7 +30,8 @@ __global__ void barrier_timeout_kernel(GridBarrier gb) {
 using namespace excmg;
 
 extern "C" int excmg_selftest_wait_timeout(int which, long long limit) {
-    if (which != 0 || limit < 1 || limit > 100000000ll) return EXCMG_ERR_ARG;
+    if (which < 0 || which > 2 || limit < 1 || limit > 100000000ll) return EXCMG_ERR_ARG;
+    if (which > 0) return resident_wait_selftest(which, limit);
     void* words = nullptr;
     void* status = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&words, g_selftest_barrier);

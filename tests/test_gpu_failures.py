@@ -102,3 +102,21 @@ def test_bounded_waits_give_up():
     assert B.selftest_wait_timeout("barrier", 20000) == ERR_TIMEOUT
     assert B.selftest_wait_timeout("barrier", 20000) == ERR_TIMEOUT   # and again: nothing left behind
     still_works(B.Context())
+
+
+@pytest.mark.parametrize("which", ["exchange 1", "exchange 2"])
+def test_bounded_waits_of_the_on_chip_kernel_give_up(which):
+    """An exchange that misses one CTA gives up after 20000 polls in every other
+    one and is reported as EXCMG_ERR_TIMEOUT, also where the words it did not get
+    hold a NaN (exchange 2); the GPU stays usable."""
+    assert B.selftest_wait_timeout(which, 20000) == ERR_TIMEOUT
+    assert B.selftest_wait_timeout(which, 20000) == ERR_TIMEOUT
+    still_works(B.Context())
+
+
+@pytest.mark.parametrize("n", [88, 100])
+def test_iteration_cap_on_launched_kernels(n):
+    ctx = B.Context()
+    x = torch.zeros((n + 1,) * 3, dtype=torch.float64, device=DEV)
+    it, rel, rc = B.bicg_solve(B.Level(n, 1, ctx), dev(P.random_field(n, 8)), x, 1e-14, 1)
+    assert rc == ERR_NOCONV and it == 1 and rel > 1e-14
