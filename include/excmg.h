@@ -161,8 +161,9 @@ const char *excmg_last_error(const excmg_ctx *ctx);
 
 /* Instrumentation.  excmg_launch_count: kernel launches the library has
  * made in this process (all contexts).  excmg_ctx_profile(ctx, 1) makes the
- * context time every operator launch inside Bi-CG with CUDA events on its
- * stream (and clears earlier records); excmg_ctx_profile_read returns, for
+ * context time every operator launch inside Bi-CG, on grids above 64^3, with
+ * CUDA events on its stream (and clears earlier records); while it is on, grids
+ * up to 81^3 run on the launched kernels from 65^3 on; excmg_ctx_profile_read returns, for
  * grids with n intervals, the summed device time (ms), the number of
  * operator launches timed since and (bytes may be NULL) the algorithmic
  * bytes those launches read and wrote: 8 B per unknown for every field in

@@ -105,7 +105,9 @@ int bicg_run(excmg_ctx* ctx, int n, int bc_kind, const double* b, double* x, dou
     // 64^3.  The node words of the first take the place of r and q, so that it needs no
     // more memory than launched kernels do (three vectors shadow-elided, five in full)
     // and no budget and no earlier call decides between them.
-    const bool resident = fused && shadow == nullptr && resident_ctas(n, 0) > 0;
+    // (Operator timing has launches to time above 64^3, where it always had.)
+    const bool timed = ctx->profile && n > kPersistentMaxN;
+    const bool resident = fused && shadow == nullptr && resident_ctas(n, 0) > 0 && !timed;
     const bool persistent = resident || (fused && shadow != nullptr && n <= kPersistentMaxN);
     double* r = resident ? nullptr : ctx_buffer(ctx, "bicg_r", bytes, &st);
     double* rs = (st || elide) ? nullptr : ctx_buffer(ctx, "bicg_rs", bytes, &st);

@@ -120,3 +120,27 @@ def test_given_shadow_that_is_the_residual(n, schedule):
     fields = 4 * 3 if schedule == "separate" else 3 + 3 * 7
     assert moved["same"] == fields * 8.0 * (n - 1) ** 3
     assert moved["one node off"] == moved["same"] + 4 * 8.0 * (n - 1) ** 3
+
+
+@pytest.mark.parametrize("n", [65, 81, 82])
+@pytest.mark.parametrize("schedule", ["separate", "fused"])
+def test_operator_timing_has_launches_above_64(n, schedule):
+    """Every iteration's operator launch is timed from 65^3 on, also where the
+    call runs on chip without timing; the iterates are those of either path within
+    the bound of the repository's fixed-iteration comparisons."""
+    b = dev(P.random_field(n, 88))
+    got = []
+    for timed in (False, True):
+        ctx = B.Context(DEV)
+        ctx.set_schedule(schedule)
+        ctx.profile(timed)
+        x = torch.zeros((n + 1,) * 3, dtype=torch.float64, device=DEV)
+        it, _, _ = B.bicg_solve(B.Level(n, 1, ctx), b, x, 0.0, 7)
+        assert it == 7
+        ms, launches, moved = ctx.profile_read(n)
+        assert launches == (7 if timed else 0)
+        if timed:
+            fields = 7 * 3 if schedule == "separate" else 3 + 6 * 7
+            assert ms > 0 and moved == fields * 8.0 * (n - 1) ** 3
+        got.append(x.cpu().numpy())
+    assert rel_max(got[1], got[0]) <= 1e-10
