@@ -408,25 +408,26 @@ struct excmg_batch {
     int next_id = 0;
     std::vector<Instance*> live;
     std::vector<Instance*> finished;
-    // per-slot Bi-CG states of the cooperative launches (device, pinned host)
+    // per-slot Bi-CG states: of the cooperative launches on the device; what every
+    // launch left, in pinned host memory
     BatchState* d_states = nullptr;
     BatchState* h_states = nullptr;
     double* d_norms = nullptr;   // per-slot norms
     double* h_norms = nullptr;
     int inner_chunk = 256;       // iterations per cooperative launch
-    int launched_rounds = 16;    // iterations per launched-mode group launch
+    int launched_rounds = 16;    // iterations enqueued for a launched-mode member at a time
     std::string last_error;
     long long launches = 0;
     excmg_batch_profile prof{};
-    // launched mode: a Bi-CG state and a partial-sum array per slot, and a
-    // pinned host copy of the states
+    // on-chip launches and launched mode: a Bi-CG state and a partial-sum array
+    // per slot, and a pinned host copy of the states
     BicgState* d_bstate = nullptr;
     BicgState* h_bstate = nullptr;
     double* d_bpart = nullptr;
     std::vector<int> free_slots;
-    // One cooperative launch per level group (instances of one precision at
-    // one grid size), each on its own stream with its own tables, partial
-    // sums, barrier and counters, harvested as soon as it completes.
+    // One launch under way: a member on chip or in launched mode, or a level group of
+    // correction solves (instances at one grid size) in a cooperative kernel, with
+    // its own stream, tables, partial sums, barrier and counters, harvested as soon as it completes.
     struct Group {
         cudaStream_t stream = nullptr;
         cudaEvent_t start = nullptr, done = nullptr;
@@ -1107,10 +1108,9 @@ int excmg_batch_submit(excmg_batch* b, int n_finest, int n_coarsest, int bc_kind
 // Advance the live instances: take back every group launch that has
 // completed, run the per-instance steps of every instance not on the GPU
 // (level set-up, direct solves, FP64 true residuals and the decisions of
-// Alg. 1 they drive), start one cooperative launch per level group of
-// instances ready for Bi-CG iterations (instances of one precision at one
-// grid size, each group on its own stream), then wait for at least one
-// running group.  *n_live receives the number of instances still running.
+// Alg. 1 they drive), start the launches of those ready for Bi-CG iterations,
+// then wait for at least one that is running.  *n_live receives the number of
+// instances still running.
 int excmg_batch_step(excmg_batch* b, int* n_live) {
     if (!b) return EXCMG_ERR_ARG;
     const double t_enter = now_s();
@@ -1220,35 +1220,17 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
                 // a Bi-CG call of Alg. 1's WHILE loop: x = u, r_0 = the true
                 // residual just formed with its copies r*_0 = p_0 = p*_0,
                 // rho_0 = (r_0, r_0); stop at ||r|| <= eps ||f_h||
-                BatchState& hs = b->h_states[slot];
-                hs = BatchState{};
-                hs.rho = b->h_norms[k];   // (r_0, r_0) exactly as summed
-                hs.rr = b->h_norms[k];
-                hs.tol = level_eps(in, l) * in->fnorm;
-                hs.max_iter = cap;
-                hs.done = 0;
-                hs.status = kRunning;
-                // h_states is pinned: the slot's state is not touched again
-                // before its group launch has completed
-                if (e == cudaSuccess)
-                    e = cudaMemcpyAsync(b->d_states + slot, b->h_states + slot, sizeof(BatchState),
-                                        cudaMemcpyHostToDevice, s);
-                {
-                    // the same call in the single solver's state layout
-                    BicgState& bs = b->h_bstate[slot];
-                    bs = BicgState{};
-                    bs.rho = b->h_norms[k];
-                    bs.rr = b->h_norms[k];
-                    bs.bnorm = in->fnorm;
-                    bs.tol = level_eps(in, l);
-                    bs.max_iter = cap;
-                    bs.status = kRunning;
-                    in->launched_k = 0;
-                    in->dir_in_p2 = false;
-                    if (e == cudaSuccess)
-                        e = cudaMemcpyAsync(b->d_bstate + slot, b->h_bstate + slot, sizeof(BicgState),
-                                            cudaMemcpyHostToDevice, s);
-                }
+                BicgState& bs = b->h_bstate[slot];   // (pinned, and not touched again before the launch has completed)
+                bs = BicgState{};
+                bs.rho = b->h_norms[k];   // (r_0, r_0) exactly as summed
+                bs.rr = b->h_norms[k];
+                bs.bnorm = in->fnorm;
+                bs.tol = level_eps(in, l);
+                bs.max_iter = cap;
+                bs.status = kRunning;
+                in->launched_k = 0;
+                in->dir_in_p2 = false;
+                e = cudaMemcpyAsync(b->d_bstate + slot, b->h_bstate + slot, sizeof(BicgState), cudaMemcpyHostToDevice, s);
             } else {
                 // FP32 correction solve on A e = r / ||r||
                 in->scale = rn;
