@@ -188,3 +188,42 @@ def test_small_entries_beside_large_ones(n, bc_kind):
     tap, eps = np.ldexp(np.longdouble(1), -55), np.ldexp(np.longdouble(1), -53)
     bound = a0 * a1 * 144 * tap + 64 * eps * (a0 * np.abs(v) + a1 * ((1 + beta) * np.abs(v) + a0 * np.abs(q0)))
     assert float((off / bound).max()) <= 1.0
+
+
+@pytest.mark.parametrize("n,bc_kind", [(54, 1), (67, 2), (81, 1)])
+def test_elided_bits_with_vectors_in_shared_memory(n, bc_kind):
+    """Six and eight nodes per thread keep x, r*, p* in shared memory; the elided
+    form has no r*, p* there and gives the same bits."""
+    b, x0 = dev(P.random_field(n, 305)), dev(P.random_field(n, 306) * 0.1)
+    got = []
+    for mode in ("full", "elided"):
+        ctx = B.Context()
+        ctx.set_shadow_mode(mode)
+        x = x0.clone()
+        got.append((x, B.bicg_solve(B.Level(n, bc_kind, ctx), b, x, 0.0, 40)))
+    assert got[0][1] == got[1][1] and torch.equal(got[0][0], got[1][0])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_eighty_cubed_alone_and_in_a_batch(precision):
+    """The largest on-chip grid of a cascade (80 = 5 * 16, eight nodes per thread), also
+    as a batch member: the finest level's residual, formed again here, meets the
+    tolerance (1e-3 for the two ways of forming it), and in FP64 the two agree within the
+    1e-9 of a full solve."""
+    n, nc, kind, tol = 80, 5, 2, 1e-8
+    f, g1, g2 = (dev(a) for a in P.exp_sum().data(n, kind))
+    uh = torch.empty((n + 1,) * 3, dtype=torch.float64, device=DEV)
+    ut, stats = B.excmg_solve(n, nc, kind, f, g1, g2, tol, u_h_out=uh, return_stats=True, precision=precision)
+    assert all(s["relres"] <= tol and not s["stagnated"] for s in stats[2:])
+    lvl = B.Level(n, kind)
+    fh = B.excmg_assemble_rhs(lvl, n, f, g1, g2)
+    assert float((fh - B.stencil_apply(lvl, uh)).norm() / fh.norm()) <= tol * (1 + 1e-3)
+    batch = B.Batch(max_instances=2)
+    ids = [batch.submit(n, nc, kind, f, g1, g2, tol, precision=precision) for _ in range(2)]
+    batch.run()
+    for k, u in ids:
+        q = batch.query(k)
+        assert q["status"] == 0 and all(s["relres"] <= tol for s in q["stats"][2:])
+        assert torch.equal(u, ids[0][1])
+        if precision == "fp64":
+            assert float((u - ut).abs().max()) <= 1e-9 * float(ut.abs().max())
