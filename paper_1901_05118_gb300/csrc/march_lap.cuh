@@ -270,6 +270,7 @@ __device__ __forceinline__ double lap_march(const MarchArrays& a, int n, int sig
         }
         if (kStep && !kElide) {
             // the same bits in: the same bits out, without another FP64 instruction
+            // (always so in the calls that come here; compared on principle, as in resident.cuh)
             long long diff = 0;
 #pragma unroll
             for (int s = 0; s < 2; ++s) {

@@ -47,9 +47,12 @@ int resident_ctas(int n, int max_ctas) {
 int resident2d_ctas(int n) { return n > kPersistentMaxN2d ? 0 : resident_geometry_cached(2, n, device_sms()).ctas; }
 
 // CTAs of a grid in the batch engine: fewer than a single solve takes, so that several instances run side by
-// side, and a number that depends on the grid alone (the sums do, too).  32^3 on 16 CTAs takes about 1.5
-// times as long per iteration as on its own 64, and nine fit beside each other.  (64^3 on 72 CTAs: 18 against
-// 11 us per iteration; eight mixed requests then take 74 instead of 50 ms, as the last one waits for itself.)
+// side, and a number that depends on the grid alone (the sums do, too).  The on-chip levels of a cascade are
+// 16, 20, 24, 28, 32, 40, 48, 56, 64 and 80 (c 2^k, c = 4 .. 8); only between these does it matter where the lines lie.
+// Eight first-kind requests on 32^3: 12.7 ms on 16 CTAs, 17.7 on 72 (two: 6.4, 4.5; nine fit beside each other);
+// 40^3 does not fit on 16: 29.6 ms on 72, 48.8 on all SMs; 48^3 54.0 and 76.0 (one alone: 15.0, 12.4); 56^3 116
+// on 72 and 125 on all (two: 32.4, 33.2), not taken so far; 64^3 74 ms on 72 against 50 for eight mixed requests,
+// as the last one waits for itself; 80^3 needs all.
 int resident_batch_limit(int n) { return n <= 32 ? 16 : n <= 52 ? 72 : 0; }
 
 namespace {

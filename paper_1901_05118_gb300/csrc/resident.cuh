@@ -39,7 +39,9 @@
 // bit for bit where p* = p (march_fx.cuh), so q serves both; r* and p* are
 // updated entry by entry, with the primal result reused where the operands
 // of a thread agree bit for bit; the other case is kept out of the FP64 pipe's
-// way (opaque in reduce.cuh).  kElide: r*, p* are not kept (the same bits).
+// way (opaque in reduce.cuh).  From such a start they always agree: the
+// comparison is there on principle, so that the full mode's r*, p* are what Alg. 2 makes of
+// their own values.  kElide: r*, p* are not kept (the same bits).
 //
 // DIM = 2: the 2D problem's 13-point rows (excmg2d.cu), with the second axis in
 // the place of z and no third one.

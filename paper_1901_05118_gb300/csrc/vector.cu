@@ -186,7 +186,8 @@ bicg_sigma_kernel(const double* __restrict__ ps, const double* __restrict__ q, s
 // once; a thread that meets a differing entry continues with separate sums
 // from the identical partial sums it has so far.  FP64 issue is scarce on
 // GB300: this saves two of the five FMAs per entry.
-// kOneQ: A^T p* is A p bit for bit and read once, from q.
+// kOneQ: A^T p* is A p bit for bit and read once, from q (r* is r then, too;
+// compared on principle, as in resident.cuh).
 template <int kLd, bool kOneQ>
 __global__ void __launch_bounds__(kVecThreads)
 bicg_update_kernel(double* __restrict__ x, const double* __restrict__ p, double* __restrict__ r,
