@@ -166,7 +166,7 @@ __device__ __noinline__ bool root_at_most(double a, double b) { return sqrt(a) <
 // it, A p kept fewer bits.  The error of the iterates against 64 bits after 48
 // to 96 iterations on 16^3 .. 32^3 (geometric means of 16 right-hand sides) was then 1.57 times the
 // per-node form's (0.75 to 2.5 by grid and kind), it is 0.73 times now (0.43 to 0.99), for
-// 10.8 instead of 10.7 us per iteration on 64^3, 0.7 % of a 32^3 solve.
+// 0.1 of 10.7 us per iteration on 64^3 and 0.7 % of a 32^3 solve.
 __device__ __forceinline__ long long to_brick(double v, int E) {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
     const unsigned e = (hi >> 20) & 0x7FFu;

@@ -1,6 +1,6 @@
-"""The resident Bi-CG kernels (grids up to 64^3, every vector on chip) at the
+"""The resident Bi-CG kernels (grids up to 81^3, every vector on chip) at the
 edges of their brick decompositions: smallest and largest grids, bricks cut
-short by the boundary, one to four nodes per thread, a call longer than one
+short by the boundary, one to eight nodes per thread, a call longer than one
 launch, the FP32 correction solves."""
 import numpy as np
 import pytest
