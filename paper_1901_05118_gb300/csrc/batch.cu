@@ -594,29 +594,6 @@ SmPlaces places(const excmg_batch* b) {
     return p;
 }
 
-// The group record's stream, events and fixed tables (made once).
-int group_init(excmg_batch* b, excmg_batch::Group& g) {
-    if (g.stream) return EXCMG_OK;
-    const size_t mi = (size_t)b->max_instances;
-    bool ok = cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreate(&g.start) == cudaSuccess && cudaEventCreate(&g.done) == cudaSuccess &&
-              cudaMalloc(&g.d_inst, mi * sizeof(BatchInst)) == cudaSuccess &&
-              cudaMalloc(&g.d_unit_begin, mi * sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&g.d_chunk_begin, mi * sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&g.d_active, sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&g.d_rounds, sizeof(int)) == cudaSuccess &&
-              cudaMallocHost(&g.h_active, 2 * sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&g.d_barrier, 4 * sizeof(unsigned int)) == cudaSuccess &&
-              cudaMalloc(&g.slots, resident_slot_bytes()) == cudaSuccess &&
-              cudaMemsetAsync(g.slots, 0, resident_slot_bytes(), g.stream) == cudaSuccess;
-    if (!ok) {
-        cudaGetLastError();
-        return bfail(b, EXCMG_ERR_OOM, "batch group buffers");
-    }
-    g.h_rounds = g.h_active + 1;
-    return EXCMG_OK;
-}
-
 void group_free(excmg_batch::Group& g) {
     if (g.stream) cudaStreamSynchronize(g.stream);
     cudaFree(g.d_inst);
@@ -635,11 +612,42 @@ void group_free(excmg_batch::Group& g) {
     g = excmg_batch::Group{};
 }
 
+// What a group record needs for the kind of launch it is to run, made once: its
+// stream and events, the tables of a cooperative launch, the slot words of an on-chip
+// one (of which at most ten run at a time: 15 CTAs on the smallest level).
+enum GroupUse { kUseMember, kUseCooperative, kUseOnChip };
+int group_init(excmg_batch* b, excmg_batch::Group& g, GroupUse use) {
+    const size_t mi = (size_t)b->max_instances;
+    bool ok = true;
+    if (!g.h_active)
+        ok = cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreate(&g.start) == cudaSuccess && cudaEventCreate(&g.done) == cudaSuccess &&
+             cudaMallocHost(&g.h_active, 2 * sizeof(int)) == cudaSuccess;
+    if (ok && use == kUseCooperative && !g.d_barrier)
+        ok = cudaMalloc(&g.d_inst, mi * sizeof(BatchInst)) == cudaSuccess &&
+             cudaMalloc(&g.d_unit_begin, mi * sizeof(int)) == cudaSuccess &&
+             cudaMalloc(&g.d_chunk_begin, mi * sizeof(int)) == cudaSuccess &&
+             cudaMalloc(&g.d_active, sizeof(int)) == cudaSuccess &&
+             cudaMalloc(&g.d_rounds, sizeof(int)) == cudaSuccess &&
+             cudaMalloc(&g.d_barrier, 4 * sizeof(unsigned int)) == cudaSuccess;
+    if (ok && use == kUseOnChip && !g.slots) {
+        ok = cudaMalloc(&g.slots, resident_slot_bytes()) == cudaSuccess &&
+             cudaMemsetAsync(g.slots, 0, resident_slot_bytes(), g.stream) == cudaSuccess;
+    }
+    if (!ok) {
+        cudaGetLastError();
+        group_free(g);   // (not busy: nothing of it is in use)
+        return bfail(b, EXCMG_ERR_OOM, "batch group buffers");
+    }
+    g.h_rounds = g.h_active + 1;
+    return EXCMG_OK;
+}
+
 // One cooperative launch of up to b->inner_chunk Bi-CG iterations for the
 // instances `list` (one precision, one grid size) on group record g, with
 // `ctas` CTAs, after the context stream's state uploads.
 int launch_group(excmg_batch* b, excmg_batch::Group& g, const std::vector<Instance*>& list, int ctas, int cand) {
-    int st = group_init(b, g);
+    int st = group_init(b, g, kUseCooperative);
     if (st) return st;
     std::vector<BatchInst> tab;
     std::vector<int> ub, cb;
@@ -719,7 +727,7 @@ bool launched_level(const Instance* in) { return in->prec == EXCMG_PRECISION_FP6
 // iterations of its current call.  Its node words lie in the instance
 // (node_words), so a call goes on with any group record and needs no further memory.
 int launch_resident(excmg_batch* b, excmg_batch::Group& g, Instance* in, int ctas) {
-    int st = group_init(b, g);
+    int st = group_init(b, g, kUseOnChip);
     if (st) return st;
     const int N = in->nc << in->level;
     cudaStream_t s = g.stream;
@@ -754,7 +762,7 @@ int launch_resident(excmg_batch* b, excmg_batch::Group& g, Instance* in, int cta
 }
 
 int launch_member(excmg_batch* b, excmg_batch::Group& g, Instance* in) {
-    int st = group_init(b, g);
+    int st = group_init(b, g, kUseMember);
     if (st) return st;
     cudaStream_t s = g.stream;
     const int K = b->launched_rounds, N = in->nc << in->level;
@@ -1265,9 +1273,11 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
         for (auto& kv : ready)
             order.push_back({-(long long)kv.second.size() * node_count(kv.first.second), kv.first});
         std::sort(order.begin(), order.end());
-        auto free_group = [&]() -> excmg_batch::Group& {
-            for (auto& g : b->groups)
-                if (!g.busy) return g;
+        // a record that is free, one that has what the launch needs first
+        auto free_group = [&](GroupUse use) -> excmg_batch::Group& {
+            for (int any = 0; any < 2; ++any)
+                for (auto& g : b->groups)
+                    if (!g.busy && (any || (g.slots != nullptr) == (use == kUseOnChip))) return g;
             b->groups.emplace_back();
             return b->groups.back();
         };
@@ -1275,7 +1285,7 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
         // for a step in which they do
         auto start_on_chip = [&](Instance* in, int ctas) -> bool {
             if (!on_chip_fits(places(b), ctas)) return false;
-            st = launch_resident(b, free_group(), in, ctas);
+            st = launch_resident(b, free_group(kUseOnChip), in, ctas);
             return true;
         };
         // one cooperative launch for a group's FP32 correction solves
@@ -1287,7 +1297,7 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
             const int ctas = coop_share(places(b), want);
             if (ctas == 0) return false;
             // (not the candidate's shape: not a tuning sample)
-            st = launch_group(b, free_group(), list, ctas, ctas == want ? cand : -1);
+            st = launch_group(b, free_group(kUseCooperative), list, ctas, ctas == want ? cand : -1);
             return true;
         };
         auto on_chip = [&](int n) { return resident_ctas(n, resident_batch_limit(n)); };
@@ -1321,7 +1331,7 @@ int excmg_batch_step(excmg_batch* b, int* n_live) {
             } else {
                 for (Instance* in : list) {
                     if (ctas > 0) (void)start_on_chip(in, ctas);
-                    else st = launch_member(b, free_group(), in);
+                    else st = launch_member(b, free_group(kUseMember), in);
                     if (st) return st;
                 }
             }
